@@ -120,6 +120,7 @@ struct Axis {
   int grid_dense = 0, grid_dense_small = 0;
   unsigned char* tc_t[2] = {nullptr, nullptr};  // split tensor-core operands of T, T^H (ffx_tc.cu)
   unsigned char* bf_t[2] = {nullptr, nullptr};  // FFX_TC_BF16: the BF16 operand blocks (ffx_tc16.cu)
+  unsigned char* pl_t[2] = {nullptr, nullptr};  // ... and those of the passes over planes (ffx_planes.cu)
   unsigned char* ft_ts = nullptr;                 // N = 64: T's row-block slices for the fused tensor-core launch
   float2* img[2] = {nullptr, nullptr};                      // lines <= 64: shared-memory images of T, T^H
 };
@@ -150,7 +151,7 @@ struct ffx_plan_s {
   Axis axis[3];
   int order[3] = {0, 1, 2};  // forward pass order
   // every axis has BF16 operand blocks and the driver makes TMA maps: large
-  // forward calls may run as a BF16 chain (ffx_tc16.cu), whose order -- the
+  // forward calls may run as a BF16 chain (ffx_planes.cu), whose order -- the
   // last axis first -- is then the plan's forward order
   int chain_bf16 = 0;
   void* tables = nullptr;
@@ -379,28 +380,30 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
     // split TF32
     const bool tm64 = ax.N == 64 && !acc && !grad && items <= 4 * grid;
     if (io) {
-      if (!ax.bf_t[adjoint ? 1 : 0] || tm64 || grad)
+      if (!ax.pl_t[adjoint ? 1 : 0] || tm64 || grad)
         return fail(FFX_EUNSUPPORTED, "internal: a BF16 chain pass of axis %d without the BF16 kernel", j);
       d.in_bf = io->in_bf;
       d.out_bf = io->out_bf;
       d.bf_plane = io->plane;
       d.oouter = 1;
       d.oinner = outer;
-    } else if (ax.bf_t[0] && !tm64 && !grad && inner == 1) {
+    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
       // cores' layout instead of converting them on the way
       int rc = ensure_ws(p, kWsSplit, batch);
       if (rc) return rc;
       const int64_t plane = batch * p->M;
-      e = launch_bf16_split(in, (uint32_t*)p->ws[kWsSplit], plane, plane, d.unsplit, p->sms, stream);
+      e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[kWsSplit], plane, plane, d.unsplit, p->sms, stream);
       if (e != cudaSuccess) return cuda_fail(e, "BF16 split of a pass input");
       ++p->launches;
       d.in_bf = (const uint32_t*)p->ws[kWsSplit];
       d.bf_plane = plane;
       d.in = nullptr;
     }
-    if (ax.bf_t[0] && !tm64)
+    if (d.in_bf)
+      e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
+    else if (ax.bf_t[0] && !tm64)
       e = launch_dense_bf16(d, ax.bf_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
     else
       e = launch_dense_tc(d, ax.tc_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
@@ -522,7 +525,7 @@ bool bf16_chain_ok(const ffx_plan_s* p, int64_t batch, const void* in, const voi
 // Every axis has the BF16 blocks of T_j^H too (adjoint chains).
 bool bf16_adjoint_ok(const ffx_plan_s* p) {
   for (int r = 0; r < p->ndim; ++r)
-    if (!p->axis[r].bf_t[1]) return false;
+    if (!p->axis[r].pl_t[1]) return false;
   return true;
 }
 
@@ -540,7 +543,7 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
   const int64_t plane = batch * p->M;
   const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
   const unsigned rec = trace_begin(p, s);
-  cudaError_t e = launch_bf16_split(in, (uint32_t*)p->ws[1], plane, plane, unsplit, p->sms, s);
+  cudaError_t e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit, p->sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the input");
   ++p->launches;
   trace_end(p, s, rec);
@@ -572,8 +575,8 @@ int chain_bf16_adjoint(ffx_plan_s* p, const float2* field, const float* grad, in
   const int64_t plane = batch * p->M;
   const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
   const unsigned rec = trace_begin(p, s);
-  cudaError_t e = launch_bf16_split_grad(field, grad, grad_shared, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit,
-                                         p->sms, s);
+  cudaError_t e = launch_plane_split(field, grad, grad_shared, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit,
+                                     p->sms, s);
   if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the gradient factors");
   ++p->launches;
   trace_end(p, s, rec);
@@ -1220,6 +1223,7 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
       if (dense_tc_supported(p->axis[j].N) && p->axis[j].T && (form == FFX_FORM_AUTO || form == FFX_FORM_TC)) {
         tbytes += 2 * dense_tc_t_bytes(p->axis[j].N) + (p->axis[j].N == 64 ? fused_tc_slice_bytes() : 0);
         if (bf16_ops && dense_bf16_supported(p->axis[j].N)) tbytes += 2 * dense_bf16_t_bytes(p->axis[j].N);
+        if (bf16_ops && plane_pass_supported(p->axis[j].N)) tbytes += 2 * plane_t_bytes(p->axis[j].N);
       }
     e = cudaMalloc(&p->tc_mem, tbytes);
     if (e != cudaSuccess) {
@@ -1266,6 +1270,15 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           e = launch_bf16_build_t(ax.T, ax.bf_t[0], ax.N, s);
           if (e == cudaSuccess) e = launch_bf16_build_t(ax.TH, ax.bf_t[1], ax.N, s);
           if (e == cudaSuccess) e = dense_bf16_prepare();
+        }
+        if (e == cudaSuccess && bf16_ops && plane_pass_supported(ax.N)) {
+          for (int q = 0; q < 2; ++q) {
+            ax.pl_t[q] = tcur;
+            tcur += plane_t_bytes(ax.N);
+          }
+          e = launch_plane_build_t(ax.T, ax.pl_t[0], ax.N, s);
+          if (e == cudaSuccess) e = launch_plane_build_t(ax.TH, ax.pl_t[1], ax.N, s);
+          if (e == cudaSuccess) e = plane_pass_prepare(ax.N);
         }
         if (e == cudaSuccess)
           e = dense_tc_prepare();
@@ -1331,9 +1344,9 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
       if (e != cudaSuccess) rc = cuda_fail(e, "tuning");
     }
   }
-  if (rc == FFX_OK && ndim >= 2 && dense_bf16_chain_supported()) {
+  if (rc == FFX_OK && ndim >= 2) {
     bool all = true;
-    for (int j = 0; j < ndim; ++j) all = all && p->axis[j].bf_t[0] != nullptr;
+    for (int j = 0; j < ndim; ++j) all = all && p->axis[j].pl_t[0] != nullptr;
     if (all) {
       p->chain_bf16 = 1;
       for (int r = 0; r < ndim; ++r) p->order[r] = ndim - 1 - r;

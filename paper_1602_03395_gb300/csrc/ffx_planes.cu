@@ -1,0 +1,917 @@
+// Passes of a BF16 chain (and per-axis BF16 passes over contiguous lines) on
+// the tensor cores: the per-axis map of lines of N points (N a multiple of 32
+// from 64 up to 1024), input as BF16 planes, tcgen05 kind::f16 products
+// accumulated in FP32 in tensor memory.
+//
+// Planes.  A field is a head plane bf16(v) and a tail plane bf16(v - bf16(v)),
+// each 4 bytes a point, in which every 16 consecutive points keep their 16
+// real parts and then their 16 imaginary parts.  A K step of a product (16
+// values, 32 bytes of an operand row) is then all real or all imaginary parts
+// of 16 points, and the complex map needs T's real and imaginary parts once
+// each instead of the 2 x 2 blocks [[x, -y], [y, x]] of interleaved pairs:
+//
+//   D_re += X_re T_re + (-X_im) T_im,   D_im += X_re T_im + X_im T_re
+//
+// (the instruction descriptor negates the first operand), each product as
+// head x [head; tail] of T into the accumulator pair [D1 | D2] (one product of
+// N = 2 RB columns) and tail x head into D2, so that the large accumulator D1
+// takes 2N/16 steps as before.  The dropped tail x tail term and the tails'
+// own rounding leave ~2^-17 per operand pair.
+//
+// Items are (128 lines, RB complex outputs): tensor-memory lane = line, and
+// the four accumulators of an item (D1, D2 of the real and of the imaginary
+// parts) fill 4 RB of the 512 columns.  What bounds a streaming pass is the
+// copies from L2 into shared memory and the tensor cores' own operand reads.
+// With T stored once, a chunk of 32 points costs 32 KB of X and RB x 256 B of
+// T for 12 RB/128 x 128 clocks of products: 64 KB per 1536 clocks at RB = 128,
+// against 64 KB per 768 clocks of the interleaved form with 64 complex outputs
+// an item (the kernel this one replaced: 0.095 ms per 256^3 pass).  For N =
+// 64, 96 and 128 (RB = N) T is resident in shared memory and only X streams.
+//
+// One persistent block of 384 threads per SM, warp-specialised.
+//  * warp 0 (one thread): copies.  Per chunk of 32 points, once the products
+//    of the chunk that had its stage have freed it: the X tile (head and tail,
+//    128 lines x 64 values, one 3-D TMA tile with 128-byte swizzle) and, when
+//    streaming, T's chunk (one bulk copy), on the stage's "full" barrier.
+//  * warp 1 (one thread): products.  Per chunk first those of the real
+//    accumulators, then those of the imaginary ones: the real half of an item
+//    is complete half a chunk before the imaginary one, and the next item's
+//    real half starts while the imaginary half is read back, so one set of
+//    accumulators keeps the tensor cores busy.  (RB = 64 has room for two.)
+//  * warps 4-11 (epilogue): warp w reads tensor-memory lanes 32 (w % 4) .. +31
+//    and half of the outputs; it moves an accumulator half into registers,
+//    releases it, and then writes it: planes (real and imaginary parts are
+//    separate runs, so each half is written on its own), complex64, densities,
+//    or densities summed over the batch in registers.
+// Every wait is bounded; one that runs out sets the block's abort flag, the
+// block drains its own copies and products, frees its tensor memory, counts
+// the error and exits.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <cstring>
+
+#include "ffx_internal.h"
+#include "ffx_tcgen05.cuh"
+#include "ffx_tma.h"
+
+namespace ffx {
+
+namespace {
+
+using namespace tc;
+
+constexpr int PL = 128;                 // lines per item = MMA M = tensor-memory lanes
+constexpr int PKC = 32;                 // points per chunk: two K steps of 16, real and imaginary
+constexpr int PXPART = PL * PKC * 4;    // 16 KB: one plane of an X tile (128 lines x 64 values)
+constexpr int PX = 2 * PXPART;          // head and tail
+constexpr int PTHREADS = 384;           // copies, products, two idle warps, eight epilogue warps
+constexpr int PEPIW = 8;                // epilogue warps
+constexpr int PMAXST = 5;
+
+// T's chunk: head rows, then tail rows, each RB rows of 128 bytes (32 real
+// parts, 32 imaginary parts) in the 128-byte-swizzled K-major layout
+__host__ __device__ constexpr int ppart(int rb) { return rb * PKC * 4; }
+__host__ __device__ constexpr int ptchunk(int rb) { return 2 * ppart(rb); }
+// outputs per item: the whole line up to 128 points, else 128, or 96 for 192
+__host__ __device__ constexpr int prow_block(int N) { return N <= 128 ? N : (N % 128 == 0 ? 128 : 96); }
+// stages: T resident (N = RB) leaves the rest to X tiles
+__host__ __device__ constexpr int pstages(int rb, bool res) {
+  return res ? (rb == 64 ? 5 : rb == 96 ? 4 : 3) : (rb == 96 ? 4 : 3);
+}
+__host__ __device__ constexpr int psmem(int rb, bool res) {
+  // + 1 KB to start the swizzled tiles on a 1024-byte boundary
+  return (res ? (rb / PKC) * ptchunk(rb) : 0) + pstages(rb, res) * (PX + (res ? 0 : ptchunk(rb))) + 1024;
+}
+static_assert(psmem(128, true) <= 226 * 1024 && psmem(128, false) <= 226 * 1024 && psmem(96, true) <= 226 * 1024 &&
+                  psmem(96, false) <= 226 * 1024 && psmem(64, true) <= 226 * 1024,
+              "shared memory");
+
+// the instruction descriptor's "negate A" bit
+constexpr uint32_t kNegA = 1u << 13;
+
+__device__ __forceinline__ uint32_t bf2(float lo, float hi) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h);
+}
+__device__ __forceinline__ float bf_lo(uint32_t h) { return __uint_as_float(h << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t h) { return __uint_as_float(h & 0xffff0000u); }
+
+// Advance a store pointer.  The compiler would otherwise keep all multiples
+// of the stride in registers across the items (and spill).
+template <class T>
+__device__ __forceinline__ void advance(T*& o, int64_t by) {
+  o += by;
+  asm volatile("" : "+l"(o));
+}
+
+// Contiguous lines: v is 16 bytes of this lane's line at o, w the next 16.  The
+// lanes of a pair swap, so that each of the two stores covers whole 32-byte
+// sectors: first the even lane's line (its lane the first half), then the odd
+// lane's (lanes storing their own 16 bytes alone left every sector half
+// written: 0.0045 ms more per 2^22 points of a field).  other: the pair's
+// other line has o at o + other bytes; even/odd lane as `odd` says.
+__device__ __forceinline__ void store_pair(void* o, int64_t other, bool odd, bool self, bool peer, float4 v, float4 w) {
+  const float4 send = odd ? v : w;
+  float4 r;
+  r.x = __shfl_xor_sync(0xffffffffu, send.x, 1);
+  r.y = __shfl_xor_sync(0xffffffffu, send.y, 1);
+  r.z = __shfl_xor_sync(0xffffffffu, send.z, 1);
+  r.w = __shfl_xor_sync(0xffffffffu, send.w, 1);
+  char* const p = static_cast<char*>(o);
+  if (odd ? peer : self) *reinterpret_cast<float4*>(odd ? p + other + 16 : p) = odd ? r : v;
+  if (odd ? self : peer) *reinterpret_cast<float4*>(odd ? p + 16 : p + other) = odd ? w : r;
+}
+
+// What a pass writes: planes (inside a chain), the complex field, densities, or
+// densities summed over the batch.
+enum POut { kOutPlanes = 0, kOutComplex = 1, kOutDensity = 2, kOutSum = 3 };
+constexpr int kPOuts = 4;
+
+// The products of one accumulator half [D1 | D2] (real or imaginary parts, at
+// tensor-memory column d) with one chunk: X's tile at xs (head plane, then
+// tail plane: K step ks has X's real parts at 64 ks and its imaginary parts at
+// 64 ks + 32 bytes of the rows), T's rows at t2 (heads and tails, both columns
+// sets) and t1 (heads alone), real parts at 32 ks and imaginary parts at 64 +
+// 32 ks.  The real half takes T's real parts with X's real ones and T's
+// imaginary parts with X's negated imaginary ones, the imaginary half the other
+// two.  CG: CTAs per product.  Called by the whole warp.
+template <int CG, int RB, bool IMAG>
+__device__ __forceinline__ void plane_half(uint32_t d, uint32_t xs, uint32_t t2, uint32_t t1, uint32_t id1,
+                                           uint32_t id2, bool first, bool unsplit) {
+  auto mma = [](uint32_t dd, uint32_t al, uint32_t bl, uint32_t id, uint32_t acc) {
+    if constexpr (CG == 2)
+      mma2_sw128(dd, al, bl, id, acc);
+    else
+      mma_sw128(dd, al, bl, id, acc);
+  };
+  constexpr uint32_t o0 = IMAG ? 64 : 0, o1 = IMAG ? 0 : 64, neg = IMAG ? 0u : kNegA;
+  const uint32_t x0 = desc_lo(xs), b2 = desc_lo(t2), b1 = desc_lo(t1);
+  if (unsplit) {
+#pragma unroll
+    for (uint32_t ks = 0; ks < 2; ++ks) {
+      mma(d, x0 + ks * 4, b1 + ks * 2 + o0 / 16, id1, (first && ks == 0) ? 0u : 1u);
+      mma(d, x0 + ks * 4 + 2, b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
+    }
+    return;
+  }
+#pragma unroll
+  for (uint32_t ks = 0; ks < 2; ++ks) {
+    mma(d, x0 + ks * 4, b2 + ks * 2 + o0 / 16, id2, (first && ks == 0) ? 0u : 1u);
+    mma(d, x0 + ks * 4 + 2, b2 + ks * 2 + o1 / 16, id2 | neg, 1u);
+    mma(d + RB, x0 + PXPART / 16 + ks * 4, b1 + ks * 2 + o0 / 16, id1, 1u);
+    mma(d + RB, x0 + PXPART / 16 + ks * 4 + 2, b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
+  }
+}
+
+// The epilogue warps of a block (warps 4-11): items first, first + step, ...;
+// item w covers line tiles (w / mtiles) * tiles_per_item + tile (this block's)
+// and row block w % mtiles.  accf: the accumulator halves' "complete" barriers,
+// release(half): the whole warp has read its part of a half.
+template <int RB, int OUT, class Release>
+__device__ __forceinline__ void plane_epilogue(const DenseArgs& a, int warp, int lane, uint32_t tmem, uint32_t accf,
+                                               int64_t first, int64_t step, int64_t my_items, int mtiles,
+                                               int tiles_per_item, int tile, int nb, bool unsplit,
+                                               volatile int* s_abort, const Release& release) {
+  constexpr int NBUF = RB == 64 ? 2 : 1;  // accumulator sets
+  constexpr int H = RB / 2;               // outputs per epilogue thread
+  constexpr bool ACC = OUT == kOutSum;
+  const int N = a.N;
+  const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
+  const int col0 = ((warp - 4) >> 2) * H;  // first of this warp's outputs
+  const int r = q * 32 + lane;            // line within the item
+  const uint32_t tlane = (uint32_t)(q * 32) << 16;
+  const int64_t inner = a.oinner;  // the output's decomposition
+  const int64_t per = a.oouter * a.oinner;
+  // planes: the even lane of a pair of neighbouring lines keeps its real part
+  // and sends the imaginary one, the odd lane the other way round
+  const bool odd = lane & 1;
+  const uint32_t sel_send = odd ? 0x5410u : 0x7632u;
+  const uint32_t sel_h = odd ? 0x3254u : 0x5410u, sel_l = odd ? 0x3276u : 0x7610u;
+  const int64_t pword = (lane & 16) + ((lane & 15) >> 1) + (odd ? 8 : 0) - lane;  // its word, relative to the line's own
+  float racc[ACC ? H : 1];
+  if (ACC) {
+#pragma unroll
+    for (int m = 0; m < H; ++m) racc[m] = 0.f;
+  }
+  int64_t sub = 0;
+  bool ok = true;
+  // an accumulator half (columns d .. d + RB and d + RB .. d + 2 RB), 16
+  // outputs at a time to take(first output, values); released once read
+  auto read_half = [&](int half, auto&& take) -> bool {
+    const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
+    const int64_t v = NBUF == 2 ? sub >> 1 : sub;
+    const int bar = 2 * buf + half;
+    // lane 0 polls; the outcome is the warp's (its tensor-memory loads need the whole warp)
+    bool got = true;
+    if (lane == 0) got = mbar_wait(accf + 8u * (uint32_t)bar, (uint32_t)(v & 1), s_abort);
+    if (__shfl_sync(0xffffffffu, got ? 1 : 0, 0) == 0) return false;
+    tc_fence_after();
+    const uint32_t d = tmem + tlane + (uint32_t)((2 * bar) * RB + col0);
+#pragma unroll
+    for (int j = 0; j < H; j += 16) {
+      uint32_t x[16], z[16];
+      tmem_ld16(d + (uint32_t)j, x);
+      tmem_ld16(d + (uint32_t)(RB + j), z);  // unsplit: not written, not used
+      tmem_wait_ld();
+      float y[16];
+#pragma unroll
+      for (int m = 0; m < 16; ++m) y[m] = unsplit ? __uint_as_float(x[m]) : __uint_as_float(x[m]) + __uint_as_float(z[m]);
+      take(j, y);
+    }
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) release(bar);
+    return true;
+  };
+#pragma unroll 1
+  for (int64_t it = 0; ok && it < my_items; ++it) {
+    const int64_t w = first + it * step;
+    const int64_t wt = w / mtiles;
+    const int n0 = (int)(w - wt * mtiles) * RB + col0;
+    const int64_t c = (wt * tiles_per_item + tile) * PL + r;
+    const bool valid = c < a.ncols;  // whole warps: the lines come in multiples of 32 where planes are written
+    const int64_t bo = c / per;      // realization (0 when accumulating)
+    const int64_t rho = c - bo * per;
+    const int64_t oo = rho / inner;
+    // (contiguous lines follow one another, across realizations too)
+    const bool pvalid = (c ^ 1) < a.ncols;
+    const int64_t other = odd ? -N : N;
+    const int64_t base = bo * a.M + oo * (int64_t)N * inner + (rho - oo * inner) + (int64_t)n0 * inner;
+    if constexpr (ACC) {
+#pragma unroll 1
+      for (int b = 0; b < nb; ++b, ++sub) {
+        auto add = [&](int j, const float* y) {
+#pragma unroll
+          for (int m = 0; m < 16; ++m) racc[j + m] += y[m] * y[m];
+        };
+        ok = read_half(0, add) && read_half(1, add);
+        if (!ok) break;
+      }
+      if (valid && ok) {
+        float* o = a.out_d + base;
+        if (inner == 1) {
+#pragma unroll
+          for (int m = 0; m < H; m += 4) {
+            float4 cur = *reinterpret_cast<float4*>(o + m);
+            cur.x += racc[m], cur.y += racc[m + 1], cur.z += racc[m + 2], cur.w += racc[m + 3];
+            *reinterpret_cast<float4*>(o + m) = cur;
+          }
+        } else {
+#pragma unroll
+          for (int m0 = 0; m0 < H; m0 += 8) {
+            float cur[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) cur[m] = o[m * inner];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) o[m * inner] = cur[m] + racc[m0 + m];
+            advance(o, 8 * inner);
+          }
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < H; ++m) racc[m] = 0.f;
+    } else if constexpr (OUT == kOutPlanes) {
+      // BF16 head and tail planes for the next pass of a chain: both halves in
+      // registers, then a lane pair exchanges (real, imaginary) parts, so that
+      // the even lane stores the pair's real parts and the odd lane its
+      // imaginary parts: a warp's store covers 128 consecutive bytes
+      float y[H], z[H];
+      ok = read_half(0, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) y[j + m] = v[m];
+      });
+      ok = ok && read_half(1, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) z[j + m] = v[m];
+      });
+      ++sub;
+      if (ok && valid) {
+        uint32_t* o = a.out_bf + base + pword;
+        // eight outputs at a time, step by step, so that their exchanges and
+        // stores overlap (one output after the other: 0.020 ms more per 256^3
+        // pass, the epilogue's latency on the critical path)
+#pragma unroll
+        for (int m0 = 0; m0 < H; m0 += 8) {
+          uint32_t h[8], l[8], x[8];
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            h[m] = bf2(y[m0 + m], z[m0 + m]);
+            l[m] = bf2(y[m0 + m] - bf_lo(h[m]), z[m0 + m] - bf_hi(h[m]));
+            x[m] = __byte_perm(h[m], l[m], sel_send);
+          }
+#pragma unroll
+          for (int m = 0; m < 8; ++m) x[m] = __shfl_xor_sync(0xffffffffu, x[m], 1);
+#pragma unroll
+          for (int m = 0; m < 8; ++m) {
+            o[m * inner] = __byte_perm(h[m], x[m], sel_h);
+            if (!unsplit) o[a.bf_plane + m * inner] = __byte_perm(l[m], x[m], sel_l);
+          }
+          advance(o, 8 * inner);
+        }
+      }
+    } else if constexpr (OUT == kOutComplex) {
+      // both halves in registers before the first store: the imaginary half is
+      // released without waiting for stores
+      float y[H], z[H];
+      ok = read_half(0, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) y[j + m] = v[m];
+      });
+      ok = ok && read_half(1, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) z[j + m] = v[m];
+      });
+      ++sub;
+      if (ok && inner == 1) {
+        float2* o = a.out_c + base;
+#pragma unroll
+        for (int m = 0; m < H; m += 4)
+          store_pair(o + m, other * (int64_t)sizeof(float2), odd, valid, pvalid,
+                     make_float4(y[m], z[m], y[m + 1], z[m + 1]),
+                     make_float4(y[m + 2], z[m + 2], y[m + 3], z[m + 3]));
+      } else if (ok && valid) {
+        float2* o = a.out_c + base;
+#pragma unroll
+        for (int m0 = 0; m0 < H; m0 += 8) {
+#pragma unroll
+          for (int m = 0; m < 8; ++m) o[m * inner] = make_float2(y[m0 + m], z[m0 + m]);
+          advance(o, 8 * inner);
+        }
+      }
+    } else {
+      float y[H];
+      float* o = a.out_d + base;
+      ok = read_half(0, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) y[j + m] = v[m] * v[m];
+      });
+      ok = ok && read_half(1, [&](int j, const float* v) {
+#pragma unroll
+        for (int m = 0; m < 16; ++m) y[j + m] += v[m] * v[m];
+      });
+      if (ok && inner == 1) {
+#pragma unroll
+        for (int m = 0; m < H; m += 8)
+          store_pair(o + m, other * (int64_t)sizeof(float), odd, valid, pvalid,
+                     make_float4(y[m], y[m + 1], y[m + 2], y[m + 3]),
+                     make_float4(y[m + 4], y[m + 5], y[m + 6], y[m + 7]));
+      } else if (ok && valid) {
+#pragma unroll
+        for (int m0 = 0; m0 < H; m0 += 8) {
+#pragma unroll
+          for (int m = 0; m < 8; ++m) o[m * inner] = y[m0 + m];
+          advance(o, 8 * inner);
+        }
+      }
+      ++sub;
+    }
+  }
+}
+
+// RB outputs per item, T resident (RES) or streamed.
+template <int RB, bool RES, int OUT>
+__global__ void __launch_bounds__(PTHREADS, 1)
+    plane_pass_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
+                      const __grid_constant__ CUtensorMap xmap) {
+  constexpr int NST = pstages(RB, RES);
+  constexpr int TCH = ptchunk(RB), TPART = ppart(RB);
+  constexpr int STAGE = PX + (RES ? 0 : TCH);
+  constexpr int NBUF = RB == 64 ? 2 : 1;  // accumulator sets
+  constexpr bool ACC = OUT == kOutSum;
+  extern __shared__ __align__(1024) unsigned char psm_raw[];
+  unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], t_bar;
+  __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_abort;
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int N = a.N;
+  const int mtiles = RES ? 1 : N / RB;
+  const int kchunks = N / PKC;
+  const int64_t items = ((a.ncols + PL - 1) / PL) * mtiles;
+  const int64_t my_items = (items - blockIdx.x + gridDim.x - 1) / gridDim.x;
+  if (my_items <= 0) return;
+  const int nb = ACC ? (int)a.batch : 1;
+  const bool unsplit = a.unsplit != 0;
+
+  if (warp == 1) tmem_alloc(&tmem_slot, 512);
+  if (tid == 0) {
+    for (int s = 0; s < NST; ++s) {
+      mbar_init(smem_u32(&full_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), 1);
+    }
+    mbar_init(smem_u32(&t_bar), 1);
+    for (int b = 0; b < 2 * NBUF; ++b) {
+      mbar_init(smem_u32(&accf_bar[b]), 1);
+      mbar_init(smem_u32(&acce_bar[b]), PEPIW);
+    }
+    mbar_init(smem_u32(&done_bar), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_abort = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  // T resident: its chunks first, then the stages
+  const uint32_t t_res = smem_u32(psm);
+  const uint32_t stages = t_res + (uint32_t)(RES ? (RB / PKC) * TCH : 0);
+
+  if (warp == 0) {
+    // ---------------- copies ----------------
+    if (lane == 0) {
+      const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
+      const uint32_t xbytes = unsplit ? (uint32_t)PXPART : (uint32_t)PX;
+      const uint32_t tbytes = unsplit ? (uint32_t)TPART : (uint32_t)TCH;  // unsplit: the head rows
+      if (RES) {
+        mbar_expect_tx(smem_u32(&t_bar), tbytes * (uint32_t)kchunks);
+        for (int kc = 0; kc < kchunks; ++kc)
+          bulk_g2s(t_res + (uint32_t)(kc * TCH), Tblk + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
+      }
+      const int64_t total = my_items * nb * kchunks;
+      int64_t iw = blockIdx.x, u = 0;
+      int ib = 0, ikc = 0, is = 0;
+#pragma unroll 1
+      for (int64_t ci = 0; ci < total; ++ci) {
+        // chunk ci into stage `is` once the products of chunk ci - NST freed it
+        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
+        const int64_t ct = RES ? iw : iw / mtiles;
+        const uint32_t st = stages + (uint32_t)(is * STAGE);
+        const uint32_t fb = smem_u32(&full_bar[is]);
+        mbar_expect_tx(fb, xbytes + (RES ? 0u : tbytes));
+        // rows: the tile's lines (realization ib's when accumulating); x: the
+        // chunk's 64 values; z: the head plane (and the tail plane)
+        const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
+        asm volatile(
+            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+            "[%5];" ::"r"(st),
+            "l"(map_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
+            : "memory");
+        if (!RES) {
+          const int mt = (int)(iw - ct * mtiles);
+          bulk_g2s(st + (uint32_t)PX, Tblk + ((size_t)mt * kchunks + ikc) * TCH, tbytes, fb);
+        }
+        if (++is == NST) {
+          is = 0;
+          ++u;
+        }
+        if (++ikc == kchunks) {
+          ikc = 0;
+          if (++ib == nb) {
+            ib = 0;
+            iw += gridDim.x;
+          }
+        }
+      }
+      // nothing of this thread's may still be in flight at exit
+      if (RES) mbar_wait_own(smem_u32(&t_bar), 0u, &s_abort);
+      for (int q = 0; q < NST; ++q) {
+        const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+        if (uq >= 0) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
+      }
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    // ---------------- products: the whole warp, one elected lane issuing ----------------
+    int64_t u = 0;
+    int s = 0;
+    bool ok = !RES || mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
+    const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
+#pragma unroll 1
+    for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
+      const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
+      const int64_t v = NBUF == 2 ? sub >> 1 : sub;
+      const uint32_t prev = (uint32_t)((v - 1) & 1);
+      const uint32_t dre = tmem + (uint32_t)(buf * 4 * RB), dim = dre + 2 * RB;
+#pragma unroll 1
+      for (int kc = 0; kc < kchunks; ++kc) {
+        const bool last = kc == kchunks - 1;
+        ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+             (kc > 0 || v == 0 || mbar_wait(smem_u32(&acce_bar[2 * buf]), prev, &s_abort));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t st = stages + (uint32_t)(s * STAGE);
+        const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
+        plane_half<1, RB, false>(dre, st, tb, tb, id1, id2, kc == 0, unsplit);
+        if (last) {
+          if (elect_one()) mma_commit(smem_u32(&accf_bar[2 * buf]));
+          __syncwarp();
+        }
+        if (kc == 0 && v > 0) {
+          ok = mbar_wait(smem_u32(&acce_bar[2 * buf + 1]), prev, &s_abort);
+          if (!ok) break;
+          tc_fence_after();
+        }
+        plane_half<1, RB, true>(dim, st, tb, tb, id1, id2, kc == 0, unsplit);
+        if (elect_one()) {
+          mma_commit(smem_u32(&empty_bar[s]));
+          if (last) mma_commit(smem_u32(&accf_bar[2 * buf + 1]));
+        }
+        __syncwarp();
+        if (++s == NST) {
+          s = 0;
+          ++u;
+        }
+      }
+    }
+    // whatever happened, the tensor cores finish this warp's work before exit
+    if (elect_one()) mma_commit(smem_u32(&done_bar));
+    __syncwarp();
+    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
+  } else if (warp >= 4) {
+    // ---------------- epilogue ----------------
+    plane_epilogue<RB, OUT>(a, warp, lane, tmem, smem_u32(&accf_bar[0]), blockIdx.x, gridDim.x, my_items, mtiles, 1, 0,
+                            nb, unsplit, &s_abort, [&](int bar) {
+                              mbar_arrive(smem_u32(&acce_bar[bar]));
+                            });
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && s_abort && err) atomicAdd(err, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_free(tmem, 512);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The streaming passes of whole 128-output row blocks (N = 256, 384, ... 1024)
+// on CTA pairs (clusters of two, cta_group::2): a product covers 256 lines, 128
+// per CTA, against one copy of T split between the two CTAs.  On one CTA the
+// streaming kernel reads 160 KB of operands per chunk from shared memory and
+// writes 64 KB of copies to it: 1792 clocks of its 128 bytes a clock, against
+// 1536 clocks of products (measured there: 61-66 us of kernel time per 256^3
+// pass, the products issuing at full rate and then waiting ~300 clocks a chunk
+// for copies).  In a pair each CTA's tensor core reads its own lines and half
+// of T's rows: 112 KB read and 56 KB written per chunk.
+//
+// B operands of a product must lie at one offset in both CTAs, the even CTA
+// holding the first half of the N columns' rows.  Per chunk a CTA therefore
+// holds TP (16 KB: T's head rows in the even CTA, its tail rows in the odd one:
+// the second operand of head x [head; tail], N = 256) and TQ (8 KB: head rows
+// 0-63 in the even CTA, 64-127 in the odd one: tail x head, N = 128).
+//
+// The even CTA issues all products.  Both CTAs' copies (TMA tiles, T's too)
+// complete on its "full" barrier.  Completed products are signalled to both
+// CTAs (multicast commits), and both CTAs' epilogue warps release accumulator
+// halves on the even CTA's barriers.  Chunks go two at a time -- real parts of
+// both, then imaginary parts of both -- so that an item's real half is complete
+// a chunk's time before its imaginary half and the epilogue's reading of one
+// hides behind products of the other (waits of ~930 clocks per half and item
+// with one chunk at a time).
+constexpr int QST = 4;                    // stages
+constexpr int QTP = 128 * 128, QTQ = 64 * 128;
+constexpr int QSTAGE = PX + QTP + QTQ;    // 56 KB
+constexpr int QSMEM = QST * QSTAGE + 1024;
+static_assert(QSMEM <= 226 * 1024, "shared memory");
+
+template <int OUT>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
+    plane_pair_kernel(const DenseArgs a, int* err,
+                      const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap tmap) {
+  constexpr int RB = 128;
+  constexpr bool ACC = OUT == kOutSum;
+  extern __shared__ __align__(1024) unsigned char psm_raw[];
+  unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t full_bar[QST], empty_bar[QST];
+  __shared__ __align__(8) uint64_t accf_bar[2], acce_bar[2], done_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_abort;
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int rank = (int)cluster_rank();
+  const int N = a.N;
+  const int mtiles = N / RB;
+  const int kchunks = N / PKC;  // even
+  const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
+  const int64_t items = ((a.ncols + 2 * PL - 1) / (2 * PL)) * mtiles;
+  const int64_t my_items = (items - pair + npairs - 1) / npairs;
+  if (my_items <= 0) return;  // both CTAs of the pair
+  const int nb = ACC ? (int)a.batch : 1;
+  const bool unsplit = a.unsplit != 0;
+
+  if (warp == 1) tmem2_alloc(&tmem_slot, 512);
+  if (tid == 0) {
+    for (int s = 0; s < QST; ++s) {
+      mbar_init(smem_u32(&full_bar[s]), 1);
+      mbar_init(smem_u32(&empty_bar[s]), 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(smem_u32(&accf_bar[b]), 1);
+      mbar_init(smem_u32(&acce_bar[b]), 2 * PEPIW);
+    }
+    mbar_init(smem_u32(&done_bar), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_abort = 0;
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync();  // the peer's barriers are initialised before any remote arrival
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t stages = smem_u32(psm);
+  const int64_t total = my_items * nb * kchunks;
+
+  if (warp == 0) {
+    // ---------------- copies: each CTA's own, completing on the even CTA's barriers ----------------
+    if (lane == 0) {
+      const uint64_t xmap_addr = reinterpret_cast<uint64_t>(&xmap), tmap_addr = reinterpret_cast<uint64_t>(&tmap);
+      const uint32_t bytes = unsplit ? (uint32_t)(PXPART + QTQ) : (uint32_t)QSTAGE;
+      const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
+      int64_t iw = pair, u = 0;
+      int ib = 0, ikc = 0, is = 0;
+#pragma unroll 1
+      for (int64_t ci = 0; ci < total; ++ci) {
+        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
+        const int64_t wt = iw / mtiles;
+        const int mt = (int)(iw - wt * mtiles);
+        const uint32_t st = stages + (uint32_t)(is * QSTAGE);
+        const uint32_t fb = full0 + 8u * (uint32_t)is;
+        if (rank == 0) mbar_expect_tx(smem_u32(&full_bar[is]), 2u * bytes);
+        // a tile past the last line reads zeros
+        const int row = (int)((2 * wt + rank) * PL + (ACC ? (int64_t)ib * a.outer : 0));
+        asm volatile(
+            "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+            "%4}], [%5];" ::"r"(st),
+            "l"(xmap_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
+            : "memory");
+        // T's rows of the chunk, 64 a tile
+        const int trow = (mt * kchunks + ikc) * (2 * RB);
+        auto copy_t = [&](uint32_t dst, int r) {
+          asm volatile(
+              "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+              "[%4];" ::"r"(dst),
+              "l"(tmap_addr), "r"(0), "r"(trow + r), "r"(fb)
+              : "memory");
+        };
+        if (!unsplit) {
+          copy_t(st + (uint32_t)PX, rank * RB);
+          copy_t(st + (uint32_t)(PX + QTQ), rank * RB + 64);
+        }
+        copy_t(st + (uint32_t)(PX + QTP), rank * 64);
+        if (++is == QST) {
+          is = 0;
+          ++u;
+        }
+        if (++ikc == kchunks) {
+          ikc = 0;
+          if (++ib == nb) {
+            ib = 0;
+            iw += npairs;
+          }
+        }
+      }
+      // no copy of either CTA may still be in flight at exit (the odd CTA
+      // leaves after the cluster barrier below)
+      if (rank == 0)
+        for (int q = 0; q < QST; ++q) {
+          const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+          if (uq >= 0) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
+        }
+    }
+    __syncwarp();
+  } else if (warp == 1 && rank == 0) {
+    // ---------------- products: the whole warp, one elected lane issuing ----------------
+    bool ok = true;
+    int s = 0;
+    int64_t u = 0;
+    const uint32_t id1 = idesc_bf16(2 * PL, RB), id2 = idesc_bf16(2 * PL, 2 * RB);
+    const uint32_t dre = tmem, dim = tmem + 2 * RB;
+#pragma unroll 1
+    for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
+      const uint32_t prev = (uint32_t)((sub - 1) & 1);
+#pragma unroll 1
+      for (int kc = 0; kc < kchunks; kc += 2) {
+        const int s0 = s, s1 = s + 1;  // QST is even: a pair of chunks never wraps
+        const uint32_t ph = (uint32_t)(u & 1);
+        const uint32_t st0 = stages + (uint32_t)(s0 * QSTAGE), st1 = st0 + QSTAGE;
+        const bool last = kc == kchunks - 2;
+        ok = mbar_wait_cluster(smem_u32(&full_bar[s0]), ph, &s_abort) &&
+             (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
+        if (!ok) break;
+        tc_fence_after();
+        plane_half<2, RB, false>(dre, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+        ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
+        if (!ok) break;
+        tc_fence_after();
+        plane_half<2, RB, false>(dre, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+        if (last) {
+          if (elect_one()) mma2_commit_both(smem_u32(&accf_bar[0]));
+          __syncwarp();
+        }
+        if (kc == 0 && sub > 0) {
+          ok = mbar_wait_cluster(smem_u32(&acce_bar[1]), prev, &s_abort);
+          if (!ok) break;
+          tc_fence_after();
+        }
+        plane_half<2, RB, true>(dim, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+        if (elect_one()) mma2_commit_both(smem_u32(&empty_bar[s0]));
+        __syncwarp();
+        plane_half<2, RB, true>(dim, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+        if (elect_one()) {
+          mma2_commit_both(smem_u32(&empty_bar[s1]));
+          if (last) mma2_commit_both(smem_u32(&accf_bar[1]));
+        }
+        __syncwarp();
+        s += 2;
+        if (s == QST) {
+          s = 0;
+          ++u;
+        }
+      }
+    }
+    // whatever happened, the tensor cores finish this warp's work before exit
+    if (elect_one()) mma2_commit(smem_u32(&done_bar));
+    __syncwarp();
+    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
+  } else if (warp >= 4) {
+    // ---------------- epilogue ----------------
+    const uint32_t acce0 = map_rank(smem_u32(&acce_bar[0]), 0u);
+    plane_epilogue<RB, OUT>(a, warp, lane, tmem, smem_u32(&accf_bar[0]), pair, npairs, my_items, mtiles, 2, rank, nb,
+                            unsplit, &s_abort, [&](int bar) { mbar_arrive_cluster_relaxed(acce0 + 8u * (uint32_t)bar); });
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && s_abort && err) atomicAdd(err, 1);
+  // neither CTA leaves while the other's products may read its shared memory
+  // or its threads arrive on its barriers
+  cluster_sync();
+  if (warp == 1) {
+    tc_fence_after();
+    tmem2_free(tmem, 512);
+  }
+  cluster_sync();
+}
+
+// T's chunks from the complex map T [N][N]: for row block mt and chunk kc the
+// head rows and the tail rows of the block's RB outputs (32 real parts, 32
+// imaginary parts), 16-byte piece c of row r stored at c ^ (r % 8).
+__global__ void plane_build_t_kernel(const float2* __restrict__ T, unsigned char* __restrict__ Tblk, int N, int RB) {
+  const int kchunks = N / PKC;
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < (int64_t)N * N;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int n = (int)(idx / N), k = (int)(idx - (int64_t)n * N);
+    const int mt = n / RB, rr = n - mt * RB, kc = k / PKC, kk = k % PKC;
+    const float2 t = T[idx];
+    unsigned char* row = Tblk + ((size_t)mt * kchunks + kc) * ptchunk(RB) + rr * 128 + (kk & 7) * 2;
+    const int re = ((kk >> 3) ^ (rr & 7)) << 4, im = ((4 + (kk >> 3)) ^ (rr & 7)) << 4;
+    const __nv_bfloat16 xh = __float2bfloat16_rn(t.x), yh = __float2bfloat16_rn(t.y);
+    const int part = ppart(RB);
+    *reinterpret_cast<__nv_bfloat16*>(row + re) = xh;
+    *reinterpret_cast<__nv_bfloat16*>(row + im) = yh;
+    *reinterpret_cast<__nv_bfloat16*>(row + part + re) = __float2bfloat16_rn(t.x - __bfloat162float(xh));
+    *reinterpret_cast<__nv_bfloat16*>(row + part + im) = __float2bfloat16_rn(t.y - __bfloat162float(yh));
+  }
+}
+
+// FP32 points into planes: each thread splits eight points (four 16-byte loads
+// in flight) into 16 bytes of real and of imaginary parts per plane.  GRAD: the
+// points are 2 g psi, g per point of each realization or one [M] array shared
+// by the batch (m8 = M / 8).  HBM-bound: 2^24 points (268 MB) in 0.042 ms.
+template <bool GRAD>
+__global__ void __launch_bounds__(256)
+    plane_split_kernel(const float4* __restrict__ in, const float2* __restrict__ grad, int64_t m8, int shared,
+                       uint4* __restrict__ hi, uint4* __restrict__ lo, int64_t n8, int unsplit) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
+    float4 v[4];
+    uint32_t r[4], m[4], rl[4], ml[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) v[k] = in[4 * i + k];
+    if (GRAD) {
+      const int64_t j = 4 * (shared ? i % m8 : i);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float2 g = grad[j + k];
+        v[k].x *= 2.f * g.x, v[k].y *= 2.f * g.x, v[k].z *= 2.f * g.y, v[k].w *= 2.f * g.y;
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      r[k] = bf2(v[k].x, v[k].z);
+      m[k] = bf2(v[k].y, v[k].w);
+      rl[k] = bf2(v[k].x - bf_lo(r[k]), v[k].z - bf_hi(r[k]));
+      ml[k] = bf2(v[k].y - bf_lo(m[k]), v[k].w - bf_hi(m[k]));
+    }
+    // a group of 16 points is two threads: real parts, then imaginary parts
+    const int64_t o = (i >> 1) * 4 + (i & 1);
+    hi[o] = make_uint4(r[0], r[1], r[2], r[3]);
+    hi[o + 2] = make_uint4(m[0], m[1], m[2], m[3]);
+    if (!unsplit) {
+      lo[o] = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+      lo[o + 2] = make_uint4(ml[0], ml[1], ml[2], ml[3]);
+    }
+  }
+}
+
+// passes that run on CTA pairs: streaming, in whole row blocks
+bool pair_pass(int N) { return N >= 256 && N % 128 == 0; }
+
+using PKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap);
+using QKernel = void (*)(const DenseArgs, int*, const CUtensorMap, const CUtensorMap);
+const QKernel kPair[kPOuts] = {plane_pair_kernel<kOutPlanes>, plane_pair_kernel<kOutComplex>,
+                               plane_pair_kernel<kOutDensity>, plane_pair_kernel<kOutSum>};
+template <int RB, bool RES>
+struct PVariant {
+  static constexpr PKernel fn[kPOuts] = {plane_pass_kernel<RB, RES, kOutPlanes>, plane_pass_kernel<RB, RES, kOutComplex>,
+                                         plane_pass_kernel<RB, RES, kOutDensity>, plane_pass_kernel<RB, RES, kOutSum>};
+};
+PKernel single_kernel(int N, int out) {
+  switch (N) {
+    case 64: return PVariant<64, true>::fn[out];
+    case 96: return PVariant<96, true>::fn[out];
+    case 128: return PVariant<128, true>::fn[out];
+    default: return PVariant<96, false>::fn[out];  // 192
+  }
+}
+int single_smem(int N) { return N <= 128 ? psmem(N, true) : psmem(96, false); }
+
+// `rows` rows of 64 BF16 values in tiles of box_rows, `planes` of them `stride`
+// bytes apart
+bool row_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int planes, int64_t stride, int box_rows,
+             bool swizzle) {
+  std::memset(map, 0, sizeof(*map));
+  const EncodeTiledFn enc = encode_tiled();
+  if (!enc) return false;
+  const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+  const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)stride};
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)planes}, estr[3] = {1, 1, 1};
+  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, stride ? 3 : 2, const_cast<void*>(base), dims, strides, box, estr,
+             CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+}  // namespace
+
+bool plane_pass_supported(int N) {
+  return encode_tiled() != nullptr && N <= kDenseMaxN && (N == 64 || N == 96 || N == 192 || (N >= 128 && N % 128 == 0));
+}
+
+size_t plane_t_bytes(int N) { return (size_t)N * N * 8; }
+
+cudaError_t plane_pass_prepare(int N) {
+  cudaError_t e = cudaSuccess;
+  for (int k = 0; k < kPOuts && e == cudaSuccess; ++k)
+    e = pair_pass(N) ? cudaFuncSetAttribute((const void*)kPair[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM)
+                     : cudaFuncSetAttribute((const void*)single_kernel(N, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            single_smem(N));
+  return e;
+}
+
+cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s) {
+  plane_build_t_kernel<<<256, 256, 0, s>>>(T, Tblk, N, prow_block(N));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
+                               int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s) {
+  if (n <= 0) return cudaSuccess;
+  const int64_t n8 = n / 8;  // whole lines of a multiple of 32 points
+  int64_t grid = (n8 + 255) / 256;
+  if (grid > 16 * (int64_t)sms) grid = 16 * (int64_t)sms;
+  const float4* i4 = reinterpret_cast<const float4*>(in);
+  const float2* g2 = reinterpret_cast<const float2*>(grad);
+  uint4* hi = reinterpret_cast<uint4*>(planes);
+  uint4* lo = reinterpret_cast<uint4*>(planes + plane);
+  if (grad)
+    plane_split_kernel<true><<<(int)grid, 256, 0, s>>>(i4, g2, M / 8, grad_shared, hi, lo, n8, unsplit);
+  else
+    plane_split_kernel<false><<<(int)grid, 256, 0, s>>>(i4, nullptr, M / 8, 0, hi, lo, n8, unsplit);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
+  DenseArgs a = args;
+  if (a.oinner == 0) {
+    a.oouter = a.outer;
+    a.oinner = a.inner;
+  }
+  if (a.inner != 1 || !a.in_bf) return cudaErrorInvalidValue;
+  // [plane][line][2N values]: every realization's lines, the tail plane
+  // bf_plane points after the head plane
+  CUtensorMap xmap, tmap;
+  if (!row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
+    return cudaErrorInvalidValue;
+  const int out = a.out_bf ? kOutPlanes : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
+  // one block per SM, or one pair of blocks per two
+  const int per = pair_pass(a.N) ? 2 : 1;
+  int64_t grid = (a.ncols + per * PL - 1) / (per * PL) * (a.N / prow_block(a.N));
+  if (grid > sms / per) grid = sms / per;
+  if (grid < 1) grid = 1;
+  grid *= per;
+  if (per == 2) {
+    // T's chunks as rows of 128 bytes (stored swizzled)
+    if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
+    kPair[out]<<<(int)grid, PTHREADS, QSMEM, s>>>(a, err, xmap, tmap);
+  } else {
+    single_kernel(a.N, out)<<<(int)grid, PTHREADS, single_smem(a.N), s>>>(a, Tblk, err, xmap);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace ffx

@@ -42,17 +42,11 @@
 // Items are (128 lines, 128 real rows) of the output, numbered row block
 // fastest so that blocks running together share the lines' inputs in L2.
 //
-// BF16 pass chains: the d passes of a forward map run from the last axis to
-// the first, and every pass but the last writes its output as BF16 head and
-// tail planes, transposed: point n' of line rho (of R lines per realization)
-// goes to n' R + rho, so that the next axis is the contiguous one for the next
-// pass and, after the pass along axis 0, the lattice is back in its own
-// order.  The epilogue makes the split the next pass would have made of the
-// same FP32 value (bitwise the same operands), and writes 32 consecutive
-// lines per warp store.  A pass with BF16 planes as input needs no producers:
-// thread 0 loads each chunk's head and tail rows as one TMA tile (a 3-D map
-// over [plane][line][2N], 128-byte swizzle) straight into the layout the
-// tensor cores read (K-major, 128-byte swizzle), next to the T chunk.
+// This kernel takes FP32 input (strided lines, backward passes); passes over
+// BF16 planes run in ffx_planes.cu, and the many-instance phases below have
+// their own plane input and output: interleaved (re, im) pairs, transposed
+// between the passes (point n' of line rho of R lines at n' R + rho), read as
+// one TMA tile per chunk into the tensor cores' 128-byte-swizzled layout.
 // Every wait is bounded; one that runs out sets the block's abort flag, the
 // block drains its own copies and products, frees its tensor memory, counts
 // the error and exits.
@@ -64,6 +58,7 @@
 #include "ffx_internal.h"
 #include "ffx_tc_many.h"
 #include "ffx_tcgen05.cuh"
+#include "ffx_tma.h"
 
 namespace ffx {
 
@@ -147,21 +142,6 @@ __device__ __forceinline__ long long bline(const DenseArgs& a, int64_t c, int b,
   return bo * (int64_t)a.N * a.inner + i;
 }
 
-// The same for the output, with the output's decomposition (oouter, oinner).
-__device__ __forceinline__ long long bline_o(const DenseArgs& a, int64_t c, int b, int& br) {
-  br = 0;
-  if (c >= a.ncols) return -1;
-  int64_t bo = c / a.oinner;
-  const int64_t i = c - bo * a.oinner;
-  if (a.acc) {
-    br = b;
-    bo += (int64_t)b * a.oouter;
-  } else {
-    br = (int)(c / (a.oouter * a.oinner));
-  }
-  return bo * (int64_t)a.N * a.oinner + i;
-}
-
 __device__ __forceinline__ uint32_t pack_bf16(float lo_k, float hi_k) {
   const __nv_bfloat162 h = __floats2bfloat162_rn(lo_k, hi_k);  // .x (element k) in the low half
   return *reinterpret_cast<const uint32_t*>(&h);
@@ -193,18 +173,16 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo, boo
 // thread converts its own bytes, with no barrier).  Measured on 256^3
 // passes: contiguous lines 0.17 ms by TMA against 0.20 ms per thread; strided
 // lines 0.17 ms per thread against 0.21 ms by a 3-D TMA tile.
-// BF16 planes (a pass of a chain): the head and tail rows as one TMA tile.
+// BF16 planes (many-instance chains): the head and tail rows as one TMA tile.
 enum BLoad { kTmaContiguous = 0, kInPlace = 1, kTmaPlanes = 2 };
 
 // FULL: every row block has BR rows (2N a multiple of 128).  GRAD: backward
 // passes, whose input element is 2 grad * psi (the factors come through their
 // own ring; two stages).  ACC: the batch's |.|^2 summed in shared memory.
-// INBF: the input is BF16 planes (mode kTmaPlanes; never with GRAD).
-template <bool FULL, bool GRAD, bool ACC, bool INBF>
+template <bool FULL, bool GRAD, bool ACC>
 __global__ void __launch_bounds__(BTHREADS, 1)
     dense_bf16_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
                       const __grid_constant__ CUtensorMap xmap, const int mode) {
-  static_assert(!(GRAD && INBF), "backward passes take FP32 input");
   constexpr int BSTAGES = bstages(GRAD, ACC);
   extern __shared__ __align__(1024) unsigned char bsm_raw[];
   // the stages on a 1024-byte boundary (the launch adds 1 KB for it)
@@ -246,62 +224,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
   const uint32_t tmem = tmem_slot;
   const uint32_t smem_base = smem_u32(bsm);
 
-  if (INBF && warp < BMMA_WARP) {
-    // ---------------- loads of a BF16-plane input: thread 0 alone ----------------
-    if (tid == 0) {
-      const int64_t total = my_items * nb * kchunks;
-      const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
-      const uint32_t xbytes = unsplit ? (uint32_t)BPART : (uint32_t)BXAREA;
-      int64_t iw = blockIdx.x, u = 0;
-      int ib = 0, ikc = 0, is = 0;
-      int last_u[BSMAX];
-#pragma unroll
-      for (int q = 0; q < BSMAX; ++q) last_u[q] = -1;
-#pragma unroll 1
-      for (int64_t ci = 0; ci < total; ++ci) {
-        // chunk ci into stage is once the products of chunk ci - BSTAGES freed it
-        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
-        const int mt = (int)(iw % mtiles);
-        const int64_t ct = iw / mtiles;
-        const uint32_t st = smem_u32(bsm + is * BSTAGE);
-        const uint32_t part = (uint32_t)(FULL ? BR : brow_count(N, mt)) * (BKC * 2);
-        const uint32_t cb = smem_u32(&copy_bar[is]);
-        mbar_expect_tx(cb, (unsplit ? part : 2 * part) + xbytes);
-        const unsigned char* src = Tblk + ((size_t)mt * kchunks + ikc) * BTCHUNK;
-        if (unsplit) {
-          bulk_g2s(st, src, part, cb);
-        } else if (part == (uint32_t)BPART) {
-          bulk_g2s(st, src, BTCHUNK, cb);
-        } else {
-          bulk_g2s(st, src, part, cb);
-          bulk_g2s(st + BPART, src + BPART, part, cb);
-        }
-        // rows: the tile's lines (realization ib's when accumulating); x: the
-        // chunk's 64 real K; z: the head plane (and the tail plane)
-        const int row = (int)(ct * BL + (ACC ? (int64_t)ib * a.outer : 0));
-        asm volatile(
-            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-            "[%5];" ::"r"(st + (uint32_t)BTCHUNK),
-            "l"(map_addr), "r"(ikc * BKC), "r"(row), "r"(0), "r"(cb)
-            : "memory");
-        last_u[is] = (int)(u & 1);
-        if (++is == BSTAGES) {
-          is = 0;
-          ++u;
-        }
-        if (++ikc == kchunks) {
-          ikc = 0;
-          if (++ib == nb) {
-            ib = 0;
-            iw += gridDim.x;
-          }
-        }
-      }
-      // nothing of this thread's may still be in flight at exit
-      for (int q = 0; q < BSTAGES; ++q)
-        if (last_u[q] >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)last_u[q], &s_abort);
-    }
-  } else if (warp < BMMA_WARP) {
+  if (warp < BMMA_WARP) {
     // ---------------- producers ----------------
     const int t = tid;
     const int64_t inner = a.inner;
@@ -523,7 +446,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             const int s = (int)(g % BSTAGES);
             const int64_t u = g / BSTAGES;
             if (!mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) ||
-                (!INBF && !mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort))) {
+                !mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort)) {
               ok = false;
               break;
             }
@@ -533,15 +456,13 @@ __global__ void __launch_bounds__(BTHREADS, 1)
 #pragma unroll
             for (int ks = 0; ks < BKC / 16; ++ks) {
               const uint32_t o = (uint32_t)(ks * 2 * BCORE);
-              // X: core matrices of the producers, or the swizzled TMA tile (32 bytes per K step)
-              const uint64_t dxh = INBF ? make_desc_sw128(xh + (uint32_t)(ks * 32)) : make_desc(xh + o, BCORE, BSBO);
+              const uint64_t dxh = make_desc(xh + o, BCORE, BSBO);
               const uint64_t dth = make_desc(th + o, BCORE, BSBO);
               const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
               if (unsplit) {
                 mma_f16(d1, dxh, dth, idesc, more);
               } else {
-                const uint64_t dxl =
-                    INBF ? make_desc_sw128(xl + (uint32_t)(ks * 32)) : make_desc(xl + o, BCORE, BSBO);
+                const uint64_t dxl = make_desc(xl + o, BCORE, BSBO);
                 if (FULL) {
                   mma_f16(d1, dxh, dth, idesc_bf16(BL, 2 * BR), more);
                 } else {
@@ -565,7 +486,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     // ---------------- epilogue ----------------
     const int q = warp & 3;       // tensor-memory lane quarter this warp may read
     const int r = q * 32 + lane;  // line within the item
-    const int64_t inner = a.oinner;  // the output's decomposition
+    const int64_t inner = a.inner;
     const bool contiguous = (inner == 1);
     float* racc = reinterpret_cast<float*>(bsm + BSTAGES * BSTAGE);  // accumulating launches only
     if (ACC)
@@ -588,7 +509,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         if (!ok) break;
         tc_fence_after();
         int br;
-        const long long base = bline_o(a, ct * BL + r, b, br);
+        const long long base = bline(a, ct * BL + r, b, br);
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BR);
 #pragma unroll 1
         for (int j0 = 0; j0 < rows; j0 += 16) {
@@ -605,19 +526,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             for (int m = 0; m < 8; ++m)
               racc[(j0 / 2 + m) * BL + r] += y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
           } else if (base >= 0) {
-            if (a.out_bf) {
-              // BF16 head and tail planes for the next pass of a chain
-#pragma unroll
-              for (int m = 0; m < 8; ++m) {
-                const __nv_bfloat162 hb = __floats2bfloat162_rn(y[2 * m], y[2 * m + 1]);
-                const int64_t e = base + (int64_t)(n0 + m) * inner;
-                a.out_bf[e] = *reinterpret_cast<const uint32_t*>(&hb);
-                if (!unsplit) {
-                  const float2 hf = __bfloat1622float2(hb);
-                  a.out_bf[a.bf_plane + e] = pack_bf16(y[2 * m] - hf.x, y[2 * m + 1] - hf.y);
-                }
-              }
-            } else if (a.out_c) {
+            if (a.out_c) {
               if (contiguous) {
                 float4* o = reinterpret_cast<float4*>(a.out_c + base + n0);
 #pragma unroll
@@ -703,23 +612,6 @@ __global__ void bf16_build_t_kernel(const float2* __restrict__ T, unsigned char*
     const int off = (rr >> 3) * BSBO + (kk >> 3) * BCORE + (rr & 7) * 16 + (kk & 7) * 2;
     *reinterpret_cast<__nv_bfloat16*>(blk + off) = hi;
     *reinterpret_cast<__nv_bfloat16*>(blk + BPART + off) = lo;
-  }
-}
-
-// The first pass of a BF16 chain reads its FP32 input as BF16 planes too:
-// every (re, im) pair v becomes bf16(v) in the head plane and bf16(v - bf16(v))
-// in the tail plane (the split the pass would make on the fly), in the same
-// order; two pairs per thread step, 16-byte loads.
-__global__ void __launch_bounds__(256) bf16_split_kernel(const float4* __restrict__ in, uint2* __restrict__ hi,
-                                                          uint2* __restrict__ lo, int64_t n2, int unsplit) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
-    const float4 v = in[i];
-    const __nv_bfloat162 h0 = __floats2bfloat162_rn(v.x, v.y), h1 = __floats2bfloat162_rn(v.z, v.w);
-    hi[i] = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
-    if (!unsplit) {
-      const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
-      lo[i] = make_uint2(pack_bf16(v.x - f0.x, v.y - f0.y), pack_bf16(v.z - f1.x, v.w - f1.y));
-    }
   }
 }
 
@@ -1262,32 +1154,11 @@ __global__ void __launch_bounds__(256) bf16_split_grad_kernel(const float4* __re
 
 }  // namespace
 
-cudaError_t launch_bf16_split_grad(const float2* field, const float* grad, int grad_shared, int64_t M,
-                                   uint32_t* planes, int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int grid = bf16_split_grid(n, sms);
-  bf16_split_grad_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4*>(field),
-                                              reinterpret_cast<const float2*>(grad), reinterpret_cast<uint2*>(planes),
-                                              reinterpret_cast<uint2*>(planes + plane), n / 2, M / 2, grad_shared,
-                                              unsplit);
-  return cudaGetLastError();
-}
-
 const void* bf16_split_grad_func() { return (const void*)bf16_split_grad_kernel; }
 int bf16_split_grid(int64_t n, int sms) {
   int64_t grid = (n / 2 + 255) / 256;
   if (grid > 8 * (int64_t)sms) grid = 8 * (int64_t)sms;
   return grid < 1 ? 1 : (int)grid;
-}
-
-cudaError_t launch_bf16_split(const float2* in, uint32_t* planes, int64_t n, int64_t plane, int unsplit, int sms,
-                              cudaStream_t s) {
-  if (n <= 0) return cudaSuccess;
-  const int64_t n2 = n / 2;  // n is even: whole realizations of lattices of >= 64 points
-  const int grid = bf16_split_grid(n, sms);
-  bf16_split_kernel<<<grid, 256, 0, s>>>(reinterpret_cast<const float4*>(in), reinterpret_cast<uint2*>(planes),
-                                              reinterpret_cast<uint2*>(planes + plane), n2, unsplit);
-  return cudaGetLastError();
 }
 
 bool dense_bf16_supported(int N) { return N >= 64 && N <= kDenseMaxN && N % 32 == 0; }
@@ -1296,21 +1167,18 @@ size_t dense_bf16_t_bytes(int N) { return (size_t)((2 * N + BR - 1) / BR) * ((2 
 
 namespace {
 
-// the kernel's variants, indexed [FULL][kind], kind 0 plain, 1 ACC, 2 GRAD,
-// 3 INBF, 4 INBF + ACC
+// the kernel's variants, indexed [FULL][kind], kind 0 plain, 1 ACC, 2 GRAD
 using BKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap, const int);
-constexpr int kBKinds = 5;
+constexpr int kBKinds = 3;
 BKernel bf16_kernel(bool full, int kind) {
   static const BKernel k[2][kBKinds] = {
-      {dense_bf16_kernel<false, false, false, false>, dense_bf16_kernel<false, false, true, false>,
-       dense_bf16_kernel<false, true, false, false>, dense_bf16_kernel<false, false, false, true>,
-       dense_bf16_kernel<false, false, true, true>},
-      {dense_bf16_kernel<true, false, false, false>, dense_bf16_kernel<true, false, true, false>,
-       dense_bf16_kernel<true, true, false, false>, dense_bf16_kernel<true, false, false, true>,
-       dense_bf16_kernel<true, false, true, true>}};
+      {dense_bf16_kernel<false, false, false>, dense_bf16_kernel<false, false, true>,
+       dense_bf16_kernel<false, true, false>},
+      {dense_bf16_kernel<true, false, false>, dense_bf16_kernel<true, false, true>,
+       dense_bf16_kernel<true, true, false>}};
   return k[full ? 1 : 0][kind];
 }
-int bf16_kind_smem(int kind) { return bsmem_launch(kind == 2, kind == 1 || kind == 4); }
+int bf16_kind_smem(int kind) { return bsmem_launch(kind == 2, kind == 1); }
 
 }  // namespace
 
@@ -1350,51 +1218,14 @@ cudaError_t launch_bf16_build_t(const float2* T, unsigned char* Tblk, int N, cud
 
 namespace {
 
-using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-// cuTensorMapEncodeTiled through the runtime's driver entry point (no link
-// against the driver library); NULL if the driver does not offer it
-EncodeTiledFn encode_tiled() {
-  static const EncodeTiledFn fn = []() -> EncodeTiledFn {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess) {
-      cudaGetLastError();
-      return nullptr;
-    }
-    return reinterpret_cast<EncodeTiledFn>(p);
-  }();
-  return fn;
-}
-
-// The input tile map of a launch and how the kernel loads its chunks: BF16
-// planes as 3-D TMA tiles; FP32 TMA tiles for contiguous lines of forward and
-// adjoint passes; in place otherwise (or when the FP32 map cannot be made).
-// Returns false when BF16 planes come without a map.
-bool input_map(const DenseArgs& a, CUtensorMap* map, int* mode) {
+// The input tile map of a launch and how the kernel loads its chunks: FP32 TMA
+// tiles for contiguous lines of forward and adjoint passes; in place otherwise
+// (or when the map cannot be made).
+void input_map(const DenseArgs& a, CUtensorMap* map, int* mode) {
   std::memset(map, 0, sizeof(*map));
   *mode = kInPlace;
   const EncodeTiledFn enc = encode_tiled();
-  if (a.in_bf) {
-    // [plane][line][2N bf16]: the lines of every realization (contiguous:
-    // inner == 1), the tail plane bf_plane pairs after the head plane; a box
-    // of 64 values x 128 lines x the planes the launch reads
-    if (!enc || a.inner != 1 || a.grad) return false;
-    const cuuint64_t rows = (cuuint64_t)a.batch * (cuuint64_t)a.outer;
-    const cuuint64_t dims[3] = {(cuuint64_t)(2 * a.N), rows, a.unsplit ? 1u : 2u};
-    const cuuint64_t strides[2] = {(cuuint64_t)(2 * a.N) * 2, (cuuint64_t)a.bf_plane * 4};
-    const cuuint32_t box[3] = {(cuuint32_t)BKC, (cuuint32_t)BL, a.unsplit ? 1u : 2u}, estr[3] = {1, 1, 1};
-    if (enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)a.in_bf, dims, strides, box, estr,
-            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
-      return false;
-    *mode = kTmaPlanes;
-    return true;
-  }
-  if (a.grad || a.inner != 1 || !enc) return true;
+  if (a.grad || a.inner != 1 || !enc) return;
   const cuuint64_t rows = (cuuint64_t)a.batch * (cuuint64_t)a.outer;  // every realization's lines
   const cuuint64_t dims[2] = {(cuuint64_t)(2 * a.N), rows};
   const cuuint64_t strides[1] = {(cuuint64_t)(2 * a.N) * 4};
@@ -1405,12 +1236,9 @@ bool input_map(const DenseArgs& a, CUtensorMap* map, int* mode) {
     *mode = kTmaContiguous;
   else
     std::memset(map, 0, sizeof(*map));
-  return true;
 }
 
 }  // namespace
-
-bool dense_bf16_chain_supported() { return encode_tiled() != nullptr; }
 
 bool many_bf16_line_map(const float2* base, int N, int64_t lines, void* map) {
   // [lines][2N floats], boxes of 32 floats x 128 lines, 128-byte swizzle: the
@@ -1449,18 +1277,12 @@ bool many_bf16_plane_map(const uint32_t* head, int N, int64_t lines, int64_t pla
   return true;
 }
 
-cudaError_t launch_dense_bf16(const DenseArgs& args, const unsigned char* Tblk, int* err, int grid, cudaStream_t s) {
-  DenseArgs a = args;
-  if (a.oinner == 0) {
-    a.oouter = a.outer;
-    a.oinner = a.inner;
-  }
+cudaError_t launch_dense_bf16(const DenseArgs& a, const unsigned char* Tblk, int* err, int grid, cudaStream_t s) {
   CUtensorMap map;
   int mode;
-  if (!input_map(a, &map, &mode)) return cudaErrorInvalidValue;
+  input_map(a, &map, &mode);
   const bool full = (2 * a.N) % BR == 0;
-  // backward passes never accumulate over the batch, nor read BF16 planes
-  const int kind = a.grad ? 2 : a.in_bf ? (a.acc ? 4 : 3) : (a.acc ? 1 : 0);
+  const int kind = a.grad ? 2 : (a.acc ? 1 : 0);  // backward passes never accumulate over the batch
   bf16_kernel(full, kind)<<<grid, BTHREADS, bf16_kind_smem(kind), s>>>(a, Tblk, err, map, mode);
   return cudaGetLastError();
 }

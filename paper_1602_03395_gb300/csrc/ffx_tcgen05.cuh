@@ -134,6 +134,100 @@ __device__ __forceinline__ void mma_f16(uint32_t tmem_d, uint64_t adesc, uint64_
       : "memory");
 }
 
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(r));
+  return r != 0;
+}
+
+// Products of operands in 128-byte-swizzled K-major tiles given by their
+// shared-memory addresses (descriptor fields of make_desc_sw128: only the low
+// word varies, which keeps the address arithmetic of an issuing warp short).
+// Issued by one elected lane; every lane of the warp calls them.
+constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
+__device__ __forceinline__ void mma_sw128(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, e;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+      " mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+      " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(kDescHiSw128)
+      : "memory");
+}
+__device__ __forceinline__ void mma2_sw128(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p, e;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+      " mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+      " @e tcgen05.mma.cta_group::2.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem_d),
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(kDescHiSw128)
+      : "memory");
+}
+
+// ---- two CTAs of a cluster on one product (cta_group::2) -------------------
+// One thread of the even CTA issues the product: D is M = 256 rows, 128 in each
+// CTA's tensor memory; each CTA holds its 128 rows of A and N / 2 rows of B at
+// the same shared-memory offsets.
+// Completion of the issuing thread's products, on the barrier at this offset in
+// both CTAs, or in the issuing one alone.
+__device__ __forceinline__ void mma2_commit_both(uint32_t mbar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(mbar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+__device__ __forceinline__ void mma2_commit(uint32_t mbar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar) : "memory");
+}
+// Both CTAs' warps allocate (free) the same columns together.
+__device__ __forceinline__ void tmem2_alloc(uint32_t* slot, uint32_t cols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(slot)), "r"(cols)
+               : "memory");
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem2_free(uint32_t tmem, uint32_t cols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols) : "memory");
+}
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// The shared::cluster address of this offset in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
+  return r;
+}
+// Arrive on a barrier of either CTA (a shared::cluster address) without
+// ordering this thread's earlier memory writes: for barriers that only pass on
+// tensor-memory columns already read back.  (A release at cluster scope waits
+// for the thread's global stores in flight: measured ~2000 clocks.)
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
+// mbar_wait for a barrier that threads of both CTAs arrive on.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t mbar, uint32_t parity, volatile int* abort_flag) {
+  for (long long i = 0; i < kSpinLimit; ++i) {
+    uint32_t done;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
+        " selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(done)
+        : "r"(mbar), "r"(parity)
+        : "memory");
+    if (done) return true;
+    if (*abort_flag) return false;
+  }
+  *abort_flag = 1;
+  return false;
+}
+
 // 32 lanes x 16 consecutive 32-bit columns of tensor memory (the calling
 // warp's lane quarter); complete with tmem_wait_ld().
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t* x) {

@@ -1,0 +1,68 @@
+"""The passes over BF16 planes (csrc/ffx_planes.cu) against the FP64 oracle, at
+the sizes where their tiling can go wrong: every row-block variant (64, 96, 128
+outputs with T resident, 192 and 256 ... 1024 streamed, the latter on CTA
+pairs), line counts that are not whole tiles or leave half a pair without
+lines, chains (transposed planes between the passes) and single passes over
+contiguous lines, and every kind of output: planes, fields, densities, the
+ensemble sum, and the adjoint.
+
+Split operands: each operand is hi + lo to 2^-17 relative and the lo*lo term is
+dropped, a few 2^-18 per pass of random sign, within the FP32 path's 2e-5 bar
+(DENSITY_TOL, FIELD_TOL; the gradient runs twice the passes, within the same
+bar).  Unsplit: 2^-9 per operand, the 1e-2 class."""
+
+import numpy as np
+import pytest
+
+import oracle as O
+from gpu_common import DENSITY_TOL, FIELD_TOL, random_field, rel_l2, require_gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+UNSPLIT_TOL = 1e-2
+
+CASES = [
+    # chains: lines per pass (axis 1, axis 0)
+    ((256, 96), (5, 9), 1),       # 256 lines of 96; 96 lines of 256 (one tile, half a pair empty)
+    ((256, 96), (5, 9), 3),       # 288 lines of 256: three tiles, the last pair's second past the end
+    ((384, 128), (3, 30), 2),     # three row blocks; T resident at 128
+    ((512, 192), (4, 7), 1),      # four row blocks; 192 in two blocks of 96
+    ((1024, 32 * 3), (6, 5), 1),  # eight row blocks
+    ((64, 64, 256), (4, 5, 6), 3),
+    # single passes over contiguous lines (a 1-D field has no chain)
+    ((256,), (100,), 5), ((256,), (3,), 129), ((768,), (7,), 257), ((128,), (9,), 131), ((192,), (4,), 3),
+    ((96,), (11,), 400),
+]
+
+
+@pytest.fixture(scope="module")
+def ffx():
+    return require_gpu()
+
+
+@pytest.mark.parametrize("dims,lam,batch", CASES)
+def test_plane_passes(ffx, dims, lam, batch):
+    rng = np.random.default_rng(7 * batch + sum(dims))
+    dx, t = (0.25,) * len(dims), 6.0
+    psi = random_field(rng, (batch,) + dims)
+    grad = rng.normal(size=(batch,) + dims).astype(np.float32)
+    ref = O.expand_field(psi, dx, t, lam)
+    dens = np.abs(ref) ** 2
+    x = to_dev(psi)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
+        rho = ffx.ffx_expand(plan, x).cpu().numpy()
+        fld = ffx.ffx_expand_field(plan, x).cpu().numpy()
+        g = ffx.ffx_expand_backward(plan, x, to_dev(grad)).cpu().numpy()
+        assert plan.device_errors() == 0
+    start = rng.random(dims).astype(np.float32)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, accumulate=True) as plan:
+        acc = ffx.ffx_expand(plan, x, to_dev(start.copy())).cpu().numpy()
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, unsplit=True) as plan:
+        rough = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.device_errors() == 0
+    assert rel_l2(rho, dens) < DENSITY_TOL
+    assert rel_l2(fld, ref) < FIELD_TOL
+    assert rel_l2(acc, start + dens.sum(0)) < DENSITY_TOL
+    assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
+    assert rel_l2(rough, dens) < UNSPLIT_TOL
