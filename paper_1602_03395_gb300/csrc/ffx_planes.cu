@@ -52,6 +52,7 @@
 #include <cstring>
 
 #include "ffx_internal.h"
+#include "ffx_pdl.h"
 #include "ffx_tcgen05.cuh"
 #include "ffx_tma.h"
 
@@ -177,6 +178,7 @@ __device__ __forceinline__ void plane_epilogue(const DenseArgs& a, int warp, int
   constexpr int H = RB / 2;               // outputs per epilogue thread
   constexpr bool ACC = OUT == kOutSum;
   const int N = a.N;
+  pdl_wait();  // before any store: the predecessor may still read the output's memory
   const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
   const int col0 = ((warp - 4) >> 2) * H;  // first of this warp's outputs
   const int r = q * 32 + lane;            // line within the item
@@ -412,6 +414,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
   }
+  pdl_trigger();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -431,6 +434,7 @@ __global__ void __launch_bounds__(PTHREADS, 1)
         for (int kc = 0; kc < kchunks; ++kc)
           bulk_g2s(t_res + (uint32_t)(kc * TCH), Tblk + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
       }
+      pdl_wait();  // T is the plan's own; the lines may be the predecessor's output
       const int64_t total = my_items * nb * kchunks;
       int64_t iw = blockIdx.x, u = 0;
       int ib = 0, ikc = 0, is = 0;
@@ -609,6 +613,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     s_abort = 0;
   }
+  pdl_trigger();
   tc_fence_before();
   __syncthreads();
   cluster_sync();  // the peer's barriers are initialised before any remote arrival
@@ -623,6 +628,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
       const uint64_t xmap_addr = reinterpret_cast<uint64_t>(&xmap), tmap_addr = reinterpret_cast<uint64_t>(&tmap);
       const uint32_t bytes = unsplit ? (uint32_t)(PXPART + QTQ) : (uint32_t)QSTAGE;
       const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
+      pdl_wait();
       int64_t iw = pair, u = 0;
       int ib = 0, ikc = 0, is = 0;
 #pragma unroll 1
@@ -778,6 +784,8 @@ template <bool GRAD>
 __global__ void __launch_bounds__(256)
     plane_split_kernel(const float4* __restrict__ in, const float2* __restrict__ grad, int64_t m8, int shared,
                        uint4* __restrict__ hi, uint4* __restrict__ lo, int64_t n8, int unsplit) {
+  pdl_trigger();
+  pdl_wait();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n8; i += (int64_t)gridDim.x * blockDim.x) {
     float4 v[4];
     uint32_t r[4], m[4], rl[4], ml[4];
@@ -879,10 +887,9 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
   uint4* hi = reinterpret_cast<uint4*>(planes);
   uint4* lo = reinterpret_cast<uint4*>(planes + plane);
   if (grad)
-    plane_split_kernel<true><<<(int)grid, 256, 0, s>>>(i4, g2, M / 8, grad_shared, hi, lo, n8, unsplit);
-  else
-    plane_split_kernel<false><<<(int)grid, 256, 0, s>>>(i4, nullptr, M / 8, 0, hi, lo, n8, unsplit);
-  return cudaGetLastError();
+    return launch_pdl(plane_split_kernel<true>, (int)grid, 256, 0, s, i4, g2, M / 8, grad_shared, hi, lo, n8, unsplit);
+  return launch_pdl(plane_split_kernel<false>, (int)grid, 256, 0, s, i4, (const float2*)nullptr, M / 8, 0, hi, lo, n8,
+                    unsplit);
 }
 
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
@@ -907,11 +914,9 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   if (per == 2) {
     // T's chunks as rows of 128 bytes (stored swizzled)
     if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
-    kPair[out]<<<(int)grid, PTHREADS, QSMEM, s>>>(a, err, xmap, tmap);
-  } else {
-    single_kernel(a.N, out)<<<(int)grid, PTHREADS, single_smem(a.N), s>>>(a, Tblk, err, xmap);
+    return launch_pdl(kPair[out], (int)grid, PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
-  return cudaGetLastError();
+  return launch_pdl(single_kernel(a.N, out), (int)grid, PTHREADS, single_smem(a.N), s, a, Tblk, err, xmap);
 }
 
 }  // namespace ffx

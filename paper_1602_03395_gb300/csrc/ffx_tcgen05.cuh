@@ -166,6 +166,16 @@ __device__ __forceinline__ void mma2_sw128(uint32_t tmem_d, uint32_t alo, uint32
       : "memory");
 }
 
+// ---- programmatic dependent launches ------------------------------------------
+// A kernel launched with launch_pdl may start while its predecessor on the
+// stream ends; everything it reads or writes that an earlier kernel of the
+// stream may touch comes after pdl_wait(), in every thread that touches it
+// (the wait covers the predecessor's completion, which in turn waited for its
+// own).  pdl_trigger() lets the successor's blocks in once every block called
+// it or ended.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- two CTAs of a cluster on one product (cta_group::2) -------------------
 // One thread of the even CTA issues the product: D is M = 256 rows, 128 in each
 // CTA's tensor memory; each CTA holds its 128 rows of A and N / 2 rows of B at
