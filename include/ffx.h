@@ -89,7 +89,8 @@ extern "C" {
 #define FFX_TUNE        0x20u
 /* ffx_expand writes the SUM over the batch of |Psibar|^2, added to what
  * out_density holds ([M_0..M_{d-1}], out += sum_b rho_b), instead of one
- * density per realization.  The sum runs over b in order (deterministic). */
+ * density per realization.  The order of the sum depends on the
+ * lattice and the batch alone (deterministic). */
 #define FFX_ACCUMULATE  0x10u
 /* Keep one launch per axis pass.  Without it, a plan with two or three axes
  * that all take a dense form with at most 64 points runs ffx_expand and

@@ -137,7 +137,7 @@ using namespace ffx;
 // fused launch's grid-barrier counters (+64), its tile counters (+1024).
 constexpr size_t kTcHeader = 1024 + kFusedTileFlags * sizeof(unsigned);
 
-constexpr int kWs = 5, kWsSplit = 4;
+constexpr int kWs = 6, kWsSplit = 4, kWsSum = 5;
 
 struct ffx_plan_s {
   int ndim = 0;
@@ -173,9 +173,10 @@ struct ffx_plan_s {
   size_t fused_smem_bytes = 0;
   // workspace buffers, grown on demand: [0], [1] the passes' fields; [2] the
   // detector densities, or a positive-P pair's first field; [3] its second;
-  // [4] the BF16 planes a per-axis BF16 pass splits its FP32 input into
-  void* ws[kWs] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  size_t ws_bytes[kWs] = {0, 0, 0, 0, 0};
+  // [4] the BF16 planes a per-axis BF16 pass splits its FP32 input into; [5]
+  // partial densities of an ensemble sum's groups
+  void* ws[kWs] = {};
+  size_t ws_bytes[kWs] = {};
   int64_t launches = 0;  // kernels the plan's calls have launched (ffx_plan_launch_count)
   void* stage[2] = {nullptr, nullptr};  // ffx_expand_host: device copies of the input and the densities
   size_t stage_bytes[2] = {0, 0};
@@ -270,8 +271,7 @@ int ensure_stage(ffx_plan_s* p, int k, size_t need) {
   return FFX_OK;
 }
 
-int ensure_ws(ffx_plan_s* p, int which, int64_t batch) {
-  const size_t need = (size_t)batch * (size_t)p->M * sizeof(float2);
+int ensure_bytes(ffx_plan_s* p, int which, size_t need) {
   if (need <= p->ws_bytes[which]) return FFX_OK;
   if (p->ws[which]) {
     cudaFree(p->ws[which]);  // synchronizes the device: queued users of the old buffer finish first
@@ -286,6 +286,10 @@ int ensure_ws(ffx_plan_s* p, int which, int64_t batch) {
   }
   p->ws_bytes[which] = need;
   return FFX_OK;
+}
+
+int ensure_ws(ffx_plan_s* p, int which, int64_t batch) {
+  return ensure_bytes(p, which, (size_t)batch * (size_t)p->M * sizeof(float2));
 }
 
 bool inplace_ok(const Axis& ax) {
@@ -340,21 +344,24 @@ struct ChainIo {
   int64_t plane;
 };
 
-// Launch one pass of axis j (forward or adjoint) with the axis's form, or,
-// with `io`, a pass of a BF16 chain.
-int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* grad, int grad_shared,
-             float2* out_c, float* out_d, int acc, int64_t batch, cudaStream_t stream, const ChainIo* io = nullptr) {
+// The lines one launch of a pass covers: `batch` realizations of M points laid
+// out [outer][N][inner] (summed over the batch with acc).  A launch that sums an
+// ensemble's realizations r, r + G, r + 2 G, ... for every r < G at once is such
+// a layout too, with G outer, G M and batch / G in their place.
+struct PassGeom {
+  int64_t outer, inner, M, batch;
+  int64_t real_lines;  // lines of one realization (what an FFT pass's q-split depends on)
+  int64_t groups;      // 32-point tensor-core sums: DenseArgs::groups (0: none)
+};
+
+// Launch one pass of axis j (forward or adjoint) in the form cform, or, with
+// `io`, a pass of a BF16 chain.
+int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, const float2* in, const float* grad,
+             int grad_shared, float2* out_c, float* out_d, int acc, cudaStream_t stream, const ChainIo* io) {
   const Axis& ax = p->axis[j];
-  int64_t outer, inner;
-  axis_outer_inner(p, j, &outer, &inner);
-  if (io) {
-    outer = p->M / ax.N;
-    inner = 1;
-  }
-  const unsigned rec_flags = trace_begin(p, stream);
+  const int64_t outer = gm.outer, inner = gm.inner, M = gm.M, batch = gm.batch;
+  const int64_t ncols = acc ? outer * inner : batch * outer * inner;
   cudaError_t e;
-  const int64_t lines = acc ? outer * inner : batch * outer * inner;
-  const int cform = call_form(p, ax, lines);  // this call's form
   if (cform == FFX_FORM_TC && tc_aligned(in, out_c, out_d)) {
     DenseArgs d;
     std::memset(&d, 0, sizeof(d));
@@ -365,15 +372,16 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
     d.out_d = out_d;
     d.outer = outer;
     d.inner = inner;
-    d.M = p->M;
+    d.M = M;
     d.batch = batch;
     d.acc = acc;
+    d.groups = gm.groups;
     d.unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
-    d.ncols = acc ? outer * inner : batch * outer * inner;
+    d.ncols = ncols;
     d.N = ax.N;
     const int64_t items = dense_tc_tiles(ax.N, d.ncols);
     int64_t grid = items;
-    if (grid > p->sms) grid = p->sms;
+    if (grid > p->sms || gm.groups) grid = p->sms;
     if (grid < 1) grid = 1;
     // BF16 operands on the streaming kernel's passes; the tensor-memory
     // kernels (64-point plain passes with at most four items per block) keep
@@ -385,16 +393,16 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
       d.in_bf = io->in_bf;
       d.out_bf = io->out_bf;
       d.bf_plane = io->plane;
-      d.oouter = 1;
-      d.oinner = outer;
+      d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
+      d.oouter = outer / d.oinner;
     } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
       // cores' layout instead of converting them on the way
-      int rc = ensure_ws(p, kWsSplit, batch);
+      const int64_t plane = batch * M;
+      int rc = ensure_ws(p, kWsSplit, plane / p->M);
       if (rc) return rc;
-      const int64_t plane = batch * p->M;
-      e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[kWsSplit], plane, plane, d.unsplit, p->sms, stream);
+      e = launch_plane_split(in, nullptr, 0, M, (uint32_t*)p->ws[kWsSplit], plane, plane, d.unsplit, p->sms, stream);
       if (e != cudaSuccess) return cuda_fail(e, "BF16 split of a pass input");
       ++p->launches;
       d.in_bf = (const uint32_t*)p->ws[kWsSplit];
@@ -420,10 +428,10 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
     d.out_d = out_d;
     d.outer = outer;
     d.inner = inner;
-    d.M = p->M;
+    d.M = M;
     d.batch = batch;
     d.acc = acc;
-    d.ncols = acc ? outer * inner : batch * outer * inner;
+    d.ncols = ncols;
     d.N = ax.N;
     d.Aimg = adjoint ? ax.img[1] : ax.img[0];
     d.err = p->dev_err;
@@ -451,10 +459,10 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
     a.out_d = out_d;
     a.outer = outer;
     a.inner = inner;
-    a.M = p->M;
+    a.M = M;
     a.batch = batch;
     a.acc = acc;
-    a.nlines = acc ? outer * inner : batch * outer * inner;
+    a.nlines = ncols;
     a.lam = ax.lam;
     a.g = ax.g;
     a.Np = ax.Np;
@@ -474,7 +482,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
       const int capacity = adjoint ? ax.grid_adj : (cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold);
       // The split depends on one realization's lines only, so a realization's
       // result does not depend on the batch it came in (bitwise).
-      a.qg = choose_qg(info, outer * inner, ax.lam, capacity);
+      a.qg = choose_qg(info, gm.real_lines, ax.lam, capacity);
       const int lines = pass_lines_per_tile(info, a.qg);
       const int64_t ntiles = (a.nlines + lines - 1) / lines;
       int64_t grid = capacity;
@@ -485,6 +493,118 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   }
   if (e != cudaSuccess) return cuda_fail(e, "pass launch");
   ++p->launches;
+  return FFX_OK;
+}
+
+// Whether the pass runs on the 32-point tensor-core kernel that sums groups of
+// realizations itself.
+bool tm32_sum(const Axis& ax, int cform, const float2* in, const float* out_d) {
+  return ax.N == 32 && cform == FFX_FORM_TC && ax.tc_t[0] && tc_aligned(in, nullptr, out_d);
+}
+
+// Groups an ensemble sum over `batch` realizations runs in.  A block sums the
+// realizations of its lines one after the other, so the lines of one
+// realization alone (a 1-D field: one line) leave most of the chip idle; with G
+// groups G times as many blocks work, each on batch / G realizations, into
+// partial densities that are added at the end.  The rule counts steps, waves of
+// resident blocks times realizations each: the fewest groups within 5% of the
+// fewest steps, and one group unless that saves a fifth of them.  (The mean of
+// 512 realizations of one 2048-point line, lam = 20: 97 ms in one group, 0.41 ms
+// in 512.)  The partial densities take at most kSumBytes.
+constexpr size_t kSumBytes = size_t(256) << 20;
+int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, bool tm32, int64_t lines,
+                   int64_t batch) {
+  if (batch * lines < kDenseFewLines && cform == FFX_FORM_DENSE) return 1;  // the few-lines kernel
+  auto steps = [&](int64_t ncols) -> int64_t {  // waves of a launch over ncols lines
+    int64_t tiles, cap;
+    if (cform == FFX_FORM_TC && tm32) {
+      tiles = (ncols + 127) / 128;
+      cap = 2 * p->sms;
+    } else if (cform == FFX_FORM_TC && planes) {
+      tiles = plane_pass_tiles(ax.N, ncols, p->sms, &cap);
+    } else if (cform == FFX_FORM_TC) {
+      tiles = dense_tc_tiles(ax.N, ncols);
+      cap = p->sms;
+    } else if (cform == FFX_FORM_DENSE) {
+      tiles = ax.N <= kDenseInPlaceMaxN ? dense_small_tiles(ax.N, ncols) : dense_tiles(ax.N, ncols);
+      cap = ax.N <= kDenseInPlaceMaxN ? ax.grid_dense_small : ax.grid_dense;
+    } else {
+      const PassKernelInfo& info = cform == FFX_FORM_PAPER ? ax.paper : ax.foldk;
+      cap = cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold;
+      const int per = pass_lines_per_tile(info, choose_qg(info, lines, ax.lam, (int)cap));
+      tiles = (ncols + per - 1) / per;
+    }
+    return (tiles + cap - 1) / cap;
+  };
+  const int64_t gmax = std::min<int64_t>(batch, std::max<int64_t>(1, (int64_t)(kSumBytes / (p->M * sizeof(float)))));
+  auto cost = [&](int64_t g) -> int64_t {
+    const int64_t rem = batch % g;
+    return steps(g * lines) * (batch / g) + (rem ? steps(rem * lines) : 0);
+  };
+  // candidates: every g up to 64, then each an eighth more, and the most
+  auto next = [&](int64_t g) { return g >= gmax ? gmax + 1 : std::min(gmax, g < 64 ? g + 1 : g + g / 8); };
+  const int64_t one = cost(1);
+  int64_t best = one;
+  for (int64_t g = 2; g <= gmax; g = next(g)) best = std::min(best, cost(g));
+  if (5 * best > 4 * one) return 1;
+  for (int64_t g = 2; g <= gmax; g = next(g))
+    if (20 * cost(g) <= 21 * best) return g;
+  return 1;
+}
+
+// Launch one pass of axis j (forward or adjoint) with the axis's form, or,
+// with `io`, a pass of a BF16 chain.
+int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* grad, int grad_shared,
+             float2* out_c, float* out_d, int acc, int64_t batch, cudaStream_t stream, const ChainIo* io = nullptr) {
+  const Axis& ax = p->axis[j];
+  int64_t outer, inner;
+  axis_outer_inner(p, j, &outer, &inner);
+  if (io) {
+    outer = p->M / ax.N;
+    inner = 1;
+  }
+  const unsigned rec_flags = trace_begin(p, stream);
+  const int64_t lines = outer * inner;
+  const int cform = call_form(p, ax, acc ? lines : batch * lines);  // this call's form
+  int rc = FFX_OK;
+  int64_t groups = 1;
+  bool tm32 = false;
+  if (acc && batch > 1) {
+    tm32 = !io && tm32_sum(ax, cform, in, out_d);
+    groups = sum_groups(p, ax, cform, io || (inner == 1 && ax.pl_t[0]), tm32, lines, batch);
+  }
+  if (groups > 1 || tm32) {
+    // partial densities of the groups, then their sum
+    const size_t bytes = (size_t)groups * (size_t)p->M * sizeof(float);
+    if ((rc = ensure_bytes(p, kWsSum, bytes))) return rc;
+    float* part = (float*)p->ws[kWsSum];
+    if (tm32) {
+      rc = run_pass(p, j, adjoint, cform, {outer, inner, p->M, batch, lines, groups}, in, nullptr, 0, nullptr, part, acc,
+                    stream, io);
+    } else {
+      cudaError_t e = cudaMemsetAsync(part, 0, bytes, stream);
+      if (e != cudaSuccess) return cuda_fail(e, "partial densities");
+      const int64_t whole = batch / groups, rem = batch % groups;
+      // realization b G + g is line block g of "realization" b of a layout G times as large
+      rc = run_pass(p, j, adjoint, cform, {groups * outer, inner, groups * p->M, whole, lines, 0}, in, nullptr, 0,
+                    nullptr, part, acc, stream, io);
+      if (!rc && rem) {
+        const int64_t off = whole * groups * p->M;
+        ChainIo rest;
+        if (io) rest = {io->in_bf + off, nullptr, io->plane};
+        rc = run_pass(p, j, adjoint, cform, {rem * outer, inner, rem * p->M, 1, lines, 0}, in ? in + off : nullptr, nullptr,
+                      0, nullptr, part, acc, stream, io ? &rest : nullptr);
+      }
+    }
+    if (rc) return rc;
+    cudaError_t e = launch_group_sum(part, groups, p->M, out_d, stream);
+    if (e != cudaSuccess) return cuda_fail(e, "sum of the partial densities");
+    ++p->launches;
+  } else {
+    rc = run_pass(p, j, adjoint, cform, {outer, inner, p->M, batch, lines, 0}, in, grad, grad_shared, out_c, out_d, acc,
+                  stream, io);
+    if (rc) return rc;
+  }
   trace_end(p, stream, rec_flags);
   return FFX_OK;
 }

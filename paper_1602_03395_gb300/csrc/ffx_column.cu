@@ -47,6 +47,35 @@ __global__ void axis_sum_kernel(const float* __restrict__ rho, int64_t outer, in
   }
 }
 
+// out[i] += sum_g part[g][i], the partial densities of an ensemble sum: a block
+// takes 32 points, its eight warps every eighth group with eight loads in
+// flight; the warps' sums are added in order (deterministic).
+__global__ void __launch_bounds__(256) group_sum_kernel(const float* __restrict__ part, int64_t groups, int64_t M,
+                                                         float* __restrict__ out) {
+  __shared__ float s_sum[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int64_t i = blockIdx.x * (int64_t)32 + lane;
+  float s = 0.f;
+  if (i < M) {
+    int64_t g = w;
+    for (; g + 56 < groups; g += 64) {
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = part[(g + 8 * k) * M + i];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) s += v[k];
+    }
+    for (; g < groups; g += 8) s += part[g * M + i];
+  }
+  s_sum[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && i < M) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += s_sum[k][lane];
+    out[i] += s;
+  }
+}
+
 __device__ __forceinline__ double y_at(double y0, double dy, int64_t j) {
   return __dadd_rn(y0, __dmul_rn(dy, (double)j));  // no contraction: y0 + dy * j as written
 }
@@ -97,6 +126,11 @@ __global__ void fringe_kernel(const float* __restrict__ img, int64_t rows, int64
 }
 
 }  // namespace
+
+cudaError_t launch_group_sum(const float* part, int64_t groups, int64_t M, float* out, cudaStream_t s) {
+  group_sum_kernel<<<(unsigned)((M + 31) / 32), 256, 0, s>>>(part, groups, M, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_axis_sum(const float* rho, int64_t outer, int N, int64_t inner, float scale, int acc, float* out,
                             int sms, cudaStream_t s) {

@@ -100,6 +100,9 @@ struct DenseArgs {
   int N;
   int acc, grad_shared;
   int unsplit;  // tensor-core kernels: one TF32 product (operands rounded, no tails)
+  // 32-point tensor-core passes of an ensemble sum: the realizations in this
+  // many groups, group g's partial densities (not added to) at out_d + g M
+  int64_t groups;
   // passes over BF16 planes (ffx_planes.cu, and the many-instance chains of
   // ffx_tc16.cu): the input (in_bf) and, inside a chain, the output (out_bf)
   // as head and tail planes of 4 bytes a point, bf_plane points apart (the tail
@@ -152,6 +155,8 @@ cudaError_t plane_pass_prepare(int N);
 cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s);
 cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
                                int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s);
+// work items of a pass over ncols lines, and how many run at once
+int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once);
 cudaError_t launch_plane_pass(const DenseArgs& a, const unsigned char* Tblk, int* err, int sms, cudaStream_t s);
 cudaError_t launch_identity(float2* I, int N, cudaStream_t s);
 
@@ -200,6 +205,8 @@ const void* fused_func();
 int fused_threads();
 cudaError_t launch_fused(const FusedArgs& a, int grid, size_t smem, cudaStream_t stream);
 
+// out[i] += sum over g < groups of part[g M + i] (ffx_column.cu).
+cudaError_t launch_group_sum(const float* part, int64_t groups, int64_t M, float* out, cudaStream_t s);
 // Detector readout (ffx_column.cu): sums of a density [outer][N][inner] along
 // N, and the fringe phase of eq. dphase2 per image row.
 cudaError_t launch_axis_sum(const float* rho, int64_t outer, int N, int64_t inner, float scale, int acc, float* out,

@@ -49,6 +49,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstring>
 
 #include "ffx_internal.h"
@@ -892,6 +893,13 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
                     unsplit);
 }
 
+int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
+  // one block per SM, or one pair of blocks per two
+  const int per = pair_pass(N) ? 2 : 1;
+  *at_once = std::max(1, sms / per);
+  return (ncols + per * PL - 1) / (per * PL) * (N / prow_block(N));
+}
+
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
   DenseArgs a = args;
   if (a.oinner == 0) {
@@ -905,13 +913,11 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   if (!row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
     return cudaErrorInvalidValue;
   const int out = a.out_bf ? kOutPlanes : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
-  // one block per SM, or one pair of blocks per two
-  const int per = pair_pass(a.N) ? 2 : 1;
-  int64_t grid = (a.ncols + per * PL - 1) / (per * PL) * (a.N / prow_block(a.N));
-  if (grid > sms / per) grid = sms / per;
+  int64_t at_once;
+  int64_t grid = std::min(plane_pass_tiles(a.N, a.ncols, sms, &at_once), at_once);
   if (grid < 1) grid = 1;
-  grid *= per;
-  if (per == 2) {
+  if (pair_pass(a.N)) {
+    grid *= 2;
     // T's chunks as rows of 128 bytes (stored swizzled)
     if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
     return launch_pdl(kPair[out], (int)grid, PTHREADS, QSMEM, s, a, err, xmap, tmap);

@@ -643,7 +643,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) dense_tc_kernel(const TcParams P)
 // per SM (all 512 columns), [X_hi T_hi | X_hi T_lo] in one N = 256 product
 // (the row block's head and tail rows are contiguous), then X_lo T_hi.
 // NP = 32: 256 columns and 64 KB per block, two blocks per SM (one loads while
-// the other multiplies); three N = 64 products per K-step.  Unsplit launches
+// the other multiplies); three N = 64 products per K-step.  SUM (NP = 32): the
+// ensemble sum; items are (line tile, group of realizations), a block walks a
+// group's realizations in order and keeps the tile's sums of |.|^2 in
+// registers (16 a thread), stored as the group's partial densities (DenseArgs::
+// groups; ffx_column.cu adds the groups).  Bound by a step's latency (loads,
+// split, products, sums, ~2.9 us with two blocks per SM): 256 realizations of
+// 32x32x512 in 0.315 ms, where the streaming kernel, one block per tile, took
+// 0.634 ms.  Unsplit launches
 // write the values rounded to TF32 and run one product per K-step.
 // ---------------------------------------------------------------------------
 constexpr int TM_THREADS = 256;
@@ -661,7 +668,7 @@ struct TmLayout {
   static constexpr int PER_THREAD = NP;                // floats: half a line
 };
 
-template <int NP>
+template <int NP, bool SUM>
 __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
     dense_tm_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err) {
   using L = TmLayout<NP>;
@@ -671,7 +678,9 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int64_t items = (a.ncols + LINES - 1) / LINES;
+  const int64_t tiles = (a.ncols + LINES - 1) / LINES;
+  const int64_t groups = SUM ? a.groups : 1;
+  const int64_t items = tiles * groups;
   if ((int64_t)blockIdx.x >= items) return;
   const int64_t my_items = (items - blockIdx.x + gridDim.x - 1) / gridDim.x;
   const bool unsplit = a.unsplit != 0;
@@ -703,7 +712,15 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
     return bo * NP * inner + i;
   };
   float x[L::PER_THREAD];
-  long long base = line_base((int64_t)blockIdx.x * LINES + 32 * q + lane);
+  // SUM: the next lines to load are those of realization nxt_b of item nxt_w
+  int64_t nxt_w = blockIdx.x, nxt_b = SUM ? nxt_w / tiles : 0;
+  long long base = line_base((SUM ? nxt_w % tiles : nxt_w) * LINES + 32 * q + lane);
+  if (SUM && base >= 0) base += nxt_b * a.M;
+  float racc[SUM ? NP / 2 : 1];
+  if (SUM) {
+#pragma unroll
+    for (int m = 0; m < NP / 2; ++m) racc[m] = 0.f;
+  }
   auto load = [&](long long bs) {
     if (contiguous) {
 #pragma unroll
@@ -729,9 +746,24 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
   bool slices = false, issued = false;
   const uint32_t trow = tmem + ((uint32_t)(32 * q) << 16);
   const uint32_t a_hi = trow + L::A_HI + (uint32_t)(NP * h), a_lo = trow + L::A_LO + (uint32_t)(NP * h);
-  for (int64_t it = 0; it < my_items && !s_abort; ++it) {
+  // steps: an item each, or with SUM an item's realization each (item w's
+  // group w / tiles holds realizations w / tiles, w / tiles + groups, ...)
+  for (int64_t it = 0; it < my_items && !s_abort;) {
     const int64_t ct = blockIdx.x + it * gridDim.x;
     const long long cur = base;
+    const int64_t cur_w = nxt_w;
+    bool more_steps;
+    if (SUM) {
+      nxt_b += groups;
+      if (nxt_b >= a.batch) {
+        nxt_w += gridDim.x;
+        nxt_b = nxt_w / tiles;
+      }
+      more_steps = nxt_w < items;
+    } else {
+      more_steps = it + 1 < my_items;
+    }
+    const bool item_done = !SUM || nxt_w != cur_w;
     // this item's values and tails into tensor memory (the previous item's MMAs are done)
     if (unsplit) {
 #pragma unroll
@@ -759,8 +791,9 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
     tc_fence_before();
     __syncthreads();
     // the next item's lines, in flight during this item's product and stores
-    if (it + 1 < my_items) {
-      base = line_base((ct + gridDim.x) * LINES + 32 * q + lane);
+    if (more_steps) {
+      base = line_base((SUM ? nxt_w % tiles : ct + gridDim.x) * LINES + 32 * q + lane);
+      if (SUM && base >= 0) base += nxt_b * a.M;
       load(base);
     }
     if (tid == 0 && !slices) slices = mbar_wait(smem_u32(&tbar), 0u, &s_abort);
@@ -813,7 +846,17 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
         for (int m = 0; m < 16; ++m) y[m] = __uint_as_float(x1[m]) + __uint_as_float(x2[m]);
       }
       const int n0 = (NP / 2) * h + j0 / 2;  // complex outputs n0 .. n0 + 7
-      if (a.out_c) {
+      if constexpr (SUM) {
+        // (static register indices: j0 is 0 or 16)
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+          const float d = y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
+          if (j0 == 0)
+            racc[m] += d;
+          else
+            racc[8 + m] += d;
+        }
+      } else if (a.out_c) {
         if (contiguous) {
           float4* o = reinterpret_cast<float4*>(a.out_c + cur + n0);
 #pragma unroll
@@ -836,6 +879,20 @@ __global__ void __launch_bounds__(TM_THREADS, TmLayout<NP>::BLOCKS)
         }
       }
     }
+    if constexpr (SUM) {
+      if (item_done) {
+        // the group's partial densities of the tile's lines
+        const long long b0 = line_base((cur_w % tiles) * LINES + 32 * q + lane);
+        if (b0 >= 0) {
+          float* o = a.out_d + (cur_w / tiles) * a.M + b0 + (int64_t)((NP / 2) * h) * inner;
+#pragma unroll
+          for (int m = 0; m < NP / 2; ++m) o[(int64_t)m * inner] = racc[m];
+        }
+#pragma unroll
+        for (int m = 0; m < NP / 2; ++m) racc[m] = 0.f;
+      }
+    }
+    if (item_done) ++it;
     tc_fence_before();
     __syncthreads();  // accumulators read before the next item's product
   }
@@ -897,9 +954,11 @@ cudaError_t dense_tc_prepare() {
     e = cudaFuncSetAttribute(dense_tc_kernel<true, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              TcLayout<true>::SMEM);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dense_tm_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, TmLayout<64>::SMEM);
+    e = cudaFuncSetAttribute(dense_tm_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TmLayout<64>::SMEM);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(dense_tm_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, TmLayout<32>::SMEM);
+    e = cudaFuncSetAttribute(dense_tm_kernel<32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, TmLayout<32>::SMEM);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(dense_tm_kernel<32, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, TmLayout<32>::SMEM);
   return e;
 }
 size_t dense_tc_t_bytes(int N) {
@@ -914,14 +973,18 @@ cudaError_t launch_dense_tc(const DenseArgs& a, const unsigned char* Tblk, int* 
   P.tblk = Tblk;
   P.err = err;
   const int64_t items = (a.ncols + LINES - 1) / LINES;
-  if (a.N == 32 && !a.acc && !a.grad) {
+  if (a.N == 32 && a.groups > 0) {
+    const int64_t units = items * a.groups;
+    const int64_t g = std::min<int64_t>(units, 2 * (int64_t)grid);
+    dense_tm_kernel<32, true><<<(unsigned)g, TM_THREADS, TmLayout<32>::SMEM, stream>>>(a, Tblk, err);
+  } else if (a.N == 32 && !a.acc && !a.grad) {
     // two blocks per SM (grid = the SMs when the pass has more items than SMs)
     const int64_t g = items > grid ? std::min<int64_t>(items, 2 * (int64_t)grid) : grid;
-    dense_tm_kernel<32><<<(unsigned)g, TM_THREADS, TmLayout<32>::SMEM, stream>>>(a, Tblk, err);
+    dense_tm_kernel<32, false><<<(unsigned)g, TM_THREADS, TmLayout<32>::SMEM, stream>>>(a, Tblk, err);
   } else if (a.N == 64 && !a.acc && !a.grad && items <= 4 * (int64_t)grid) {
     // a few items per block: the input operand in tensor memory, no pipeline
     // to fill (measured 7-14% faster at up to ~2 items per SM, 6% slower at 13)
-    dense_tm_kernel<64><<<grid, TM_THREADS, TmLayout<64>::SMEM, stream>>>(a, Tblk, err);
+    dense_tm_kernel<64, false><<<grid, TM_THREADS, TmLayout<64>::SMEM, stream>>>(a, Tblk, err);
   } else if (a.N == 64 && !a.acc && !a.grad) {
     // T (128 KB) stays in shared memory for the whole launch
     dense_tc_kernel<true, false, true><<<grid, NTHREADS, TcLayout<true>::SMEM, stream>>>(P);
