@@ -740,7 +740,9 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
     fused_call = plan.fused and B_ <= plan.fused_max_batch  # all d passes in one launch
     call_forms = plan.call_forms(B_)  # the kernel each axis runs at this batch
     # BF16 chain: one launch splits the input into BF16 planes, then the passes
+    # (a chain whose first pass runs on CTA pairs has no split launch)
     chain = plan.bf16_chain(B_) and args.column is None
+    split = chain and plan.chain_split(B_)
     if args.column is None:
         out_shape = (B_,) + tuple(w.dims)
 
@@ -869,7 +871,7 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
         mean_ms = [ms / args.steps]
         launch_time = "one launch per step: the timed region's step time (CUDA events at its ends)"
     # the lattice axis of each traced launch (None: the BF16 split of a chain)
-    launch_axis = ([None] if chain else []) + list(order)
+    launch_axis = ([None] if split else []) + list(order)
     dom = max((k for k in range(launches) if fused_call or launch_axis[k] is not None), key=lambda k: mean_ms[k])
     pk, pk_src = peaks()
     sm_max = float(pk.get("sm_max_mhz", 2070.0))
@@ -1043,7 +1045,7 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
                          "peak": hbm_peak, "unit": "GB/s",
                          "frac": bytes_launch / (mean_ms[dom] * 1e-3) / 1e9 / hbm_peak,
                          "note": f"of {pk_src} hbm_gbs; one read + one write of the batch"},
-        "hbm_step": hbm_step_record(w, B_, chain, fused_call, out_bytes, ms / args.steps, hbm_peak, pk_src),
+        "hbm_step": hbm_step_record(w, B_, split, fused_call, out_bytes, ms / args.steps, hbm_peak, pk_src),
         "pass_ms": {pass_names[k]: mean_ms[k] for k in range(launches)},
         "e2e": {"value": e2e_value, "unit": UNIT, "api": e2e_api, "lanes": lanes_used,
                 "h2d_bytes_per_step": B_ * M * 8,

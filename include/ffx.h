@@ -436,8 +436,8 @@ int ffx_plan_axis_form(ffx_plan_t plan, int axis);
 
 /* Number of kernel launches one ffx_expand / ffx_expand_backward call makes
  * with a batch of one.  A call that runs as a BF16 chain
- * (ffx_plan_bf16_chain) makes one more: the split of its input into BF16
- * planes (in ffx_expand_backward: the forward half of a 3-D plan). */
+ * (ffx_plan_bf16_chain) makes one more where ffx_plan_chain_split says so: the
+ * split of its input into BF16 planes (in ffx_expand_backward: the forward half of a 3-D plan). */
 int ffx_launches_per_call(ffx_plan_t plan, int backward);
 
 /* The largest batch for which ffx_expand and ffx_expand_field run as one
@@ -484,6 +484,12 @@ int64_t ffx_plan_launch_count(ffx_plan_t plan);
  * split it into, so the results are those of the per-axis passes in the same
  * order).  The planes use the plan's two field workspaces. */
 int ffx_plan_bf16_chain(ffx_plan_t plan, int64_t batch);
+
+/* 1 if such a chain starts with a launch that splits its FP32 input into
+ * planes; 0 if its first pass reads the FP32 input itself (a last axis of 256
+ * points or more, in multiples of 128, with enough lines to fill the chip) or
+ * the call is no chain. */
+int ffx_plan_chain_split(ffx_plan_t plan, int64_t batch);
 
 /* Forward pass order: writes the lattice axis of pass k to order[k],
  * k = 0..ndim-1.  The adjoint runs the same axes in reverse. */

@@ -390,12 +390,12 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
     if (io) {
       if (!ax.pl_t[adjoint ? 1 : 0] || tm64 || grad)
         return fail(FFX_EUNSUPPORTED, "internal: a BF16 chain pass of axis %d without the BF16 kernel", j);
-      d.in_bf = io->in_bf;
+      d.in_bf = io->in_bf;  // or NULL: the FP32 lines `in`
       d.out_bf = io->out_bf;
       d.bf_plane = io->plane;
       d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
       d.oouter = outer / d.oinner;
-    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1) {
+    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_splits(ax.N, d.ncols, p->sms)) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
       // cores' layout instead of converting them on the way
@@ -409,7 +409,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.bf_plane = plane;
       d.in = nullptr;
     }
-    if (d.in_bf)
+    if (io || (ax.pl_t[0] && !tm64 && !grad && inner == 1))
       e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
     else if (ax.bf_t[0] && !tm64)
       e = launch_dense_bf16(d, ax.bf_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
@@ -649,33 +649,44 @@ bool bf16_adjoint_ok(const ffx_plan_s* p) {
   return true;
 }
 
+// Whether a forward chain starts with a split of its input (else its first pass
+// reads the FP32 input itself).
+bool chain_splits(const ffx_plan_s* p, int64_t batch) {
+  const Axis& ax = p->axis[p->order[0]];
+  return !plane_pass_splits(ax.N, batch * (p->M / ax.N), p->sms);
+}
+
 // The forward map of a batch as a BF16 chain: the input split into BF16
 // planes in ws[1] (head plane, then tail plane: 8 bytes a point, the size of
 // a complex64 field), then the passes in the plan's order (the last axis
 // first), each reading planes and writing planes (ws[0], ws[1], ...), the
 // last one the caller's field (out_c) or densities (out_d, summed over the
-// batch with FFX_ACCUMULATE).  `in` is read by the split alone, so out_c may
-// equal it; it must not be ws[1].
+// batch with FFX_ACCUMULATE).  `in` is read by the split (or the first pass,
+// which writes ws[0]) alone, so out_c may equal it; it must not be ws[1] or, if
+// the first pass reads it, ws[0].
 int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, float* out_d, cudaStream_t s) {
   const int d = p->ndim;
   int rc;
   if ((rc = ensure_ws(p, 0, batch)) || (rc = ensure_ws(p, 1, batch))) return rc;
   const int64_t plane = batch * p->M;
   const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
-  const unsigned rec = trace_begin(p, s);
-  cudaError_t e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit, p->sms, s);
-  if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the input");
-  ++p->launches;
-  trace_end(p, s, rec);
-  const uint32_t* cur_bf = (const uint32_t*)p->ws[1];
+  const uint32_t* cur_bf = nullptr;
+  if (chain_splits(p, batch)) {
+    const unsigned rec = trace_begin(p, s);
+    cudaError_t e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit, p->sms, s);
+    if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the input");
+    ++p->launches;
+    trace_end(p, s, rec);
+    cur_bf = (const uint32_t*)p->ws[1];
+  }
   for (int r = 0; r < d; ++r) {
     const bool last = r == d - 1;
     ChainIo io;
     io.in_bf = cur_bf;
     io.out_bf = last ? nullptr : (uint32_t*)p->ws[r & 1];
     io.plane = plane;
-    rc = run_axis(p, p->order[r], false, nullptr, nullptr, 0, last ? out_c : nullptr, last ? out_d : nullptr,
-                  last && out_d ? p->acc : 0, batch, s, &io);
+    rc = run_axis(p, p->order[r], false, cur_bf ? nullptr : in, nullptr, 0, last ? out_c : nullptr,
+                  last ? out_d : nullptr, last && out_d ? p->acc : 0, batch, s, &io);
     if (rc) return rc;
     cur_bf = io.out_bf;
   }
@@ -1615,6 +1626,11 @@ int ffx_plan_bf16_chain(ffx_plan_t p, int64_t batch) {
   if (p->many || batch <= p->fused) return 0;
   const void* aligned = (const void*)(uintptr_t)16;
   return bf16_chain_ok(p, batch, aligned, aligned, aligned) ? 1 : 0;
+}
+
+int ffx_plan_chain_split(ffx_plan_t p, int64_t batch) {
+  if (ffx_plan_bf16_chain(p, batch) != 1) return 0;
+  return chain_splits(p, batch) ? 1 : 0;
 }
 
 int64_t ffx_plan_launch_count(ffx_plan_t p) { return p ? p->launches : -1; }

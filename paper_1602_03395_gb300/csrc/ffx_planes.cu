@@ -50,7 +50,6 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
-#include <cstring>
 
 #include "ffx_internal.h"
 #include "ffx_pdl.h"
@@ -574,15 +573,64 @@ constexpr int QSTAGE = PX + QTP + QTQ;    // 56 KB
 constexpr int QSMEM = QST * QSTAGE + 1024;
 static_assert(QSMEM <= 226 * 1024, "shared memory");
 
-template <int OUT>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
+// F32: the input is contiguous FP32 lines, split on the way in (the first pass
+// of a chain, or a single pass).  The FP32 tile of a chunk (two boxes of 16
+// points a line, 128-byte swizzle) is exactly as large as its head and tail
+// rows and lands where they go: row n of the first box on head row n, of the
+// second on tail row n.  Four producer warps (12-15), a thread a line, read
+// their line's 256 bytes, split them and write the two rows over them, so no
+// thread waits for another.  Registers move from the control and producer warps
+// to the epilogue's (setmaxnreg): 56 + 2 x 176 + 104 a thread of the four
+// warpgroups, the 4 x 128 of the launch.  Splitting loads shared memory with 64
+// KB more a chunk (232 KB, 1812 clocks against 1536 of products), and every row
+// block splits its lines again, but the separate split reads and writes 16
+// bytes a point of HBM.
+constexpr int QTHREADS_F32 = PTHREADS + 128;
+static_assert(QTHREADS_F32 == 512 && 56 + 2 * 176 + 104 == 4 * 128, "register split");
+static_assert(PL == 128, "a producer thread per line");
+
+// Splits line n of a chunk's FP32 tile at x into its head and tail rows.
+__device__ __forceinline__ void split_line(unsigned char* x, int n, bool unsplit) {
+  unsigned char* const row = x + n * 128;
+  const int sw = n & 7;
+  float4 v[2][8];
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[g][c] = *reinterpret_cast<const float4*>(row + g * PXPART + ((c ^ sw) << 4));
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      // eight points of group g: 16 bytes of real and of imaginary parts
+      uint32_t r[4], m[4], rl[4], ml[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4 f = v[g][4 * k + c];
+        r[c] = bf2(f.x, f.z);
+        m[c] = bf2(f.y, f.w);
+        rl[c] = bf2(f.x - bf_lo(r[c]), f.z - bf_hi(r[c]));
+        ml[c] = bf2(f.y - bf_lo(m[c]), f.w - bf_hi(m[c]));
+      }
+      const int ore = ((4 * g + k) ^ sw) << 4, oim = ((4 * g + 2 + k) ^ sw) << 4;
+      *reinterpret_cast<uint4*>(row + ore) = make_uint4(r[0], r[1], r[2], r[3]);
+      *reinterpret_cast<uint4*>(row + oim) = make_uint4(m[0], m[1], m[2], m[3]);
+      if (!unsplit) {
+        *reinterpret_cast<uint4*>(row + PXPART + ore) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+        *reinterpret_cast<uint4*>(row + PXPART + oim) = make_uint4(ml[0], ml[1], ml[2], ml[3]);
+      }
+    }
+}
+
+template <int OUT, bool F32>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? QTHREADS_F32 : PTHREADS, 1)
     plane_pair_kernel(const DenseArgs a, int* err,
                       const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap tmap) {
   constexpr int RB = 128;
   constexpr bool ACC = OUT == kOutSum;
   extern __shared__ __align__(1024) unsigned char psm_raw[];
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t full_bar[QST], empty_bar[QST];
+  __shared__ __align__(8) uint64_t full_bar[QST], empty_bar[QST], raw_bar[QST];
   __shared__ __align__(8) uint64_t accf_bar[2], acce_bar[2], done_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
@@ -603,7 +651,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
   if (warp == 1) tmem2_alloc(&tmem_slot, 512);
   if (tid == 0) {
     for (int s = 0; s < QST; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), 1);
+      // FP32 input: and the eight producer warps of the pair
+      mbar_init(smem_u32(&full_bar[s]), F32 ? 9 : 1);
+      mbar_init(smem_u32(&raw_bar[s]), 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -623,124 +673,164 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(PTHREADS, 1)
   const uint32_t stages = smem_u32(psm);
   const int64_t total = my_items * nb * kchunks;
 
-  if (warp == 0) {
-    // ---------------- copies: each CTA's own, completing on the even CTA's barriers ----------------
-    if (lane == 0) {
-      const uint64_t xmap_addr = reinterpret_cast<uint64_t>(&xmap), tmap_addr = reinterpret_cast<uint64_t>(&tmap);
-      const uint32_t bytes = unsplit ? (uint32_t)(PXPART + QTQ) : (uint32_t)QSTAGE;
-      const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
-      pdl_wait();
-      int64_t iw = pair, u = 0;
-      int ib = 0, ikc = 0, is = 0;
+  if (warp < 4) {
+    if constexpr (F32) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (warp == 0) {
+      // ---------------- copies: each CTA's own, completing on the even CTA's barriers ----------------
+      if (lane == 0) {
+        const uint64_t xmap_addr = reinterpret_cast<uint64_t>(&xmap), tmap_addr = reinterpret_cast<uint64_t>(&tmap);
+        const uint32_t bytes = unsplit ? (uint32_t)((F32 ? 0 : PXPART) + QTQ) : (uint32_t)(QSTAGE - (F32 ? PX : 0));
+        const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
+        pdl_wait();
+        int64_t iw = pair, u = 0;
+        int ib = 0, ikc = 0, is = 0;
 #pragma unroll 1
-      for (int64_t ci = 0; ci < total; ++ci) {
-        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
-        const int64_t wt = iw / mtiles;
-        const int mt = (int)(iw - wt * mtiles);
-        const uint32_t st = stages + (uint32_t)(is * QSTAGE);
-        const uint32_t fb = full0 + 8u * (uint32_t)is;
-        if (rank == 0) mbar_expect_tx(smem_u32(&full_bar[is]), 2u * bytes);
-        // a tile past the last line reads zeros
-        const int row = (int)((2 * wt + rank) * PL + (ACC ? (int64_t)ib * a.outer : 0));
-        asm volatile(
-            "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-            "%4}], [%5];" ::"r"(st),
-            "l"(xmap_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
-            : "memory");
-        // T's rows of the chunk, 64 a tile
-        const int trow = (mt * kchunks + ikc) * (2 * RB);
-        auto copy_t = [&](uint32_t dst, int r) {
-          asm volatile(
-              "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-              "[%4];" ::"r"(dst),
-              "l"(tmap_addr), "r"(0), "r"(trow + r), "r"(fb)
-              : "memory");
-        };
-        if (!unsplit) {
-          copy_t(st + (uint32_t)PX, rank * RB);
-          copy_t(st + (uint32_t)(PX + QTQ), rank * RB + 64);
+        for (int64_t ci = 0; ci < total; ++ci) {
+          if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
+          const int64_t wt = iw / mtiles;
+          const int mt = (int)(iw - wt * mtiles);
+          const uint32_t st = stages + (uint32_t)(is * QSTAGE);
+          const uint32_t fb = full0 + 8u * (uint32_t)is;
+          if (rank == 0) mbar_expect_tx(smem_u32(&full_bar[is]), 2u * bytes);
+          // a tile past the last line reads zeros
+          const int row = (int)((2 * wt + rank) * PL + (ACC ? (int64_t)ib * a.outer : 0));
+          if (F32) {
+            const uint32_t rb = smem_u32(&raw_bar[is]);
+            mbar_expect_tx(rb, PX);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              asm volatile(
+                  "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                  "[%4];" ::"r"(st + (uint32_t)(h * PXPART)),
+                  "l"(xmap_addr), "r"(ikc * 2 * PKC + 32 * h), "r"(row), "r"(rb)
+                  : "memory");
+          } else {
+            asm volatile(
+                "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+                "%3, %4}], [%5];" ::"r"(st),
+                "l"(xmap_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
+                : "memory");
+          }
+          // T's rows of the chunk, 64 a tile
+          const int trow = (mt * kchunks + ikc) * (2 * RB);
+          auto copy_t = [&](uint32_t dst, int r) {
+            asm volatile(
+                "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                "[%4];" ::"r"(dst),
+                "l"(tmap_addr), "r"(0), "r"(trow + r), "r"(fb)
+                : "memory");
+          };
+          if (!unsplit) {
+            copy_t(st + (uint32_t)PX, rank * RB);
+            copy_t(st + (uint32_t)(PX + QTQ), rank * RB + 64);
+          }
+          copy_t(st + (uint32_t)(PX + QTP), rank * 64);
+          if (++is == QST) {
+            is = 0;
+            ++u;
+          }
+          if (++ikc == kchunks) {
+            ikc = 0;
+            if (++ib == nb) {
+              ib = 0;
+              iw += npairs;
+            }
+          }
         }
-        copy_t(st + (uint32_t)(PX + QTP), rank * 64);
-        if (++is == QST) {
-          is = 0;
-          ++u;
+        // no copy of either CTA may still be in flight at exit (the odd CTA
+        // leaves after the cluster barrier below)
+        for (int q = 0; q < QST; ++q) {
+          const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+          if (uq < 0) continue;
+          if (F32) mbar_wait_own(smem_u32(&raw_bar[q]), (uint32_t)(uq & 1), &s_abort);
+          if (rank == 0) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
         }
-        if (++ikc == kchunks) {
-          ikc = 0;
-          if (++ib == nb) {
-            ib = 0;
-            iw += npairs;
+      }
+      __syncwarp();
+    } else if (warp == 1 && rank == 0) {
+      // ---------------- products: the whole warp, one elected lane issuing ----------------
+      bool ok = true;
+      int s = 0;
+      int64_t u = 0;
+      const uint32_t id1 = idesc_bf16(2 * PL, RB), id2 = idesc_bf16(2 * PL, 2 * RB);
+      const uint32_t dre = tmem, dim = tmem + 2 * RB;
+#pragma unroll 1
+      for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
+        const uint32_t prev = (uint32_t)((sub - 1) & 1);
+#pragma unroll 1
+        for (int kc = 0; kc < kchunks; kc += 2) {
+          const int s0 = s, s1 = s + 1;  // QST is even: a pair of chunks never wraps
+          const uint32_t ph = (uint32_t)(u & 1);
+          const uint32_t st0 = stages + (uint32_t)(s0 * QSTAGE), st1 = st0 + QSTAGE;
+          const bool last = kc == kchunks - 2;
+          ok = mbar_wait_cluster(smem_u32(&full_bar[s0]), ph, &s_abort) &&
+               (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
+          if (!ok) break;
+          tc_fence_after();
+          plane_half<2, RB, false>(dre, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
+          if (!ok) break;
+          tc_fence_after();
+          plane_half<2, RB, false>(dre, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          if (last) {
+            if (elect_one()) mma2_commit_both(smem_u32(&accf_bar[0]));
+            __syncwarp();
+          }
+          if (kc == 0 && sub > 0) {
+            ok = mbar_wait_cluster(smem_u32(&acce_bar[1]), prev, &s_abort);
+            if (!ok) break;
+            tc_fence_after();
+          }
+          plane_half<2, RB, true>(dim, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          if (elect_one()) mma2_commit_both(smem_u32(&empty_bar[s0]));
+          __syncwarp();
+          plane_half<2, RB, true>(dim, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          if (elect_one()) {
+            mma2_commit_both(smem_u32(&empty_bar[s1]));
+            if (last) mma2_commit_both(smem_u32(&accf_bar[1]));
+          }
+          __syncwarp();
+          s += 2;
+          if (s == QST) {
+            s = 0;
+            ++u;
           }
         }
       }
-      // no copy of either CTA may still be in flight at exit (the odd CTA
-      // leaves after the cluster barrier below)
-      if (rank == 0)
-        for (int q = 0; q < QST; ++q) {
-          const int64_t uq = q < is ? u : u - 1;  // stage q's last use
-          if (uq >= 0) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
-        }
+      // whatever happened, the tensor cores finish this warp's work before exit
+      if (elect_one()) mma2_commit(smem_u32(&done_bar));
+      __syncwarp();
+      mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
     }
-    __syncwarp();
-  } else if (warp == 1 && rank == 0) {
-    // ---------------- products: the whole warp, one elected lane issuing ----------------
-    bool ok = true;
-    int s = 0;
-    int64_t u = 0;
-    const uint32_t id1 = idesc_bf16(2 * PL, RB), id2 = idesc_bf16(2 * PL, 2 * RB);
-    const uint32_t dre = tmem, dim = tmem + 2 * RB;
+  } else if (warp < 12) {
+    // ---------------- epilogue ----------------
+    if constexpr (F32) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+    const uint32_t acce0 = map_rank(smem_u32(&acce_bar[0]), 0u);
+    plane_epilogue<RB, OUT>(a, warp, lane, tmem, smem_u32(&accf_bar[0]), pair, npairs, my_items, mtiles, 2, rank, nb,
+                            unsplit, &s_abort, [&](int bar) { mbar_arrive_cluster_relaxed(acce0 + 8u * (uint32_t)bar); });
+  } else {
+    // ---------------- FP32 input: split into the stages ----------------
+    if constexpr (F32) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+      const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
+      const int n = tid - 384;  // the tile's line
+      int s = 0;
+      int64_t u = 0;
 #pragma unroll 1
-    for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
-      const uint32_t prev = (uint32_t)((sub - 1) & 1);
-#pragma unroll 1
-      for (int kc = 0; kc < kchunks; kc += 2) {
-        const int s0 = s, s1 = s + 1;  // QST is even: a pair of chunks never wraps
-        const uint32_t ph = (uint32_t)(u & 1);
-        const uint32_t st0 = stages + (uint32_t)(s0 * QSTAGE), st1 = st0 + QSTAGE;
-        const bool last = kc == kchunks - 2;
-        ok = mbar_wait_cluster(smem_u32(&full_bar[s0]), ph, &s_abort) &&
-             (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
-        if (!ok) break;
-        tc_fence_after();
-        plane_half<2, RB, false>(dre, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
-        ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
-        if (!ok) break;
-        tc_fence_after();
-        plane_half<2, RB, false>(dre, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
-        if (last) {
-          if (elect_one()) mma2_commit_both(smem_u32(&accf_bar[0]));
-          __syncwarp();
-        }
-        if (kc == 0 && sub > 0) {
-          ok = mbar_wait_cluster(smem_u32(&acce_bar[1]), prev, &s_abort);
-          if (!ok) break;
-          tc_fence_after();
-        }
-        plane_half<2, RB, true>(dim, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
-        if (elect_one()) mma2_commit_both(smem_u32(&empty_bar[s0]));
+      for (int64_t ci = 0; ci < total; ++ci) {
+        bool ok = true;
+        if (lane == 0) ok = mbar_wait(smem_u32(&raw_bar[s]), (uint32_t)(u & 1), &s_abort);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        split_line(psm + s * QSTAGE, n, unsplit);
+        fence_async_smem();
         __syncwarp();
-        plane_half<2, RB, true>(dim, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
-        if (elect_one()) {
-          mma2_commit_both(smem_u32(&empty_bar[s1]));
-          if (last) mma2_commit_both(smem_u32(&accf_bar[1]));
-        }
-        __syncwarp();
-        s += 2;
-        if (s == QST) {
+        if (lane == 0) mbar_arrive_cluster(full0 + 8u * (uint32_t)s);
+        if (++s == QST) {
           s = 0;
           ++u;
         }
       }
     }
-    // whatever happened, the tensor cores finish this warp's work before exit
-    if (elect_one()) mma2_commit(smem_u32(&done_bar));
-    __syncwarp();
-    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
-  } else if (warp >= 4) {
-    // ---------------- epilogue ----------------
-    const uint32_t acce0 = map_rank(smem_u32(&acce_bar[0]), 0u);
-    plane_epilogue<RB, OUT>(a, warp, lane, tmem, smem_u32(&accf_bar[0]), pair, npairs, my_items, mtiles, 2, rank, nb,
-                            unsplit, &s_abort, [&](int bar) { mbar_arrive_cluster_relaxed(acce0 + 8u * (uint32_t)bar); });
   }
 
   tc_fence_before();
@@ -823,8 +913,11 @@ bool pair_pass(int N) { return N >= 256 && N % 128 == 0; }
 
 using PKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap);
 using QKernel = void (*)(const DenseArgs, int*, const CUtensorMap, const CUtensorMap);
-const QKernel kPair[kPOuts] = {plane_pair_kernel<kOutPlanes>, plane_pair_kernel<kOutComplex>,
-                               plane_pair_kernel<kOutDensity>, plane_pair_kernel<kOutSum>};
+template <bool F32>
+struct QVariant {
+  static constexpr QKernel fn[kPOuts] = {plane_pair_kernel<kOutPlanes, F32>, plane_pair_kernel<kOutComplex, F32>,
+                                         plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>};
+};
 template <int RB, bool RES>
 struct PVariant {
   static constexpr PKernel fn[kPOuts] = {plane_pass_kernel<RB, RES, kOutPlanes>, plane_pass_kernel<RB, RES, kOutComplex>,
@@ -840,19 +933,23 @@ PKernel single_kernel(int N, int out) {
 }
 int single_smem(int N) { return N <= 128 ? psmem(N, true) : psmem(96, false); }
 
-// `rows` rows of 64 BF16 values in tiles of box_rows, `planes` of them `stride`
-// bytes apart
+// `rows` rows of `cols` FP32 values (a multiple of 32) in tiles of 32 x box_rows
+bool f32_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int box_rows) {
+  const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
+  const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
+  const cuuint32_t box[2] = {32, (cuuint32_t)box_rows};
+  return make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+// `rows` rows of `cols` BF16 values in tiles of 64 x box_rows, `planes` of them
+// `stride` bytes apart
 bool row_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int planes, int64_t stride, int box_rows,
              bool swizzle) {
-  std::memset(map, 0, sizeof(*map));
-  const EncodeTiledFn enc = encode_tiled();
-  if (!enc) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
   const cuuint64_t strides[2] = {(cuuint64_t)cols * 2, (cuuint64_t)stride};
-  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)planes}, estr[3] = {1, 1, 1};
-  return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, stride ? 3 : 2, const_cast<void*>(base), dims, strides, box, estr,
-             CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
-             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+  const cuuint32_t box[3] = {64, (cuuint32_t)box_rows, (cuuint32_t)planes};
+  return make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, stride ? 3 : 2, base, dims, strides, box,
+                       swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
 }  // namespace
@@ -866,9 +963,14 @@ size_t plane_t_bytes(int N) { return (size_t)N * N * 8; }
 cudaError_t plane_pass_prepare(int N) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < kPOuts && e == cudaSuccess; ++k)
-    e = pair_pass(N) ? cudaFuncSetAttribute((const void*)kPair[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM)
-                     : cudaFuncSetAttribute((const void*)single_kernel(N, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                            single_smem(N));
+    if (pair_pass(N)) {
+      e = cudaFuncSetAttribute((const void*)QVariant<false>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
+      if (e == cudaSuccess)
+        e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
+    } else {
+      e = cudaFuncSetAttribute((const void*)single_kernel(N, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               single_smem(N));
+    }
   return e;
 }
 
@@ -893,6 +995,11 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
                     unsplit);
 }
 
+bool plane_pass_splits(int N, int64_t ncols, int sms) {
+  int64_t at_once;
+  return pair_pass(N) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
+}
+
 int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
   // one block per SM, or one pair of blocks per two
   const int per = pair_pass(N) ? 2 : 1;
@@ -906,11 +1013,13 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     a.oouter = a.outer;
     a.oinner = a.inner;
   }
-  if (a.inner != 1 || !a.in_bf) return cudaErrorInvalidValue;
+  const bool f32 = !a.in_bf;
+  if (a.inner != 1 || a.grad || (f32 && !pair_pass(a.N))) return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
-  // bf_plane points after the head plane
+  // bf_plane points after the head plane; or the FP32 lines
   CUtensorMap xmap, tmap;
-  if (!row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
+  if (f32 ? !f32_map(&xmap, a.in, 2 * a.N, a.batch * a.outer, PL)
+          : !row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
     return cudaErrorInvalidValue;
   const int out = a.out_bf ? kOutPlanes : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
   int64_t at_once;
@@ -920,7 +1029,8 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     grid *= 2;
     // T's chunks as rows of 128 bytes (stored swizzled)
     if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
-    return launch_pdl(kPair[out], (int)grid, PTHREADS, QSMEM, s, a, err, xmap, tmap);
+    return launch_pdl(f32 ? QVariant<true>::fn[out] : QVariant<false>::fn[out], (int)grid,
+                      f32 ? QTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
   return launch_pdl(single_kernel(a.N, out), (int)grid, PTHREADS, single_smem(a.N), s, a, Tblk, err, xmap);
 }

@@ -1224,18 +1224,13 @@ namespace {
 void input_map(const DenseArgs& a, CUtensorMap* map, int* mode) {
   std::memset(map, 0, sizeof(*map));
   *mode = kInPlace;
-  const EncodeTiledFn enc = encode_tiled();
-  if (a.grad || a.inner != 1 || !enc) return;
+  if (a.grad || a.inner != 1) return;
   const cuuint64_t rows = (cuuint64_t)a.batch * (cuuint64_t)a.outer;  // every realization's lines
   const cuuint64_t dims[2] = {(cuuint64_t)(2 * a.N), rows};
   const cuuint64_t strides[1] = {(cuuint64_t)(2 * a.N) * 4};
-  const cuuint32_t box[2] = {32, (cuuint32_t)BL}, estr[2] = {1, 1};
-  if (enc(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)a.in, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)
+  const cuuint32_t box[2] = {32, (cuuint32_t)BL};
+  if (make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.in, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
     *mode = kTmaContiguous;
-  else
-    std::memset(map, 0, sizeof(*map));
 }
 
 }  // namespace
@@ -1244,37 +1239,25 @@ bool many_bf16_line_map(const float2* base, int N, int64_t lines, void* map) {
   // [lines][2N floats], boxes of 32 floats x 128 lines, 128-byte swizzle: the
   // map of the uniform kernel's TMA tiles of contiguous lines
   std::memset(map, 0, sizeof(CUtensorMap));
-  const EncodeTiledFn enc = encode_tiled();
-  if (!enc || lines < 1 || (reinterpret_cast<uintptr_t>(base) & 15u)) return false;
+  if (lines < 1 || (reinterpret_cast<uintptr_t>(base) & 15u)) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)(2 * N), (cuuint64_t)lines};
   const cuuint64_t strides[1] = {(cuuint64_t)(2 * N) * 4};
-  const cuuint32_t box[2] = {32, (cuuint32_t)BL}, estr[2] = {1, 1};
-  if (enc(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void*)base, dims, strides, box, estr,
-          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
-    std::memset(map, 0, sizeof(CUtensorMap));
-    return false;
-  }
-  return true;
+  const cuuint32_t box[2] = {32, (cuuint32_t)BL};
+  return make_tile_map(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box,
+                       CU_TENSOR_MAP_SWIZZLE_128B);
 }
 static_assert(sizeof(CUtensorMap) == 128, "tile maps are 128 bytes");
 
 bool many_bf16_plane_map(const uint32_t* head, int N, int64_t lines, int64_t plane, void* map) {
   // [plane][line][2N bf16], boxes of 64 values x 128 lines x both planes, 128-byte
-  // swizzle: the map of the uniform kernel's BF16-plane tiles
+  // swizzle
   std::memset(map, 0, sizeof(CUtensorMap));
-  const EncodeTiledFn enc = encode_tiled();
-  if (!enc || lines < 1 || (reinterpret_cast<uintptr_t>(head) & 15u) || ((plane * 4) & 15)) return false;
+  if (lines < 1 || (reinterpret_cast<uintptr_t>(head) & 15u) || ((plane * 4) & 15)) return false;
   const cuuint64_t dims[3] = {(cuuint64_t)(2 * N), (cuuint64_t)lines, 2u};
   const cuuint64_t strides[2] = {(cuuint64_t)(2 * N) * 2, (cuuint64_t)plane * 4};
-  const cuuint32_t box[3] = {(cuuint32_t)BKC, (cuuint32_t)BL, 2u}, estr[3] = {1, 1, 1};
-  if (enc(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)head, dims, strides, box,
-          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS) {
-    std::memset(map, 0, sizeof(CUtensorMap));
-    return false;
-  }
-  return true;
+  const cuuint32_t box[3] = {(cuuint32_t)BKC, (cuuint32_t)BL, 2u};
+  return make_tile_map(reinterpret_cast<CUtensorMap*>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, head, dims, strides, box,
+                       CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 cudaError_t launch_dense_bf16(const DenseArgs& a, const unsigned char* Tblk, int* err, int grid, cudaStream_t s) {

@@ -214,6 +214,11 @@ __device__ __forceinline__ uint32_t map_rank(uint32_t saddr, uint32_t rank) {
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(saddr), "r"(rank));
   return r;
 }
+// Arrive on a barrier of either CTA (a shared::cluster address), after this
+// thread's shared-memory writes.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t mbar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(mbar) : "memory");
+}
 // Arrive on a barrier of either CTA (a shared::cluster address) without
 // ordering this thread's earlier memory writes: for barriers that only pass on
 // tensor-memory columns already read back.  (A release at cluster scope waits

@@ -66,3 +66,72 @@ def test_plane_passes(ffx, dims, lam, batch):
     assert rel_l2(acc, start + dens.sum(0)) < DENSITY_TOL
     assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
     assert rel_l2(rough, dens) < UNSPLIT_TOL
+
+
+# passes that fill the chip on CTA pairs read their FP32 lines themselves: whole
+# and ragged last tiles, chains and single passes, several row blocks
+FP32_CASES = [
+    ((96, 64, 256), (4, 5, 6), 4),     # chain: 24576 lines of 256
+    ((64, 1024), (5, 6), 160),         # chain: 10240 lines of 1024, eight row blocks
+    ((512,), (7,), 4900),              # single pass: a last tile of 36 lines
+    ((384,), (5,), 13001),             # ... and half a pair without lines
+    ((32, 32, 256), (3, 4, 5), 10),    # per-axis passes behind it
+]
+
+
+@pytest.mark.parametrize("dims,lam,batch", FP32_CASES)
+def test_pair_pass_of_fp32_lines(ffx, dims, lam, batch):
+    rng = np.random.default_rng(batch + sum(dims))
+    dx, t = (0.25,) * len(dims), 6.0
+    psi = random_field(rng, (batch,) + dims)
+    ref = O.expand_field(psi, dx, t, lam)
+    dens = np.abs(ref) ** 2
+    x = to_dev(psi)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
+        n0 = plan.launch_count()
+        rho = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.launch_count() - n0 == len(dims)  # no split launch
+        fld = ffx.ffx_expand_field(plan, x).cpu().numpy()
+        y = x.clone()
+        ffx.ffx_expand_field(plan, y, y)              # in place
+        assert np.array_equal(y.cpu().numpy(), fld)
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, accumulate=True) as plan:
+        acc = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, unsplit=True) as plan:
+        rough = ffx.ffx_expand(plan, x).cpu().numpy()
+    assert rel_l2(rho, dens) < DENSITY_TOL
+    assert rel_l2(fld, ref) < FIELD_TOL
+    assert rel_l2(acc, dens.sum(0)) < DENSITY_TOL
+    assert rel_l2(rough, dens) < UNSPLIT_TOL
+
+
+def test_first_cuda_call_of_a_thread(ffx):
+    """A call that starts with a tile map, from a thread that made no CUDA call
+    yet (as an autograd worker may): the same result as from this thread."""
+    import threading
+
+    import torch
+
+    dims, lam, batch = (96, 64, 256), (4, 5, 6), 4
+    x = to_dev(random_field(np.random.default_rng(3), (batch,) + dims))
+    stream = torch.cuda.current_stream()
+    with ffx.Plan(dims, (0.25,) * 3, 6.0, lam) as plan:
+        want = ffx.ffx_expand(plan, x)
+        out = torch.zeros_like(want)
+        torch.cuda.synchronize()
+        failures = []
+
+        def work():
+            try:
+                ffx.ffx_expand(plan, x, out, stream)
+            except Exception as e:  # reported by the assert below
+                failures.append(e)
+
+        thread = threading.Thread(target=work)
+        thread.start()
+        thread.join()
+        torch.cuda.synchronize()
+    assert not failures
+    assert torch.equal(out, want)
