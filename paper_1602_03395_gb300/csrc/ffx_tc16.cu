@@ -664,6 +664,57 @@ __device__ __forceinline__ BView many_view(const TcParams& P, int64_t w) {
   return v;
 }
 
+// An item and its pass's description come from global memory, two dependent
+// loads.  Every role therefore walks its items with the item after next and the
+// next item's description in flight while it works on the current one (a role
+// that loaded them at the switch waited ~1500 clocks an item).
+struct BDesc {  // a pass's description, pointers not rebased
+  const unsigned char* tblk;
+  const void *out_c, *out_d, *out_bf;
+  int64_t ncols, bf_plane;
+  int xmap, N, outc_base, outd_base, out_planes;
+};
+template <bool OUT>
+__device__ __forceinline__ BDesc many_desc(const TcParams& P, int arg) {
+  const TcPassArg& pa = P.args[arg];
+  BDesc c;
+  c.tblk = pa.tblk;
+  c.xmap = pa.xmap;
+  c.N = pa.d.N;
+  if (OUT) {
+    c.out_c = pa.d.out_c, c.out_d = pa.d.out_d, c.out_bf = pa.d.out_bf;
+    c.outc_base = pa.outc_base, c.outd_base = pa.outd_base, c.out_planes = pa.out_planes;
+    c.ncols = pa.d.ncols, c.bf_plane = pa.d.bf_plane;
+  }
+  return c;
+}
+template <bool OUT>  // with the output's fields
+struct BItems {
+  const TcParams& P;
+  int64_t w, last;
+  TcItem item, nitem, aitem;
+  BDesc d, nd;
+  __device__ __forceinline__ BItems(const TcParams& p, int64_t first, int64_t end) : P(p), w(first), last(end) {
+    item = P.items[first];
+    nitem = P.items[min((long long)(first + 1), (long long)(last - 1))];
+    aitem = P.items[min((long long)(first + 2), (long long)(last - 1))];
+    d = many_desc<OUT>(P, item.arg);
+    nd = many_desc<OUT>(P, nitem.arg);
+  }
+  __device__ __forceinline__ bool more() const { return w < last; }
+  __device__ __forceinline__ void next() {
+    ++w;
+    item = nitem;
+    d = nd;
+    nitem = aitem;
+    nd = many_desc<OUT>(P, nitem.arg);
+    aitem = P.items[min((long long)(w + 2), (long long)(last - 1))];
+  }
+  __device__ __forceinline__ const void* xmap() const {
+    return (const void*)((const unsigned char*)P.xmaps + (size_t)d.xmap * 128);
+  }
+};
+
 // First point of line c of an item's pass (a batch of one), or -1 past the end.
 __device__ __forceinline__ long long many_line(const BView& v, int64_t c) {
   if (c >= v.ncols) return -1;
@@ -686,6 +737,11 @@ __device__ __forceinline__ int prod_off(bool contiguous, int t, int i) {
 }
 
 constexpr int BMANY_STAGES = 3;
+// eight epilogue warps, two per tensor-memory lane quarter on every other 16
+// columns (four warps, one row block's 64 outputs each thread, took longer over
+// an item than its copies and products)
+constexpr int BMANY_EPIW = 8;
+constexpr int BMANY_THREADS = BPROD + 32 + 32 * BMANY_EPIW;
 // the stages, and 1 KB to start them on a 1024-byte boundary (the swizzled
 // tiles' atoms)
 constexpr int BMANY_SMEM = BMANY_STAGES * BSTAGE + 1024;
@@ -703,7 +759,7 @@ constexpr int BMANY_SMEM = BMANY_STAGES * BSTAGE + 1024;
 // TOUT: the output transposed so, also for FP32 input (a chain's first pass
 // reading the caller's input).
 template <int XM, bool TOUT>
-__global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcParams P) {
+__global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const TcParams P) {
   constexpr int BSTAGES = BMANY_STAGES;
   constexpr bool TMA = XM == kTmaContiguous;
   constexpr bool PLANES = XM == kTmaPlanes;
@@ -729,7 +785,7 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&accf_bar[b]), 1);
-      mbar_init(smem_u32(&acce_bar[b]), BEPI);
+      mbar_init(smem_u32(&acce_bar[b]), BMANY_EPIW);
     }
     mbar_init(smem_u32(&done_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -744,24 +800,21 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
   if (PLANES && warp < BMMA_WARP) {
     // ---------------- loads of BF16 planes: thread 0 alone ----------------
     if (tid == 0) {
-      int64_t iw = first, ci = 0;
+      int64_t u = 0;
       int ikc = 0, is = 0;
-      BView iv = many_view(P, first);
-      int ikch = (2 * iv.N + BKC - 1) / BKC;
-      int last_u[BSTAGES];
-#pragma unroll
-      for (int q = 0; q < BSTAGES; ++q) last_u[q] = -1;
-      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(iv.xmap) : "memory");
+      BItems<false> li(P, first, last);
+      int ikch = (2 * li.d.N + BKC - 1) / BKC;
+      int cur = li.d.xmap;
+      asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
 #pragma unroll 1
-      while (iw < last) {
-        // chunk ci into stage is once the products of chunk ci - BSTAGES freed it
-        const int64_t u = ci / BSTAGES;
+      while (li.more()) {
+        // the next chunk into stage `is` once its previous chunk's products freed it
         if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
         const uint32_t st = smem_u32(bsm + is * BSTAGE);
-        const uint32_t part = (uint32_t)brow_count(iv.N, iv.mt) * (BKC * 2);
+        const uint32_t part = (uint32_t)brow_count(li.d.N, li.item.mt) * (BKC * 2);
         const uint32_t cb = smem_u32(&copy_bar[is]);
         mbar_expect_tx(cb, 2 * part + (uint32_t)BXAREA);
-        const unsigned char* src = iv.tblk + ((size_t)iv.mt * ikch + ikc) * BTCHUNK;
+        const unsigned char* src = li.d.tblk + ((size_t)li.item.mt * ikch + ikc) * BTCHUNK;
         if (part == (uint32_t)BPART) {
           bulk_g2s(st, src, BTCHUNK, cb);
         } else {
@@ -773,25 +826,27 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
         asm volatile(
             "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
             "%4}], [%5];" ::"r"(st + (uint32_t)BTCHUNK),
-            "l"(reinterpret_cast<uint64_t>(iv.xmap)), "r"(ikc * BKC), "r"((int)(iv.ct * BL)), "r"(0), "r"(cb)
+            "l"(reinterpret_cast<uint64_t>(li.xmap())), "r"(ikc * BKC), "r"((int)(li.item.ct * BL)), "r"(0), "r"(cb)
             : "memory");
-        last_u[is] = (int)(u & 1);
-        ++ci;
-        is = is + 1 == BSTAGES ? 0 : is + 1;
+        if (++is == BSTAGES) {
+          is = 0;
+          ++u;
+        }
         if (++ikc == ikch) {
           ikc = 0;
-          if (++iw < last) {
-            const void* prev = iv.xmap;
-            iv = many_view(P, iw);
-            ikch = (2 * iv.N + BKC - 1) / BKC;
-            if (iv.xmap != prev)
-              asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(iv.xmap) : "memory");
+          li.next();
+          ikch = (2 * li.d.N + BKC - 1) / BKC;
+          if (li.d.xmap != cur) {
+            cur = li.d.xmap;
+            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
           }
         }
       }
       // nothing of this thread's may still be in flight at exit
-      for (int q = 0; q < BSTAGES; ++q)
-        if (last_u[q] >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)last_u[q], &s_abort);
+      for (int q = 0; q < BSTAGES; ++q) {
+        const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+        if (uq >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)(uq & 1), &s_abort);
+      }
     }
   } else if (warp < BMMA_WARP) {
     // ---------------- producers ----------------
@@ -802,27 +857,29 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
     // boxes, 128-byte swizzle) on the stage's "copy" barrier, else every
     // thread its points of the input.  The chunk's position (item iw, K chunk
     // ikc) advances incrementally.
-    int64_t iw = first, ci = 0;
+    int64_t ci = 0;
     int ikc = 0, is = 0;
-    BView iv = many_view(P, first);
-    int ikch = (2 * iv.N + BKC - 1) / BKC;
+    BItems<false> li(P, first, last);
+    BView iv;  // in place: the lines' geometry
+    if (!TMA) iv = many_view(P, first);
+    int ikch = (2 * li.d.N + BKC - 1) / BKC;
     long long ilb[2] = {-1, -1};
     bool lines_ok = false;
     int last_u[BSTAGES];
 #pragma unroll
     for (int q = 0; q < BSTAGES; ++q) last_u[q] = -1;
     auto issue = [&]() -> bool {
-      if (iw < last) {
+      if (li.more()) {
         const int64_t u = ci / BSTAGES;
         if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) return false;
         unsigned char* st = bsm + is * BSTAGE;
         const uint32_t xh = smem_u32(st + BTCHUNK), xl = xh + BPART;
         const bool tma = TMA;
         if (t == 0) {
-          const uint32_t part = (uint32_t)brow_count(iv.N, iv.mt) * (BKC * 2);
+          const uint32_t part = (uint32_t)brow_count(li.d.N, li.item.mt) * (BKC * 2);
           const uint32_t cb = smem_u32(&copy_bar[is]);
           mbar_expect_tx(cb, 2 * part + (tma ? (uint32_t)BXAREA : 0u));
-          const unsigned char* src = iv.tblk + ((size_t)iv.mt * ikch + ikc) * BTCHUNK;
+          const unsigned char* src = li.d.tblk + ((size_t)li.item.mt * ikch + ikc) * BTCHUNK;
           const uint32_t dst = smem_u32(st);
           if (part == (uint32_t)BPART) {
             bulk_g2s(dst, src, BTCHUNK, cb);  // head and tail in one copy
@@ -833,8 +890,8 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
           if (tma) {
             // rows: the tile's lines (past the pass's end: zeros); x: the
             // chunk's 64 real K (past 2N: zeros) in two 32-float boxes
-            const uint64_t map_addr = reinterpret_cast<uint64_t>(iv.xmap);
-            const int row = (int)(iv.ct * BL);
+            const uint64_t map_addr = reinterpret_cast<uint64_t>(li.xmap());
+            const int row = (int)(li.item.ct * BL);
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               asm volatile(
@@ -901,32 +958,30 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
         if (++ikc == ikch) {
           ikc = 0;
           lines_ok = false;
-          if (++iw < last) {
-            const void* prev = iv.xmap;
-            iv = many_view(P, iw);
-            ikch = (2 * iv.N + BKC - 1) / BKC;
-            // a map written before the launch, read by the tensor copies
-            if (TMA && t == 0 && iv.xmap != prev)
-              asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(iv.xmap) : "memory");
-          }
+          const int prev = li.d.xmap;
+          li.next();
+          if (!TMA && li.more()) iv = many_view(P, li.w);
+          ikch = (2 * li.d.N + BKC - 1) / BKC;
+          // a map written before the launch, read by the tensor copies
+          if (TMA && t == 0 && li.d.xmap != prev)
+            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
         }
       } else {
         asm volatile("cp.async.commit_group;" ::: "memory");  // an empty group past the end keeps the count
       }
       return true;
     };
-    if (TMA && t == 0) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(iv.xmap) : "memory");
+    if (TMA && t == 0) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
     bool ok = true;
 #pragma unroll 1
     for (int r = 0; r < BSTAGES - 1; ++r) ok = issue() && ok;
     // Conversion side: its own position (item cw, K chunk ckc), BSTAGES - 1
     // chunks behind the issue side.
-    int64_t cw = first;
     int ckc = 0;
-    int cN = P.args[P.items[first].arg].d.N;
-    bool ccontig = P.args[P.items[first].arg].d.inner == 1;
+    BItems<false> wi(P, first, last);
+    bool ccontig = TMA || P.args[wi.item.arg].d.inner == 1;
 #pragma unroll 1
-    for (int64_t c = 0; cw < last; ++c) {
+    for (int64_t c = 0; wi.more(); ++c) {
       const int s = (int)(c % BSTAGES);
       unsigned char* xa = bsm + s * BSTAGE + BTCHUNK;
       if (TMA) {
@@ -976,13 +1031,10 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
       mbar_arrive(smem_u32(&full_bar[s]));
       // the copies of chunk c + BSTAGES - 1, into the stage chunk c - 1 used
       ok = issue() && ok;
-      if (++ckc == (2 * cN + BKC - 1) / BKC) {
+      if (++ckc == (2 * wi.d.N + BKC - 1) / BKC) {
         ckc = 0;
-        if (++cw < last) {
-          const TcPassArg& pa = P.args[P.items[cw].arg];
-          cN = pa.d.N;
-          ccontig = pa.d.inner == 1;
-        }
+        wi.next();
+        if (!TMA && wi.more()) ccontig = P.args[wi.item.arg].d.inner == 1;
       }
     }
     // nothing of this thread's may still be in flight at exit
@@ -991,134 +1043,153 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
       for (int q = 0; q < BSTAGES; ++q)
         if (last_u[q] >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)last_u[q], &s_abort);
   } else if (warp == BMMA_WARP) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int64_t g = 0, sub = 0;
-      bool ok = true;
-      for (int64_t w = first; ok && w < last; ++w, ++sub) {
-        const TcItem item = P.items[w];
-        const int N = P.args[item.arg].d.N;
-        const int rows = brow_count(N, item.mt);
-        const int kchunks = (2 * N + BKC - 1) / BKC;
-        const uint32_t idesc = idesc_bf16(BL, rows);
-        const bool whole = rows == BR;
-        const int buf = (int)(sub & 1);
-        const int64_t v = sub >> 1;
-        if (v >= 1 && !mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort)) {
-          ok = false;
-          break;
-        }
+    // ---------------- products: the whole warp, one elected lane issuing ----------------
+    int64_t sub = 0, u = 0;
+    int s = 0;
+    bool ok = true;
+    // descriptor words (see mma_lo): T's core matrices, and X's, the producers'
+    // core matrices or the swizzled TMA tile
+    constexpr uint32_t hi_core = (uint32_t)(BSBO >> 4) | (1u << 14), lo_core = (uint32_t)(BCORE >> 4) << 16;
+    constexpr uint32_t hi_x = PLANES ? kDescHiSw128 : hi_core, lo_x = PLANES ? 1u << 16 : lo_core;
+    constexpr uint32_t xstep = PLANES ? 2 : 2 * BCORE / 16;  // a K step's bytes / 16
+    constexpr uint32_t id_whole = idesc_bf16(BL, 2 * BR);
+    BItems<false> mi(P, first, last);
+    for (; ok && mi.more(); mi.next(), ++sub) {
+      const int rows = brow_count(mi.d.N, mi.item.mt);
+      const int kchunks = (2 * mi.d.N + BKC - 1) / BKC;
+      const uint32_t idesc = idesc_bf16(BL, rows);
+      const bool whole = rows == BR;
+      const int buf = (int)(sub & 1);
+      const int64_t v = sub >> 1;
+      ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
+#pragma unroll 1
+      for (int kc = 0; kc < kchunks; ++kc) {
+        ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+             (PLANES || mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort));
+        if (!ok) break;
         tc_fence_after();
-        const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
-        for (int kc = 0; kc < kchunks; ++kc, ++g) {
-          const int s = (int)(g % BSTAGES);
-          const int64_t u = g / BSTAGES;
-          if (!mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) ||
-              (!PLANES && !mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort))) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t th = smem_base + (uint32_t)(s * BSTAGE), tl = th + BPART;
-          const uint32_t xh = th + BTCHUNK, xl = xh + BPART;
+        const uint32_t st = smem_base + (uint32_t)(s * BSTAGE);
+        const uint32_t th = (st >> 4) | lo_core, tl = th + BPART / 16;
+        const uint32_t xh = ((st + BTCHUNK) >> 4) | lo_x, xl = xh + BPART / 16;
 #pragma unroll
-          for (int ks = 0; ks < BKC / 16; ++ks) {
-            const uint32_t o = (uint32_t)(ks * 2 * BCORE);
-            // X: the producers' core matrices, or the swizzled TMA tile (32 bytes per K step)
-            const uint64_t dxh = PLANES ? make_desc_sw128(xh + (uint32_t)(ks * 32)) : make_desc(xh + o, BCORE, BSBO);
-            const uint64_t dxl = PLANES ? make_desc_sw128(xl + (uint32_t)(ks * 32)) : make_desc(xl + o, BCORE, BSBO);
-            const uint64_t dth = make_desc(th + o, BCORE, BSBO);
-            const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
-            if (whole) {
-              // the T chunk's 256 rows (head rows, then tail rows) into [d1 | d2]
-              mma_f16(d1, dxh, dth, idesc_bf16(BL, 2 * BR), more);
-            } else {
-              mma_f16(d1, dxh, dth, idesc, more);
-              mma_f16(d2, dxh, make_desc(tl + o, BCORE, BSBO), idesc, more);
-            }
-            mma_f16(d2, dxl, dth, idesc, 1u);
+        for (uint32_t ks = 0; ks < BKC / 16; ++ks) {
+          const uint32_t o = ks * (2 * BCORE / 16);
+          const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
+          if (whole) {
+            // the T chunk's 256 rows (head rows, then tail rows) into [d1 | d2]
+            mma_lo<hi_x, hi_core>(d1, xh + ks * xstep, th + o, id_whole, more);
+          } else {
+            mma_lo<hi_x, hi_core>(d1, xh + ks * xstep, th + o, idesc, more);
+            mma_lo<hi_x, hi_core>(d2, xh + ks * xstep, tl + o, idesc, more);
           }
-          mma_commit(smem_u32(&empty_bar[s]));
+          mma_lo<hi_x, hi_core>(d2, xl + ks * xstep, th + o, idesc, 1u);
         }
-        if (ok) mma_commit(smem_u32(&accf_bar[buf]));
+        if (elect_one()) {
+          mma_commit(smem_u32(&empty_bar[s]));
+          if (kc == kchunks - 1) mma_commit(smem_u32(&accf_bar[buf]));
+        }
+        __syncwarp();
+        if (++s == BSTAGES) {
+          s = 0;
+          ++u;
+        }
       }
-      // whatever happened, the tensor cores finish this thread's work before exit
-      mma_commit(smem_u32(&done_bar));
-      mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
     }
+    // whatever happened, the tensor cores finish this warp's work before exit
+    if (elect_one()) mma_commit(smem_u32(&done_bar));
     __syncwarp();
+    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
   } else {
     // ---------------- epilogue ----------------
-    const int q = warp & 3;       // tensor-memory lane quarter this warp may read
-    const int r = q * 32 + lane;  // line within the item
+    const int q = warp & 3;                           // tensor-memory lane quarter this warp may read
+    const int j_first = 16 * ((warp - BMMA_WARP - 1) >> 2);  // its columns: 16 of every 32
+    const int r = q * 32 + lane;                      // line within the item
     int64_t sub = 0;
-    bool ok = true;
-    for (int64_t w = first; ok && w < last; ++w, ++sub) {
-      const BView ev = many_view(P, w);
-      // the output's stride between a line's points: the input's, or (chains)
-      // the transposed order's, the pass's line count
-      const int64_t inner = TOUT ? ev.ncols : ev.inner;
-      const bool contiguous = !TOUT && inner == 1;
-      const int nbase = ev.mt * (BR / 2);
-      const int rows = brow_count(ev.N, ev.mt);
+    BItems<true> ei(P, first, last);
+    for (; ei.more(); ei.next(), ++sub) {
+      const int rows = brow_count(ei.d.N, ei.item.mt);
       const int buf = (int)(sub & 1);
       const int64_t v = sub >> 1;
       // lane 0 polls; the outcome is the warp's (its tensor-memory loads need the whole warp)
       bool got = true;
       if (lane == 0) got = mbar_wait(smem_u32(&accf_bar[buf]), (uint32_t)(v & 1), &s_abort);
-      ok = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
-      if (!ok) break;
+      if (__shfl_sync(0xffffffffu, got ? 1 : 0, 0) == 0) break;
       tc_fence_after();
-      const int64_t line = ev.ct * BL + r;
-      const long long base = TOUT ? (line < ev.ncols ? line : -1) : many_line(ev, line);
+      const int nbase = ei.item.mt * (BR / 2);
+      const int64_t line = ei.item.ct * BL + r;
+      // the output's stride between a line's points: the input's, or (chains)
+      // the transposed order's, the pass's line count
+      int64_t inner = ei.d.ncols;
+      long long base = line < ei.d.ncols ? line : -1;
+      if (!TOUT) {
+        const BView ev = many_view(P, ei.w);
+        inner = ev.inner;
+        base = many_line(ev, line);
+      }
+      const bool contiguous = !TOUT && inner == 1;
+      uint32_t* const out_bf =
+          TOUT && ei.d.out_planes ? (uint32_t*)many_rebase(P.call, ei.d.outc_base, ei.d.out_bf) : nullptr;
+      float2* const out_c = ei.d.out_planes ? nullptr : (float2*)many_rebase(P.call, ei.d.outc_base, ei.d.out_c);
+      float* const out_d = (float*)many_rebase(P.call, ei.d.outd_base, ei.d.out_d);
       const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BR);
+      uint32_t x[16], z[16];
+      tmem_ld16(taddr + (uint32_t)j_first, x);
+      tmem_ld16(taddr + (uint32_t)(BR + j_first), z);
 #pragma unroll 1
-      for (int j0 = 0; j0 < rows; j0 += 16) {
-        uint32_t x[16], z[16];
-        tmem_ld16(taddr + (uint32_t)j0, x);
-        tmem_ld16(taddr + (uint32_t)(BR + j0), z);
+      for (int j0 = j_first; j0 < rows; j0 += 32) {
         tmem_wait_ld();
         float y[16];
 #pragma unroll
         for (int m = 0; m < 16; ++m) y[m] = __uint_as_float(x[m]) + __uint_as_float(z[m]);
+        if (j0 + 32 < rows) {
+          // the next columns, in flight while these are written
+          tmem_ld16(taddr + (uint32_t)(j0 + 32), x);
+          tmem_ld16(taddr + (uint32_t)(BR + j0 + 32), z);
+        }
         const int n0 = nbase + j0 / 2;  // complex outputs n0 .. n0 + 7 of this line
-        if (base < 0) continue;
-        if (TOUT && ev.out_bf) {
-          // BF16 head and tail planes for the next pass (the split that pass
-          // would make of the same FP32 value)
+        if (base >= 0) {
+          if (TOUT && out_bf) {
+            // BF16 head and tail planes for the next pass (the split that pass
+            // would make of the same FP32 value)
+            uint32_t* o = out_bf + base + (int64_t)n0 * inner;
 #pragma unroll
-          for (int m = 0; m < 8; ++m) {
-            const __nv_bfloat162 hb = __floats2bfloat162_rn(y[2 * m], y[2 * m + 1]);
-            const int64_t e = base + (int64_t)(n0 + m) * inner;
-            ev.out_bf[e] = *reinterpret_cast<const uint32_t*>(&hb);
-            const float2 hf = __bfloat1622float2(hb);
-            ev.out_bf[ev.bf_plane + e] = pack_bf16(y[2 * m] - hf.x, y[2 * m + 1] - hf.y);
-          }
-        } else if (ev.out_c) {
-          if (contiguous) {
-            float4* o = reinterpret_cast<float4*>(ev.out_c + base + n0);
+            for (int m = 0; m < 8; ++m) {
+              const __nv_bfloat162 hb = __floats2bfloat162_rn(y[2 * m], y[2 * m + 1]);
+              const float2 hf = __bfloat1622float2(hb);
+              o[m * inner] = *reinterpret_cast<const uint32_t*>(&hb);
+              o[ei.d.bf_plane + m * inner] = pack_bf16(y[2 * m] - hf.x, y[2 * m + 1] - hf.y);
+            }
+          } else if (out_c) {
+            if (contiguous) {
+              float4* o = reinterpret_cast<float4*>(out_c + base + n0);
 #pragma unroll
-            for (int m = 0; m < 4; ++m) o[m] = make_float4(y[4 * m], y[4 * m + 1], y[4 * m + 2], y[4 * m + 3]);
+              for (int m = 0; m < 4; ++m) o[m] = make_float4(y[4 * m], y[4 * m + 1], y[4 * m + 2], y[4 * m + 3]);
+            } else {
+#pragma unroll
+              for (int m = 0; m < 8; ++m) out_c[base + (int64_t)(n0 + m) * inner] = make_float2(y[2 * m], y[2 * m + 1]);
+            }
           } else {
+            float dd[8];
 #pragma unroll
-            for (int m = 0; m < 8; ++m) ev.out_c[base + (int64_t)(n0 + m) * inner] = make_float2(y[2 * m], y[2 * m + 1]);
-          }
-        } else {
-          float dd[8];
+            for (int m = 0; m < 8; ++m) dd[m] = y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
+            if (contiguous) {
+              float4* o = reinterpret_cast<float4*>(out_d + base + n0);
+              o[0] = make_float4(dd[0], dd[1], dd[2], dd[3]);
+              o[1] = make_float4(dd[4], dd[5], dd[6], dd[7]);
+            } else {
 #pragma unroll
-          for (int m = 0; m < 8; ++m) dd[m] = y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
-          if (contiguous) {
-            float4* o = reinterpret_cast<float4*>(ev.out_d + base + n0);
-            o[0] = make_float4(dd[0], dd[1], dd[2], dd[3]);
-            o[1] = make_float4(dd[4], dd[5], dd[6], dd[7]);
-          } else {
-#pragma unroll
-            for (int m = 0; m < 8; ++m) ev.out_d[base + (int64_t)(n0 + m) * inner] = dd[m];
+              for (int m = 0; m < 8; ++m) out_d[base + (int64_t)(n0 + m) * inner] = dd[m];
+            }
           }
         }
+        __syncwarp();  // the next columns are read by the whole warp
       }
       tc_fence_before();
-      mbar_arrive(smem_u32(&acce_bar[buf]));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acce_bar[buf]));
     }
   }
 
@@ -1199,7 +1270,7 @@ const void* many_bf16_func(int mode) {
     default: return (const void*)dense_bf16_many_kernel<kInPlace, false>;
   }
 }
-int many_bf16_threads() { return BTHREADS; }
+int many_bf16_threads() { return BMANY_THREADS; }
 size_t many_bf16_smem() { return (size_t)BMANY_SMEM; }
 cudaError_t many_bf16_prepare() {
   cudaError_t e = cudaSuccess;

@@ -149,13 +149,17 @@ __device__ __forceinline__ bool elect_one() {
 // Issued by one elected lane; every lane of the warp calls them.
 constexpr uint32_t kDescHiSw128 = (1024u >> 4) | (1u << 14) | (2u << 29);
 __device__ __forceinline__ uint32_t desc_lo(uint32_t saddr) { return (saddr >> 4) | (1u << 16); }
-__device__ __forceinline__ void mma_sw128(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
+template <uint32_t AHI, uint32_t BHI>
+__device__ __forceinline__ void mma_lo(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p, e;\n .reg .b64 da, db;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
-      " mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+      " mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %6};\n"
       " @e tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(tmem_d),
-      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(kDescHiSw128)
+      "r"(alo), "r"(blo), "r"(idesc), "r"(acc), "n"(AHI), "n"(BHI)
       : "memory");
+}
+__device__ __forceinline__ void mma_sw128(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
+  mma_lo<kDescHiSw128, kDescHiSw128>(tmem_d, alo, blo, idesc, acc);
 }
 __device__ __forceinline__ void mma2_sw128(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t idesc, uint32_t acc) {
   asm volatile(
