@@ -750,7 +750,7 @@ constexpr int BMANY_SMEM = BMANY_STAGES * BSTAGE + 1024;
 //  * kInPlace: FP32 input by per-thread copies, each producer polling for
 //    itself and the warps moving on independently;
 //  * kTmaContiguous: FP32 contiguous lines by TMA tiles (a tile map per
-//    pass), thread 0 polling and a producer barrier passing the outcome on;
+//    pass), split in place by a thread per line;
 //  * kTmaPlanes (BF16 chains): BF16 head and tail planes of contiguous lines
 //    by one 3-D TMA tile per chunk straight into the tensor cores' swizzled
 //    K-major layout (thread 0 alone; no conversion), output transposed
@@ -779,7 +779,7 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
   if (warp == BMMA_WARP) tmem_alloc(&tmem_slot, BCOLS);
   if (tid == 0) {
     for (int s = 0; s < BSTAGES; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), BPROD);
+      mbar_init(smem_u32(&full_bar[s]), TMA ? 4 : BPROD);
       mbar_init(smem_u32(&empty_bar[s]), 1);
       mbar_init(smem_u32(&copy_bar[s]), 1);
     }
@@ -797,8 +797,8 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
   const uint32_t tmem = tmem_slot;
   const uint32_t smem_base = smem_u32(bsm);
 
-  if (PLANES && warp < BMMA_WARP) {
-    // ---------------- loads of BF16 planes: thread 0 alone ----------------
+  if ((PLANES || TMA) && warp < BMMA_WARP) {
+    // ---------------- copies: thread 0 alone ----------------
     if (tid == 0) {
       int64_t u = 0;
       int ikc = 0, is = 0;
@@ -822,12 +822,24 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
           bulk_g2s(st + BPART, src + BPART, part, cb);
         }
         // x: the chunk's 64 real K (past 2N: zeros); rows: the tile's lines
-        // (past the pass's end: zeros); z: the head and tail planes
-        asm volatile(
-            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-            "%4}], [%5];" ::"r"(st + (uint32_t)BTCHUNK),
-            "l"(reinterpret_cast<uint64_t>(li.xmap())), "r"(ikc * BKC), "r"((int)(li.item.ct * BL)), "r"(0), "r"(cb)
-            : "memory");
+        // (past the pass's end: zeros); planes: both, else two 32-float boxes
+        const uint64_t map_addr = reinterpret_cast<uint64_t>(li.xmap());
+        const int row = (int)(li.item.ct * BL);
+        if (PLANES) {
+          asm volatile(
+              "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+              "%4}], [%5];" ::"r"(st + (uint32_t)BTCHUNK),
+              "l"(map_addr), "r"(ikc * BKC), "r"(row), "r"(0), "r"(cb)
+              : "memory");
+        } else {
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                "[%4];" ::"r"(st + (uint32_t)(BTCHUNK + h * BPART)),
+                "l"(map_addr), "r"(ikc * BKC + 32 * h), "r"(row), "r"(cb)
+                : "memory");
+        }
         if (++is == BSTAGES) {
           is = 0;
           ++u;
@@ -847,21 +859,58 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
         const int64_t uq = q < is ? u : u - 1;  // stage q's last use
         if (uq >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)(uq & 1), &s_abort);
       }
+    } else if (TMA && warp >= 4) {
+      // ---------------- FP32 lines: a thread each ----------------
+      // Line n's 256 bytes (row n of both boxes) lie where its head and tail
+      // rows go (the planes' tile layout): read, split, written over in place,
+      // no thread waiting for another (with two barriers of 256 threads a chunk
+      // the first phase of 66 M points took 0.280 ms, against 0.242 ms).
+      const int n = tid - 128, sw = n & 7;
+      int s = 0, ckc = 0;
+      int64_t u = 0;
+      BItems<false> wi(P, first, last);
+      while (wi.more()) {
+        bool ok = true;
+        if (lane == 0) ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        unsigned char* const row = bsm + s * BSTAGE + BTCHUNK + n * 128;
+        float4 v[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          v[c] = *reinterpret_cast<const float4*>(row + (c >> 3) * BPART + (((c & 7) ^ sw) << 4));
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+          const float f[8] = {v[2 * c].x,     v[2 * c].y,     v[2 * c].z,     v[2 * c].w,
+                              v[2 * c + 1].x, v[2 * c + 1].y, v[2 * c + 1].z, v[2 * c + 1].w};
+          uint4 hi, lo;
+          split8(f, hi, lo, false);
+          *reinterpret_cast<uint4*>(row + ((c ^ sw) << 4)) = hi;
+          *reinterpret_cast<uint4*>(row + BPART + ((c ^ sw) << 4)) = lo;
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&full_bar[s]));
+        if (++s == BSTAGES) {
+          s = 0;
+          ++u;
+        }
+        if (++ckc == (2 * wi.d.N + BKC - 1) / BKC) {
+          ckc = 0;
+          wi.next();
+        }
+      }
     }
+    __syncwarp();
   } else if (warp < BMMA_WARP) {
-    // ---------------- producers ----------------
+    // ---------------- producers (in place) ----------------
     const int t = tid;
     // Issue side: chunk j of the block's run into stage j % BSTAGES once the
     // products of chunk j - BSTAGES have freed it; thread 0 copies the T chunk
-    // (and, where the pass has a tile map, the input tile: two 128 x 32-float
-    // boxes, 128-byte swizzle) on the stage's "copy" barrier, else every
-    // thread its points of the input.  The chunk's position (item iw, K chunk
-    // ikc) advances incrementally.
+    // on the stage's "copy" barrier, every thread its points of the input.
     int64_t ci = 0;
     int ikc = 0, is = 0;
     BItems<false> li(P, first, last);
-    BView iv;  // in place: the lines' geometry
-    if (!TMA) iv = many_view(P, first);
+    BView iv = many_view(P, first);  // the lines' geometry
     int ikch = (2 * li.d.N + BKC - 1) / BKC;
     long long ilb[2] = {-1, -1};
     bool lines_ok = false;
@@ -874,11 +923,10 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
         if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) return false;
         unsigned char* st = bsm + is * BSTAGE;
         const uint32_t xh = smem_u32(st + BTCHUNK), xl = xh + BPART;
-        const bool tma = TMA;
         if (t == 0) {
           const uint32_t part = (uint32_t)brow_count(li.d.N, li.item.mt) * (BKC * 2);
           const uint32_t cb = smem_u32(&copy_bar[is]);
-          mbar_expect_tx(cb, 2 * part + (tma ? (uint32_t)BXAREA : 0u));
+          mbar_expect_tx(cb, 2 * part);
           const unsigned char* src = li.d.tblk + ((size_t)li.item.mt * ikch + ikc) * BTCHUNK;
           const uint32_t dst = smem_u32(st);
           if (part == (uint32_t)BPART) {
@@ -887,34 +935,18 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
             bulk_g2s(dst, src, part, cb);
             bulk_g2s(dst + BPART, src + BPART, part, cb);
           }
-          if (tma) {
-            // rows: the tile's lines (past the pass's end: zeros); x: the
-            // chunk's 64 real K (past 2N: zeros) in two 32-float boxes
-            const uint64_t map_addr = reinterpret_cast<uint64_t>(li.xmap());
-            const int row = (int)(li.item.ct * BL);
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-              asm volatile(
-                  "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
-                  "%3}], [%4];" ::"r"(xh + (uint32_t)(h * BPART)),
-                  "l"(map_addr), "r"(ikc * BKC + 32 * h), "r"(row), "r"(cb)
-                  : "memory");
-          }
           last_u[is] = (int)(u & 1);
         }
         const int64_t inner = iv.inner;
         const bool contiguous = (inner == 1);
-        if (tma) {
-          // nothing for the other threads to copy (an empty group keeps the count)
-        } else if (!lines_ok) {
+        if (!lines_ok) {
           ilb[0] = many_line(iv, iv.ct * BL + prod_line(contiguous, t, 0));
           if (contiguous) ilb[1] = many_line(iv, iv.ct * BL + prod_line(contiguous, t, 2));
           lines_ok = true;
         }
         // lines past the pass's end, and K past 2N in the last chunk of a
         // 2N = 32 mod 64 axis, read nothing and land as zeros (source size 0)
-        if (tma) {
-        } else if (contiguous) {
+        if (contiguous) {
           // lanes t and t ^ 8 hold the rows (line, kp) and (line, kp + 1) of
           // a row pair, 8 complex points: the even lane copies points 0-1 and
           // 4-5 (the head rows), the odd lane 2-3 and 6-7 (the tail rows), so
@@ -958,20 +990,15 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
         if (++ikc == ikch) {
           ikc = 0;
           lines_ok = false;
-          const int prev = li.d.xmap;
           li.next();
-          if (!TMA && li.more()) iv = many_view(P, li.w);
+          if (li.more()) iv = many_view(P, li.w);
           ikch = (2 * li.d.N + BKC - 1) / BKC;
-          // a map written before the launch, read by the tensor copies
-          if (TMA && t == 0 && li.d.xmap != prev)
-            asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
         }
       } else {
         asm volatile("cp.async.commit_group;" ::: "memory");  // an empty group past the end keeps the count
       }
       return true;
     };
-    if (TMA && t == 0) asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(li.xmap()) : "memory");
     bool ok = true;
 #pragma unroll 1
     for (int r = 0; r < BSTAGES - 1; ++r) ok = issue() && ok;
@@ -979,46 +1006,26 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
     // chunks behind the issue side.
     int ckc = 0;
     BItems<false> wi(P, first, last);
-    bool ccontig = TMA || P.args[wi.item.arg].d.inner == 1;
+    bool ccontig = P.args[wi.item.arg].d.inner == 1;
 #pragma unroll 1
     for (int64_t c = 0; wi.more(); ++c) {
       const int s = (int)(c % BSTAGES);
       unsigned char* xa = bsm + s * BSTAGE + BTCHUNK;
-      if (TMA) {
-        // the tile has landed: thread 0 polls the copy barrier, the barrier
-        // passes the outcome and the data on
-        if (t == 0) ok = ok && mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)((c / BSTAGES) & 1), &s_abort);
-        if (!prod_all(ok)) break;
-      } else {
-        // this thread's points of the chunk have landed (of its groups only
-        // the BSTAGES - 2 newer ones may be pending); the warp stops as one
-        // and sees the partner lane's halves of this thread's rows
-        asm volatile("cp.async.wait_group %0;" ::"n"(BSTAGES - 2) : "memory");
-        if (!__all_sync(0xffffffffu, ok)) break;
-        if (ccontig) __syncwarp();
-      }
+      // this thread's points of the chunk have landed (of its groups only
+      // the BSTAGES - 2 newer ones may be pending); the warp stops as one
+      // and sees the partner lane's halves of this thread's rows
+      asm volatile("cp.async.wait_group %0;" ::"n"(BSTAGES - 2) : "memory");
+      if (!__all_sync(0xffffffffu, ok)) break;
+      if (ccontig) __syncwarp();
       float v[BITEMS][8];
 #pragma unroll
       for (int i = 0; i < BITEMS; ++i) {
-        if (TMA) {
-          // box kp / 4, row n, 16-byte chunks 2 (kp % 4) and + 1, swizzled by n % 8
-          const int n = prod_line(true, t, i), kp = prod_kp(true, t, i);
-          const unsigned char* row = xa + (kp >> 2) * BPART + n * 128;
-          const int c0 = 2 * (kp & 3);
-          const float4 r0 = *reinterpret_cast<const float4*>(row + ((c0 ^ (n & 7)) << 4));
-          const float4 r1 = *reinterpret_cast<const float4*>(row + (((c0 + 1) ^ (n & 7)) << 4));
-          v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
-          v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
-        } else {
-          const int off = prod_off(ccontig, t, i);
-          const float4 r0 = *reinterpret_cast<const float4*>(xa + off);
-          const float4 r1 = *reinterpret_cast<const float4*>(xa + BPART + off);
-          v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
-          v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
-        }
+        const int off = prod_off(ccontig, t, i);
+        const float4 r0 = *reinterpret_cast<const float4*>(xa + off);
+        const float4 r1 = *reinterpret_cast<const float4*>(xa + BPART + off);
+        v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
+        v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
       }
-      // every producer has read its input before any overwrites the tile with BF16 rows
-      if (TMA) prod_sync();
 #pragma unroll
       for (int i = 0; i < BITEMS; ++i) {
         const int off = prod_off(ccontig, t, i);
@@ -1034,7 +1041,7 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
       if (++ckc == (2 * wi.d.N + BKC - 1) / BKC) {
         ckc = 0;
         wi.next();
-        if (!TMA && wi.more()) ccontig = P.args[wi.item.arg].d.inner == 1;
+        if (wi.more()) ccontig = P.args[wi.item.arg].d.inner == 1;
       }
     }
     // nothing of this thread's may still be in flight at exit
@@ -1047,11 +1054,12 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
     int64_t sub = 0, u = 0;
     int s = 0;
     bool ok = true;
-    // descriptor words (see mma_lo): T's core matrices, and X's, the producers'
-    // core matrices or the swizzled TMA tile
+    // descriptor words (see mma_lo): T's core matrices, and X's, the in-place
+    // producers' core matrices or the swizzled TMA tile
     constexpr uint32_t hi_core = (uint32_t)(BSBO >> 4) | (1u << 14), lo_core = (uint32_t)(BCORE >> 4) << 16;
-    constexpr uint32_t hi_x = PLANES ? kDescHiSw128 : hi_core, lo_x = PLANES ? 1u << 16 : lo_core;
-    constexpr uint32_t xstep = PLANES ? 2 : 2 * BCORE / 16;  // a K step's bytes / 16
+    constexpr bool SW = PLANES || TMA;
+    constexpr uint32_t hi_x = SW ? kDescHiSw128 : hi_core, lo_x = SW ? 1u << 16 : lo_core;
+    constexpr uint32_t xstep = SW ? 2 : 2 * BCORE / 16;  // a K step's bytes / 16
     constexpr uint32_t id_whole = idesc_bf16(BL, 2 * BR);
     BItems<false> mi(P, first, last);
     for (; ok && mi.more(); mi.next(), ++sub) {
