@@ -1739,7 +1739,11 @@ int ffx_expand_column(ffx_plan_t p, const void* psi0, int64_t batch, int axis, f
     cudaError_t e = cudaMemsetAsync(rho, 0, (size_t)p->M * sizeof(float), s);
     if (e != cudaSuccess) return cuda_fail(e, "density scratch");
   }
-  if ((rc = forward_density(p, axes, (const float2*)psi0, batch, rho, s))) return rc;
+  // (the sum takes whole densities, so the passes may run in any order: that of
+  // the BF16 chain where the call can take one.  128^3 x 4: 158 us with strided
+  // FP32 passes ahead of the integrated axis, 106 us as a chain.)
+  const int* passes = bf16_chain_ok(p, batch, psi0, nullptr, rho) ? p->order : axes;
+  if ((rc = forward_density(p, passes, (const float2*)psi0, batch, rho, s))) return rc;
   int64_t outer, inner;
   axis_outer_inner(p, axis, &outer, &inner);
   const Axis& ax = p->axis[axis];
