@@ -23,7 +23,7 @@
 // the stage itself, each thread's bytes where its own BF16 rows go, and is
 // converted in place: no separate input ring, three 64 KB stages.
 //
-// Kernel: one persistent block of 416 threads per SM, warp-specialised.
+// Kernel: one persistent block of 544 threads per SM, warp-specialised.
 //  * warps 0-7 (producers), per K chunk of 64 real K, once the products of
 //    the chunk three back have freed its stage: thread 0 starts a bulk copy of
 //    the pre-split T chunk (head and tail, 128 rows x 64 K each, already in
@@ -32,11 +32,12 @@
 //    into the stage (cp.async); two chunks later the thread converts its share
 //    into BF16 heads and tails in place (16-byte core-matrix rows, conflict
 //    free) and arrives on "full".
-//  * warp 8 (MMA): waits "copy" and "full", issues 4 K-steps x 3 products of
+//  * warp 8 (MMA; one elected lane issues): waits "copy" and "full", issues 4 K-steps x 3 products of
 //    tcgen05.mma kind::f16 (M = 128 lines, N = 128 rows, K = 16) into one of
 //    two accumulator pairs; tcgen05.commit frees the stage ("empty") and,
 //    after an item's last chunk, hands the accumulator on ("acc_full").
-//  * warps 9-12 (epilogue): read their 32-lane quarter of the accumulators,
+//  * warps 9-16 (epilogue): read their 32-lane quarter of the accumulators, two
+//    warps on every other 16 columns of one,
 //    store complex64 or |.|^2 (or add |.|^2 over the batch in shared memory),
 //    and arrive on "acc_empty".
 // Items are (128 lines, 128 real rows) of the output, numbered row block
@@ -78,9 +79,12 @@ constexpr int BTCHUNK = 2 * BPART;           // T chunk: head, tail
 // input of the chunk (32 KB) lands first
 constexpr int BXAREA = 2 * BPART;
 constexpr int BSTAGE = BTCHUNK + BXAREA;     // 64 KB
-constexpr int BPROD = 256, BEPI = 128;
-constexpr int BTHREADS = BPROD + 32 + BEPI;  // 416
-constexpr int BMMA_WARP = BPROD / 32;        // warp 8; warps 9-12 are the epilogue
+// eight epilogue warps, two per tensor-memory lane quarter on every other 16
+// columns (four warps, a row block's 64 outputs each thread, took longer over a
+// short item than its copies and products)
+constexpr int BPROD = 256, BEPIW = 8;
+constexpr int BTHREADS = BPROD + 32 + 32 * BEPIW;  // 544
+constexpr int BMMA_WARP = BPROD / 32;              // warp 8; warps 9-16 are the epilogue
 constexpr int BITEMS = BL * (BKC / 8) / BPROD;  // 4 core-matrix rows (8 real K) per producer thread per chunk
 constexpr int BGRAD_CHUNK = BPROD * BITEMS * 16;  // 16 KB: a chunk's gradient factors (backward passes)
 constexpr int BEXTRA = (BR / 2) * BL * 4;       // accumulating launches: |.|^2 over the batch, [row][line]
@@ -94,21 +98,6 @@ __host__ __device__ constexpr int bsmem(bool grad, bool acc) {
 // 1024-byte boundary (the swizzled tiles' atoms)
 __host__ __device__ constexpr int bsmem_launch(bool grad, bool acc) { return bsmem(grad, acc) + 1024; }
 static_assert(bsmem_launch(false, true) <= 227 * 1024 && bsmem_launch(true, false) <= 227 * 1024, "shared memory");
-
-// The 256 producer threads' named barrier (id 1): every thread passes its
-// flag and gets the AND of all of them, so that a decision to stop is the
-// same in every producer thread; a plain one (id 2) orders their shared-memory
-// accesses.
-__device__ __forceinline__ bool prod_all(bool v) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.and.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(r)
-      : "r"((uint32_t)v), "n"(BPROD)
-      : "memory");
-  return r != 0;
-}
-__device__ __forceinline__ void prod_sync() { asm volatile("bar.sync 2, %0;" ::"n"(BPROD) : "memory"); }
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
@@ -165,15 +154,12 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo, boo
   lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-// How a chunk's input reaches the stage: a TMA tile of contiguous lines (a
-// 2-D map over [lines][2N floats], two 128 x 32-float boxes with 128-byte
-// swizzle; the producers read it, meet at a barrier, and write the BF16 rows
-// over it), or per-thread cp.async that lands each thread's points on the
-// bytes of its own BF16 rows (strided lines and backward passes; every
-// thread converts its own bytes, with no barrier).  Measured on 256^3
-// passes: contiguous lines 0.17 ms by TMA against 0.20 ms per thread; strided
-// lines 0.17 ms per thread against 0.21 ms by a 3-D TMA tile.
-// BF16 planes (many-instance chains): the head and tail rows as one TMA tile.
+// How a chunk's input reaches the stage: per-thread cp.async that lands each
+// thread's points on the bytes of its own BF16 rows (the uniform kernel, whose
+// strided lines and backward passes take this way; every thread converts its
+// own bytes, with no barrier); or, in many-instance phases, FP32 contiguous
+// lines as a TMA tile (two 128 x 32-float boxes with 128-byte swizzle), or BF16
+// planes, the head and tail rows as one TMA tile.
 enum BLoad { kTmaContiguous = 0, kInPlace = 1, kTmaPlanes = 2 };
 
 // FULL: every row block has BR rows (2N a multiple of 128).  GRAD: backward
@@ -181,8 +167,7 @@ enum BLoad { kTmaContiguous = 0, kInPlace = 1, kTmaPlanes = 2 };
 // own ring; two stages).  ACC: the batch's |.|^2 summed in shared memory.
 template <bool FULL, bool GRAD, bool ACC>
 __global__ void __launch_bounds__(BTHREADS, 1)
-    dense_bf16_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
-                      const __grid_constant__ CUtensorMap xmap, const int mode) {
+    dense_bf16_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err) {
   constexpr int BSTAGES = bstages(GRAD, ACC);
   extern __shared__ __align__(1024) unsigned char bsm_raw[];
   // the stages on a 1024-byte boundary (the launch adds 1 KB for it)
@@ -212,7 +197,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&accf_bar[b]), 1);
-      mbar_init(smem_u32(&acce_bar[b]), BEPI);
+      mbar_init(smem_u32(&acce_bar[b]), BEPIW);
     }
     mbar_init(smem_u32(&done_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -229,7 +214,6 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     const int t = tid;
     const int64_t inner = a.inner;
     const bool contiguous = (inner == 1);
-    const bool tma = mode == kTmaContiguous;
     const int64_t total = my_items * nb * kchunks;
     unsigned char* graw = bsm + BSTAGES * BSTAGE;  // gradient factors, one slot per stage (backward)
     // this thread's 4 core-matrix rows of a chunk: line n_i, K group kp_i
@@ -257,17 +241,13 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     int last_u[BSMAX];
 #pragma unroll
     for (int q = 0; q < BSMAX; ++q) last_u[q] = -1;
-    const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
     auto issue = [&]() -> bool {
       if (ci < total) {
         const int64_t u = ci / BSTAGES;
-        // the stage's previous products are done: with TMA thread 0 polls
-        // (the next barrier passes the outcome on); in place every producer
-        // polls for itself and moves on by itself (no barrier couples the
-        // warps there: measured 20% faster than a barrier after thread 0's poll)
-        if ((tma ? t == 0 : true) && u >= 1 &&
-            !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort))
-          return false;
+        // the stage's previous products are done: every producer polls for
+        // itself and moves on by itself (no barrier couples the warps: measured
+        // 20% faster than a barrier after thread 0's poll)
+        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) return false;
         unsigned char* st = bsm + is * BSTAGE;
         const int mt = (int)(iw % mtiles);
         const int64_t ct = iw / mtiles;
@@ -275,7 +255,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         if (t == 0) {
           const uint32_t part = (uint32_t)(FULL ? BR : brow_count(N, mt)) * (BKC * 2);
           const uint32_t cb = smem_u32(&copy_bar[is]);
-          mbar_expect_tx(cb, (unsplit ? part : 2 * part) + (tma ? (uint32_t)BXAREA : 0u));
+          mbar_expect_tx(cb, unsplit ? part : 2 * part);
           const unsigned char* src = Tblk + ((size_t)mt * kchunks + ikc) * BTCHUNK;
           const uint32_t dst = smem_u32(st);
           if (unsplit) {
@@ -286,61 +266,47 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             bulk_g2s(dst, src, part, cb);
             bulk_g2s(dst + BPART, src + BPART, part, cb);
           }
-          if (tma) {
-            // rows: the tile's lines (realization ib's when accumulating); x: the
-            // chunk's 64 real K in two 32-float boxes
-            const int row = (int)(ct * BL + (ACC ? (int64_t)ib * a.outer : 0));
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-              asm volatile(
-                  "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
-                  "[%4];" ::"r"(xh + (uint32_t)(h * BPART)),
-                  "l"(map_addr), "r"(ikc * BKC + 32 * h), "r"(row), "r"(cb)
-                  : "memory");
-          }
           last_u[is] = (int)(u & 1);
         }
-        if (!tma) {
-          if (!lines_ok) {
-            ilb[0] = bline(a, ct * BL + item_line(0), ib, ibr[0]);
-            if (contiguous) ilb[1] = bline(a, ct * BL + item_line(2), ib, ibr[1]);
-            lines_ok = true;
-          }
-          const uint32_t gdst0 = smem_u32(graw + is * BGRAD_CHUNK) + (uint32_t)t * 16;
-#pragma unroll
-          for (int i = 0; i < BITEMS; ++i) {
-            const int li = contiguous ? (i >> 1) : 0;
-            const long long lb = ilb[li];
-            const bool valid = lb >= 0;
-            const int k0 = ikc * (BKC / 2) + 4 * item_kp(i);  // first complex point
-            const int64_t addr = valid ? lb + (int64_t)k0 * inner : 0;
-            const uint32_t off = (uint32_t)item_off(i);
-            // invalid lines read nothing and land as zeros (source size 0)
-            if (contiguous) {
-              cp_async16(xh + off, a.in + addr, valid ? 16 : 0);
-              cp_async16(xl + off, a.in + addr + (valid ? 2 : 0), valid ? 16 : 0);
-            } else {
-              // point k0 + j of the line into half j % 2 of the head (j < 2) or
-              // tail row; lanes 8-15 and 24-31 take the points in the order
-              // 1, 0, 3, 2 so that each copy instruction's 8-byte pieces fall
-              // on every bank twice (two wavefronts) instead of four times
-#pragma unroll
-              for (int j0 = 0; j0 < 4; ++j0) {
-                const int j = j0 ^ ((t >> 3) & 1);
-                cp_async8((j < 2 ? xh : xl) + off + (uint32_t)((j & 1) * 8), a.in + addr + (valid ? j * inner : 0),
-                          valid ? 8 : 0);
-              }
-            }
-            if (GRAD) {
-              const int64_t gaddr = valid && a.grad_shared ? addr - (int64_t)ibr[li] * a.M : addr;
-              const uint32_t gd = gdst0 + (uint32_t)(i * BPROD * 16);
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                cp_async4(gd + 4 * j, a.grad + gaddr + (valid ? j * inner : 0), valid ? 4 : 0);
-            }
-          }
-          asm volatile("cp.async.commit_group;" ::: "memory");
+        if (!lines_ok) {
+          ilb[0] = bline(a, ct * BL + item_line(0), ib, ibr[0]);
+          if (contiguous) ilb[1] = bline(a, ct * BL + item_line(2), ib, ibr[1]);
+          lines_ok = true;
         }
+        const uint32_t gdst0 = smem_u32(graw + is * BGRAD_CHUNK) + (uint32_t)t * 16;
+#pragma unroll
+        for (int i = 0; i < BITEMS; ++i) {
+          const int li = contiguous ? (i >> 1) : 0;
+          const long long lb = ilb[li];
+          const bool valid = lb >= 0;
+          const int k0 = ikc * (BKC / 2) + 4 * item_kp(i);  // first complex point
+          const int64_t addr = valid ? lb + (int64_t)k0 * inner : 0;
+          const uint32_t off = (uint32_t)item_off(i);
+          // invalid lines read nothing and land as zeros (source size 0)
+          if (contiguous) {
+            cp_async16(xh + off, a.in + addr, valid ? 16 : 0);
+            cp_async16(xl + off, a.in + addr + (valid ? 2 : 0), valid ? 16 : 0);
+          } else {
+            // point k0 + j of the line into half j % 2 of the head (j < 2) or
+            // tail row; lanes 8-15 and 24-31 take the points in the order
+            // 1, 0, 3, 2 so that each copy instruction's 8-byte pieces fall
+            // on every bank twice (two wavefronts) instead of four times
+#pragma unroll
+            for (int j0 = 0; j0 < 4; ++j0) {
+              const int j = j0 ^ ((t >> 3) & 1);
+              cp_async8((j < 2 ? xh : xl) + off + (uint32_t)((j & 1) * 8), a.in + addr + (valid ? j * inner : 0),
+                        valid ? 8 : 0);
+            }
+          }
+          if (GRAD) {
+            const int64_t gaddr = valid && a.grad_shared ? addr - (int64_t)ibr[li] * a.M : addr;
+            const uint32_t gd = gdst0 + (uint32_t)(i * BPROD * 16);
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              cp_async4(gd + 4 * j, a.grad + gaddr + (valid ? j * inner : 0), valid ? 4 : 0);
+          }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
         ++ci;
         is = is + 1 == BSTAGES ? 0 : is + 1;
         if (++ikc == kchunks) {
@@ -351,7 +317,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
             iw += gridDim.x;
           }
         }
-      } else if (!tma) {
+      } else {
         asm volatile("cp.async.commit_group;" ::: "memory");  // an empty group past the end keeps the count
       }
       return true;
@@ -365,37 +331,17 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       unsigned char* xa = bsm + s * BSTAGE + BTCHUNK;
       const float4* gs = reinterpret_cast<const float4*>(graw + s * BGRAD_CHUNK) + t;
       float v[BITEMS][8];
-      if (tma) {
-        // the tile has landed: thread 0 polls the copy barrier, the barrier
-        // passes the outcome and the data on
-        if (t == 0) ok = ok && mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)((c / BSTAGES) & 1), &s_abort);
-        if (!prod_all(ok)) break;
+      // this thread's points of the chunk have landed (of its groups only the
+      // BSTAGES - 2 newer ones may be pending); it alone touches their bytes
+      asm volatile("cp.async.wait_group %0;" ::"n"(BSTAGES - 2) : "memory");
+      if (!ok) break;
 #pragma unroll
-        for (int i = 0; i < BITEMS; ++i) {
-          // box kp / 4, row n, 16-byte chunks 2 (kp % 4) and + 1, swizzled by n % 8
-          const int n = item_line(i), kp = item_kp(i);
-          const unsigned char* row = xa + (kp >> 2) * BPART + n * 128;
-          const int c0 = 2 * (kp & 3);
-          const float4 r0 = *reinterpret_cast<const float4*>(row + ((c0 ^ (n & 7)) << 4));
-          const float4 r1 = *reinterpret_cast<const float4*>(row + (((c0 + 1) ^ (n & 7)) << 4));
-          v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
-          v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
-        }
-        // every producer has read its input before any overwrites the tile with BF16 rows
-        prod_sync();
-      } else {
-        // this thread's points of the chunk have landed (of its groups only the
-        // BSTAGES - 2 newer ones may be pending); it alone touches their bytes
-        asm volatile("cp.async.wait_group %0;" ::"n"(BSTAGES - 2) : "memory");
-        if (!ok) break;
-#pragma unroll
-        for (int i = 0; i < BITEMS; ++i) {
-          const int off = item_off(i);
-          const float4 r0 = *reinterpret_cast<const float4*>(xa + off);
-          const float4 r1 = *reinterpret_cast<const float4*>(xa + BPART + off);
-          v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
-          v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
-        }
+      for (int i = 0; i < BITEMS; ++i) {
+        const int off = item_off(i);
+        const float4 r0 = *reinterpret_cast<const float4*>(xa + off);
+        const float4 r1 = *reinterpret_cast<const float4*>(xa + BPART + off);
+        v[i][0] = r0.x, v[i][1] = r0.y, v[i][2] = r0.z, v[i][3] = r0.w;
+        v[i][4] = r1.x, v[i][5] = r1.y, v[i][6] = r1.z, v[i][7] = r1.w;
       }
 #pragma unroll
       for (int i = 0; i < BITEMS; ++i) {
@@ -423,74 +369,76 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       for (int q = 0; q < BSTAGES; ++q)
         if (last_u[q] >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)last_u[q], &s_abort);
   } else if (warp == BMMA_WARP) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int64_t g = 0, sub = 0;
-      bool ok = true;
-      for (int64_t it = 0; ok && it < my_items; ++it) {
-        const int mt = (int)((blockIdx.x + it * gridDim.x) % mtiles);
-        const uint32_t idesc = idesc_bf16(BL, FULL ? BR : brow_count(N, mt));
-        // whole row blocks: X_hi against [T_hi; T_lo] (the T chunk's 256 rows,
-        // head rows then tail rows) in one N = 256 product into the adjacent
-        // accumulators [d1 | d2] -- the operand X_hi is read once for both
-        for (int b = 0; ok && b < nb; ++b, ++sub) {
-          const int buf = (int)(sub & 1);
-          const int64_t v = sub >> 1;
-          if (v >= 1 && !mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort)) {
-            ok = false;
-            break;
-          }
+    // ---------------- products: the whole warp, one elected lane issuing ----------------
+    int64_t sub = 0, u = 0;
+    int s = 0;
+    bool ok = true;
+    // descriptor words of both operands' core matrices (see mma_lo)
+    constexpr uint32_t hi_core = (uint32_t)(BSBO >> 4) | (1u << 14), lo_core = (uint32_t)(BCORE >> 4) << 16;
+    for (int64_t it = 0; ok && it < my_items; ++it) {
+      const int mt = (int)((blockIdx.x + it * gridDim.x) % mtiles);
+      const uint32_t idesc = idesc_bf16(BL, FULL ? BR : brow_count(N, mt));
+      // whole row blocks: X_hi against [T_hi; T_lo] (the T chunk's 256 rows,
+      // head rows then tail rows) in one N = 256 product into the adjacent
+      // accumulators [d1 | d2] -- the operand X_hi is read once for both
+      for (int b = 0; ok && b < nb; ++b, ++sub) {
+        const int buf = (int)(sub & 1);
+        const int64_t v = sub >> 1;
+        ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
+#pragma unroll 1
+        for (int kc = 0; kc < kchunks; ++kc) {
+          ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+               mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
+          if (!ok) break;
           tc_fence_after();
-          const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
-          for (int kc = 0; kc < kchunks; ++kc, ++g) {
-            const int s = (int)(g % BSTAGES);
-            const int64_t u = g / BSTAGES;
-            if (!mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) ||
-                !mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t th = smem_base + (uint32_t)(s * BSTAGE), tl = th + BPART;
-            const uint32_t xh = th + BTCHUNK, xl = xh + BPART;
+          const uint32_t th = ((smem_base + (uint32_t)(s * BSTAGE)) >> 4) | lo_core, tl = th + BPART / 16;
+          const uint32_t xh = th + BTCHUNK / 16, xl = xh + BPART / 16;
 #pragma unroll
-            for (int ks = 0; ks < BKC / 16; ++ks) {
-              const uint32_t o = (uint32_t)(ks * 2 * BCORE);
-              const uint64_t dxh = make_desc(xh + o, BCORE, BSBO);
-              const uint64_t dth = make_desc(th + o, BCORE, BSBO);
-              const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
-              if (unsplit) {
-                mma_f16(d1, dxh, dth, idesc, more);
+          for (uint32_t ks = 0; ks < BKC / 16; ++ks) {
+            const uint32_t o = ks * (2 * BCORE / 16);
+            const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
+            if (unsplit) {
+              mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
+            } else {
+              if (FULL) {
+                mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc_bf16(BL, 2 * BR), more);
               } else {
-                const uint64_t dxl = make_desc(xl + o, BCORE, BSBO);
-                if (FULL) {
-                  mma_f16(d1, dxh, dth, idesc_bf16(BL, 2 * BR), more);
-                } else {
-                  mma_f16(d1, dxh, dth, idesc, more);
-                  mma_f16(d2, dxh, make_desc(tl + o, BCORE, BSBO), idesc, more);
-                }
-                mma_f16(d2, dxl, dth, idesc, 1u);
+                mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
+                mma_lo<hi_core, hi_core>(d2, xh + o, tl + o, idesc, more);
               }
+              mma_lo<hi_core, hi_core>(d2, xl + o, th + o, idesc, 1u);
             }
-            mma_commit(smem_u32(&empty_bar[s]));
           }
-          if (ok) mma_commit(smem_u32(&accf_bar[buf]));
+          if (elect_one()) {
+            mma_commit(smem_u32(&empty_bar[s]));
+            if (kc == kchunks - 1) mma_commit(smem_u32(&accf_bar[buf]));
+          }
+          __syncwarp();
+          if (++s == BSTAGES) {
+            s = 0;
+            ++u;
+          }
         }
       }
-      // whatever happened, the tensor cores finish this thread's work before exit
-      mma_commit(smem_u32(&done_bar));
-      mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
     }
+    // whatever happened, the tensor cores finish this warp's work before exit
+    if (elect_one()) mma_commit(smem_u32(&done_bar));
     __syncwarp();
+    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
   } else {
     // ---------------- epilogue ----------------
-    const int q = warp & 3;       // tensor-memory lane quarter this warp may read
-    const int r = q * 32 + lane;  // line within the item
+    const int q = warp & 3;                                  // tensor-memory lane quarter this warp may read
+    const int j_first = 16 * ((warp - BMMA_WARP - 1) >> 2);  // its columns: 16 of every 32
+    const int r = q * 32 + lane;                             // line within the item
     const int64_t inner = a.inner;
     const bool contiguous = (inner == 1);
     float* racc = reinterpret_cast<float*>(bsm + BSTAGES * BSTAGE);  // accumulating launches only
     if (ACC)
-      for (int m = 0; m < BR / 2; ++m) racc[m * BL + r] = 0.f;
+      for (int j0 = j_first; j0 < BR; j0 += 32)
+        for (int m = 0; m < 8; ++m) racc[(j0 / 2 + m) * BL + r] = 0.f;
     int64_t sub = 0;
     bool ok = true;
     for (int64_t it = 0; ok && it < my_items; ++it) {
@@ -511,15 +459,21 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         int br;
         const long long base = bline(a, ct * BL + r, b, br);
         const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BR);
+        uint32_t x[16], z[16];
+        tmem_ld16(taddr + (uint32_t)j_first, x);
+        tmem_ld16(taddr + (uint32_t)(BR + j_first), z);  // unsplit: not written, not used
 #pragma unroll 1
-        for (int j0 = 0; j0 < rows; j0 += 16) {
-          uint32_t x[16], z[16];
-          tmem_ld16(taddr + (uint32_t)j0, x);
-          if (!unsplit) tmem_ld16(taddr + (uint32_t)(BR + j0), z);
+        for (int j0 = j_first; j0 < rows; j0 += 32) {
           tmem_wait_ld();
           float y[16];
 #pragma unroll
-          for (int m = 0; m < 16; ++m) y[m] = __uint_as_float(x[m]) + (unsplit ? 0.f : __uint_as_float(z[m]));
+          for (int m = 0; m < 16; ++m)
+            y[m] = unsplit ? __uint_as_float(x[m]) : __uint_as_float(x[m]) + __uint_as_float(z[m]);
+          if (j0 + 32 < rows) {
+            // the next columns, in flight while these are written
+            tmem_ld16(taddr + (uint32_t)(j0 + 32), x);
+            tmem_ld16(taddr + (uint32_t)(BR + j0 + 32), z);
+          }
           const int n0 = nbase + j0 / 2;  // complex outputs n0 .. n0 + 7 of this line
           if (ACC) {
 #pragma unroll
@@ -549,29 +503,23 @@ __global__ void __launch_bounds__(BTHREADS, 1)
               }
             }
           }
+          __syncwarp();  // the next columns are read by the whole warp
         }
         tc_fence_before();
-        mbar_arrive(smem_u32(&acce_bar[buf]));
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&acce_bar[buf]));
         if (ACC && b == nb - 1) {
           if (base >= 0) {
             const int64_t o0 = base - (int64_t)br * a.M + (int64_t)nbase * inner;
-            if (contiguous) {
-              float4* o = reinterpret_cast<float4*>(a.out_d + o0);
 #pragma unroll 1
-              for (int m = 0; m < rows / 8; ++m) {
-                float4 cur = o[m];
-                cur.x += racc[(4 * m) * BL + r];
-                cur.y += racc[(4 * m + 1) * BL + r];
-                cur.z += racc[(4 * m + 2) * BL + r];
-                cur.w += racc[(4 * m + 3) * BL + r];
-                o[m] = cur;
-              }
-            } else {
-#pragma unroll 1
-              for (int m = 0; m < rows / 2; ++m) a.out_d[o0 + (int64_t)m * inner] += racc[m * BL + r];
+            for (int j0 = j_first; j0 < rows; j0 += 32) {
+              const int m0 = j0 / 2;
+#pragma unroll
+              for (int m = m0; m < m0 + 8; ++m) a.out_d[o0 + (int64_t)m * inner] += racc[m * BL + r];
             }
           }
-          for (int m = 0; m < BR / 2; ++m) racc[m * BL + r] = 0.f;
+          for (int j0 = j_first; j0 < BR; j0 += 32)
+            for (int m = 0; m < 8; ++m) racc[(j0 / 2 + m) * BL + r] = 0.f;
         }
       }
     }
@@ -737,11 +685,6 @@ __device__ __forceinline__ int prod_off(bool contiguous, int t, int i) {
 }
 
 constexpr int BMANY_STAGES = 3;
-// eight epilogue warps, two per tensor-memory lane quarter on every other 16
-// columns (four warps, one row block's 64 outputs each thread, took longer over
-// an item than its copies and products)
-constexpr int BMANY_EPIW = 8;
-constexpr int BMANY_THREADS = BPROD + 32 + 32 * BMANY_EPIW;
 // the stages, and 1 KB to start them on a 1024-byte boundary (the swizzled
 // tiles' atoms)
 constexpr int BMANY_SMEM = BMANY_STAGES * BSTAGE + 1024;
@@ -759,7 +702,7 @@ constexpr int BMANY_SMEM = BMANY_STAGES * BSTAGE + 1024;
 // TOUT: the output transposed so, also for FP32 input (a chain's first pass
 // reading the caller's input).
 template <int XM, bool TOUT>
-__global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const TcParams P) {
+__global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcParams P) {
   constexpr int BSTAGES = BMANY_STAGES;
   constexpr bool TMA = XM == kTmaContiguous;
   constexpr bool PLANES = XM == kTmaPlanes;
@@ -785,7 +728,7 @@ __global__ void __launch_bounds__(BMANY_THREADS, 1) dense_bf16_many_kernel(const
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&accf_bar[b]), 1);
-      mbar_init(smem_u32(&acce_bar[b]), BMANY_EPIW);
+      mbar_init(smem_u32(&acce_bar[b]), BEPIW);
     }
     mbar_init(smem_u32(&done_bar), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1247,7 +1190,7 @@ size_t dense_bf16_t_bytes(int N) { return (size_t)((2 * N + BR - 1) / BR) * ((2 
 namespace {
 
 // the kernel's variants, indexed [FULL][kind], kind 0 plain, 1 ACC, 2 GRAD
-using BKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap, const int);
+using BKernel = void (*)(const DenseArgs, const unsigned char*, int*);
 constexpr int kBKinds = 3;
 BKernel bf16_kernel(bool full, int kind) {
   static const BKernel k[2][kBKinds] = {
@@ -1278,7 +1221,7 @@ const void* many_bf16_func(int mode) {
     default: return (const void*)dense_bf16_many_kernel<kInPlace, false>;
   }
 }
-int many_bf16_threads() { return BMANY_THREADS; }
+int many_bf16_threads() { return BTHREADS; }
 size_t many_bf16_smem() { return (size_t)BMANY_SMEM; }
 cudaError_t many_bf16_prepare() {
   cudaError_t e = cudaSuccess;
@@ -1294,25 +1237,6 @@ cudaError_t launch_bf16_build_t(const float2* T, unsigned char* Tblk, int N, cud
   bf16_build_t_kernel<<<256, 256, 0, s>>>(T, Tblk, N);
   return cudaGetLastError();
 }
-
-namespace {
-
-// The input tile map of a launch and how the kernel loads its chunks: FP32 TMA
-// tiles for contiguous lines of forward and adjoint passes; in place otherwise
-// (or when the map cannot be made).
-void input_map(const DenseArgs& a, CUtensorMap* map, int* mode) {
-  std::memset(map, 0, sizeof(*map));
-  *mode = kInPlace;
-  if (a.grad || a.inner != 1) return;
-  const cuuint64_t rows = (cuuint64_t)a.batch * (cuuint64_t)a.outer;  // every realization's lines
-  const cuuint64_t dims[2] = {(cuuint64_t)(2 * a.N), rows};
-  const cuuint64_t strides[1] = {(cuuint64_t)(2 * a.N) * 4};
-  const cuuint32_t box[2] = {32, (cuuint32_t)BL};
-  if (make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, a.in, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B))
-    *mode = kTmaContiguous;
-}
-
-}  // namespace
 
 bool many_bf16_line_map(const float2* base, int N, int64_t lines, void* map) {
   // [lines][2N floats], boxes of 32 floats x 128 lines, 128-byte swizzle: the
@@ -1340,12 +1264,9 @@ bool many_bf16_plane_map(const uint32_t* head, int N, int64_t lines, int64_t pla
 }
 
 cudaError_t launch_dense_bf16(const DenseArgs& a, const unsigned char* Tblk, int* err, int grid, cudaStream_t s) {
-  CUtensorMap map;
-  int mode;
-  input_map(a, &map, &mode);
   const bool full = (2 * a.N) % BR == 0;
   const int kind = a.grad ? 2 : (a.acc ? 1 : 0);  // backward passes never accumulate over the batch
-  bf16_kernel(full, kind)<<<grid, BTHREADS, bf16_kind_smem(kind), s>>>(a, Tblk, err, map, mode);
+  bf16_kernel(full, kind)<<<grid, BTHREADS, bf16_kind_smem(kind), s>>>(a, Tblk, err);
   return cudaGetLastError();
 }
 
