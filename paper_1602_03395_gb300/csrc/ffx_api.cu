@@ -477,6 +477,8 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       // one or two terms on lines of 16, 64, 256 or 1024 points: the kernel
       // with four-step line transforms in registers
       e = launch_conv(a, kind, ax.N, p->sms, stream);
+    } else if (line3_supported(ax.N, inner, ax.g)) {
+      e = launch_line3(a, kind, ax.N, p->sms, stream);
     } else {
       const PassKernelInfo& info = adjoint ? ax.adj : (cform == FFX_FORM_PAPER ? ax.paper : ax.foldk);
       const int capacity = adjoint ? ax.grid_adj : (cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold);
@@ -509,11 +511,11 @@ bool tm32_sum(const Axis& ax, int cform, const float2* in, const float* out_d) {
 // partial densities that are added at the end.  The rule counts steps, waves of
 // resident blocks times realizations each: the fewest groups within 5% of the
 // fewest steps, and one group unless that saves a fifth of them.  (The mean of
-// 512 realizations of one 2048-point line, lam = 20: 97 ms in one group, 0.41 ms
-// in 512.)  The partial densities take at most kSumBytes.
+// 512 realizations of one 2048-point line, lam = 20, on the FFT engine of
+// ffx_pass.cuh: 97 ms in one group, 0.41 ms in 512.)  The partial densities take at most kSumBytes.
 constexpr size_t kSumBytes = size_t(256) << 20;
 int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, bool tm32, int64_t lines,
-                   int64_t batch) {
+                   int64_t inner, int64_t batch) {
   if (batch * lines < kDenseFewLines && cform == FFX_FORM_DENSE) return 1;  // the few-lines kernel
   auto steps = [&](int64_t ncols) -> int64_t {  // waves of a launch over ncols lines
     int64_t tiles, cap;
@@ -528,6 +530,10 @@ int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, 
     } else if (cform == FFX_FORM_DENSE) {
       tiles = ax.N <= kDenseInPlaceMaxN ? dense_small_tiles(ax.N, ncols) : dense_tiles(ax.N, ncols);
       cap = ax.N <= kDenseInPlaceMaxN ? ax.grid_dense_small : ax.grid_dense;
+    } else if (line3_supported(ax.N, inner, ax.g)) {
+      const int per = line3_lines(ax.N);
+      tiles = (ncols + per - 1) / per;
+      cap = 2 * (int64_t)p->sms;
     } else {
       const PassKernelInfo& info = cform == FFX_FORM_PAPER ? ax.paper : ax.foldk;
       cap = cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold;
@@ -571,7 +577,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   bool tm32 = false;
   if (acc && batch > 1) {
     tm32 = !io && tm32_sum(ax, cform, in, out_d);
-    groups = sum_groups(p, ax, cform, io || (inner == 1 && ax.pl_t[0]), tm32, lines, batch);
+    groups = sum_groups(p, ax, cform, io || (inner == 1 && ax.pl_t[0]), tm32, lines, inner, batch);
   }
   if (groups > 1 || tm32) {
     // partial densities of the groups, then their sum
@@ -1077,11 +1083,15 @@ int build_dense(ffx_plan_s* p, int j, float2* T, float2* TH, float2* scratch, cu
   a.tab.F = ax.F;
   a.tab.tw = ax.tw;
   a.tab.fold = ax.fold;
-  a.qg = choose_qg(ax.foldk, N, ax.lam, ax.grid_fold);
-  const int lines = pass_lines_per_tile(ax.foldk, a.qg);
-  int64_t grid = (N + lines - 1) / lines;
-  if (grid > ax.grid_fold) grid = ax.grid_fold;
-  e = ax.foldk.launch(a, (int)grid, s);
+  if (line3_supported(N, 1, ax.g)) {
+    e = launch_line3(a, KIND_FWD_FOLD, N, p->sms, s);
+  } else {
+    a.qg = choose_qg(ax.foldk, N, ax.lam, ax.grid_fold);
+    const int lines = pass_lines_per_tile(ax.foldk, a.qg);
+    int64_t grid = (N + lines - 1) / lines;
+    if (grid > ax.grid_fold) grid = ax.grid_fold;
+    e = ax.foldk.launch(a, (int)grid, s);
+  }
   if (e == cudaSuccess) e = launch_dense_build(O, T, TH, N, s);
   if (e != cudaSuccess) return cuda_fail(e, "dense map");
   ax.T = T;

@@ -81,6 +81,13 @@ bool supported_length(int64_t N);
 bool conv_supported(int N, int lam, int acc, int kind);
 cudaError_t launch_conv(const PassArgs& a, int kind, int N, int sms, cudaStream_t s);
 
+// FFT-form passes along contiguous lines of 512, 1024 or 2048 points with
+// gcd(lam, N) <= 16 (ffx_line3.cu); lines per block, and the blocks that run at
+// once are 2 per SM
+bool line3_supported(int N, int64_t inner, int g);
+int line3_lines(int N);
+cudaError_t launch_line3(const PassArgs& a, int kind, int N, int sms, cudaStream_t s);
+
 // Set the calling thread's message for ffx_last_error().
 void set_last_error_message(const char* msg);
 
