@@ -32,7 +32,7 @@
 #include "ffx_internal.h"
 
 #ifndef FFX_PASS_MIN_BLOCKS
-#define FFX_PASS_MIN_BLOCKS 3  // resident 256-thread blocks per SM the register budget aims for
+#define FFX_PASS_MIN_BLOCKS 3  // resident 256-thread blocks per SM the register budget aims for, 8 points a thread
 #endif
 
 namespace ffx {
@@ -414,8 +414,17 @@ __device__ __forceinline__ void pass_tiles(const PassArgs& a, int64_t first, int
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
+// Threads of 12 or 16 points spill 0.2-1 KB at three blocks per SM (85
+// registers): with two, fold passes at lam = 20 take 0.240 ms instead of 0.273
+// (4096 lines of 384 points) and three of 96 points 0.466 ms instead of 0.558;
+// with 8 points three blocks stay ahead (8192 lines of 256: 0.337 against 0.349).
+template <class P>
+constexpr int pass_min_blocks() {
+  return P::E >= 12 ? 2 : FFX_PASS_MIN_BLOCKS;
+}
+
 template <class P, int KIND, int G>
-__global__ void __launch_bounds__(P::T * G, FFX_PASS_MIN_BLOCKS) pass_kernel(const PassArgs a) {
+__global__ void __launch_bounds__(P::T * G, pass_min_blocks<P>()) pass_kernel(const PassArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   pass_tiles<P, KIND, G>(a, blockIdx.x, INT64_MAX, gridDim.x, smem);
 }
