@@ -553,8 +553,13 @@ int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, 
   int64_t best = one;
   for (int64_t g = 2; g <= gmax; g = next(g)) best = std::min(best, cost(g));
   if (5 * best > 4 * one) return 1;
+  // a step is at least ~2 us, in the FFT forms ~2 us a term; the partial
+  // densities cost ~6 us of launches and their traffic, and have to be gained
+  // twice over (256x16x64 x 7: 85 us in one group, 100 us in several)
+  const double step_us = cform == FFX_FORM_PAPER || cform == FFX_FORM_FOLD ? 2.0 * ax.lam : 2.0;
   for (int64_t g = 2; g <= gmax; g = next(g))
-    if (20 * cost(g) <= 21 * best) return g;
+    if (20 * cost(g) <= 21 * best)
+      return (double)(one - cost(g)) * step_us > 2.0 * (6.0 + (double)g * (double)p->M * 8e-6 / 5.0) ? g : 1;
   return 1;
 }
 
