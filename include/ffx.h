@@ -486,9 +486,8 @@ int64_t ffx_plan_launch_count(ffx_plan_t plan);
 int ffx_plan_bf16_chain(ffx_plan_t plan, int64_t batch);
 
 /* 1 if such a chain starts with a launch that splits its FP32 input into
- * planes; 0 if its first pass reads the FP32 input itself (a last axis of 256
- * points or more, in multiples of 128, with enough lines to fill the chip) or
- * the call is no chain. */
+ * planes; 0 if its first pass reads the FP32 input itself (a last axis of any
+ * length but 192, with enough lines to fill the chip) or the call is no chain. */
 int ffx_plan_chain_split(ffx_plan_t plan, int64_t batch);
 
 /* Forward pass order: writes the lattice axis of pass k to order[k],

@@ -163,7 +163,8 @@ cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cu
 cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
                                int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s);
 // whether the pass takes FP32 lines as they are (DenseArgs::in) and splits them
-// itself: lengths that run on CTA pairs, with an item for every pair
+// itself: every length but 192, with an item for every block (pair of blocks)
+// that runs at once
 bool plane_pass_splits(int N, int64_t ncols, int sms);
 // work items of a pass over ncols lines, and how many run at once
 int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once);

@@ -77,15 +77,13 @@ __host__ __device__ constexpr int ptchunk(int rb) { return 2 * ppart(rb); }
 // outputs per item: the whole line up to 128 points, else 128, or 96 for 192
 __host__ __device__ constexpr int prow_block(int N) { return N <= 128 ? N : (N % 128 == 0 ? 128 : 96); }
 // stages: T resident (N = RB) leaves the rest to X tiles
-__host__ __device__ constexpr int pstages(int rb, bool res) {
-  return res ? (rb == 64 ? 5 : rb == 96 ? 4 : 3) : (rb == 96 ? 4 : 3);
-}
+__host__ __device__ constexpr int pstages(int rb, bool res) { return res ? (rb == 64 ? 5 : rb == 96 ? 4 : 3) : 4; }
 __host__ __device__ constexpr int psmem(int rb, bool res) {
   // + 1 KB to start the swizzled tiles on a 1024-byte boundary
   return (res ? (rb / PKC) * ptchunk(rb) : 0) + pstages(rb, res) * (PX + (res ? 0 : ptchunk(rb))) + 1024;
 }
-static_assert(psmem(128, true) <= 226 * 1024 && psmem(128, false) <= 226 * 1024 && psmem(96, true) <= 226 * 1024 &&
-                  psmem(96, false) <= 226 * 1024 && psmem(64, true) <= 226 * 1024,
+static_assert(psmem(128, true) <= 226 * 1024 && psmem(96, true) <= 226 * 1024 && psmem(96, false) <= 226 * 1024 &&
+                  psmem(64, true) <= 226 * 1024 && psmem(64, false) <= 226 * 1024,
               "shared memory");
 
 // the instruction descriptor's "negate A" bit
@@ -371,19 +369,93 @@ __device__ __forceinline__ void plane_epilogue(const DenseArgs& a, int warp, int
   }
 }
 
-// RB outputs per item, T resident (RES) or streamed.
-template <int RB, bool RES, int OUT>
-__global__ void __launch_bounds__(PTHREADS, 1)
+// FP32 input (F32 kernels): contiguous FP32 lines, split on the way in (the first
+// pass of a chain, or a single pass).  The FP32 tile of a chunk (two boxes of 16
+// points a line, 128-byte swizzle) is exactly as large as its head and tail
+// rows and lands where they go: row n of the first box on head row n, of the
+// second on tail row n.  Four producer warps (12-15), a thread a line, read
+// their line's 256 bytes, split them and write the two rows over them, so no
+// thread waits for another.  Registers move from the control and producer warps
+// to the epilogue's (setmaxnreg): 56 + 2 x 176 + 104 a thread of the four
+// warpgroups, the 4 x 128 of the launch.  Splitting loads shared memory with 64
+// KB more a chunk (232 KB, 1812 clocks against 1536 of products on a CTA pair), and every
+// row block splits its lines again, but the separate split reads and writes 16
+// bytes a point of HBM.
+constexpr int PTHREADS_F32 = PTHREADS + 128;
+static_assert(PTHREADS_F32 == 512 && 56 + 2 * 176 + 104 == 4 * 128, "register split");
+static_assert(PL == 128, "a producer thread per line");
+
+// Splits line n of a chunk's FP32 tile at x into its head and tail rows.
+__device__ __forceinline__ void split_line(unsigned char* x, int n, bool unsplit) {
+  unsigned char* const row = x + n * 128;
+  const int sw = n & 7;
+  float4 v[2][8];
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[g][c] = *reinterpret_cast<const float4*>(row + g * PXPART + ((c ^ sw) << 4));
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      // eight points of group g: 16 bytes of real and of imaginary parts
+      uint32_t r[4], m[4], rl[4], ml[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4 f = v[g][4 * k + c];
+        r[c] = bf2(f.x, f.z);
+        m[c] = bf2(f.y, f.w);
+        rl[c] = bf2(f.x - bf_lo(r[c]), f.z - bf_hi(r[c]));
+        ml[c] = bf2(f.y - bf_lo(m[c]), f.w - bf_hi(m[c]));
+      }
+      const int ore = ((4 * g + k) ^ sw) << 4, oim = ((4 * g + 2 + k) ^ sw) << 4;
+      *reinterpret_cast<uint4*>(row + ore) = make_uint4(r[0], r[1], r[2], r[3]);
+      *reinterpret_cast<uint4*>(row + oim) = make_uint4(m[0], m[1], m[2], m[3]);
+      if (!unsplit) {
+        *reinterpret_cast<uint4*>(row + PXPART + ore) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+        *reinterpret_cast<uint4*>(row + PXPART + oim) = make_uint4(ml[0], ml[1], ml[2], ml[3]);
+      }
+    }
+}
+
+// The producer threads' loop over the block's chunks: line n of each tile, once
+// it has landed (raw_bar); done(stage): the warp has split its lines.
+template <int NST, int STAGE, class Done>
+__device__ __forceinline__ void split_tiles(unsigned char* stages, int n, int lane, int64_t total, bool unsplit,
+                                            uint64_t* raw_bar, volatile int* s_abort, const Done& done) {
+  int s = 0;
+  int64_t u = 0;
+#pragma unroll 1
+  for (int64_t ci = 0; ci < total; ++ci) {
+    bool ok = true;
+    if (lane == 0) ok = mbar_wait(smem_u32(&raw_bar[s]), (uint32_t)(u & 1), s_abort);
+    if (!__all_sync(0xffffffffu, ok)) break;
+    split_line(stages + s * STAGE, n, unsplit);
+    fence_async_smem();
+    __syncwarp();
+    if (lane == 0) done(s);
+    if (++s == NST) {
+      s = 0;
+      ++u;
+    }
+  }
+}
+
+// RB outputs per item, T resident (RES) or streamed; F32 (with RES): FP32 input.
+template <int RB, bool RES, int OUT, bool F32>
+__global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
     plane_pass_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
                       const __grid_constant__ CUtensorMap xmap) {
   constexpr int NST = pstages(RB, RES);
   constexpr int TCH = ptchunk(RB), TPART = ppart(RB);
   constexpr int STAGE = PX + (RES ? 0 : TCH);
+  constexpr int TB = !RES && RB == 64 ? 128 : RB;  // T's rows per block
   constexpr int NBUF = RB == 64 ? 2 : 1;  // accumulator sets
   constexpr bool ACC = OUT == kOutSum;
   extern __shared__ __align__(1024) unsigned char psm_raw[];
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], t_bar;
+  static_assert(RES || !F32, "FP32 input comes with resident T");
+  __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], raw_bar[PMAXST], t_bar;
   __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
@@ -402,8 +474,9 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   if (warp == 1) tmem_alloc(&tmem_slot, 512);
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), 1);
+      mbar_init(smem_u32(&full_bar[s]), F32 ? 4 : 1);  // FP32 input: the producer warps
       mbar_init(smem_u32(&empty_bar[s]), 1);
+      mbar_init(smem_u32(&raw_bar[s]), 1);
     }
     mbar_init(smem_u32(&t_bar), 1);
     for (int b = 0; b < 2 * NBUF; ++b) {
@@ -423,114 +496,140 @@ __global__ void __launch_bounds__(PTHREADS, 1)
   const uint32_t t_res = smem_u32(psm);
   const uint32_t stages = t_res + (uint32_t)(RES ? (RB / PKC) * TCH : 0);
 
-  if (warp == 0) {
-    // ---------------- copies ----------------
-    if (lane == 0) {
-      const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
-      const uint32_t xbytes = unsplit ? (uint32_t)PXPART : (uint32_t)PX;
-      const uint32_t tbytes = unsplit ? (uint32_t)TPART : (uint32_t)TCH;  // unsplit: the head rows
-      if (RES) {
-        mbar_expect_tx(smem_u32(&t_bar), tbytes * (uint32_t)kchunks);
-        for (int kc = 0; kc < kchunks; ++kc)
-          bulk_g2s(t_res + (uint32_t)(kc * TCH), Tblk + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
-      }
-      pdl_wait();  // T is the plan's own; the lines may be the predecessor's output
-      const int64_t total = my_items * nb * kchunks;
-      int64_t iw = blockIdx.x, u = 0;
-      int ib = 0, ikc = 0, is = 0;
+  if (warp < 4) {
+    if constexpr (F32) asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (warp == 0) {
+      // ---------------- copies ----------------
+      if (lane == 0) {
+        const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
+        const uint32_t xbytes = unsplit ? (uint32_t)PXPART : (uint32_t)PX;
+        const uint32_t tbytes = unsplit ? (uint32_t)TPART : (uint32_t)TCH;  // unsplit: the head rows
+        if (RES) {
+          mbar_expect_tx(smem_u32(&t_bar), tbytes * (uint32_t)kchunks);
+          for (int kc = 0; kc < kchunks; ++kc)
+            bulk_g2s(t_res + (uint32_t)(kc * TCH), Tblk + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
+        }
+        pdl_wait();  // T is the plan's own; the lines may be the predecessor's output
+        const int64_t total = my_items * nb * kchunks;
+        int64_t iw = blockIdx.x, u = 0;
+        int ib = 0, ikc = 0, is = 0;
 #pragma unroll 1
-      for (int64_t ci = 0; ci < total; ++ci) {
-        // chunk ci into stage `is` once the products of chunk ci - NST freed it
-        if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
-        const int64_t ct = RES ? iw : iw / mtiles;
-        const uint32_t st = stages + (uint32_t)(is * STAGE);
-        const uint32_t fb = smem_u32(&full_bar[is]);
-        mbar_expect_tx(fb, xbytes + (RES ? 0u : tbytes));
-        // rows: the tile's lines (realization ib's when accumulating); x: the
-        // chunk's 64 values; z: the head plane (and the tail plane)
-        const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
-        asm volatile(
-            "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-            "[%5];" ::"r"(st),
-            "l"(map_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
-            : "memory");
-        if (!RES) {
-          const int mt = (int)(iw - ct * mtiles);
-          bulk_g2s(st + (uint32_t)PX, Tblk + ((size_t)mt * kchunks + ikc) * TCH, tbytes, fb);
+        for (int64_t ci = 0; ci < total; ++ci) {
+          // chunk ci into stage `is` once the products of chunk ci - NST freed it
+          if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
+          const int64_t ct = RES ? iw : iw / mtiles;
+          const uint32_t st = stages + (uint32_t)(is * STAGE);
+          const uint32_t fb = smem_u32(F32 ? &raw_bar[is] : &full_bar[is]);
+          mbar_expect_tx(fb, F32 ? (uint32_t)PX : xbytes + (RES ? 0u : tbytes));
+          // rows: the tile's lines (realization ib's when accumulating); x: the
+          // chunk's 64 values; z: the head plane (and the tail plane)
+          const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
+          if (F32) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              asm volatile(
+                  "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                  "[%4];" ::"r"(st + (uint32_t)(h * PXPART)),
+                  "l"(map_addr), "r"(ikc * 2 * PKC + 32 * h), "r"(row), "r"(fb)
+                  : "memory");
+          } else {
+            asm volatile(
+                "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                "%4}], [%5];" ::"r"(st),
+                "l"(map_addr), "r"(ikc * 2 * PKC), "r"(row), "r"(0), "r"(fb)
+                : "memory");
+          }
+          if (!RES) {
+            const int mt = (int)(iw - ct * mtiles);
+            if (RB == TB) {
+              bulk_g2s(st + (uint32_t)PX, Tblk + ((size_t)mt * kchunks + ikc) * TCH, tbytes, fb);
+            } else {
+              // half of a 128-row block: its head rows, then its tail rows
+              const unsigned char* src = Tblk + ((size_t)(mt >> 1) * kchunks + ikc) * ptchunk(TB) + (mt & 1) * TPART;
+              bulk_g2s(st + (uint32_t)PX, src, TPART, fb);
+              if (!unsplit) bulk_g2s(st + (uint32_t)(PX + TPART), src + ppart(TB), TPART, fb);
+            }
+          }
+          if (++is == NST) {
+            is = 0;
+            ++u;
+          }
+          if (++ikc == kchunks) {
+            ikc = 0;
+            if (++ib == nb) {
+              ib = 0;
+              iw += gridDim.x;
+            }
+          }
         }
-        if (++is == NST) {
-          is = 0;
-          ++u;
+        // nothing of this thread's may still be in flight at exit
+        if (RES) mbar_wait_own(smem_u32(&t_bar), 0u, &s_abort);
+        for (int q = 0; q < NST; ++q) {
+          const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+          if (uq >= 0) mbar_wait_own(smem_u32(F32 ? &raw_bar[q] : &full_bar[q]), (uint32_t)(uq & 1), &s_abort);
         }
-        if (++ikc == kchunks) {
-          ikc = 0;
-          if (++ib == nb) {
-            ib = 0;
-            iw += gridDim.x;
+      }
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---------------- products: the whole warp, one elected lane issuing ----------------
+      int64_t u = 0;
+      int s = 0;
+      bool ok = !RES || mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
+      const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
+#pragma unroll 1
+      for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
+        const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
+        const int64_t v = NBUF == 2 ? sub >> 1 : sub;
+        const uint32_t prev = (uint32_t)((v - 1) & 1);
+        const uint32_t dre = tmem + (uint32_t)(buf * 4 * RB), dim = dre + 2 * RB;
+#pragma unroll 1
+        for (int kc = 0; kc < kchunks; ++kc) {
+          const bool last = kc == kchunks - 1;
+          ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+               (kc > 0 || v == 0 || mbar_wait(smem_u32(&acce_bar[2 * buf]), prev, &s_abort));
+          if (!ok) break;
+          tc_fence_after();
+          const uint32_t st = stages + (uint32_t)(s * STAGE);
+          const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
+          plane_half<1, RB, false>(dre, st, tb, tb, id1, id2, kc == 0, unsplit);
+          if (last) {
+            if (elect_one()) mma_commit(smem_u32(&accf_bar[2 * buf]));
+            __syncwarp();
+          }
+          if (kc == 0 && v > 0) {
+            ok = mbar_wait(smem_u32(&acce_bar[2 * buf + 1]), prev, &s_abort);
+            if (!ok) break;
+            tc_fence_after();
+          }
+          plane_half<1, RB, true>(dim, st, tb, tb, id1, id2, kc == 0, unsplit);
+          if (elect_one()) {
+            mma_commit(smem_u32(&empty_bar[s]));
+            if (last) mma_commit(smem_u32(&accf_bar[2 * buf + 1]));
+          }
+          __syncwarp();
+          if (++s == NST) {
+            s = 0;
+            ++u;
           }
         }
       }
-      // nothing of this thread's may still be in flight at exit
-      if (RES) mbar_wait_own(smem_u32(&t_bar), 0u, &s_abort);
-      for (int q = 0; q < NST; ++q) {
-        const int64_t uq = q < is ? u : u - 1;  // stage q's last use
-        if (uq >= 0) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
-      }
+      // whatever happened, the tensor cores finish this warp's work before exit
+      if (elect_one()) mma_commit(smem_u32(&done_bar));
+      __syncwarp();
+      mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
     }
-    __syncwarp();
-  } else if (warp == 1) {
-    // ---------------- products: the whole warp, one elected lane issuing ----------------
-    int64_t u = 0;
-    int s = 0;
-    bool ok = !RES || mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
-    const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
-#pragma unroll 1
-    for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
-      const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
-      const int64_t v = NBUF == 2 ? sub >> 1 : sub;
-      const uint32_t prev = (uint32_t)((v - 1) & 1);
-      const uint32_t dre = tmem + (uint32_t)(buf * 4 * RB), dim = dre + 2 * RB;
-#pragma unroll 1
-      for (int kc = 0; kc < kchunks; ++kc) {
-        const bool last = kc == kchunks - 1;
-        ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-             (kc > 0 || v == 0 || mbar_wait(smem_u32(&acce_bar[2 * buf]), prev, &s_abort));
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t st = stages + (uint32_t)(s * STAGE);
-        const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
-        plane_half<1, RB, false>(dre, st, tb, tb, id1, id2, kc == 0, unsplit);
-        if (last) {
-          if (elect_one()) mma_commit(smem_u32(&accf_bar[2 * buf]));
-          __syncwarp();
-        }
-        if (kc == 0 && v > 0) {
-          ok = mbar_wait(smem_u32(&acce_bar[2 * buf + 1]), prev, &s_abort);
-          if (!ok) break;
-          tc_fence_after();
-        }
-        plane_half<1, RB, true>(dim, st, tb, tb, id1, id2, kc == 0, unsplit);
-        if (elect_one()) {
-          mma_commit(smem_u32(&empty_bar[s]));
-          if (last) mma_commit(smem_u32(&accf_bar[2 * buf + 1]));
-        }
-        __syncwarp();
-        if (++s == NST) {
-          s = 0;
-          ++u;
-        }
-      }
-    }
-    // whatever happened, the tensor cores finish this warp's work before exit
-    if (elect_one()) mma_commit(smem_u32(&done_bar));
-    __syncwarp();
-    mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
-  } else if (warp >= 4) {
+  } else if (warp < 12) {
     // ---------------- epilogue ----------------
+    if constexpr (F32) asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
     plane_epilogue<RB, OUT>(a, warp, lane, tmem, smem_u32(&accf_bar[0]), blockIdx.x, gridDim.x, my_items, mtiles, 1, 0,
-                            nb, unsplit, &s_abort, [&](int bar) {
-                              mbar_arrive(smem_u32(&acce_bar[bar]));
-                            });
+                            nb, unsplit, &s_abort, [&](int bar) { mbar_arrive(smem_u32(&acce_bar[bar])); });
+  } else {
+    // ---------------- FP32 input: split into the stages ----------------
+    if constexpr (F32) {
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+      split_tiles<NST, STAGE>(psm + (RB / PKC) * TCH, tid - 384, lane, my_items * nb * kchunks, unsplit, raw_bar, &s_abort,
+                              [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
+    }
   }
 
   tc_fence_before();
@@ -573,57 +672,9 @@ constexpr int QSTAGE = PX + QTP + QTQ;    // 56 KB
 constexpr int QSMEM = QST * QSTAGE + 1024;
 static_assert(QSMEM <= 226 * 1024, "shared memory");
 
-// F32: the input is contiguous FP32 lines, split on the way in (the first pass
-// of a chain, or a single pass).  The FP32 tile of a chunk (two boxes of 16
-// points a line, 128-byte swizzle) is exactly as large as its head and tail
-// rows and lands where they go: row n of the first box on head row n, of the
-// second on tail row n.  Four producer warps (12-15), a thread a line, read
-// their line's 256 bytes, split them and write the two rows over them, so no
-// thread waits for another.  Registers move from the control and producer warps
-// to the epilogue's (setmaxnreg): 56 + 2 x 176 + 104 a thread of the four
-// warpgroups, the 4 x 128 of the launch.  Splitting loads shared memory with 64
-// KB more a chunk (232 KB, 1812 clocks against 1536 of products), and every row
-// block splits its lines again, but the separate split reads and writes 16
-// bytes a point of HBM.
-constexpr int QTHREADS_F32 = PTHREADS + 128;
-static_assert(QTHREADS_F32 == 512 && 56 + 2 * 176 + 104 == 4 * 128, "register split");
-static_assert(PL == 128, "a producer thread per line");
-
-// Splits line n of a chunk's FP32 tile at x into its head and tail rows.
-__device__ __forceinline__ void split_line(unsigned char* x, int n, bool unsplit) {
-  unsigned char* const row = x + n * 128;
-  const int sw = n & 7;
-  float4 v[2][8];
-#pragma unroll
-  for (int g = 0; g < 2; ++g)
-#pragma unroll
-    for (int c = 0; c < 8; ++c) v[g][c] = *reinterpret_cast<const float4*>(row + g * PXPART + ((c ^ sw) << 4));
-#pragma unroll
-  for (int g = 0; g < 2; ++g)
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      // eight points of group g: 16 bytes of real and of imaginary parts
-      uint32_t r[4], m[4], rl[4], ml[4];
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        const float4 f = v[g][4 * k + c];
-        r[c] = bf2(f.x, f.z);
-        m[c] = bf2(f.y, f.w);
-        rl[c] = bf2(f.x - bf_lo(r[c]), f.z - bf_hi(r[c]));
-        ml[c] = bf2(f.y - bf_lo(m[c]), f.w - bf_hi(m[c]));
-      }
-      const int ore = ((4 * g + k) ^ sw) << 4, oim = ((4 * g + 2 + k) ^ sw) << 4;
-      *reinterpret_cast<uint4*>(row + ore) = make_uint4(r[0], r[1], r[2], r[3]);
-      *reinterpret_cast<uint4*>(row + oim) = make_uint4(m[0], m[1], m[2], m[3]);
-      if (!unsplit) {
-        *reinterpret_cast<uint4*>(row + PXPART + ore) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
-        *reinterpret_cast<uint4*>(row + PXPART + oim) = make_uint4(ml[0], ml[1], ml[2], ml[3]);
-      }
-    }
-}
-
+// F32: FP32 lines, split in the stages as in plane_pass_kernel.
 template <int OUT, bool F32>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? QTHREADS_F32 : PTHREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
     plane_pair_kernel(const DenseArgs a, int* err,
                       const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap tmap) {
   constexpr int RB = 128;
@@ -813,23 +864,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? QTHREADS_F32 :
     if constexpr (F32) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
       const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
-      const int n = tid - 384;  // the tile's line
-      int s = 0;
-      int64_t u = 0;
-#pragma unroll 1
-      for (int64_t ci = 0; ci < total; ++ci) {
-        bool ok = true;
-        if (lane == 0) ok = mbar_wait(smem_u32(&raw_bar[s]), (uint32_t)(u & 1), &s_abort);
-        if (!__all_sync(0xffffffffu, ok)) break;
-        split_line(psm + s * QSTAGE, n, unsplit);
-        fence_async_smem();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(full0 + 8u * (uint32_t)s);
-        if (++s == QST) {
-          s = 0;
-          ++u;
-        }
-      }
+      split_tiles<QST, QSTAGE>(psm, tid - 384, lane, total, unsplit, raw_bar, &s_abort,
+                               [&](int st) { mbar_arrive_cluster(full0 + 8u * (uint32_t)st); });
     }
   }
 
@@ -908,8 +944,14 @@ __global__ void __launch_bounds__(256)
   }
 }
 
-// passes that run on CTA pairs: streaming, in whole row blocks
-bool pair_pass(int N) { return N >= 256 && N % 128 == 0; }
+// lengths that run on CTA pairs: streaming, in whole row blocks
+bool pair_length(int N) { return N >= 256 && N % 128 == 0; }
+int64_t pair_items(int N, int64_t ncols) { return (ncols + 2 * PL - 1) / (2 * PL) * (N / 128); }
+// Passes with fewer items than half the pairs leave most of the chip idle, and
+// their time is one item's: 128 lines x 64 outputs on single CTAs then, four
+// times as many items of a quarter of the work (a call over 745 lines of 1024
+// points: 40.6 us as 24 pairs' items, 34.2 us as 96 blocks').
+bool pair_pass(int N, int64_t ncols, int sms) { return pair_length(N) && 4 * pair_items(N, ncols) >= sms; }
 
 using PKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap);
 using QKernel = void (*)(const DenseArgs, int*, const CUtensorMap, const CUtensorMap);
@@ -918,20 +960,23 @@ struct QVariant {
   static constexpr QKernel fn[kPOuts] = {plane_pair_kernel<kOutPlanes, F32>, plane_pair_kernel<kOutComplex, F32>,
                                          plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>};
 };
-template <int RB, bool RES>
+template <int RB, bool RES, bool F32>
 struct PVariant {
-  static constexpr PKernel fn[kPOuts] = {plane_pass_kernel<RB, RES, kOutPlanes>, plane_pass_kernel<RB, RES, kOutComplex>,
-                                         plane_pass_kernel<RB, RES, kOutDensity>, plane_pass_kernel<RB, RES, kOutSum>};
+  static constexpr PKernel fn[kPOuts] = {
+      plane_pass_kernel<RB, RES, kOutPlanes, F32>, plane_pass_kernel<RB, RES, kOutComplex, F32>,
+      plane_pass_kernel<RB, RES, kOutDensity, F32>, plane_pass_kernel<RB, RES, kOutSum, F32>};
 };
-PKernel single_kernel(int N, int out) {
+PKernel single_kernel(int N, int out, bool f32) {
   switch (N) {
-    case 64: return PVariant<64, true>::fn[out];
-    case 96: return PVariant<96, true>::fn[out];
-    case 128: return PVariant<128, true>::fn[out];
-    default: return PVariant<96, false>::fn[out];  // 192
+    case 64: return f32 ? PVariant<64, true, true>::fn[out] : PVariant<64, true, false>::fn[out];
+    case 96: return f32 ? PVariant<96, true, true>::fn[out] : PVariant<96, true, false>::fn[out];
+    case 128: return f32 ? PVariant<128, true, true>::fn[out] : PVariant<128, true, false>::fn[out];
+    case 192: return PVariant<96, false, false>::fn[out];
+    default: return PVariant<64, false, false>::fn[out];
   }
 }
-int single_smem(int N) { return N <= 128 ? psmem(N, true) : psmem(96, false); }
+int single_rows(int N) { return N <= 128 ? N : N == 192 ? 96 : 64; }  // outputs per item
+int single_smem(int N) { return psmem(single_rows(N), N <= 128); }
 
 // `rows` rows of `cols` FP32 values (a multiple of 32) in tiles of 32 x box_rows
 bool f32_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int box_rows) {
@@ -962,15 +1007,17 @@ size_t plane_t_bytes(int N) { return (size_t)N * N * 8; }
 
 cudaError_t plane_pass_prepare(int N) {
   cudaError_t e = cudaSuccess;
-  for (int k = 0; k < kPOuts && e == cudaSuccess; ++k)
-    if (pair_pass(N)) {
+  for (int k = 0; k < kPOuts && e == cudaSuccess; ++k) {
+    if (pair_length(N)) {
       e = cudaFuncSetAttribute((const void*)QVariant<false>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-    } else {
-      e = cudaFuncSetAttribute((const void*)single_kernel(N, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               single_smem(N));
     }
+    for (bool f32 : {false, true})
+      if (e == cudaSuccess && (!f32 || N <= 128))
+        e = cudaFuncSetAttribute((const void*)single_kernel(N, k, f32), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 single_smem(N));
+  }
   return e;
 }
 
@@ -995,16 +1042,16 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
                     unsplit);
 }
 
-bool plane_pass_splits(int N, int64_t ncols, int sms) {
-  int64_t at_once;
-  return pair_pass(N) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
+int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
+  // one pair of blocks per two SMs, or one block per SM
+  const bool pair = pair_pass(N, ncols, sms);
+  *at_once = std::max(1, pair ? sms / 2 : sms);
+  return pair ? pair_items(N, ncols) : (ncols + PL - 1) / PL * (N / single_rows(N));
 }
 
-int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
-  // one block per SM, or one pair of blocks per two
-  const int per = pair_pass(N) ? 2 : 1;
-  *at_once = std::max(1, sms / per);
-  return (ncols + per * PL - 1) / (per * PL) * (N / prow_block(N));
+bool plane_pass_splits(int N, int64_t ncols, int sms) {
+  int64_t at_once;
+  return (N <= 128 || pair_pass(N, ncols, sms)) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
 }
 
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
@@ -1014,7 +1061,8 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     a.oinner = a.inner;
   }
   const bool f32 = !a.in_bf;
-  if (a.inner != 1 || a.grad || (f32 && !pair_pass(a.N))) return cudaErrorInvalidValue;
+  const bool pair = pair_pass(a.N, a.ncols, sms);
+  if (a.inner != 1 || a.grad || (f32 && !pair && a.N > 128)) return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines
   CUtensorMap xmap, tmap;
@@ -1025,14 +1073,15 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   int64_t at_once;
   int64_t grid = std::min(plane_pass_tiles(a.N, a.ncols, sms, &at_once), at_once);
   if (grid < 1) grid = 1;
-  if (pair_pass(a.N)) {
+  if (pair) {
     grid *= 2;
     // T's chunks as rows of 128 bytes (stored swizzled)
     if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
     return launch_pdl(f32 ? QVariant<true>::fn[out] : QVariant<false>::fn[out], (int)grid,
-                      f32 ? QTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
+                      f32 ? PTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
-  return launch_pdl(single_kernel(a.N, out), (int)grid, PTHREADS, single_smem(a.N), s, a, Tblk, err, xmap);
+  return launch_pdl(single_kernel(a.N, out, f32), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,
+                    err, xmap);
 }
 
 }  // namespace ffx

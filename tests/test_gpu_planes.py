@@ -29,6 +29,7 @@ CASES = [
     ((512, 192), (4, 7), 1),      # four row blocks; 192 in two blocks of 96
     ((1024, 32 * 3), (6, 5), 1),  # eight row blocks
     ((64, 64, 256), (4, 5, 6), 3),
+    ((512, 64), (4, 5), 40),      # 64-output items on single CTAs (too few for pairs) and on pairs
     # single passes over contiguous lines (a 1-D field has no chain)
     ((256,), (100,), 5), ((256,), (3,), 129), ((768,), (7,), 257), ((128,), (9,), 131), ((192,), (4,), 3),
     ((96,), (11,), 400),
@@ -68,19 +69,23 @@ def test_plane_passes(ffx, dims, lam, batch):
     assert rel_l2(rough, dens) < UNSPLIT_TOL
 
 
-# passes that fill the chip on CTA pairs read their FP32 lines themselves: whole
-# and ragged last tiles, chains and single passes, several row blocks
+# passes that fill the chip read their FP32 lines themselves (all lengths but
+# 192): whole and ragged last tiles, chains and single passes, several row blocks
 FP32_CASES = [
     ((96, 64, 256), (4, 5, 6), 4),     # chain: 24576 lines of 256
     ((64, 1024), (5, 6), 160),         # chain: 10240 lines of 1024, eight row blocks
     ((512,), (7,), 4900),              # single pass: a last tile of 36 lines
     ((384,), (5,), 13001),             # ... and half a pair without lines
     ((32, 32, 256), (3, 4, 5), 10),    # per-axis passes behind it
+    ((64, 64, 64), (5, 3, 7), 6),      # T resident: chains and single passes
+    ((64, 128), (5, 9), 310),
+    ((96,), (5,), 19537),
+    ((128,), (7,), 20001),
 ]
 
 
 @pytest.mark.parametrize("dims,lam,batch", FP32_CASES)
-def test_pair_pass_of_fp32_lines(ffx, dims, lam, batch):
+def test_pass_of_fp32_lines(ffx, dims, lam, batch):
     rng = np.random.default_rng(batch + sum(dims))
     dx, t = (0.25,) * len(dims), 6.0
     psi = random_field(rng, (batch,) + dims)
