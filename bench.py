@@ -694,18 +694,18 @@ def backward_record(args, torch, ffx, plan, w, pool_in, distinct, stream, M):
             "timing": "CUDA events around direct calls on the stream, inputs rotating through the pool"}
 
 
-def hbm_step_record(w, batch, chain, fused_call, out_bytes, step_ms, hbm_peak, pk_src):
+def hbm_step_record(w, batch, split, fused_call, out_bytes, step_ms, hbm_peak, pk_src, square=False):
     """Whole-step HBM view: the algorithmic bytes of a step (read psi0, 8 B
     per point, write the output) and the bytes the implementation's launches
     move (the BF16 chain's input split, 16 B per point; every pass one read
-    and one write of the batch, 8 + 8 B per point, 4 B for densities; the fused
-    launch keeps its intermediates in L2), over the step's time."""
+    and one write of the batch, 8 + 8 B per point, 4 B for densities; `square`:
+    one pass covers two axes; the fused launch keeps its intermediates in L2), over the step's time."""
     pts = batch * int(np.prod(w.dims))
     algo = pts * 8 + out_bytes
     if fused_call:
         impl = algo
     else:
-        impl = (16 * pts if chain else 0) + (len(w.dims) - 1) * 16 * pts + pts * 8 + out_bytes
+        impl = (16 * pts if split else 0) + (len(w.dims) - 1 - square) * 16 * pts + pts * 8 + out_bytes
     sec = step_ms * 1e-3
     return {"algorithmic_bytes": algo, "implementation_bytes": impl, "unit": "GB/s", "peak": hbm_peak,
             "algorithmic_gbs": algo / sec / 1e9, "algorithmic_frac": algo / sec / 1e9 / hbm_peak,
@@ -743,6 +743,7 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
     # (a chain whose first pass runs on CTA pairs has no split launch)
     chain = plan.bf16_chain(B_) and args.column is None
     split = chain and plan.chain_split(B_)
+    square = chain and plan.chain_square(B_)  # one launch covers the last two axes
     if args.column is None:
         out_shape = (B_,) + tuple(w.dims)
 
@@ -871,7 +872,7 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
         mean_ms = [ms / args.steps]
         launch_time = "one launch per step: the timed region's step time (CUDA events at its ends)"
     # the lattice axis of each traced launch (None: the BF16 split of a chain)
-    launch_axis = ([None] if split else []) + list(order)
+    launch_axis = ([None] if split else []) + (list(order[:1]) + list(order[2:]) if square else list(order))
     dom = max((k for k in range(launches) if fused_call or launch_axis[k] is not None), key=lambda k: mean_ms[k])
     pk, pk_src = peaks()
     sm_max = float(pk.get("sm_max_mhz", 2070.0))
@@ -903,16 +904,21 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
         N, lam = w.dims[axis], w.lam[axis]
         axis_form = call_forms[axis]
         flops = pass_flops(N, lam, B_ * M // N, axis_form)
+        if square and dom == 0:  # both its axes
+            flops += pass_flops(w.dims[order[1]], w.lam[order[1]], B_ * M // w.dims[order[1]], axis_form)
         # HBM view of the same launch: it reads and writes the batch once
         # (complex64; the last pass writes float32 densities)
         last = dom == launches - 1
-        kernel_key = f"pass_{axis_form}_N{N}_lam{lam}_{w.key}" + ("_bf16" if bf16_launch else "")
+        kernel_key = (f"square_N{N}_{w.key}" if square and dom == 0 else
+                      f"pass_{axis_form}_N{N}_lam{lam}_{w.key}" + ("_bf16" if bf16_launch else ""))
         if args.column is not None:
             kernel_key += f"_column{args.column}"
         traffic = load_traffic(f"{kernel_key}_b{B_}" + ("_density" if last else ""))
         bytes_launch = B_ * M * (8 + (4 if last else 8))
         pass_names = ["split_bf16_planes" if j is None else f"axis{j}_N{w.dims[j]}_lam{w.lam[j]}_{call_forms[j]}"
                       for j in launch_axis]
+        if square:
+            pass_names[0] = "_".join(f"axis{j}_N{w.dims[j]}_lam{w.lam[j]}" for j in order[:2]) + "_tc"
     achieved = flops / (mean_ms[dom] * 1e-3) / 1e12
     if axis_form == "tc":
         # split contraction on the tensor cores; `achieved` counts the
@@ -1045,7 +1051,7 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
                          "peak": hbm_peak, "unit": "GB/s",
                          "frac": bytes_launch / (mean_ms[dom] * 1e-3) / 1e9 / hbm_peak,
                          "note": f"of {pk_src} hbm_gbs; one read + one write of the batch"},
-        "hbm_step": hbm_step_record(w, B_, split, fused_call, out_bytes, ms / args.steps, hbm_peak, pk_src),
+        "hbm_step": hbm_step_record(w, B_, split, fused_call, out_bytes, ms / args.steps, hbm_peak, pk_src, square),
         "pass_ms": {pass_names[k]: mean_ms[k] for k in range(launches)},
         "e2e": {"value": e2e_value, "unit": UNIT, "api": e2e_api, "lanes": lanes_used,
                 "h2d_bytes_per_step": B_ * M * 8,

@@ -437,7 +437,8 @@ int ffx_plan_axis_form(ffx_plan_t plan, int axis);
 /* Number of kernel launches one ffx_expand / ffx_expand_backward call makes
  * with a batch of one.  A call that runs as a BF16 chain
  * (ffx_plan_bf16_chain) makes one more where ffx_plan_chain_split says so: the
- * split of its input into BF16 planes (in ffx_expand_backward: the forward half of a 3-D plan). */
+ * split of its input into BF16 planes (in ffx_expand_backward: the forward half of a 3-D plan),
+ * and one fewer where ffx_plan_chain_square says so. */
 int ffx_launches_per_call(ffx_plan_t plan, int backward);
 
 /* The largest batch for which ffx_expand and ffx_expand_field run as one
@@ -489,6 +490,10 @@ int ffx_plan_bf16_chain(ffx_plan_t plan, int64_t batch);
  * planes; 0 if its first pass reads the FP32 input itself (a last axis of any
  * length but 192, with enough lines to fill the chip) or the call is no chain. */
 int ffx_plan_chain_split(ffx_plan_t plan, int64_t batch);
+
+/* 1 if such a chain covers its last two axes (64 points each) in one launch,
+ * so that the call makes one launch fewer; it splits its input on the way in. */
+int ffx_plan_chain_square(ffx_plan_t plan, int64_t batch);
 
 /* Forward pass order: writes the lattice axis of pass k to order[k],
  * k = 0..ndim-1.  The adjoint runs the same axes in reverse. */

@@ -342,6 +342,7 @@ struct ChainIo {
   const uint32_t* in_bf;
   uint32_t* out_bf;
   int64_t plane;
+  int points;  // in_bf is chain_square's output (lines not contiguous)
 };
 
 // The lines one launch of a pass covers: `batch` realizations of M points laid
@@ -393,6 +394,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.in_bf = io->in_bf;  // or NULL: the FP32 lines `in`
       d.out_bf = io->out_bf;
       d.bf_plane = io->plane;
+      d.in_points = io->points;
       d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
       d.oouter = outer / d.oinner;
     } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_splits(ax.N, d.ncols, p->sms)) {
@@ -602,7 +604,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
       if (!rc && rem) {
         const int64_t off = whole * groups * p->M;
         ChainIo rest;
-        if (io) rest = {io->in_bf + off, nullptr, io->plane};
+        if (io) rest = {io->in_bf + (io->points ? off / 2 : off), nullptr, io->plane, io->points};
         rc = run_pass(p, j, adjoint, cform, {rem * outer, inner, rem * p->M, 1, lines, 0}, in ? in + off : nullptr, nullptr,
                       0, nullptr, part, acc, stream, io ? &rest : nullptr);
       }
@@ -660,11 +662,23 @@ bool bf16_adjoint_ok(const ffx_plan_s* p) {
   return true;
 }
 
+// Whether a forward chain's first two passes, along the last two axes, are one
+// (plane_square_kernel): 64 points each, the first axis one whose pass keeps T
+// resident, or none (2-D lattices; their ensemble sums stay with the passes).
+// 44 bytes a point of HBM become 28 on 3-D lattices (density, 64 realizations
+// of 64^3: @@), 28 become 12 on 2-D ones (@@).
+bool chain_square(const ffx_plan_s* p) {
+  const int d = p->ndim;
+  if (d < 2 || p->axis[d - 1].N != 64 || p->axis[d - 2].N != 64 || p->order[0] != d - 1 || p->order[1] != d - 2)
+    return false;
+  return d == 2 ? !p->acc : p->axis[0].N == 64 || p->axis[0].N == 96 || p->axis[0].N == 128;
+}
+
 // Whether a forward chain starts with a split of its input (else its first pass
 // reads the FP32 input itself).
 bool chain_splits(const ffx_plan_s* p, int64_t batch) {
   const Axis& ax = p->axis[p->order[0]];
-  return !plane_pass_splits(ax.N, batch * (p->M / ax.N), p->sms);
+  return !chain_square(p) && !plane_pass_splits(ax.N, batch * (p->M / ax.N), p->sms);
 }
 
 // The forward map of a batch as a BF16 chain: the input split into BF16
@@ -672,16 +686,38 @@ bool chain_splits(const ffx_plan_s* p, int64_t batch) {
 // a complex64 field), then the passes in the plan's order (the last axis
 // first), each reading planes and writing planes (ws[0], ws[1], ...), the
 // last one the caller's field (out_c) or densities (out_d, summed over the
-// batch with FFX_ACCUMULATE).  `in` is read by the split (or the first pass,
+// batch with FFX_ACCUMULATE).  With chain_square the first two passes are one
+// that writes ws[1].  `in` is read by the split (or the first pass,
 // which writes ws[0]) alone, so out_c may equal it; it must not be ws[1] or, if
 // the first pass reads it, ws[0].
 int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, float* out_d, cudaStream_t s) {
   const int d = p->ndim;
+  const bool square = chain_square(p);
   int rc;
-  if ((rc = ensure_ws(p, 0, batch)) || (rc = ensure_ws(p, 1, batch))) return rc;
+  if ((!square && (rc = ensure_ws(p, 0, batch))) || ((!square || d > 2) && (rc = ensure_ws(p, 1, batch)))) return rc;
   const int64_t plane = batch * p->M;
   const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
   const uint32_t* cur_bf = nullptr;
+  if (square) {
+    DenseArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.in = in;
+    a.out_bf = d > 2 ? (uint32_t*)p->ws[1] : nullptr;
+    a.bf_plane = plane;
+    a.out_c = d > 2 ? nullptr : out_c;
+    a.out_d = d > 2 ? nullptr : out_d;
+    a.ncols = plane / 64;
+    a.N = 64;
+    a.unsplit = unsplit;
+    const unsigned rec = trace_begin(p, s);
+    cudaError_t e = launch_plane_square(a, p->axis[d - 1].pl_t[0], p->axis[d - 2].pl_t[0], p->dev_err, p->sms, s);
+    if (e != cudaSuccess) return cuda_fail(e, "pass launch");
+    ++p->launches;
+    trace_end(p, s, rec);
+    if (d == 2) return FFX_OK;
+    ChainIo io = {(const uint32_t*)p->ws[1], nullptr, plane, 1};
+    return run_axis(p, p->order[2], false, nullptr, nullptr, 0, out_c, out_d, out_d ? p->acc : 0, batch, s, &io);
+  }
   if (chain_splits(p, batch)) {
     const unsigned rec = trace_begin(p, s);
     cudaError_t e = launch_plane_split(in, nullptr, 0, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit, p->sms, s);
@@ -696,6 +732,7 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
     io.in_bf = cur_bf;
     io.out_bf = last ? nullptr : (uint32_t*)p->ws[r & 1];
     io.plane = plane;
+    io.points = 0;
     rc = run_axis(p, p->order[r], false, cur_bf ? nullptr : in, nullptr, 0, last ? out_c : nullptr,
                   last ? out_d : nullptr, last && out_d ? p->acc : 0, batch, s, &io);
     if (rc) return rc;
@@ -729,6 +766,7 @@ int chain_bf16_adjoint(ffx_plan_s* p, const float2* field, const float* grad, in
     io.in_bf = cur_bf;
     io.out_bf = last ? nullptr : (uint32_t*)p->ws[r & 1];
     io.plane = plane;
+    io.points = 0;
     rc = run_axis(p, p->order[r], true, nullptr, nullptr, 0, last ? out : nullptr, nullptr, 0, batch, s, &io);
     if (rc) return rc;
     cur_bf = io.out_bf;
@@ -1425,6 +1463,7 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           e = launch_plane_build_t(ax.T, ax.pl_t[0], ax.N, s);
           if (e == cudaSuccess) e = launch_plane_build_t(ax.TH, ax.pl_t[1], ax.N, s);
           if (e == cudaSuccess) e = plane_pass_prepare(ax.N);
+          if (e == cudaSuccess && ax.N == 64) e = plane_square_prepare();
         }
         if (e == cudaSuccess)
           e = dense_tc_prepare();
@@ -1641,6 +1680,11 @@ int ffx_plan_bf16_chain(ffx_plan_t p, int64_t batch) {
   if (p->many || batch <= p->fused) return 0;
   const void* aligned = (const void*)(uintptr_t)16;
   return bf16_chain_ok(p, batch, aligned, aligned, aligned) ? 1 : 0;
+}
+
+int ffx_plan_chain_square(ffx_plan_t p, int64_t batch) {
+  if (ffx_plan_bf16_chain(p, batch) != 1) return 0;
+  return chain_square(p) ? 1 : 0;
 }
 
 int ffx_plan_chain_split(ffx_plan_t p, int64_t batch) {

@@ -119,6 +119,7 @@ struct DenseArgs {
   uint32_t* out_bf;
   int64_t bf_plane;
   int64_t oouter, oinner;
+  int in_points;  // in_bf is a square pass's output (plane_square_kernel)
 };
 const void* dense_kernel_func();
 cudaError_t launch_dense(const DenseArgs& a, int grid, cudaStream_t stream);
@@ -168,6 +169,11 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
 bool plane_pass_splits(int N, int64_t ncols, int sms);
 // work items of a pass over ncols lines, and how many run at once
 int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once);
+// the last two axes of 64 points in one pass: a.ncols contiguous FP32 lines (64
+// for each 64 x 64 square), T1 the last axis's T, T2 the other's
+cudaError_t plane_square_prepare();
+cudaError_t launch_plane_square(const DenseArgs& a, const unsigned char* T1, const unsigned char* T2, int* err, int sms,
+                                cudaStream_t s);
 cudaError_t launch_plane_pass(const DenseArgs& a, const unsigned char* Tblk, int* err, int sms, cudaStream_t s);
 cudaError_t launch_identity(float2* I, int N, cudaStream_t s);
 

@@ -50,6 +50,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "ffx_internal.h"
 #include "ffx_pdl.h"
@@ -127,16 +128,39 @@ __device__ __forceinline__ void store_pair(void* o, int64_t other, bool odd, boo
 enum POut { kOutPlanes = 0, kOutComplex = 1, kOutDensity = 2, kOutSum = 3 };
 constexpr int kPOuts = 4;
 
+// Where the first operand of a chunk lies: descriptor words (low) of its real
+// and imaginary parts, head and tail, at K step ks.
+//  * rows along K (a line a row): head plane, then tail plane, K step ks has the
+//    real parts at 64 ks and the imaginary parts at 64 ks + 32 bytes of the rows;
+//  * rows along the lines (a point a row, 64 lines of 128 bytes; tiles of real
+//    heads, imaginary heads, real tails, imaginary tails `part` bytes apart,
+//    the next 64 lines `atom` bytes on): K step ks starts at row 16 ks.
+struct XLines {
+  uint32_t x0;
+  __device__ __forceinline__ explicit XLines(uint32_t saddr) : x0(desc_lo(saddr)) {}
+  __device__ __forceinline__ uint32_t at(uint32_t ks, bool imag, bool tail) const {
+    return x0 + ks * 4 + (imag ? 2 : 0) + (tail ? PXPART / 16 : 0);
+  }
+};
+struct XPoints {
+  uint32_t x0, part;
+  __device__ __forceinline__ XPoints(uint32_t saddr, uint32_t part_bytes, uint32_t atom)
+      : x0((saddr >> 4) | ((atom >> 4) << 16)), part(part_bytes >> 4) {}
+  __device__ __forceinline__ uint32_t at(uint32_t ks, bool imag, bool tail) const {
+    return x0 + ks * 128 + ((imag ? 1 : 0) + (tail ? 2 : 0)) * part;
+  }
+};
+// the instruction descriptor's "first operand's rows run along its rows" bit
+constexpr uint32_t kMajorA = 1u << 15;
+
 // The products of one accumulator half [D1 | D2] (real or imaginary parts, at
-// tensor-memory column d) with one chunk: X's tile at xs (head plane, then
-// tail plane: K step ks has X's real parts at 64 ks and its imaginary parts at
-// 64 ks + 32 bytes of the rows), T's rows at t2 (heads and tails, both columns
-// sets) and t1 (heads alone), real parts at 32 ks and imaginary parts at 64 +
-// 32 ks.  The real half takes T's real parts with X's real ones and T's
-// imaginary parts with X's negated imaginary ones, the imaginary half the other
-// two.  CG: CTAs per product.  Called by the whole warp.
-template <int CG, int RB, bool IMAG>
-__device__ __forceinline__ void plane_half(uint32_t d, uint32_t xs, uint32_t t2, uint32_t t1, uint32_t id1,
+// tensor-memory column d) with one chunk: X's operands (above), T's rows at t2
+// (heads and tails, both column sets) and t1 (heads alone), real parts at 32 ks
+// and imaginary parts at 64 + 32 ks.  The real half takes T's real parts with
+// X's real ones and T's imaginary parts with X's negated imaginary ones, the
+// imaginary half the other two.  CG: CTAs per product.  Called by the whole warp.
+template <int CG, int RB, bool IMAG, class X>
+__device__ __forceinline__ void plane_half(uint32_t d, const X& x, uint32_t t2, uint32_t t1, uint32_t id1,
                                            uint32_t id2, bool first, bool unsplit) {
   auto mma = [](uint32_t dd, uint32_t al, uint32_t bl, uint32_t id, uint32_t acc) {
     if constexpr (CG == 2)
@@ -145,21 +169,21 @@ __device__ __forceinline__ void plane_half(uint32_t d, uint32_t xs, uint32_t t2,
       mma_sw128(dd, al, bl, id, acc);
   };
   constexpr uint32_t o0 = IMAG ? 64 : 0, o1 = IMAG ? 0 : 64, neg = IMAG ? 0u : kNegA;
-  const uint32_t x0 = desc_lo(xs), b2 = desc_lo(t2), b1 = desc_lo(t1);
+  const uint32_t b2 = desc_lo(t2), b1 = desc_lo(t1);
   if (unsplit) {
 #pragma unroll
     for (uint32_t ks = 0; ks < 2; ++ks) {
-      mma(d, x0 + ks * 4, b1 + ks * 2 + o0 / 16, id1, (first && ks == 0) ? 0u : 1u);
-      mma(d, x0 + ks * 4 + 2, b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
+      mma(d, x.at(ks, false, false), b1 + ks * 2 + o0 / 16, id1, (first && ks == 0) ? 0u : 1u);
+      mma(d, x.at(ks, true, false), b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
     }
     return;
   }
 #pragma unroll
   for (uint32_t ks = 0; ks < 2; ++ks) {
-    mma(d, x0 + ks * 4, b2 + ks * 2 + o0 / 16, id2, (first && ks == 0) ? 0u : 1u);
-    mma(d, x0 + ks * 4 + 2, b2 + ks * 2 + o1 / 16, id2 | neg, 1u);
-    mma(d + RB, x0 + PXPART / 16 + ks * 4, b1 + ks * 2 + o0 / 16, id1, 1u);
-    mma(d + RB, x0 + PXPART / 16 + ks * 4 + 2, b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
+    mma(d, x.at(ks, false, false), b2 + ks * 2 + o0 / 16, id2, (first && ks == 0) ? 0u : 1u);
+    mma(d, x.at(ks, true, false), b2 + ks * 2 + o1 / 16, id2 | neg, 1u);
+    mma(d + RB, x.at(ks, false, true), b1 + ks * 2 + o0 / 16, id1, 1u);
+    mma(d + RB, x.at(ks, true, true), b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
   }
 }
 
@@ -441,9 +465,15 @@ __device__ __forceinline__ void split_tiles(unsigned char* stages, int n, int la
   }
 }
 
-// RB outputs per item, T resident (RES) or streamed; F32 (with RES): FP32 input.
-template <int RB, bool RES, int OUT, bool F32>
-__global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
+// What a pass reads: planes of contiguous lines; contiguous FP32 lines; or the
+// square kernel's four planes (below), in which a line's points are a.oinner
+// points apart (tiles of 64 lines x 32 points of each).
+enum PIn { kInPlanes = 0, kInF32 = 1, kInPoints = 2 };
+
+// RB outputs per item, T resident (RES) or streamed; other input than planes
+// comes with RES.
+template <int RB, bool RES, int OUT, int IN>
+__global__ void __launch_bounds__(IN == kInF32 ? PTHREADS_F32 : PTHREADS, 1)
     plane_pass_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
                       const __grid_constant__ CUtensorMap xmap) {
   constexpr int NST = pstages(RB, RES);
@@ -454,7 +484,8 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
   constexpr bool ACC = OUT == kOutSum;
   extern __shared__ __align__(1024) unsigned char psm_raw[];
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
-  static_assert(RES || !F32, "FP32 input comes with resident T");
+  constexpr bool F32 = IN == kInF32, POINTS = IN == kInPoints;
+  static_assert(RES || IN == kInPlanes, "FP32 and point-row input come with resident T");
   __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], raw_bar[PMAXST], t_bar;
   __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
   __shared__ uint32_t tmem_slot;
@@ -532,6 +563,17 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
                   "[%4];" ::"r"(st + (uint32_t)(h * PXPART)),
                   "l"(map_addr), "r"(ikc * 2 * PKC + 32 * h), "r"(row), "r"(fb)
                   : "memory");
+          } else if (POINTS) {
+            // the tile's two groups of 64 lines (realization rb's, from line m0)
+            const int64_t rb = row / a.oinner;
+            const int m0 = (int)(row - rb * a.oinner);
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+              asm volatile(
+                  "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                  "%5}], [%6];" ::"r"(st + (uint32_t)(h * PXPART)),
+                  "l"(map_addr), "r"(m0 + 64 * h), "r"(ikc * PKC), "r"((int)rb), "r"(0), "r"(fb)
+                  : "memory");
           } else {
             asm volatile(
                 "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
@@ -575,7 +617,8 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
       int64_t u = 0;
       int s = 0;
       bool ok = !RES || mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
-      const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
+      constexpr uint32_t major = POINTS ? kMajorA : 0u;
+      const uint32_t id1 = idesc_bf16(PL, RB) | major, id2 = idesc_bf16(PL, 2 * RB) | major;
 #pragma unroll 1
       for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
         const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
@@ -591,7 +634,13 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
           tc_fence_after();
           const uint32_t st = stages + (uint32_t)(s * STAGE);
           const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
-          plane_half<1, RB, false>(dre, st, tb, tb, id1, id2, kc == 0, unsplit);
+          auto half = [&](auto imag, uint32_t dd) {
+            if constexpr (POINTS)
+              plane_half<1, RB, decltype(imag)::value>(dd, XPoints(st, PXPART / 4, PXPART), tb, tb, id1, id2, kc == 0, unsplit);
+            else
+              plane_half<1, RB, decltype(imag)::value>(dd, XLines(st), tb, tb, id1, id2, kc == 0, unsplit);
+          };
+          half(std::false_type(), dre);
           if (last) {
             if (elect_one()) mma_commit(smem_u32(&accf_bar[2 * buf]));
             __syncwarp();
@@ -601,7 +650,7 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
             if (!ok) break;
             tc_fence_after();
           }
-          plane_half<1, RB, true>(dim, st, tb, tb, id1, id2, kc == 0, unsplit);
+          half(std::true_type(), dim);
           if (elect_one()) {
             mma_commit(smem_u32(&empty_bar[s]));
             if (last) mma_commit(smem_u32(&accf_bar[2 * buf + 1]));
@@ -630,6 +679,333 @@ __global__ void __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
       split_tiles<NST, STAGE>(psm + (RB / PKC) * TCH, tid - 384, lane, my_items * nb * kchunks, unsplit, raw_bar, &s_abort,
                               [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
     }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (tid == 0 && s_abort && err) atomicAdd(err, 1);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_free(tmem, 512);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The last two axes of a lattice, 64 points each, in one pass ("squares" of 64
+// x 64 points: 64^3 ensembles, stacks of 64 x 64 images).  As two passes of a
+// chain they read and write 32 bytes a point of HBM; here the intermediate
+// stays on the SM (16 bytes a point, 12 for a 2-D density).  An item is two
+// squares, 128 lines along the last axis:
+//  * step 1, the last axis: FP32 lines split in place in the stages (as the
+//    FP32-input passes above) against T resident, into tensor memory columns
+//    0-255 (lane: line (g, b) of square g; column: point j');
+//  * the epilogue warps read it (E1), split it again and write it to shared
+//    memory as the second step's operand, 64 KB: point rows b of 128 bytes, the
+//    64 columns j' of a square side by side (rows along M, so nothing is
+//    transposed: a lane's 32 columns are 64 consecutive bytes);
+//  * step 2, the other axis: that operand against the other T, also resident,
+//    into columns 256-511 (lane: (g, j'), column: point b');
+//  * E2 stores the natural order [g][b'][j'], lanes along j': the densities or
+//    the field of a 2-D lattice, or the four planes (real and imaginary heads,
+//    real and imaginary tails, 2 bytes a point each) that the first axis's pass
+//    reads with its lines' points oinner apart (kInPoints).
+// Order of the products: step 1 of item i + 1, then step 2 of item i; of the
+// epilogue: E1 of item i, then E2 of item i - 1: the products of one step hide
+// the other step's epilogue.  Shared memory bounds it: 448 KB of operands and
+// 128 KB of copies, splits and operand stores an item, 5600 clocks against 3072 of
+// products at full rate; HBM 16 bytes a point.
+constexpr int SST = 3;  // stages
+constexpr int SA2 = 4 * 2 * 64 * 128;  // the second operand: 4 parts x 2 squares x 64 rows
+constexpr int ssmem() { return 4 * ptchunk(64) + SA2 + SST * PX + 1024; }
+static_assert(ssmem() <= 232448 - 512, "shared memory of a block");
+
+template <int OUT>
+__global__ void __launch_bounds__(PTHREADS_F32, 1)
+    plane_square_kernel(const DenseArgs a, const unsigned char* __restrict__ T1, const unsigned char* __restrict__ T2,
+                        int* err, const __grid_constant__ CUtensorMap xmap) {
+  constexpr int RB = 64, H = RB / 2, TCH = ptchunk(RB), TPART = ppart(RB);
+  constexpr int PART = 2 * 64 * 128;  // a part of the second operand
+  static_assert(OUT != kOutSum, "densities are summed by the passes");
+  extern __shared__ __align__(1024) unsigned char psm_raw[];
+  unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
+  __shared__ __align__(8) uint64_t full_bar[SST], empty_bar[SST], raw_bar[SST], t_bar;
+  // D1 and D2: halves complete (f), halves read (e); the second operand written
+  __shared__ __align__(8) uint64_t d1f_bar[2], d1e_bar[2], d2f_bar[2], d2e_bar[2], a2f_bar, done_bar;
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int s_abort;
+
+  const int tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int64_t items = (a.ncols + PL - 1) / PL;
+  const int64_t my_items = (items - blockIdx.x + gridDim.x - 1) / gridDim.x;
+  if (my_items <= 0) return;
+  const bool unsplit = a.unsplit != 0;
+
+  if (warp == 1) tmem_alloc(&tmem_slot, 512);
+  if (tid == 0) {
+    for (int s = 0; s < SST; ++s) {
+      mbar_init(smem_u32(&full_bar[s]), 4);  // the producer warps
+      mbar_init(smem_u32(&empty_bar[s]), 1);
+      mbar_init(smem_u32(&raw_bar[s]), 1);
+    }
+    mbar_init(smem_u32(&t_bar), 1);
+    for (int h = 0; h < 2; ++h) {
+      mbar_init(smem_u32(&d1f_bar[h]), 1);
+      mbar_init(smem_u32(&d2f_bar[h]), 1);
+      mbar_init(smem_u32(&d1e_bar[h]), PEPIW);
+      mbar_init(smem_u32(&d2e_bar[h]), PEPIW);
+    }
+    mbar_init(smem_u32(&a2f_bar), PEPIW);
+    mbar_init(smem_u32(&done_bar), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    s_abort = 0;
+  }
+  pdl_trigger();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = tmem_slot;
+  const uint32_t t1 = smem_u32(psm), t2 = t1 + 2u * TCH, a2 = t2 + 2u * TCH, stages = a2 + (uint32_t)SA2;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (warp == 0) {
+      // ---------------- copies ----------------
+      if (lane == 0) {
+        const uint64_t map_addr = reinterpret_cast<uint64_t>(&xmap);
+        const uint32_t tbytes = unsplit ? (uint32_t)TPART : (uint32_t)TCH;  // unsplit: the head rows
+        mbar_expect_tx(smem_u32(&t_bar), 4 * tbytes);
+        for (int kc = 0; kc < 2; ++kc) {
+          bulk_g2s(t1 + (uint32_t)(kc * TCH), T1 + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
+          bulk_g2s(t2 + (uint32_t)(kc * TCH), T2 + (size_t)kc * TCH, tbytes, smem_u32(&t_bar));
+        }
+        pdl_wait();  // both T are the plan's own; the lines may be the predecessor's output
+        const int64_t total = my_items * 2;
+        int64_t u = 0;
+        int is = 0;
+#pragma unroll 1
+        for (int64_t ci = 0; ci < total; ++ci) {
+          if (u >= 1 && !mbar_wait(smem_u32(&empty_bar[is]), (uint32_t)((u - 1) & 1), &s_abort)) break;
+          const uint32_t st = stages + (uint32_t)(is * PX);
+          const uint32_t fb = smem_u32(&raw_bar[is]);
+          mbar_expect_tx(fb, (uint32_t)PX);
+          const int row = (int)((blockIdx.x + (ci >> 1) * gridDim.x) * PL);
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            asm volatile(
+                "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], "
+                "[%4];" ::"r"(st + (uint32_t)(h * PXPART)),
+                "l"(map_addr), "r"((int)(ci & 1) * 2 * PKC + 32 * h), "r"(row), "r"(fb)
+                : "memory");
+          if (++is == SST) {
+            is = 0;
+            ++u;
+          }
+        }
+        // nothing of this thread's may still be in flight at exit
+        mbar_wait_own(smem_u32(&t_bar), 0u, &s_abort);
+        for (int q = 0; q < SST; ++q) {
+          const int64_t uq = q < is ? u : u - 1;  // stage q's last use
+          if (uq >= 0) mbar_wait_own(smem_u32(&raw_bar[q]), (uint32_t)(uq & 1), &s_abort);
+        }
+      }
+      __syncwarp();
+    } else if (warp == 1) {
+      // ---------------- products: the whole warp, one elected lane issuing ----------------
+      bool ok = mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
+      const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
+      const uint32_t dre1 = tmem, dim1 = dre1 + 2 * RB, dre2 = tmem + 4 * RB, dim2 = dre2 + 2 * RB;
+      int s = 0;
+      int64_t u = 0;
+      auto commit = [&](uint64_t* bar) {
+        if (elect_one()) mma_commit(smem_u32(bar));
+        __syncwarp();
+      };
+#pragma unroll 1
+      for (int64_t i = 0; ok && i <= my_items; ++i) {
+        const uint32_t prev = (uint32_t)((i - 1) & 1);
+        if (i < my_items) {  // step 1 of item i
+#pragma unroll 1
+          for (int kc = 0; kc < 2; ++kc) {
+            ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+                 (kc > 0 || i == 0 || mbar_wait(smem_u32(&d1e_bar[0]), prev, &s_abort));
+            if (!ok) break;
+            tc_fence_after();
+            const XLines x(stages + (uint32_t)(s * PX));
+            const uint32_t tb = t1 + (uint32_t)(kc * TCH);
+            plane_half<1, RB, false>(dre1, x, tb, tb, id1, id2, kc == 0, unsplit);
+            if (kc == 1) commit(&d1f_bar[0]);
+            if (kc == 0 && i > 0) {
+              ok = mbar_wait(smem_u32(&d1e_bar[1]), prev, &s_abort);
+              if (!ok) break;
+              tc_fence_after();
+            }
+            plane_half<1, RB, true>(dim1, x, tb, tb, id1, id2, kc == 0, unsplit);
+            commit(&empty_bar[s]);
+            if (kc == 1) commit(&d1f_bar[1]);
+            if (++s == SST) {
+              s = 0;
+              ++u;
+            }
+          }
+          if (!ok) break;
+        }
+        if (i > 0) {  // step 2 of item i - 1
+          ok = mbar_wait(smem_u32(&a2f_bar), prev, &s_abort) &&
+               (i == 1 || mbar_wait(smem_u32(&d2e_bar[0]), (uint32_t)(i & 1), &s_abort));
+          if (!ok) break;
+          tc_fence_after();
+#pragma unroll
+          for (int kc = 0; kc < 2; ++kc)
+            plane_half<1, RB, false>(dre2, XPoints(a2 + (uint32_t)(kc * PKC * 128), PART, 64 * 128),
+                                     t2 + (uint32_t)(kc * TCH), t2 + (uint32_t)(kc * TCH), id1 | kMajorA, id2 | kMajorA,
+                                     kc == 0, unsplit);
+          commit(&d2f_bar[0]);
+          if (i > 1) {
+            ok = mbar_wait(smem_u32(&d2e_bar[1]), (uint32_t)(i & 1), &s_abort);
+            if (!ok) break;
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int kc = 0; kc < 2; ++kc)
+            plane_half<1, RB, true>(dim2, XPoints(a2 + (uint32_t)(kc * PKC * 128), PART, 64 * 128),
+                                    t2 + (uint32_t)(kc * TCH), t2 + (uint32_t)(kc * TCH), id1 | kMajorA, id2 | kMajorA,
+                                    kc == 0, unsplit);
+          commit(&d2f_bar[1]);  // the second operand is free as well
+        }
+      }
+      // whatever happened, the tensor cores finish this warp's work before exit
+      commit(&done_bar);
+      mbar_wait_own(smem_u32(&done_bar), 0u, &s_abort);
+    }
+  } else if (warp < 12) {
+    // ---------------- epilogue ----------------
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 176;");
+    pdl_wait();  // before any store: the predecessor may still read the output's memory
+    const int q = warp & 3;                 // tensor-memory lane quarter this warp may read
+    const int col0 = ((warp - 4) >> 2) * H;  // first of this warp's columns
+    const int r = q * 32 + lane;
+    const int g = r >> 6, b = r & 63;       // square; E1: row b, E2: column j' = b
+    const bool odd = lane & 1;
+    const uint32_t sel_send = odd ? 0x5410u : 0x7632u;
+    const uint32_t sel_h = odd ? 0x3254u : 0x5410u, sel_l = odd ? 0x3276u : 0x7610u;
+    const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)col0;
+    // this warp's 32 columns of an accumulator half, summed over its two column sets; then released
+    auto read_half = [&](uint32_t d, uint64_t* f, uint64_t* e, uint32_t parity, float* y) -> bool {
+      bool got = true;
+      if (lane == 0) got = mbar_wait(smem_u32(f), parity, &s_abort);
+      if (__shfl_sync(0xffffffffu, got ? 1 : 0, 0) == 0) return false;
+      tc_fence_after();
+#pragma unroll
+      for (int j = 0; j < H; j += 16) {
+        uint32_t x[16], z[16];
+        tmem_ld16(d + (uint32_t)j, x);
+        tmem_ld16(d + (uint32_t)(RB + j), z);  // unsplit: not written, not used
+        tmem_wait_ld();
+#pragma unroll
+        for (int m = 0; m < 16; ++m)
+          y[j + m] = unsplit ? __uint_as_float(x[m]) : __uint_as_float(x[m]) + __uint_as_float(z[m]);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(e));
+      return true;
+    };
+    // heads of 32 values in place of the first 16 of them, tails of the last 16
+    auto split32 = [](const float* y, uint32_t* h, uint32_t* l) {
+#pragma unroll
+      for (int m = 0; m < 16; ++m) {
+        h[m] = bf2(y[2 * m], y[2 * m + 1]);
+        l[m] = bf2(y[2 * m] - bf_lo(h[m]), y[2 * m + 1] - bf_hi(h[m]));
+      }
+    };
+    unsigned char* const arow = psm + 4 * TCH + g * (64 * 128) + b * 128;
+    bool ok = true;
+#pragma unroll 1
+    for (int64_t i = 0; ok && i <= my_items; ++i) {
+      if (i < my_items) {
+        // ---- E1 of item i ----
+        float y[H];
+        uint32_t hr[16], lr[16], hm[16], lm[16];
+        ok = read_half(tbase, &d1f_bar[0], &d1e_bar[0], (uint32_t)(i & 1), y);
+        if (!ok) break;
+        split32(y, hr, lr);
+        ok = read_half(tbase + 2 * RB, &d1f_bar[1], &d1e_bar[1], (uint32_t)(i & 1), y);
+        if (!ok) break;
+        split32(y, hm, lm);
+        if (i > 0) {  // step 2 of item i - 1 has read the operand
+          bool got = true;
+          if (lane == 0) got = mbar_wait(smem_u32(&d2f_bar[1]), (uint32_t)((i - 1) & 1), &s_abort);
+          ok = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
+          if (!ok) break;
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          unsigned char* o = arow + (((col0 / 8 + c) ^ (b & 7)) << 4);
+          *reinterpret_cast<uint4*>(o) = make_uint4(hr[4 * c], hr[4 * c + 1], hr[4 * c + 2], hr[4 * c + 3]);
+          *reinterpret_cast<uint4*>(o + PART) = make_uint4(hm[4 * c], hm[4 * c + 1], hm[4 * c + 2], hm[4 * c + 3]);
+          if (!unsplit) {
+            *reinterpret_cast<uint4*>(o + 2 * PART) = make_uint4(lr[4 * c], lr[4 * c + 1], lr[4 * c + 2], lr[4 * c + 3]);
+            *reinterpret_cast<uint4*>(o + 3 * PART) = make_uint4(lm[4 * c], lm[4 * c + 1], lm[4 * c + 2], lm[4 * c + 3]);
+          }
+        }
+        fence_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&a2f_bar));
+      }
+      if (i > 0) {
+        // ---- E2 of item i - 1 ----
+        const uint32_t par = (uint32_t)((i - 1) & 1);
+        float y[H], z[H];
+        ok = read_half(tbase + 4 * RB, &d2f_bar[0], &d2e_bar[0], par, y);
+        if (!ok) break;
+        ok = read_half(tbase + 6 * RB, &d2f_bar[1], &d2e_bar[1], par, z);
+        if (!ok) break;
+        const int64_t sq = 2 * (blockIdx.x + (i - 1) * (int64_t)gridDim.x) + g;
+        const bool valid = sq * 64 < a.ncols;  // whole warps
+        const int64_t base = sq * 4096 + col0 * 64 + b;
+        if constexpr (OUT == kOutPlanes) {
+          // a lane pair's two points are one word of each part: the even lane
+          // stores the real parts' words, the odd lane the imaginary parts'
+          const int64_t pw = a.bf_plane / 2;  // words a part
+          uint32_t* o = a.out_bf + (base >> 1) + (odd ? pw : 0);
+          if (valid) {
+#pragma unroll
+            for (int m0 = 0; m0 < H; m0 += 8) {
+              uint32_t h[8], l[8], x[8];
+#pragma unroll
+              for (int m = 0; m < 8; ++m) {
+                h[m] = bf2(y[m0 + m], z[m0 + m]);
+                l[m] = bf2(y[m0 + m] - bf_lo(h[m]), z[m0 + m] - bf_hi(h[m]));
+                x[m] = __byte_perm(h[m], l[m], sel_send);
+              }
+#pragma unroll
+              for (int m = 0; m < 8; ++m) x[m] = __shfl_xor_sync(0xffffffffu, x[m], 1);
+#pragma unroll
+              for (int m = 0; m < 8; ++m) {
+                o[(m0 + m) * 32] = __byte_perm(h[m], x[m], sel_h);
+                if (!unsplit) o[2 * pw + (m0 + m) * 32] = __byte_perm(l[m], x[m], sel_l);
+              }
+            }
+          }
+        } else if (valid) {
+          if constexpr (OUT == kOutComplex) {
+            float2* o = a.out_c + base;
+#pragma unroll
+            for (int m = 0; m < H; ++m) o[m * 64] = make_float2(y[m], z[m]);
+          } else {
+            float* o = a.out_d + base;
+#pragma unroll
+            for (int m = 0; m < H; ++m) o[m * 64] = y[m] * y[m] + z[m] * z[m];
+          }
+        }
+      }
+    }
+  } else {
+    // ---------------- FP32 input: split into the stages ----------------
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
+    split_tiles<SST, PX>(psm + 4 * TCH + SA2, tid - 384, lane, my_items * 2, unsplit, raw_bar, &s_abort,
+                         [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
   }
 
   tc_fence_before();
@@ -818,11 +1194,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
                (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
           if (!ok) break;
           tc_fence_after();
-          plane_half<2, RB, false>(dre, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          plane_half<2, RB, false>(dre, XLines(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
           ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
           if (!ok) break;
           tc_fence_after();
-          plane_half<2, RB, false>(dre, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          plane_half<2, RB, false>(dre, XLines(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
           if (last) {
             if (elect_one()) mma2_commit_both(smem_u32(&accf_bar[0]));
             __syncwarp();
@@ -832,10 +1208,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
             if (!ok) break;
             tc_fence_after();
           }
-          plane_half<2, RB, true>(dim, st0, st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          plane_half<2, RB, true>(dim, XLines(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
           if (elect_one()) mma2_commit_both(smem_u32(&empty_bar[s0]));
           __syncwarp();
-          plane_half<2, RB, true>(dim, st1, st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          plane_half<2, RB, true>(dim, XLines(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
           if (elect_one()) {
             mma2_commit_both(smem_u32(&empty_bar[s1]));
             if (last) mma2_commit_both(smem_u32(&accf_bar[1]));
@@ -960,20 +1336,25 @@ struct QVariant {
   static constexpr QKernel fn[kPOuts] = {plane_pair_kernel<kOutPlanes, F32>, plane_pair_kernel<kOutComplex, F32>,
                                          plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>};
 };
-template <int RB, bool RES, bool F32>
+template <int RB, bool RES, int IN>
 struct PVariant {
   static constexpr PKernel fn[kPOuts] = {
-      plane_pass_kernel<RB, RES, kOutPlanes, F32>, plane_pass_kernel<RB, RES, kOutComplex, F32>,
-      plane_pass_kernel<RB, RES, kOutDensity, F32>, plane_pass_kernel<RB, RES, kOutSum, F32>};
+      plane_pass_kernel<RB, RES, kOutPlanes, IN>, plane_pass_kernel<RB, RES, kOutComplex, IN>,
+      plane_pass_kernel<RB, RES, kOutDensity, IN>, plane_pass_kernel<RB, RES, kOutSum, IN>};
 };
-PKernel single_kernel(int N, int out, bool f32) {
+template <int IN>
+PKernel resident_kernel(int N, int out) {
   switch (N) {
-    case 64: return f32 ? PVariant<64, true, true>::fn[out] : PVariant<64, true, false>::fn[out];
-    case 96: return f32 ? PVariant<96, true, true>::fn[out] : PVariant<96, true, false>::fn[out];
-    case 128: return f32 ? PVariant<128, true, true>::fn[out] : PVariant<128, true, false>::fn[out];
-    case 192: return PVariant<96, false, false>::fn[out];
-    default: return PVariant<64, false, false>::fn[out];
+    case 64: return PVariant<64, true, IN>::fn[out];
+    case 96: return PVariant<96, true, IN>::fn[out];
+    default: return PVariant<128, true, IN>::fn[out];
   }
+}
+PKernel single_kernel(int N, int out, int in) {
+  if (N <= 128)
+    return in == kInF32 ? resident_kernel<kInF32>(N, out)
+                        : in == kInPoints ? resident_kernel<kInPoints>(N, out) : resident_kernel<kInPlanes>(N, out);
+  return N == 192 ? PVariant<96, false, kInPlanes>::fn[out] : PVariant<64, false, kInPlanes>::fn[out];
 }
 int single_rows(int N) { return N <= 128 ? N : N == 192 ? 96 : 64; }  // outputs per item
 int single_smem(int N) { return psmem(single_rows(N), N <= 128); }
@@ -997,6 +1378,23 @@ bool row_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int
                        swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE);
 }
 
+// the square kernel's four (unsplit: two) parts as [part][realization][point][line]
+bool points_map(CUtensorMap* map, const void* base, int64_t lines, int N, int64_t batch, int64_t plane, int parts) {
+  const cuuint64_t dims[4] = {(cuuint64_t)lines, (cuuint64_t)N, (cuuint64_t)batch, (cuuint64_t)parts};
+  const cuuint64_t strides[3] = {(cuuint64_t)lines * 2, (cuuint64_t)lines * N * 2, (cuuint64_t)plane * 2};
+  const cuuint32_t box[4] = {64, PKC, 1, (cuuint32_t)parts};
+  return make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+template <int OUT>
+cudaError_t launch_square(const DenseArgs& a, const unsigned char* T1, const unsigned char* T2, int* err, int sms,
+                          cudaStream_t s) {
+  CUtensorMap xmap;
+  if (!f32_map(&xmap, a.in, 2 * 64, a.ncols, PL)) return cudaErrorInvalidValue;
+  const int64_t grid = std::min<int64_t>((a.ncols + PL - 1) / PL, sms);
+  return launch_pdl(plane_square_kernel<OUT>, (int)grid, PTHREADS_F32, ssmem(), s, a, T1, T2, err, xmap);
+}
+
 }  // namespace
 
 bool plane_pass_supported(int N) {
@@ -1013,12 +1411,27 @@ cudaError_t plane_pass_prepare(int N) {
       if (e == cudaSuccess)
         e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
     }
-    for (bool f32 : {false, true})
-      if (e == cudaSuccess && (!f32 || N <= 128))
-        e = cudaFuncSetAttribute((const void*)single_kernel(N, k, f32), cudaFuncAttributeMaxDynamicSharedMemorySize,
+    for (int in : {kInPlanes, kInF32, kInPoints})
+      if (e == cudaSuccess && (in == kInPlanes || N <= 128))
+        e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
   }
   return e;
+}
+
+cudaError_t plane_square_prepare() {
+  cudaError_t e = cudaSuccess;
+  for (const void* f : {(const void*)plane_square_kernel<kOutPlanes>, (const void*)plane_square_kernel<kOutComplex>,
+                        (const void*)plane_square_kernel<kOutDensity>})
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, ssmem());
+  return e;
+}
+
+cudaError_t launch_plane_square(const DenseArgs& a, const unsigned char* T1, const unsigned char* T2, int* err, int sms,
+                                cudaStream_t s) {
+  if (a.out_bf) return launch_square<kOutPlanes>(a, T1, T2, err, sms, s);
+  if (a.out_c) return launch_square<kOutComplex>(a, T1, T2, err, sms, s);
+  return launch_square<kOutDensity>(a, T1, T2, err, sms, s);
 }
 
 cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s) {
@@ -1062,11 +1475,16 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   }
   const bool f32 = !a.in_bf;
   const bool pair = pair_pass(a.N, a.ncols, sms);
-  if (a.inner != 1 || a.grad || (f32 && !pair && a.N > 128)) return cudaErrorInvalidValue;
+  if (a.inner != 1 || a.grad || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
+    return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
-  // bf_plane points after the head plane; or the FP32 lines
+  // bf_plane points after the head plane; or the FP32 lines; or a square
+  // pass's parts
   CUtensorMap xmap, tmap;
-  if (f32 ? !f32_map(&xmap, a.in, 2 * a.N, a.batch * a.outer, PL)
+  if (a.in_points) {
+    if (!points_map(&xmap, a.in_bf, a.oinner, a.N, a.batch * a.outer / a.oinner, a.bf_plane, a.unsplit ? 2 : 4))
+      return cudaErrorInvalidValue;
+  } else if (f32 ? !f32_map(&xmap, a.in, 2 * a.N, a.batch * a.outer, PL)
           : !row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
     return cudaErrorInvalidValue;
   const int out = a.out_bf ? kOutPlanes : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
@@ -1080,7 +1498,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     return launch_pdl(f32 ? QVariant<true>::fn[out] : QVariant<false>::fn[out], (int)grid,
                       f32 ? PTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
-  return launch_pdl(single_kernel(a.N, out, f32), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,
+  return launch_pdl(single_kernel(a.N, out, a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,
                     err, xmap);
 }
 

@@ -39,7 +39,7 @@ inline bool make_tile_map(CUtensorMap* map, CUtensorMapDataType type, unsigned r
   std::memset(map, 0, sizeof(*map));
   const EncodeTiledFn enc = encode_tiled();
   if (!enc) return false;
-  const cuuint32_t estr[3] = {1, 1, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
   for (int attempt = 0; attempt < 2; ++attempt) {
     if (enc(map, type, rank, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle,
             CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS)

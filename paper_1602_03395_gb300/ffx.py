@@ -100,6 +100,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.ffx_plan_bf16_chain.restype = i32
     lib.ffx_plan_chain_split.argtypes = [vp, i64]
     lib.ffx_plan_chain_split.restype = i32
+    lib.ffx_plan_chain_square.argtypes = [vp, i64]
+    lib.ffx_plan_chain_square.restype = i32
     lib.ffx_plan_launch_count.argtypes = [vp]
     lib.ffx_plan_launch_count.restype = i64
     lib.ffx_expand_positive_p.argtypes = [vp, vp, vp, i64, vp, vp]
@@ -284,11 +286,13 @@ class Plan:
         lines adds its own split launch; launch_count() counts exactly."""
         n = len(self.dims)
         # a BF16 chain adds the split of its input, unless its first pass takes
-        # the FP32 input itself (the forward half of a
-        # backward call takes a chain except on 2-D plans, its adjoint half
-        # always, with the split of its gradient factors)
+        # the FP32 input itself; one launch may cover its last two axes (the
+        # forward half of a backward call takes a chain except on 2-D plans,
+        # its adjoint half always, with the split of its gradient factors)
         bf = self.bf16_chain(batch)
-        chain = (1 if self.chain_split(batch) and (not backward or n != 2) else 0) + (1 if bf and backward else 0)
+        chain = 1 if bf and backward else 0
+        if not backward or n != 2:
+            chain += int(self.chain_split(batch)) - int(self.chain_square(batch))
         if not backward and self.fused and batch > self.fused_max_batch:
             return n + chain
         return int(load_library().ffx_launches_per_call(self.handle, int(backward))) + chain
@@ -312,6 +316,11 @@ class Plan:
         """Whether a forward BF16 chain with this batch starts with a launch
         that splits its input (else its first pass splits on the way in)."""
         return load_library().ffx_plan_chain_split(self.handle, batch) == 1
+
+    def chain_square(self, batch: int = 1) -> bool:
+        """Whether a forward BF16 chain with this batch covers its last two
+        axes (64 points each) in one launch."""
+        return load_library().ffx_plan_chain_square(self.handle, batch) == 1
 
     def pass_order(self):
         order = (ctypes.c_int32 * len(self.dims))()

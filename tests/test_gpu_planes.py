@@ -84,6 +84,57 @@ FP32_CASES = [
 ]
 
 
+# chains whose last two axes (64 points each) are one launch: every first axis
+# it serves, no first axis (an odd number of squares), items that do and do not
+# divide by the blocks, ensemble sums in groups with a remainder
+SQUARE_CASES = [
+    ((64, 64, 64), (5, 3, 7), 20),
+    ((64, 64, 64), (9, 50, 4), 41),
+    ((96, 64, 64), (4, 5, 6), 13),
+    ((128, 64, 64), (6, 4, 3), 10),
+    ((64, 64), (5, 8), 1217),
+]
+
+
+@pytest.mark.parametrize("dims,lam,batch", SQUARE_CASES)
+def test_square_of_64_points(ffx, dims, lam, batch):
+    rng = np.random.default_rng(batch + sum(dims))
+    dx, t = (0.25, 0.3, 0.2)[:len(dims)], 6.0
+    psi = random_field(rng, (batch,) + dims)
+    ref = O.expand_field(psi, dx, t, lam)
+    dens = np.abs(ref) ** 2
+    start = rng.random(size=dims).astype(np.float32)
+    grad = rng.normal(size=(batch,) + dims).astype(np.float32)
+    x = to_dev(psi)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
+        assert plan.chain_square(batch) and not plan.chain_split(batch)
+        n0 = plan.launch_count()
+        rho = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.launch_count() - n0 == len(dims) - 1 == plan.launches_per_call(batch=batch)
+        fld = ffx.ffx_expand_field(plan, x).cpu().numpy()
+        y = x.clone()
+        ffx.ffx_expand_field(plan, y, y)  # in place
+        assert np.array_equal(y.cpu().numpy(), fld)
+        n0 = plan.launch_count()
+        g = ffx.ffx_expand_backward(plan, x, to_dev(grad)).cpu().numpy()
+        if len(dims) == 3:
+            assert plan.launch_count() - n0 == plan.launches_per_call(backward=True, batch=batch)
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, accumulate=True) as plan:
+        assert plan.chain_square(batch) == (len(dims) == 3)
+        acc = ffx.ffx_expand(plan, x, to_dev(start.copy())).cpu().numpy()
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, unsplit=True) as plan:
+        rough = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.device_errors() == 0
+    assert rel_l2(rho, dens) < DENSITY_TOL
+    assert rel_l2(fld, ref) < FIELD_TOL
+    assert rel_l2(rho, np.abs(fld) ** 2) < 1e-6
+    assert rel_l2(acc, start + dens.sum(0)) < DENSITY_TOL
+    assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
+    assert rel_l2(rough, dens) < UNSPLIT_TOL
+
+
 @pytest.mark.parametrize("dims,lam,batch", FP32_CASES)
 def test_pass_of_fp32_lines(ffx, dims, lam, batch):
     rng = np.random.default_rng(batch + sum(dims))
@@ -95,7 +146,7 @@ def test_pass_of_fp32_lines(ffx, dims, lam, batch):
     with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
         n0 = plan.launch_count()
         rho = ffx.ffx_expand(plan, x).cpu().numpy()
-        assert plan.launch_count() - n0 == len(dims)  # no split launch
+        assert plan.launch_count() - n0 == len(dims) - plan.chain_square(batch)  # no split launch
         fld = ffx.ffx_expand_field(plan, x).cpu().numpy()
         y = x.clone()
         ffx.ffx_expand_field(plan, y, y)              # in place
