@@ -495,6 +495,11 @@ int ffx_plan_chain_split(ffx_plan_t plan, int64_t batch);
  * so that the call makes one launch fewer; it splits its input on the way in. */
 int ffx_plan_chain_square(ffx_plan_t plan, int64_t batch);
 
+/* 1 if the forward half of an ffx_expand_backward call with this batch writes
+ * the factors 2 grad * field of its adjoint half itself; 0 if a launch of its
+ * own forms them. */
+int ffx_plan_chain_grad(ffx_plan_t plan, int64_t batch);
+
 /* Forward pass order: writes the lattice axis of pass k to order[k],
  * k = 0..ndim-1.  The adjoint runs the same axes in reverse. */
 int ffx_plan_pass_order(ffx_plan_t plan, int32_t* order);

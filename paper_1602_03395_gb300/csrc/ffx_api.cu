@@ -336,7 +336,7 @@ void trace_end(ffx_plan_s* p, cudaStream_t stream, unsigned rec_flags) {
 // A pass of a BF16 chain (forward only): its lines are contiguous (the
 // previous pass wrote them transposed, or the axis is the last one), read
 // from BF16 planes (in_bf) or the FP32 field `in`; its output goes to BF16
-// planes (out_bf) or the caller's buffers, transposed: point n' of line rho
+// planes (out_bf; with `grad`, of 2 grad times the result) or the caller's buffers, transposed: point n' of line rho
 // at n' (M / N) + rho of its realization.  plane: points per plane.
 struct ChainIo {
   const uint32_t* in_bf;
@@ -389,7 +389,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
     // split TF32
     const bool tm64 = ax.N == 64 && !acc && !grad && items <= 4 * grid;
     if (io) {
-      if (!ax.pl_t[adjoint ? 1 : 0] || tm64 || grad)
+      if (!ax.pl_t[adjoint ? 1 : 0] || tm64 || (grad && !io->out_bf))
         return fail(FFX_EUNSUPPORTED, "internal: a BF16 chain pass of axis %d without the BF16 kernel", j);
       d.in_bf = io->in_bf;  // or NULL: the FP32 lines `in`
       d.out_bf = io->out_bf;
@@ -666,7 +666,8 @@ bool bf16_adjoint_ok(const ffx_plan_s* p) {
 // (plane_square_kernel): 64 points each, the first axis one whose pass keeps T
 // resident, or none (2-D lattices; their ensemble sums stay with the passes).
 // 44 bytes a point of HBM become 28 on 3-D lattices (density, 64 realizations
-// of 64^3: @@), 28 become 12 on 2-D ones (@@).
+// of 64^3: 142.5 us as three passes, 108.0 us), 28 become 12 on 2-D ones (4096
+// images: 78.9 and 60.2 us).
 bool chain_square(const ffx_plan_s* p) {
   const int d = p->ndim;
   if (d < 2 || p->axis[d - 1].N != 64 || p->axis[d - 2].N != 64 || p->order[0] != d - 1 || p->order[1] != d - 2)
@@ -690,7 +691,9 @@ bool chain_splits(const ffx_plan_s* p, int64_t batch) {
 // that writes ws[1].  `in` is read by the split (or the first pass,
 // which writes ws[0]) alone, so out_c may equal it; it must not be ws[1] or, if
 // the first pass reads it, ws[0].
-int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, float* out_d, cudaStream_t s) {
+// With `grad` (3-D) the last pass writes planes of 2 grad times the field to ws[0].
+int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, float* out_d, cudaStream_t s,
+               const float* grad = nullptr, int grad_shared = 0) {
   const int d = p->ndim;
   const bool square = chain_square(p);
   int rc;
@@ -715,8 +718,8 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
     ++p->launches;
     trace_end(p, s, rec);
     if (d == 2) return FFX_OK;
-    ChainIo io = {(const uint32_t*)p->ws[1], nullptr, plane, 1};
-    return run_axis(p, p->order[2], false, nullptr, nullptr, 0, out_c, out_d, out_d ? p->acc : 0, batch, s, &io);
+    ChainIo io = {(const uint32_t*)p->ws[1], grad ? (uint32_t*)p->ws[0] : nullptr, plane, 1};
+    return run_axis(p, p->order[2], false, nullptr, grad, grad_shared, out_c, out_d, out_d ? p->acc : 0, batch, s, &io);
   }
   if (chain_splits(p, batch)) {
     const unsigned rec = trace_begin(p, s);
@@ -730,48 +733,64 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
     const bool last = r == d - 1;
     ChainIo io;
     io.in_bf = cur_bf;
-    io.out_bf = last ? nullptr : (uint32_t*)p->ws[r & 1];
+    io.out_bf = last && !grad ? nullptr : (uint32_t*)p->ws[r & 1];
     io.plane = plane;
     io.points = 0;
-    rc = run_axis(p, p->order[r], false, cur_bf ? nullptr : in, nullptr, 0, last ? out_c : nullptr,
-                  last ? out_d : nullptr, last && out_d ? p->acc : 0, batch, s, &io);
+    rc = run_axis(p, p->order[r], false, cur_bf ? nullptr : in, last ? grad : nullptr, grad_shared,
+                  last ? out_c : nullptr, last ? out_d : nullptr, last && out_d ? p->acc : 0, batch, s, &io);
     if (rc) return rc;
     cur_bf = io.out_bf;
   }
   return FFX_OK;
 }
 
-// The adjoint half of a backward call as a BF16 chain: 2 grad * field split
-// into BF16 planes in ws[1], then the adjoint passes in the chain's order
-// (T_j^H along the last axis first; the axes' factors commute), planes
-// between them in ws[0] and ws[1] as in chain_bf16, the last pass writing
-// `out`.  `field` is read by the split alone (it may be ws[0]).
-int chain_bf16_adjoint(ffx_plan_s* p, const float2* field, const float* grad, int grad_shared, int64_t batch,
-                       float2* out, cudaStream_t s) {
+// Whether the last forward pass of such a call writes planes of 2 grad times
+// the field itself, from which the adjoint half starts: calls that fill the
+// chip (the chain's input is not split apart either) and a last pass whose
+// kernel does so.  Its epilogue then reads 4 bytes a point more; the separate
+// split reads and writes 20 (backward calls: 256^3 499 -> 461 us, 64
+// realizations of 64^3 336 -> 290 us with the square pass, 20 of 96x64x96 261 ->
+// 251 us).
+bool chain_grad(const ffx_plan_s* p, int64_t batch) {
+  const Axis& ax = p->axis[p->order[p->ndim - 1]];
+  return p->ndim == 3 && !chain_splits(p, batch) && plane_pass_splits(ax.N, batch * (p->M / ax.N), p->sms) &&
+         bf16_adjoint_ok(p);
+}
+
+// The adjoint half of a backward call as a BF16 chain: the planes of 2 grad *
+// field, in ws[from], then the adjoint passes in the chain's order (T_j^H along
+// the last axis first; the axes' factors commute), planes between them in the
+// workspaces in turn, the last pass writing `out`.
+int chain_bf16_adjoint(ffx_plan_s* p, int from, int64_t batch, float2* out, cudaStream_t s) {
   const int d = p->ndim;
-  int rc;
-  if ((rc = ensure_ws(p, 0, batch)) || (rc = ensure_ws(p, 1, batch))) return rc;
-  const int64_t plane = batch * p->M;
-  const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
-  const unsigned rec = trace_begin(p, s);
-  cudaError_t e = launch_plane_split(field, grad, grad_shared, p->M, (uint32_t*)p->ws[1], plane, plane, unsplit,
-                                     p->sms, s);
-  if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the gradient factors");
-  ++p->launches;
-  trace_end(p, s, rec);
-  const uint32_t* cur_bf = (const uint32_t*)p->ws[1];
+  const uint32_t* cur_bf = (const uint32_t*)p->ws[from];
   for (int r = 0; r < d; ++r) {
     const bool last = r == d - 1;
     ChainIo io;
     io.in_bf = cur_bf;
-    io.out_bf = last ? nullptr : (uint32_t*)p->ws[r & 1];
-    io.plane = plane;
+    io.out_bf = last ? nullptr : (uint32_t*)p->ws[(from + 1 + r) & 1];
+    io.plane = batch * p->M;
     io.points = 0;
-    rc = run_axis(p, p->order[r], true, nullptr, nullptr, 0, last ? out : nullptr, nullptr, 0, batch, s, &io);
+    int rc = run_axis(p, p->order[r], true, nullptr, nullptr, 0, last ? out : nullptr, nullptr, 0, batch, s, &io);
     if (rc) return rc;
     cur_bf = io.out_bf;
   }
   return FFX_OK;
+}
+
+// ... after a split of 2 grad * field into planes in ws[1] (`field` may be ws[0]).
+int chain_bf16_split_adjoint(ffx_plan_s* p, const float2* field, const float* grad, int grad_shared, int64_t batch,
+                             float2* out, cudaStream_t s) {
+  int rc;
+  if ((rc = ensure_ws(p, 0, batch)) || (rc = ensure_ws(p, 1, batch))) return rc;
+  const int64_t plane = batch * p->M;
+  const unsigned rec = trace_begin(p, s);
+  cudaError_t e = launch_plane_split(field, grad, grad_shared, p->M, (uint32_t*)p->ws[1], plane, plane,
+                                     (p->flags & FFX_TC_UNSPLIT) ? 1 : 0, p->sms, s);
+  if (e != cudaSuccess) return cuda_fail(e, "BF16 split of the gradient factors");
+  ++p->launches;
+  trace_end(p, s, rec);
+  return chain_bf16_adjoint(p, 1, batch, out, s);
 }
 
 // Run a chain of passes (forward or adjoint) from `in` (read only) into
@@ -1462,8 +1481,9 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           }
           e = launch_plane_build_t(ax.T, ax.pl_t[0], ax.N, s);
           if (e == cudaSuccess) e = launch_plane_build_t(ax.TH, ax.pl_t[1], ax.N, s);
-          if (e == cudaSuccess) e = plane_pass_prepare(ax.N);
-          if (e == cudaSuccess && ax.N == 64) e = plane_square_prepare();
+          const bool square = ndim > 1 && p->axis[ndim - 1].N == 64 && p->axis[ndim - 2].N == 64;
+          if (e == cudaSuccess) e = plane_pass_prepare(ax.N, square && j == 0, ndim == 3 && j == 0);
+          if (e == cudaSuccess && square) e = plane_square_prepare();
         }
         if (e == cudaSuccess)
           e = dense_tc_prepare();
@@ -1685,6 +1705,11 @@ int ffx_plan_bf16_chain(ffx_plan_t p, int64_t batch) {
 int ffx_plan_chain_square(ffx_plan_t p, int64_t batch) {
   if (ffx_plan_bf16_chain(p, batch) != 1) return 0;
   return chain_square(p) ? 1 : 0;
+}
+
+int ffx_plan_chain_grad(ffx_plan_t p, int64_t batch) {
+  if (ffx_plan_bf16_chain(p, batch) != 1) return 0;
+  return chain_grad(p, batch) ? 1 : 0;
 }
 
 int ffx_plan_chain_split(ffx_plan_t p, int64_t batch) {
@@ -1934,10 +1959,17 @@ int ffx_expand_backward(ffx_plan_t p, const void* psi0, const float* grad_densit
   // grad_psi0 (ws[1] as the alternate)
   if ((rc = ensure_ws(p, 0, batch))) return rc;
   float2* field = (float2*)p->ws[0];
+  if (psi0 != p->ws[0] && psi0 != p->ws[1] && chain_grad(p, batch) &&
+      bf16_chain_ok(p, batch, psi0, grad_psi0, nullptr)) {
+    if ((rc = ensure_ws(p, 1, batch)) ||
+        (rc = chain_bf16(p, (const float2*)psi0, batch, nullptr, nullptr, s, grad_density, p->acc)))
+      return rc;
+    return chain_bf16_adjoint(p, 0, batch, (float2*)grad_psi0, s);
+  }
   if ((rc = chain_into(p, p->order, false, (const float2*)psi0, nullptr, 0, batch, field, 1, s))) return rc;
   // the adjoint half as a BF16 chain where the forward map takes one
   if (bf16_chain_ok(p, batch, field, grad_psi0, nullptr) && bf16_adjoint_ok(p))
-    return chain_bf16_adjoint(p, field, grad_density, p->acc, batch, (float2*)grad_psi0, s);
+    return chain_bf16_split_adjoint(p, field, grad_density, p->acc, batch, (float2*)grad_psi0, s);
   int axes[3];
   for (int r = 0; r < p->ndim; ++r) axes[r] = p->order[p->ndim - 1 - r];
   return chain_into(p, axes, true, field, grad_density, p->acc, batch, (float2*)grad_psi0, 1, s);

@@ -125,8 +125,10 @@ __device__ __forceinline__ void store_pair(void* o, int64_t other, bool odd, boo
 
 // What a pass writes: planes (inside a chain), the complex field, densities, or
 // densities summed over the batch.
-enum POut { kOutPlanes = 0, kOutComplex = 1, kOutDensity = 2, kOutSum = 3 };
-constexpr int kPOuts = 4;
+// kOutGrad: planes of 2 grad times the result (the last forward pass of a
+// backward call, whose adjoint half starts from them)
+enum POut { kOutPlanes = 0, kOutComplex = 1, kOutDensity = 2, kOutSum = 3, kOutGrad = 4 };
+constexpr int kPOuts = 5;
 
 // Where the first operand of a chunk lies: descriptor words (low) of its real
 // and imaginary parts, head and tail, at K step ks.
@@ -185,6 +187,13 @@ __device__ __forceinline__ void plane_half(uint32_t d, const X& x, uint32_t t2, 
     mma(d + RB, x.at(ks, false, true), b1 + ks * 2 + o0 / 16, id1, 1u);
     mma(d + RB, x.at(ks, true, true), b1 + ks * 2 + o1 / 16, id1 | neg, 1u);
   }
+}
+
+// A load that stays where it is written (hoisted loads of later outputs spill).
+__device__ __forceinline__ float load_here(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
 }
 
 // The epilogue warps of a block (warps 4-11): items first, first + step, ...;
@@ -295,7 +304,16 @@ __device__ __forceinline__ void plane_epilogue(const DenseArgs& a, int warp, int
       }
 #pragma unroll
       for (int m = 0; m < H; ++m) racc[m] = 0.f;
-    } else if constexpr (OUT == kOutPlanes) {
+    } else if constexpr (OUT == kOutPlanes || OUT == kOutGrad) {
+      // gradient factors: into L2 now (one line of 32 points per output and warp)
+      const float* gp = nullptr;
+      if constexpr (OUT == kOutGrad) {
+        gp = a.grad + base - (a.grad_shared ? bo * a.M : 0);
+        if (valid) {
+#pragma unroll 1
+          for (int m = lane; m < H; m += 32) asm volatile("prefetch.global.L2 [%0];" ::"l"(gp - lane + m * inner));
+        }
+      }
       // BF16 head and tail planes for the next pass of a chain: both halves in
       // registers, then a lane pair exchanges (real, imaginary) parts, so that
       // the even lane stores the pair's real parts and the odd lane its
@@ -318,6 +336,17 @@ __device__ __forceinline__ void plane_epilogue(const DenseArgs& a, int warp, int
 #pragma unroll
         for (int m0 = 0; m0 < H; m0 += 8) {
           uint32_t h[8], l[8], x[8];
+          if constexpr (OUT == kOutGrad) {
+            float gn[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m) gn[m] = load_here(gp + m * inner);
+#pragma unroll
+            for (int m = 0; m < 8; ++m) {
+              const float g2 = 2.f * gn[m];
+              y[m0 + m] *= g2, z[m0 + m] *= g2;
+            }
+            advance(gp, 8 * inner);
+          }
 #pragma unroll
           for (int m = 0; m < 8; ++m) {
             h[m] = bf2(y[m0 + m], z[m0 + m]);
@@ -1333,14 +1362,22 @@ using PKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUte
 using QKernel = void (*)(const DenseArgs, int*, const CUtensorMap, const CUtensorMap);
 template <bool F32>
 struct QVariant {
+  static constexpr QKernel grad() {
+    if constexpr (F32) return nullptr;
+    else return plane_pair_kernel<kOutGrad, false>;
+  }
   static constexpr QKernel fn[kPOuts] = {plane_pair_kernel<kOutPlanes, F32>, plane_pair_kernel<kOutComplex, F32>,
-                                         plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>};
+                                         plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>, grad()};
 };
 template <int RB, bool RES, int IN>
 struct PVariant {
+  static constexpr PKernel grad() {
+    if constexpr (!RES || IN == kInF32) return nullptr;
+    else return plane_pass_kernel<RB, RES, kOutGrad, IN>;
+  }
   static constexpr PKernel fn[kPOuts] = {
       plane_pass_kernel<RB, RES, kOutPlanes, IN>, plane_pass_kernel<RB, RES, kOutComplex, IN>,
-      plane_pass_kernel<RB, RES, kOutDensity, IN>, plane_pass_kernel<RB, RES, kOutSum, IN>};
+      plane_pass_kernel<RB, RES, kOutDensity, IN>, plane_pass_kernel<RB, RES, kOutSum, IN>, grad()};
 };
 template <int IN>
 PKernel resident_kernel(int N, int out) {
@@ -1403,16 +1440,17 @@ bool plane_pass_supported(int N) {
 
 size_t plane_t_bytes(int N) { return (size_t)N * N * 8; }
 
-cudaError_t plane_pass_prepare(int N) {
+cudaError_t plane_pass_prepare(int N, bool points, bool grad) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < kPOuts && e == cudaSuccess; ++k) {
+    if (k == kOutGrad && !grad) continue;
     if (pair_length(N)) {
       e = cudaFuncSetAttribute((const void*)QVariant<false>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-      if (e == cudaSuccess)
+      if (e == cudaSuccess && QVariant<true>::fn[k])
         e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
     }
     for (int in : {kInPlanes, kInF32, kInPoints})
-      if (e == cudaSuccess && (in == kInPlanes || N <= 128))
+      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && (in != kInPoints || points) && single_kernel(N, k, in))
         e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
   }
@@ -1475,7 +1513,11 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   }
   const bool f32 = !a.in_bf;
   const bool pair = pair_pass(a.N, a.ncols, sms);
-  if (a.inner != 1 || a.grad || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
+  const int out = a.out_bf ? (a.grad ? kOutGrad : kOutPlanes)
+                           : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
+  const int in = a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
+  if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
+  if (a.inner != 1 || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
     return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines; or a square
@@ -1487,7 +1529,6 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   } else if (f32 ? !f32_map(&xmap, a.in, 2 * a.N, a.batch * a.outer, PL)
           : !row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
     return cudaErrorInvalidValue;
-  const int out = a.out_bf ? kOutPlanes : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
   int64_t at_once;
   int64_t grid = std::min(plane_pass_tiles(a.N, a.ncols, sms, &at_once), at_once);
   if (grid < 1) grid = 1;
@@ -1498,7 +1539,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     return launch_pdl(f32 ? QVariant<true>::fn[out] : QVariant<false>::fn[out], (int)grid,
                       f32 ? PTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
-  return launch_pdl(single_kernel(a.N, out, a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,
+  return launch_pdl(single_kernel(a.N, out, in), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,
                     err, xmap);
 }
 

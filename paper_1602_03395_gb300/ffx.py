@@ -102,6 +102,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
     lib.ffx_plan_chain_split.restype = i32
     lib.ffx_plan_chain_square.argtypes = [vp, i64]
     lib.ffx_plan_chain_square.restype = i32
+    lib.ffx_plan_chain_grad.argtypes = [vp, i64]
+    lib.ffx_plan_chain_grad.restype = i32
     lib.ffx_plan_launch_count.argtypes = [vp]
     lib.ffx_plan_launch_count.restype = i64
     lib.ffx_expand_positive_p.argtypes = [vp, vp, vp, i64, vp, vp]
@@ -288,9 +290,9 @@ class Plan:
         # a BF16 chain adds the split of its input, unless its first pass takes
         # the FP32 input itself; one launch may cover its last two axes (the
         # forward half of a backward call takes a chain except on 2-D plans,
-        # its adjoint half always, with the split of its gradient factors)
-        bf = self.bf16_chain(batch)
-        chain = 1 if bf and backward else 0
+        # its adjoint half always, with the split of its gradient factors
+        # unless the forward half writes them)
+        chain = 1 if backward and self.bf16_chain(batch) and not self.chain_grad(batch) else 0
         if not backward or n != 2:
             chain += int(self.chain_split(batch)) - int(self.chain_square(batch))
         if not backward and self.fused and batch > self.fused_max_batch:
@@ -321,6 +323,11 @@ class Plan:
         """Whether a forward BF16 chain with this batch covers its last two
         axes (64 points each) in one launch."""
         return load_library().ffx_plan_chain_square(self.handle, batch) == 1
+
+    def chain_grad(self, batch: int = 1) -> bool:
+        """Whether the forward half of a backward call with this batch writes
+        the gradient factors of its adjoint half itself."""
+        return load_library().ffx_plan_chain_grad(self.handle, batch) == 1
 
     def pass_order(self):
         order = (ctypes.c_int32 * len(self.dims))()

@@ -191,3 +191,40 @@ def test_first_cuda_call_of_a_thread(ffx):
         torch.cuda.synchronize()
     assert not failures
     assert torch.equal(out, want)
+
+
+# backward calls whose last forward pass writes the gradient factors: every
+# kernel that does (T resident of 64, 96 and 128 points, CTA pairs, after a square
+# pass), whole and ragged last tiles; and calls with a launch of their own for them
+GRAD_CASES = [
+    ((64, 64, 64), (5, 3, 7), 20, True),
+    ((96, 64, 64), (4, 5, 6), 13, True),
+    ((128, 128, 96), (4, 5, 6), 3, True),
+    ((64, 128, 96), (5, 3, 4), 7, True),
+    ((96, 96, 128), (3, 4, 5), 5, True),
+    ((256, 96, 128), (3, 4, 5), 3, True),
+    ((192, 96, 128), (3, 4, 5), 3, False),
+    ((96, 96, 96), (3, 4, 5), 1, False),
+]
+
+
+@pytest.mark.parametrize("dims,lam,batch,fused", GRAD_CASES)
+def test_gradient_factors_of_the_last_forward_pass(ffx, dims, lam, batch, fused):
+    rng = np.random.default_rng(batch + sum(dims))
+    dx, t = (0.25, 0.3, 0.2), 6.0
+    psi = random_field(rng, (batch,) + dims)
+    grad = rng.normal(size=(batch,) + dims).astype(np.float32)
+    gsum = rng.normal(size=dims).astype(np.float32)
+    x = to_dev(psi)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
+        assert plan.chain_grad(batch) == fused
+        n0 = plan.launch_count()
+        g = ffx.ffx_expand_backward(plan, x, to_dev(grad)).cpu().numpy()
+        assert plan.launch_count() - n0 == plan.launches_per_call(backward=True, batch=batch)
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, accumulate=True) as plan:
+        gs = ffx.ffx_expand_backward(plan, x, to_dev(gsum)).cpu().numpy()
+        assert plan.device_errors() == 0
+    assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
+    ref = O.density_loss_gradient(psi, np.broadcast_to(gsum, psi.shape), dx, t, lam)
+    assert rel_l2(gs, ref) < FIELD_TOL
