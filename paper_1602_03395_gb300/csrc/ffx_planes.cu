@@ -471,11 +471,49 @@ __device__ __forceinline__ void split_line(unsigned char* x, int n, bool unsplit
     }
 }
 
-// The producer threads' loop over the block's chunks: line n of each tile, once
-// it has landed (raw_bar); done(stage): the warp has split its lines.
-template <int NST, int STAGE, class Done>
-__device__ __forceinline__ void split_tiles(unsigned char* stages, int n, int lane, int64_t total, bool unsplit,
-                                            uint64_t* raw_bar, volatile int* s_abort, const Done& done) {
+// The same for a chunk of strided lines: per group of 64 lines, 16 KB, four FP32
+// boxes of 16 lines x 32 points (a point a row of 128 bytes) become the group's
+// four parts of 64 lines x 32 points.  Two lanes of a warp share a row (lines
+// 0-31, lines 32-63), so the warp has read its rows before it writes them.
+__device__ __forceinline__ void split_points(unsigned char* x, int warp, int lane, bool unsplit) {
+  constexpr int BOX = PXPART / 4;
+  const int row = (warp & 1) * 16 + (lane & 15), side = lane >> 4, sw = row & 7;
+  unsigned char* const p = x + (warp >> 1) * PXPART + row * 128;
+  float4 v[2][8];
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) v[g][c] = *reinterpret_cast<const float4*>(p + (2 * side + g) * BOX + ((c ^ sw) << 4));
+  __syncwarp();
+#pragma unroll
+  for (int g = 0; g < 2; ++g)
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      // eight lines: 16 bytes of each part
+      uint32_t r[4], m[4], rl[4], ml[4];
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float4 f = v[g][4 * k + c];
+        r[c] = bf2(f.x, f.z);
+        m[c] = bf2(f.y, f.w);
+        rl[c] = bf2(f.x - bf_lo(r[c]), f.z - bf_hi(r[c]));
+        ml[c] = bf2(f.y - bf_lo(m[c]), f.w - bf_hi(m[c]));
+      }
+      unsigned char* const o = p + (((4 * side + 2 * g + k) ^ sw) << 4);
+      *reinterpret_cast<uint4*>(o) = make_uint4(r[0], r[1], r[2], r[3]);
+      *reinterpret_cast<uint4*>(o + BOX) = make_uint4(m[0], m[1], m[2], m[3]);
+      if (!unsplit) {
+        *reinterpret_cast<uint4*>(o + 2 * BOX) = make_uint4(rl[0], rl[1], rl[2], rl[3]);
+        *reinterpret_cast<uint4*>(o + 3 * BOX) = make_uint4(ml[0], ml[1], ml[2], ml[3]);
+      }
+    }
+}
+
+// The producer threads' loop over the block's chunks: split(stage) of each, once
+// it has landed (raw_bar); done(stage): the warp has split its share.
+template <int NST, class Split, class Done>
+__device__ __forceinline__ void split_tiles(int lane, int64_t total, uint64_t* raw_bar, volatile int* s_abort,
+                                            const Split& split, const Done& done) {
   int s = 0;
   int64_t u = 0;
 #pragma unroll 1
@@ -483,7 +521,7 @@ __device__ __forceinline__ void split_tiles(unsigned char* stages, int n, int la
     bool ok = true;
     if (lane == 0) ok = mbar_wait(smem_u32(&raw_bar[s]), (uint32_t)(u & 1), s_abort);
     if (!__all_sync(0xffffffffu, ok)) break;
-    split_line(stages + s * STAGE, n, unsplit);
+    split(s);
     fence_async_smem();
     __syncwarp();
     if (lane == 0) done(s);
@@ -496,13 +534,15 @@ __device__ __forceinline__ void split_tiles(unsigned char* stages, int n, int la
 
 // What a pass reads: planes of contiguous lines; contiguous FP32 lines; or the
 // square kernel's four planes (below), in which a line's points are a.oinner
-// points apart (tiles of 64 lines x 32 points of each).
-enum PIn { kInPlanes = 0, kInF32 = 1, kInPoints = 2 };
+// points apart (tiles of 64 lines x 32 points of each); or FP32 lines whose
+// points are a.inner (a multiple of 64) points apart.
+enum PIn { kInPlanes = 0, kInF32 = 1, kInPoints = 2, kInStrided = 3 };
+constexpr bool in_fp32(int in) { return in == kInF32 || in == kInStrided; }
 
 // RB outputs per item, T resident (RES) or streamed; other input than planes
 // comes with RES.
 template <int RB, bool RES, int OUT, int IN>
-__global__ void __launch_bounds__(IN == kInF32 ? PTHREADS_F32 : PTHREADS, 1)
+__global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
     plane_pass_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err,
                       const __grid_constant__ CUtensorMap xmap) {
   constexpr int NST = pstages(RB, RES);
@@ -513,7 +553,8 @@ __global__ void __launch_bounds__(IN == kInF32 ? PTHREADS_F32 : PTHREADS, 1)
   constexpr bool ACC = OUT == kOutSum;
   extern __shared__ __align__(1024) unsigned char psm_raw[];
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
-  constexpr bool F32 = IN == kInF32, POINTS = IN == kInPoints;
+  // F32: split in the stages; POINTS: parts with a point a row
+  constexpr bool F32 = in_fp32(IN), POINTS = IN == kInPoints || IN == kInStrided;
   static_assert(RES || IN == kInPlanes, "FP32 and point-row input come with resident T");
   __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], raw_bar[PMAXST], t_bar;
   __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
@@ -584,7 +625,23 @@ __global__ void __launch_bounds__(IN == kInF32 ? PTHREADS_F32 : PTHREADS, 1)
           // rows: the tile's lines (realization ib's when accumulating); x: the
           // chunk's 64 values; z: the head plane (and the tail plane)
           const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
-          if (F32) {
+          if (IN == kInStrided) {
+            // two groups of 64 lines: group i at line 64 (i % per) of outer block i / per
+            const int64_t per = a.inner / 64;
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int64_t gi = ct * 2 + h + (ACC ? (int64_t)ib * a.outer * per : 0);
+              const int64_t z = gi / per;
+              const int x0 = (int)(gi - z * per) * 128;
+#pragma unroll
+              for (int b = 0; b < 4; ++b)
+                asm volatile(
+                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
+                    "%4}], [%5];" ::"r"(st + (uint32_t)(h * PXPART + b * (PXPART / 4))),
+                    "l"(map_addr), "r"(x0 + 32 * b), "r"(ikc * PKC), "r"((int)z), "r"(fb)
+                    : "memory");
+            }
+          } else if (F32) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               asm volatile(
@@ -705,8 +762,16 @@ __global__ void __launch_bounds__(IN == kInF32 ? PTHREADS_F32 : PTHREADS, 1)
     // ---------------- FP32 input: split into the stages ----------------
     if constexpr (F32) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-      split_tiles<NST, STAGE>(psm + (RB / PKC) * TCH, tid - 384, lane, my_items * nb * kchunks, unsplit, raw_bar, &s_abort,
-                              [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
+      split_tiles<NST>(
+          lane, my_items * nb * kchunks, raw_bar, &s_abort,
+          [&](int st) {
+            unsigned char* const x = psm + (RB / PKC) * TCH + st * STAGE;
+            if constexpr (IN == kInStrided)
+              split_points(x, warp - 12, lane, unsplit);
+            else
+              split_line(x, tid - 384, unsplit);
+          },
+          [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
     }
   }
 
@@ -1033,8 +1098,10 @@ __global__ void __launch_bounds__(PTHREADS_F32, 1)
   } else {
     // ---------------- FP32 input: split into the stages ----------------
     asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
-    split_tiles<SST, PX>(psm + 4 * TCH + SA2, tid - 384, lane, my_items * 2, unsplit, raw_bar, &s_abort,
-                         [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
+    split_tiles<SST>(
+        lane, my_items * 2, raw_bar, &s_abort,
+        [&](int st) { split_line(psm + 4 * TCH + SA2 + st * PX, tid - 384, unsplit); },
+        [&](int st) { mbar_arrive(smem_u32(&full_bar[st])); });
   }
 
   tc_fence_before();
@@ -1269,8 +1336,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
     if constexpr (F32) {
       asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
       const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
-      split_tiles<QST, QSTAGE>(psm, tid - 384, lane, total, unsplit, raw_bar, &s_abort,
-                               [&](int st) { mbar_arrive_cluster(full0 + 8u * (uint32_t)st); });
+      split_tiles<QST>(
+          lane, total, raw_bar, &s_abort, [&](int st) { split_line(psm + st * QSTAGE, tid - 384, unsplit); },
+          [&](int st) { mbar_arrive_cluster(full0 + 8u * (uint32_t)st); });
     }
   }
 
@@ -1372,11 +1440,15 @@ struct QVariant {
 template <int RB, bool RES, int IN>
 struct PVariant {
   static constexpr PKernel grad() {
-    if constexpr (!RES || IN == kInF32) return nullptr;
+    if constexpr (!RES || in_fp32(IN)) return nullptr;
     else return plane_pass_kernel<RB, RES, kOutGrad, IN>;
   }
+  static constexpr PKernel planes() {  // strided lines: no chain
+    if constexpr (IN == kInStrided) return nullptr;
+    else return plane_pass_kernel<RB, RES, kOutPlanes, IN>;
+  }
   static constexpr PKernel fn[kPOuts] = {
-      plane_pass_kernel<RB, RES, kOutPlanes, IN>, plane_pass_kernel<RB, RES, kOutComplex, IN>,
+      planes(), plane_pass_kernel<RB, RES, kOutComplex, IN>,
       plane_pass_kernel<RB, RES, kOutDensity, IN>, plane_pass_kernel<RB, RES, kOutSum, IN>, grad()};
 };
 template <int IN>
@@ -1389,8 +1461,12 @@ PKernel resident_kernel(int N, int out) {
 }
 PKernel single_kernel(int N, int out, int in) {
   if (N <= 128)
-    return in == kInF32 ? resident_kernel<kInF32>(N, out)
-                        : in == kInPoints ? resident_kernel<kInPoints>(N, out) : resident_kernel<kInPlanes>(N, out);
+    switch (in) {
+      case kInF32: return resident_kernel<kInF32>(N, out);
+      case kInPoints: return resident_kernel<kInPoints>(N, out);
+      case kInStrided: return resident_kernel<kInStrided>(N, out);
+      default: return resident_kernel<kInPlanes>(N, out);
+    }
   return N == 192 ? PVariant<96, false, kInPlanes>::fn[out] : PVariant<64, false, kInPlanes>::fn[out];
 }
 int single_rows(int N) { return N <= 128 ? N : N == 192 ? 96 : 64; }  // outputs per item
@@ -1402,6 +1478,14 @@ bool f32_map(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int
   const cuuint64_t strides[1] = {(cuuint64_t)cols * 4};
   const cuuint32_t box[2] = {32, (cuuint32_t)box_rows};
   return make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
+}
+
+// FP32 lines `inner` points apart: [outer][N][inner] points in tiles of 16 lines x 32 points
+bool strided_map(CUtensorMap* map, const void* base, int64_t outer, int N, int64_t inner) {
+  const cuuint64_t dims[3] = {(cuuint64_t)inner * 2, (cuuint64_t)N, (cuuint64_t)outer};
+  const cuuint64_t strides[2] = {(cuuint64_t)inner * 8, (cuuint64_t)inner * N * 8};
+  const cuuint32_t box[3] = {32, PKC, 1};
+  return make_tile_map(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, CU_TENSOR_MAP_SWIZZLE_128B);
 }
 
 // `rows` rows of `cols` BF16 values in tiles of 64 x box_rows, `planes` of them
@@ -1440,7 +1524,7 @@ bool plane_pass_supported(int N) {
 
 size_t plane_t_bytes(int N) { return (size_t)N * N * 8; }
 
-cudaError_t plane_pass_prepare(int N, bool points, bool grad) {
+cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < kPOuts && e == cudaSuccess; ++k) {
     if (k == kOutGrad && !grad) continue;
@@ -1449,8 +1533,9 @@ cudaError_t plane_pass_prepare(int N, bool points, bool grad) {
       if (e == cudaSuccess && QVariant<true>::fn[k])
         e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
     }
-    for (int in : {kInPlanes, kInF32, kInPoints})
-      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && (in != kInPoints || points) && single_kernel(N, k, in))
+    for (int in : {kInPlanes, kInF32, kInPoints, kInStrided})
+      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && (in != kInPoints || points) &&
+          (in != kInStrided || strided) && single_kernel(N, k, in))
         e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
   }
@@ -1505,6 +1590,14 @@ bool plane_pass_splits(int N, int64_t ncols, int sms) {
   return (N <= 128 || pair_pass(N, ncols, sms)) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
 }
 
+// Strided FP32 lines: groups of 64 adjacent lines land by TMA with a point a row
+// and are split in place like contiguous ones; the products take them with their
+// rows along the lines, so nothing is transposed.  (The kernel of ffx_tc16.cu
+// loads such lines to registers and stores them transposed: 2^24 points of 64,
+// inner 256, in place 48.7 us, here 36.3; 4.4 M points of 96, inner 192: 32.3 and
+// 20.0; 15.7 M points of 128, inner 256: 92.1 and 53.2.)
+bool plane_pass_strided(int N, int64_t inner) { return (N == 64 || N == 96 || N == 128) && inner % 64 == 0; }
+
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
   DenseArgs a = args;
   if (a.oinner == 0) {
@@ -1515,15 +1608,19 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   const bool pair = pair_pass(a.N, a.ncols, sms);
   const int out = a.out_bf ? (a.grad ? kOutGrad : kOutPlanes)
                            : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
-  const int in = a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
+  const bool strided = plane_pass_strided(a.N, a.inner);
+  const int in = strided ? kInStrided : a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
+  if (strided && (!f32 || a.out_bf)) return cudaErrorInvalidValue;
   if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
-  if (a.inner != 1 || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
+  if ((a.inner != 1 && !strided) || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
     return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines; or a square
   // pass's parts
   CUtensorMap xmap, tmap;
-  if (a.in_points) {
+  if (strided) {
+    if (!strided_map(&xmap, a.in, a.batch * a.outer, a.N, a.inner)) return cudaErrorInvalidValue;
+  } else if (a.in_points) {
     if (!points_map(&xmap, a.in_bf, a.oinner, a.N, a.batch * a.outer / a.oinner, a.bf_plane, a.unsplit ? 2 : 4))
       return cudaErrorInvalidValue;
   } else if (f32 ? !f32_map(&xmap, a.in, 2 * a.N, a.batch * a.outer, PL)

@@ -228,3 +228,49 @@ def test_gradient_factors_of_the_last_forward_pass(ffx, dims, lam, batch, fused)
     assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
     ref = O.density_loss_gradient(psi, np.broadcast_to(gsum, psi.shape), dx, t, lam)
     assert rel_l2(gs, ref) < FIELD_TOL
+
+
+# strided FP32 lines of 64, 96 and 128 points outside a chain: a group of 64
+# lines too few for the last tile, one group per outer block, several, first and
+# middle axes, ensemble sums (one group of realizations and many)
+STRIDED_CASES = [
+    ((64, 48, 64), (5, 3, 7), 27),
+    ((32, 64, 64), (3, 5, 4), 39),
+    ((96, 64), (9, 5), 3),
+    ((96, 32, 64), (4, 5, 6), 2),
+    ((32, 96, 64), (6, 4, 3), 3),
+    ((128, 32, 32), (11, 4, 3), 5),
+    ((32, 128, 192), (3, 30, 4), 2),
+]
+
+
+@pytest.mark.parametrize("dims,lam,batch", STRIDED_CASES)
+def test_strided_lines(ffx, dims, lam, batch):
+    rng = np.random.default_rng(batch + sum(dims))
+    dx, t = (0.25, 0.3, 0.2)[:len(dims)], 6.0
+    psi = random_field(rng, (batch,) + dims)
+    ref = O.expand_field(psi, dx, t, lam)
+    dens = np.abs(ref) ** 2
+    start = rng.random(size=dims).astype(np.float32)
+    grad = rng.normal(size=(batch,) + dims).astype(np.float32)
+    x = to_dev(psi)
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True) as plan:
+        assert not plan.bf16_chain(batch)
+        rho = ffx.ffx_expand(plan, x).cpu().numpy()
+        fld = ffx.ffx_expand_field(plan, x).cpu().numpy()
+        y = x.clone()
+        ffx.ffx_expand_field(plan, y, y)  # in place
+        assert np.array_equal(y.cpu().numpy(), fld)
+        g = ffx.ffx_expand_backward(plan, x, to_dev(grad)).cpu().numpy()
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, accumulate=True) as plan:
+        acc = ffx.ffx_expand(plan, x, to_dev(start.copy())).cpu().numpy()
+        assert plan.device_errors() == 0
+    with ffx.Plan(dims, dx, t, lam, form="tc", bf16=True, unsplit=True) as plan:
+        rough = ffx.ffx_expand(plan, x).cpu().numpy()
+        assert plan.device_errors() == 0
+    assert rel_l2(rho, dens) < DENSITY_TOL
+    assert rel_l2(fld, ref) < FIELD_TOL
+    assert rel_l2(acc, start + dens.sum(0)) < DENSITY_TOL
+    assert rel_l2(g, O.density_loss_gradient(psi, grad, dx, t, lam)) < FIELD_TOL
+    assert rel_l2(rough, dens) < UNSPLIT_TOL
