@@ -411,7 +411,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.bf_plane = plane;
       d.in = nullptr;
     }
-    if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(ax.N, inner))))
+    if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(ax.N, inner, d.ncols, p->sms))))
       e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
     else if (ax.bf_t[0] && !tm64)
       e = launch_dense_bf16(d, ax.bf_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
@@ -1486,7 +1486,7 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           for (int k = j + 1; k < ndim; ++k) inner *= p->axis[k].N;
           if (e == cudaSuccess)
             e = plane_pass_prepare(ax.N, square && j == 0, ndim == 3 && j == 0,
-                                   j < ndim - 1 && plane_pass_strided(ax.N, inner));
+                                   j < ndim - 1);
           if (e == cudaSuccess && square) e = plane_square_prepare();
         }
         if (e == cudaSuccess)

@@ -162,10 +162,10 @@ size_t plane_t_bytes(int N);
 // shared-memory attributes of the kernels a plan may launch (each loads its
 // code, about 0.5 ms the first time in a process): points, grad: those that read
 // a square pass's output, those that write gradient factors; strided: those of
-// plane_pass_strided
+// strided FP32 lines
 cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided);
 // whether launch_plane_pass takes FP32 lines whose points are `inner` > 1 apart
-bool plane_pass_strided(int N, int64_t inner);
+bool plane_pass_strided(int N, int64_t inner, int64_t ncols, int sms);
 cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s);
 cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
                                int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s);

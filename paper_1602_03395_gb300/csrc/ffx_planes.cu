@@ -152,6 +152,9 @@ struct XPoints {
     return x0 + ks * 128 + ((imag ? 1 : 0) + (tail ? 2 : 0)) * part;
   }
 };
+struct XStage : XPoints {  // the parts of two groups in a stage
+  __device__ __forceinline__ explicit XStage(uint32_t saddr) : XPoints(saddr, PXPART / 4, PXPART) {}
+};
 // the instruction descriptor's "first operand's rows run along its rows" bit
 constexpr uint32_t kMajorA = 1u << 15;
 
@@ -535,9 +538,27 @@ __device__ __forceinline__ void split_tiles(int lane, int64_t total, uint64_t* r
 // What a pass reads: planes of contiguous lines; contiguous FP32 lines; or the
 // square kernel's four planes (below), in which a line's points are a.oinner
 // points apart (tiles of 64 lines x 32 points of each); or FP32 lines whose
-// points are a.inner (a multiple of 64) points apart.
+// points are a.inner (a multiple of 16) points apart.
 enum PIn { kInPlanes = 0, kInF32 = 1, kInPoints = 2, kInStrided = 3 };
 constexpr bool in_fp32(int in) { return in == kInF32 || in == kInStrided; }
+
+// Copies of a chunk of strided lines: 128 lines from line l0 (a multiple of 16),
+// in boxes of 16 that lie next to one another in memory (a.inner is a multiple
+// of 16), 64 lines' boxes a group of 16 KB.
+__device__ __forceinline__ void copy_strided(const DenseArgs& a, uint64_t map_addr, uint32_t st, uint32_t bar, int64_t l0,
+                                             int kc) {
+  const uint32_t per = (uint32_t)(a.inner / 16), u = (uint32_t)(l0 / 16);
+  uint32_t z = u / per, x = u - z * per;
+#pragma unroll
+  for (int b = 0; b < 8; ++b) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(st + (uint32_t)(b * (PXPART / 4))),
+        "l"(map_addr), "r"(x * 32u), "r"(kc * PKC), "r"(z), "r"(bar)
+        : "memory");
+    if (++x == per) x = 0, ++z;
+  }
+}
 
 // RB outputs per item, T resident (RES) or streamed; other input than planes
 // comes with RES.
@@ -626,21 +647,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
           // chunk's 64 values; z: the head plane (and the tail plane)
           const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
           if (IN == kInStrided) {
-            // two groups of 64 lines: group i at line 64 (i % per) of outer block i / per
-            const int64_t per = a.inner / 64;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              const int64_t gi = ct * 2 + h + (ACC ? (int64_t)ib * a.outer * per : 0);
-              const int64_t z = gi / per;
-              const int x0 = (int)(gi - z * per) * 128;
-#pragma unroll
-              for (int b = 0; b < 4; ++b)
-                asm volatile(
-                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, "
-                    "%4}], [%5];" ::"r"(st + (uint32_t)(h * PXPART + b * (PXPART / 4))),
-                    "l"(map_addr), "r"(x0 + 32 * b), "r"(ikc * PKC), "r"((int)z), "r"(fb)
-                    : "memory");
-            }
+            copy_strided(a, map_addr, st, fb, ct * PL + (ACC ? (int64_t)ib * a.outer * a.inner : 0), ikc);
           } else if (F32) {
 #pragma unroll
             for (int h = 0; h < 2; ++h)
@@ -722,7 +729,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
           const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
           auto half = [&](auto imag, uint32_t dd) {
             if constexpr (POINTS)
-              plane_half<1, RB, decltype(imag)::value>(dd, XPoints(st, PXPART / 4, PXPART), tb, tb, id1, id2, kc == 0, unsplit);
+              plane_half<1, RB, decltype(imag)::value>(dd, XStage(st), tb, tb, id1, id2, kc == 0, unsplit);
             else
               plane_half<1, RB, decltype(imag)::value>(dd, XLines(st), tb, tb, id1, id2, kc == 0, unsplit);
           };
@@ -1145,8 +1152,8 @@ constexpr int QSMEM = QST * QSTAGE + 1024;
 static_assert(QSMEM <= 226 * 1024, "shared memory");
 
 // F32: FP32 lines, split in the stages as in plane_pass_kernel.
-template <int OUT, bool F32>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 : PTHREADS, 1)
+template <int OUT, int IN>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
     plane_pair_kernel(const DenseArgs a, int* err,
                       const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap tmap) {
   constexpr int RB = 128;
@@ -1162,6 +1169,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
   const int warp = tid >> 5, lane = tid & 31;
   const int rank = (int)cluster_rank();
   const int N = a.N;
+  constexpr bool F32 = in_fp32(IN), STRIDED = IN == kInStrided;
   const int mtiles = N / RB;
   const int kchunks = N / PKC;  // even
   const int64_t pair = blockIdx.x >> 1, npairs = gridDim.x >> 1;
@@ -1220,6 +1228,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
           if (F32) {
             const uint32_t rb = smem_u32(&raw_bar[is]);
             mbar_expect_tx(rb, PX);
+            if (STRIDED)
+              copy_strided(a, xmap_addr, st, rb, (2 * wt + rank) * PL + (ACC ? (int64_t)ib * a.outer * a.inner : 0), ikc);
+            else
 #pragma unroll
             for (int h = 0; h < 2; ++h)
               asm volatile(
@@ -1275,7 +1286,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
       bool ok = true;
       int s = 0;
       int64_t u = 0;
-      const uint32_t id1 = idesc_bf16(2 * PL, RB), id2 = idesc_bf16(2 * PL, 2 * RB);
+      using X = std::conditional_t<STRIDED, XStage, XLines>;
+      constexpr uint32_t major = STRIDED ? kMajorA : 0u;
+      const uint32_t id1 = idesc_bf16(2 * PL, RB) | major, id2 = idesc_bf16(2 * PL, 2 * RB) | major;
       const uint32_t dre = tmem, dim = tmem + 2 * RB;
 #pragma unroll 1
       for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
@@ -1290,11 +1303,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
                (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
           if (!ok) break;
           tc_fence_after();
-          plane_half<2, RB, false>(dre, XLines(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          plane_half<2, RB, false>(dre, X(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
           ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
           if (!ok) break;
           tc_fence_after();
-          plane_half<2, RB, false>(dre, XLines(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          plane_half<2, RB, false>(dre, X(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
           if (last) {
             if (elect_one()) mma2_commit_both(smem_u32(&accf_bar[0]));
             __syncwarp();
@@ -1304,10 +1317,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
             if (!ok) break;
             tc_fence_after();
           }
-          plane_half<2, RB, true>(dim, XLines(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
+          plane_half<2, RB, true>(dim, X(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
           if (elect_one()) mma2_commit_both(smem_u32(&empty_bar[s0]));
           __syncwarp();
-          plane_half<2, RB, true>(dim, XLines(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
+          plane_half<2, RB, true>(dim, X(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
           if (elect_one()) {
             mma2_commit_both(smem_u32(&empty_bar[s1]));
             if (last) mma2_commit_both(smem_u32(&accf_bar[1]));
@@ -1337,7 +1350,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(F32 ? PTHREADS_F32 :
       asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
       const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
       split_tiles<QST>(
-          lane, total, raw_bar, &s_abort, [&](int st) { split_line(psm + st * QSTAGE, tid - 384, unsplit); },
+          lane, total, raw_bar, &s_abort, 
+          [&](int st) {
+            if constexpr (STRIDED)
+              split_points(psm + st * QSTAGE, warp - 12, lane, unsplit);
+            else
+              split_line(psm + st * QSTAGE, tid - 384, unsplit);
+          },
           [&](int st) { mbar_arrive_cluster(full0 + 8u * (uint32_t)st); });
     }
   }
@@ -1428,15 +1447,23 @@ bool pair_pass(int N, int64_t ncols, int sms) { return pair_length(N) && 4 * pai
 
 using PKernel = void (*)(const DenseArgs, const unsigned char*, int*, const CUtensorMap);
 using QKernel = void (*)(const DenseArgs, int*, const CUtensorMap, const CUtensorMap);
-template <bool F32>
+template <int IN>
 struct QVariant {
-  static constexpr QKernel grad() {
-    if constexpr (F32) return nullptr;
-    else return plane_pair_kernel<kOutGrad, false>;
+  static constexpr QKernel planes() {  // strided lines: no chain
+    if constexpr (IN == kInStrided) return nullptr;
+    else return plane_pair_kernel<kOutPlanes, IN>;
   }
-  static constexpr QKernel fn[kPOuts] = {plane_pair_kernel<kOutPlanes, F32>, plane_pair_kernel<kOutComplex, F32>,
-                                         plane_pair_kernel<kOutDensity, F32>, plane_pair_kernel<kOutSum, F32>, grad()};
+  static constexpr QKernel grad() {
+    if constexpr (in_fp32(IN)) return nullptr;
+    else return plane_pair_kernel<kOutGrad, IN>;
+  }
+  static constexpr QKernel fn[kPOuts] = {planes(), plane_pair_kernel<kOutComplex, IN>, plane_pair_kernel<kOutDensity, IN>,
+                                         plane_pair_kernel<kOutSum, IN>, grad()};
 };
+QKernel pair_kernel(int out, int in) {
+  return in == kInStrided ? QVariant<kInStrided>::fn[out]
+                          : in == kInF32 ? QVariant<kInF32>::fn[out] : QVariant<kInPlanes>::fn[out];
+}
 template <int RB, bool RES, int IN>
 struct PVariant {
   static constexpr PKernel grad() {
@@ -1528,16 +1555,14 @@ cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided) {
   cudaError_t e = cudaSuccess;
   for (int k = 0; k < kPOuts && e == cudaSuccess; ++k) {
     if (k == kOutGrad && !grad) continue;
-    if (pair_length(N)) {
-      e = cudaFuncSetAttribute((const void*)QVariant<false>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-      if (e == cudaSuccess && QVariant<true>::fn[k])
-        e = cudaFuncSetAttribute((const void*)QVariant<true>::fn[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-    }
-    for (int in : {kInPlanes, kInF32, kInPoints, kInStrided})
-      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && (in != kInPoints || points) &&
-          (in != kInStrided || strided) && single_kernel(N, k, in))
+    for (int in : {kInPlanes, kInF32, kInPoints, kInStrided}) {
+      if ((in == kInPoints && !points) || (in == kInStrided && !strided)) continue;
+      if (e == cudaSuccess && pair_length(N) && in != kInPoints && pair_kernel(k, in))
+        e = cudaFuncSetAttribute((const void*)pair_kernel(k, in), cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
+      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && single_kernel(N, k, in))
         e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
+    }
   }
   return e;
 }
@@ -1590,13 +1615,17 @@ bool plane_pass_splits(int N, int64_t ncols, int sms) {
   return (N <= 128 || pair_pass(N, ncols, sms)) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
 }
 
-// Strided FP32 lines: groups of 64 adjacent lines land by TMA with a point a row
+// Strided FP32 lines: groups of 16 adjacent lines land by TMA with a point a row
 // and are split in place like contiguous ones; the products take them with their
 // rows along the lines, so nothing is transposed.  (The kernel of ffx_tc16.cu
 // loads such lines to registers and stores them transposed: 2^24 points of 64,
 // inner 256, in place 48.7 us, here 36.3; 4.4 M points of 96, inner 192: 32.3 and
-// 20.0; 15.7 M points of 128, inner 256: 92.1 and 53.2.)
-bool plane_pass_strided(int N, int64_t inner) { return (N == 64 || N == 96 || N == 128) && inner % 64 == 0; }
+// 20.0; 15.7 M points of 128, inner 256: 92.1 and 53.2; 22 M points of 256, inner
+// 12288: 232 and 101, inner 48: 225 and 100; 16.8 M points of 512, inner 128: 318
+// and 134.)
+bool plane_pass_strided(int N, int64_t inner, int64_t ncols, int sms) {
+  return inner > 1 && inner % 16 == 0 && (N == 64 || N == 96 || N == 128 || pair_pass(N, ncols, sms));
+}
 
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
   DenseArgs a = args;
@@ -1608,7 +1637,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   const bool pair = pair_pass(a.N, a.ncols, sms);
   const int out = a.out_bf ? (a.grad ? kOutGrad : kOutPlanes)
                            : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
-  const bool strided = plane_pass_strided(a.N, a.inner);
+  const bool strided = plane_pass_strided(a.N, a.inner, a.ncols, sms);
   const int in = strided ? kInStrided : a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
   if (strided && (!f32 || a.out_bf)) return cudaErrorInvalidValue;
   if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
@@ -1633,7 +1662,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     grid *= 2;
     // T's chunks as rows of 128 bytes (stored swizzled)
     if (!row_map(&tmap, Tblk, 64, (int64_t)plane_t_bytes(a.N) / 128, 1, 0, 64, false)) return cudaErrorInvalidValue;
-    return launch_pdl(f32 ? QVariant<true>::fn[out] : QVariant<false>::fn[out], (int)grid,
+    return launch_pdl(pair_kernel(out, in), (int)grid,
                       f32 ? PTHREADS_F32 : PTHREADS, QSMEM, s, a, err, xmap, tmap);
   }
   return launch_pdl(single_kernel(a.N, out, in), (int)grid, f32 ? PTHREADS_F32 : PTHREADS, single_smem(a.N), s, a, Tblk,

@@ -230,7 +230,8 @@ def test_gradient_factors_of_the_last_forward_pass(ffx, dims, lam, batch, fused)
     assert rel_l2(gs, ref) < FIELD_TOL
 
 
-# strided FP32 lines of 64, 96 and 128 points outside a chain: a group of 64
+# strided FP32 lines of 64, 96, 128 points and (on CTA pairs) 256, 384, ...
+# outside a chain: a group of 64
 # lines too few for the last tile, one group per outer block, several, first and
 # middle axes, ensemble sums (one group of realizations and many)
 STRIDED_CASES = [
@@ -241,6 +242,14 @@ STRIDED_CASES = [
     ((32, 96, 64), (6, 4, 3), 3),
     ((128, 32, 32), (11, 4, 3), 5),
     ((32, 128, 192), (3, 30, 4), 2),
+    ((256, 32, 64), (4, 5, 6), 3),
+    ((32, 256, 64), (3, 7, 5), 5),
+    ((384, 64), (9, 5), 61),
+    ((32, 512, 32), (3, 20, 5), 2),
+    ((32, 96, 48), (3, 5, 4), 3),      # groups of 16 lines: tiles over several outer blocks
+    ((32, 128, 16), (3, 5, 4), 1),
+    ((16, 64, 48), (3, 5, 4), 103),
+    ((48, 256, 16), (3, 5, 4), 7),
 ]
 
 
