@@ -411,7 +411,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.bf_plane = plane;
       d.in = nullptr;
     }
-    if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(ax.N, inner, d.ncols, p->sms))))
+    if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(inner))))
       e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
     else if (ax.bf_t[0] && !tm64)
       e = launch_dense_bf16(d, ax.bf_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);

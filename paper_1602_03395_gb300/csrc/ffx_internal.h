@@ -165,7 +165,7 @@ size_t plane_t_bytes(int N);
 // strided FP32 lines
 cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided);
 // whether launch_plane_pass takes FP32 lines whose points are `inner` > 1 apart
-bool plane_pass_strided(int N, int64_t inner, int64_t ncols, int sms);
+bool plane_pass_strided(int64_t inner);
 cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s);
 cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
                                int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s);

@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
   // F32: split in the stages; POINTS: parts with a point a row
   constexpr bool F32 = in_fp32(IN), POINTS = IN == kInPoints || IN == kInStrided;
-  static_assert(RES || IN == kInPlanes, "FP32 and point-row input come with resident T");
+  static_assert(RES || IN == kInPlanes || IN == kInStrided, "the other inputs come with resident T");
   __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], raw_bar[PMAXST], t_bar;
   __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
   __shared__ uint32_t tmem_slot;
@@ -596,7 +596,8 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
   if (warp == 1) tmem_alloc(&tmem_slot, 512);
   if (tid == 0) {
     for (int s = 0; s < NST; ++s) {
-      mbar_init(smem_u32(&full_bar[s]), F32 ? 4 : 1);  // FP32 input: the producer warps
+      // FP32 input: the producer warps, and T's copy if streamed
+      mbar_init(smem_u32(&full_bar[s]), F32 ? (RES ? 4 : 5) : 1);
       mbar_init(smem_u32(&empty_bar[s]), 1);
       mbar_init(smem_u32(&raw_bar[s]), 1);
     }
@@ -643,6 +644,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
           const uint32_t st = stages + (uint32_t)(is * STAGE);
           const uint32_t fb = smem_u32(F32 ? &raw_bar[is] : &full_bar[is]);
           mbar_expect_tx(fb, F32 ? (uint32_t)PX : xbytes + (RES ? 0u : tbytes));
+          if (F32 && !RES) mbar_expect_tx(smem_u32(&full_bar[is]), tbytes);
           // rows: the tile's lines (realization ib's when accumulating); x: the
           // chunk's 64 values; z: the head plane (and the tail plane)
           const int row = (int)(ct * PL + (ACC ? (int64_t)ib * a.outer : 0));
@@ -676,13 +678,14 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
           }
           if (!RES) {
             const int mt = (int)(iw - ct * mtiles);
+            const uint32_t tbar = smem_u32(&full_bar[is]);
             if (RB == TB) {
-              bulk_g2s(st + (uint32_t)PX, Tblk + ((size_t)mt * kchunks + ikc) * TCH, tbytes, fb);
+              bulk_g2s(st + (uint32_t)PX, Tblk + ((size_t)mt * kchunks + ikc) * TCH, tbytes, tbar);
             } else {
               // half of a 128-row block: its head rows, then its tail rows
               const unsigned char* src = Tblk + ((size_t)(mt >> 1) * kchunks + ikc) * ptchunk(TB) + (mt & 1) * TPART;
-              bulk_g2s(st + (uint32_t)PX, src, TPART, fb);
-              if (!unsplit) bulk_g2s(st + (uint32_t)(PX + TPART), src + ppart(TB), TPART, fb);
+              bulk_g2s(st + (uint32_t)PX, src, TPART, tbar);
+              if (!unsplit) bulk_g2s(st + (uint32_t)(PX + TPART), src + ppart(TB), TPART, tbar);
             }
           }
           if (++is == NST) {
@@ -701,7 +704,9 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
         if (RES) mbar_wait_own(smem_u32(&t_bar), 0u, &s_abort);
         for (int q = 0; q < NST; ++q) {
           const int64_t uq = q < is ? u : u - 1;  // stage q's last use
-          if (uq >= 0) mbar_wait_own(smem_u32(F32 ? &raw_bar[q] : &full_bar[q]), (uint32_t)(uq & 1), &s_abort);
+          if (uq < 0) continue;
+          if (F32) mbar_wait_own(smem_u32(&raw_bar[q]), (uint32_t)(uq & 1), &s_abort);
+          if (!F32 || !RES) mbar_wait_own(smem_u32(&full_bar[q]), (uint32_t)(uq & 1), &s_abort);
         }
       }
       __syncwarp();
@@ -772,7 +777,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
       split_tiles<NST>(
           lane, my_items * nb * kchunks, raw_bar, &s_abort,
           [&](int st) {
-            unsigned char* const x = psm + (RB / PKC) * TCH + st * STAGE;
+            unsigned char* const x = psm + (RES ? (RB / PKC) * TCH : 0) + st * STAGE;
             if constexpr (IN == kInStrided)
               split_points(x, warp - 12, lane, unsplit);
             else
@@ -1494,6 +1499,7 @@ PKernel single_kernel(int N, int out, int in) {
       case kInStrided: return resident_kernel<kInStrided>(N, out);
       default: return resident_kernel<kInPlanes>(N, out);
     }
+  if (in == kInStrided) return N == 192 ? PVariant<96, false, kInStrided>::fn[out] : PVariant<64, false, kInStrided>::fn[out];
   return N == 192 ? PVariant<96, false, kInPlanes>::fn[out] : PVariant<64, false, kInPlanes>::fn[out];
 }
 int single_rows(int N) { return N <= 128 ? N : N == 192 ? 96 : 64; }  // outputs per item
@@ -1559,7 +1565,7 @@ cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided) {
       if ((in == kInPoints && !points) || (in == kInStrided && !strided)) continue;
       if (e == cudaSuccess && pair_length(N) && in != kInPoints && pair_kernel(k, in))
         e = cudaFuncSetAttribute((const void*)pair_kernel(k, in), cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-      if (e == cudaSuccess && (in == kInPlanes || N <= 128) && single_kernel(N, k, in))
+      if (e == cudaSuccess && (in == kInPlanes || in == kInStrided || N <= 128) && single_kernel(N, k, in))
         e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
     }
@@ -1623,9 +1629,7 @@ bool plane_pass_splits(int N, int64_t ncols, int sms) {
 // 20.0; 15.7 M points of 128, inner 256: 92.1 and 53.2; 22 M points of 256, inner
 // 12288: 232 and 101, inner 48: 225 and 100; 16.8 M points of 512, inner 128: 318
 // and 134.)
-bool plane_pass_strided(int N, int64_t inner, int64_t ncols, int sms) {
-  return inner > 1 && inner % 16 == 0 && (N == 64 || N == 96 || N == 128 || pair_pass(N, ncols, sms));
-}
+bool plane_pass_strided(int64_t inner) { return inner > 1 && inner % 16 == 0; }
 
 cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, int* err, int sms, cudaStream_t s) {
   DenseArgs a = args;
@@ -1637,11 +1641,11 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   const bool pair = pair_pass(a.N, a.ncols, sms);
   const int out = a.out_bf ? (a.grad ? kOutGrad : kOutPlanes)
                            : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
-  const bool strided = plane_pass_strided(a.N, a.inner, a.ncols, sms);
+  const bool strided = plane_pass_strided(a.inner);
   const int in = strided ? kInStrided : a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
   if (strided && (!f32 || a.out_bf)) return cudaErrorInvalidValue;
   if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
-  if ((a.inner != 1 && !strided) || ((f32 || a.in_points) && !pair && a.N > 128) || (a.in_points && pair))
+  if ((a.inner != 1 && !strided) || ((f32 || a.in_points) && !pair && !strided && a.N > 128) || (a.in_points && pair))
     return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines; or a square

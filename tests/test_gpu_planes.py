@@ -250,6 +250,10 @@ STRIDED_CASES = [
     ((32, 128, 16), (3, 5, 4), 1),
     ((16, 64, 48), (3, 5, 4), 103),
     ((48, 256, 16), (3, 5, 4), 7),
+    ((192, 32, 48), (3, 5, 4), 2),     # T streamed: 192, and few lines of long ones
+    ((32, 192, 16), (3, 5, 4), 3),
+    ((256, 48), (9, 5), 3),
+    ((1024, 32), (9, 5), 2),
 ]
 
 
