@@ -397,7 +397,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.in_points = io->points;
       d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
       d.oouter = outer / d.oinner;
-    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_splits(ax.N, d.ncols, p->sms)) {
+    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_fp32(ax.N, d.ncols, p->sms)) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
       // cores' layout instead of converting them on the way

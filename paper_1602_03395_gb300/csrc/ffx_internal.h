@@ -169,9 +169,10 @@ bool plane_pass_strided(int64_t inner);
 cudaError_t launch_plane_build_t(const float2* T, unsigned char* Tblk, int N, cudaStream_t s);
 cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_shared, int64_t M, uint32_t* planes,
                                int64_t n, int64_t plane, int unsplit, int sms, cudaStream_t s);
-// whether the pass takes FP32 lines as they are (DenseArgs::in) and splits them
-// itself: every length but 192, with an item for every block (pair of blocks)
-// that runs at once
+// whether the pass takes contiguous FP32 lines as they are (DenseArgs::in) and
+// splits them itself: with an item for every block (pair of blocks) that runs at
+// once; _splits: as a chain's first pass too, which 192 points are not
+bool plane_pass_fp32(int N, int64_t ncols, int sms);
 bool plane_pass_splits(int N, int64_t ncols, int sms);
 // work items of a pass over ncols lines, and how many run at once
 int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once);

@@ -576,7 +576,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
   unsigned char* const psm = psm_raw + ((1024u - (smem_u32(psm_raw) & 1023u)) & 1023u);
   // F32: split in the stages; POINTS: parts with a point a row
   constexpr bool F32 = in_fp32(IN), POINTS = IN == kInPoints || IN == kInStrided;
-  static_assert(RES || IN == kInPlanes || IN == kInStrided, "the other inputs come with resident T");
+  static_assert(RES || IN != kInPoints, "a square pass's parts come with resident T");
   __shared__ __align__(8) uint64_t full_bar[PMAXST], empty_bar[PMAXST], raw_bar[PMAXST], t_bar;
   __shared__ __align__(8) uint64_t accf_bar[2 * NBUF], acce_bar[2 * NBUF], done_bar;
   __shared__ uint32_t tmem_slot;
@@ -1475,8 +1475,8 @@ struct PVariant {
     if constexpr (!RES || in_fp32(IN)) return nullptr;
     else return plane_pass_kernel<RB, RES, kOutGrad, IN>;
   }
-  static constexpr PKernel planes() {  // strided lines: no chain
-    if constexpr (IN == kInStrided) return nullptr;
+  static constexpr PKernel planes() {  // strided lines, FP32 lines of 192: no chain
+    if constexpr (IN == kInStrided || (IN == kInF32 && !RES)) return nullptr;
     else return plane_pass_kernel<RB, RES, kOutPlanes, IN>;
   }
   static constexpr PKernel fn[kPOuts] = {
@@ -1499,6 +1499,7 @@ PKernel single_kernel(int N, int out, int in) {
       case kInStrided: return resident_kernel<kInStrided>(N, out);
       default: return resident_kernel<kInPlanes>(N, out);
     }
+  if (in == kInF32) return PVariant<96, false, kInF32>::fn[out];
   if (in == kInStrided) return N == 192 ? PVariant<96, false, kInStrided>::fn[out] : PVariant<64, false, kInStrided>::fn[out];
   return N == 192 ? PVariant<96, false, kInPlanes>::fn[out] : PVariant<64, false, kInPlanes>::fn[out];
 }
@@ -1565,7 +1566,8 @@ cudaError_t plane_pass_prepare(int N, bool points, bool grad, bool strided) {
       if ((in == kInPoints && !points) || (in == kInStrided && !strided)) continue;
       if (e == cudaSuccess && pair_length(N) && in != kInPoints && pair_kernel(k, in))
         e = cudaFuncSetAttribute((const void*)pair_kernel(k, in), cudaFuncAttributeMaxDynamicSharedMemorySize, QSMEM);
-      if (e == cudaSuccess && (in == kInPlanes || in == kInStrided || N <= 128) && single_kernel(N, k, in))
+      if (e == cudaSuccess && (in == kInPlanes || in == kInStrided || N <= 128 || (in == kInF32 && N == 192)) &&
+          single_kernel(N, k, in))
         e = cudaFuncSetAttribute((const void*)single_kernel(N, k, in), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  single_smem(N));
     }
@@ -1616,10 +1618,11 @@ int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
   return pair ? pair_items(N, ncols) : (ncols + PL - 1) / PL * (N / single_rows(N));
 }
 
-bool plane_pass_splits(int N, int64_t ncols, int sms) {
+bool plane_pass_fp32(int N, int64_t ncols, int sms) {
   int64_t at_once;
-  return (N <= 128 || pair_pass(N, ncols, sms)) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
+  return (N <= 128 || N == 192 || pair_pass(N, ncols, sms)) && plane_pass_tiles(N, ncols, sms, &at_once) >= at_once;
 }
+bool plane_pass_splits(int N, int64_t ncols, int sms) { return N != 192 && plane_pass_fp32(N, ncols, sms); }
 
 // Strided FP32 lines: groups of 16 adjacent lines land by TMA with a point a row
 // and are split in place like contiguous ones; the products take them with their
@@ -1645,7 +1648,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
   const int in = strided ? kInStrided : a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
   if (strided && (!f32 || a.out_bf)) return cudaErrorInvalidValue;
   if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
-  if ((a.inner != 1 && !strided) || ((f32 || a.in_points) && !pair && !strided && a.N > 128) || (a.in_points && pair))
+  if ((a.inner != 1 && !strided) || (f32 && !pair && !strided && a.N > 128 && a.N != 192) || (a.in_points && a.N > 128))
     return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines; or a square

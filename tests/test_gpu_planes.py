@@ -81,6 +81,8 @@ FP32_CASES = [
     ((64, 128), (5, 9), 310),
     ((96,), (5,), 19537),
     ((128,), (7,), 20001),
+    ((192,), (7,), 9801),              # T streamed: a last tile of 73 lines
+    ((48, 48, 192), (3, 4, 5), 5),
 ]
 
 
