@@ -119,7 +119,7 @@ struct Axis {
   float2* TH = nullptr;  // its adjoint
   int grid_dense = 0, grid_dense_small = 0;
   unsigned char* tc_t[2] = {nullptr, nullptr};  // split tensor-core operands of T, T^H (ffx_tc.cu)
-  unsigned char* bf_t[2] = {nullptr, nullptr};  // FFX_TC_BF16: the BF16 operand blocks (ffx_tc16.cu)
+  unsigned char* bf_th = nullptr;  // FFX_TC_BF16: T^H's BF16 operand blocks (ffx_tc16.cu)
   unsigned char* pl_t[2] = {nullptr, nullptr};  // ... and those of the passes over planes (ffx_planes.cu)
   unsigned char* ft_ts = nullptr;                 // N = 64: T's row-block slices for the fused tensor-core launch
   float2* img[2] = {nullptr, nullptr};                      // lines <= 64: shared-memory images of T, T^H
@@ -413,8 +413,8 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
     }
     if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(inner))))
       e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
-    else if (ax.bf_t[0] && !tm64)
-      e = launch_dense_bf16(d, ax.bf_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
+    else if (ax.bf_th && adjoint && !tm64 && grad)
+      e = launch_dense_bf16(d, ax.bf_th, p->dev_err, (int)grid, stream);
     else
       e = launch_dense_tc(d, ax.tc_t[adjoint ? 1 : 0], p->dev_err, (int)grid, stream);
   } else if (io) {
@@ -1425,7 +1425,7 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
     for (int j = 0; j < ndim; ++j)
       if (dense_tc_supported(p->axis[j].N) && p->axis[j].T && (form == FFX_FORM_AUTO || form == FFX_FORM_TC)) {
         tbytes += 2 * dense_tc_t_bytes(p->axis[j].N) + (p->axis[j].N == 64 ? fused_tc_slice_bytes() : 0);
-        if (bf16_ops && dense_bf16_supported(p->axis[j].N)) tbytes += 2 * dense_bf16_t_bytes(p->axis[j].N);
+        if (bf16_ops && dense_bf16_supported(p->axis[j].N)) tbytes += dense_bf16_t_bytes(p->axis[j].N);
         if (bf16_ops && plane_pass_supported(p->axis[j].N)) tbytes += 2 * plane_t_bytes(p->axis[j].N);
       }
     e = cudaMalloc(&p->tc_mem, tbytes);
@@ -1466,12 +1466,9 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           e = launch_fused_tc_slices(ax.T, ax.ft_ts, s);
         }
         if (e == cudaSuccess && bf16_ops && dense_bf16_supported(ax.N)) {
-          for (int q = 0; q < 2; ++q) {
-            ax.bf_t[q] = tcur;
-            tcur += dense_bf16_t_bytes(ax.N);
-          }
-          e = launch_bf16_build_t(ax.T, ax.bf_t[0], ax.N, s);
-          if (e == cudaSuccess) e = launch_bf16_build_t(ax.TH, ax.bf_t[1], ax.N, s);
+          ax.bf_th = tcur;
+          tcur += dense_bf16_t_bytes(ax.N);
+          e = launch_bf16_build_t(ax.TH, ax.bf_th, ax.N, s);
           if (e == cudaSuccess) e = dense_bf16_prepare();
         }
         if (e == cudaSuccess && bf16_ops && plane_pass_supported(ax.N)) {
@@ -1630,7 +1627,7 @@ int ffx_plan_tc_bf16(ffx_plan_t p) {
   if (!p) return -1;
   if (p->many) return many_bf16(p->many) ? 1 : 0;
   for (int j = 0; j < p->ndim; ++j)
-    if (p->axis[j].bf_t[0]) return 1;
+    if (p->axis[j].bf_th) return 1;
   return 0;
 }
 

@@ -21,31 +21,31 @@
 // operands; the products run at the kind::f16 rate.  The FP32 input of a chunk
 // (32 KB) is exactly the size of its BF16 head and tail parts, so it lands in
 // the stage itself, each thread's bytes where its own BF16 rows go, and is
-// converted in place: no separate input ring, three 64 KB stages.
+// converted in place: no separate input ring.  Two 64 KB stages, and two 16 KB
+// slots of gradient factors.
 //
 // Kernel: one persistent block of 544 threads per SM, warp-specialised.
 //  * warps 0-7 (producers), per K chunk of 64 real K, once the products of
-//    the chunk three back have freed its stage: thread 0 starts a bulk copy of
+//    the chunk two back have freed its stage: thread 0 starts a bulk copy of
 //    the pre-split T chunk (head and tail, 128 rows x 64 K each, already in
 //    the tensor cores' K-major no-swizzle core-matrix order) on the stage's
 //    "copy" barrier, and every producer thread copies its share of the input
-//    into the stage (cp.async); two chunks later the thread converts its share
-//    into BF16 heads and tails in place (16-byte core-matrix rows, conflict
+//    into the stage (cp.async); a chunk later the thread converts its share, times
+//    2 grad, into BF16 heads and tails in place (16-byte core-matrix rows, conflict
 //    free) and arrives on "full".
 //  * warp 8 (MMA; one elected lane issues): waits "copy" and "full", issues 4 K-steps x 3 products of
 //    tcgen05.mma kind::f16 (M = 128 lines, N = 128 rows, K = 16) into one of
 //    two accumulator pairs; tcgen05.commit frees the stage ("empty") and,
 //    after an item's last chunk, hands the accumulator on ("acc_full").
 //  * warps 9-16 (epilogue): read their 32-lane quarter of the accumulators, two
-//    warps on every other 16 columns of one,
-//    store complex64 or |.|^2 (or add |.|^2 over the batch in shared memory),
-//    and arrive on "acc_empty".
+//    warps on every other 16 columns of one, store complex64, and arrive on
+//    "acc_empty".
 // Items are (128 lines, 128 real rows) of the output, numbered row block
 // fastest so that blocks running together share the lines' inputs in L2.
 //
-// This kernel takes FP32 input (strided lines, backward passes); passes over
-// BF16 planes run in ffx_planes.cu, and the many-instance phases below have
-// their own plane input and output: interleaved (re, im) pairs, transposed
+// This kernel takes the first adjoint pass of a backward call outside a chain,
+// whose input element is 2 grad * psi; every other pass runs in ffx_planes.cu, and
+// the many-instance phases below have their own plane input and output: interleaved (re, im) pairs, transposed
 // between the passes (point n' of line rho of R lines at n' R + rho), read as
 // one TMA tile per chunk into the tensor cores' 128-byte-swizzled layout.
 // Every wait is bounded; one that runs out sets the block's abort flag, the
@@ -70,7 +70,7 @@ using namespace tc;
 constexpr int BL = 128;                      // lines per item = MMA M = tensor-memory lanes
 constexpr int BR = 128;                      // real output rows per item = MMA N
 constexpr int BKC = 64;                      // real K per chunk: four K-steps of 16
-constexpr int BSMAX = 3;  // stages: 3, or 2 in backward launches (their gradient ring)
+constexpr int BSTAGES = 2;  // and a gradient ring of as many slots
 constexpr int BCORE = 128;                   // bytes between core matrices along K
 constexpr int BSBO = (BKC / 8) * BCORE;      // 1024: between 8-row groups
 constexpr int BPART = BR * BKC * 2;          // 16 KB: one split part of a chunk (T or X)
@@ -87,17 +87,12 @@ constexpr int BTHREADS = BPROD + 32 + 32 * BEPIW;  // 544
 constexpr int BMMA_WARP = BPROD / 32;              // warp 8; warps 9-16 are the epilogue
 constexpr int BITEMS = BL * (BKC / 8) / BPROD;  // 4 core-matrix rows (8 real K) per producer thread per chunk
 constexpr int BGRAD_CHUNK = BPROD * BITEMS * 16;  // 16 KB: a chunk's gradient factors (backward passes)
-constexpr int BEXTRA = (BR / 2) * BL * 4;       // accumulating launches: |.|^2 over the batch, [row][line]
 constexpr int BCOLS = 4 * BR;                   // two accumulator pairs: all 512 columns
-__host__ __device__ constexpr int bstages(bool grad, bool acc) { return grad ? 2 : 3; }
-// stages, then the |.|^2 sums of accumulating launches or the gradient ring
-__host__ __device__ constexpr int bsmem(bool grad, bool acc) {
-  return bstages(grad, acc) * BSTAGE + (acc ? BEXTRA : 0) + (grad ? bstages(grad, acc) * BGRAD_CHUNK : 0);
-}
+constexpr int BSMEM = BSTAGES * (BSTAGE + BGRAD_CHUNK);  // stages, then the gradient ring
 // a launch's dynamic shared memory: 1 KB more, to start the stages on a
 // 1024-byte boundary (the swizzled tiles' atoms)
-__host__ __device__ constexpr int bsmem_launch(bool grad, bool acc) { return bsmem(grad, acc) + 1024; }
-static_assert(bsmem_launch(false, true) <= 227 * 1024 && bsmem_launch(true, false) <= 227 * 1024, "shared memory");
+constexpr int BSMEM_LAUNCH = BSMEM + 1024;
+static_assert(BSMEM_LAUNCH <= 227 * 1024, "shared memory");
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int bytes) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
@@ -115,19 +110,14 @@ __host__ __device__ __forceinline__ int brow_count(int N, int mt) {
   return left < BR ? left : BR;
 }
 
-// Line c of the pass (realization b when accumulating): offset of its first
-// point, or -1 past the end; br = its realization.
-__device__ __forceinline__ long long bline(const DenseArgs& a, int64_t c, int b, int& br) {
+// Line c of the pass: offset of its first point, or -1 past the end; br = its
+// realization.
+__device__ __forceinline__ long long bline(const DenseArgs& a, int64_t c, int& br) {
   br = 0;
   if (c >= a.ncols) return -1;
-  int64_t bo = c / a.inner;
+  const int64_t bo = c / a.inner;
   const int64_t i = c - bo * a.inner;
-  if (a.acc) {
-    br = b;
-    bo += (int64_t)b * a.outer;
-  } else {
-    br = (int)(c / (a.outer * a.inner));
-  }
+  br = (int)(c / (a.outer * a.inner));
   return bo * (int64_t)a.N * a.inner + i;
 }
 
@@ -155,24 +145,23 @@ __device__ __forceinline__ void split8(const float* v, uint4& hi, uint4& lo, boo
 }
 
 // How a chunk's input reaches the stage: per-thread cp.async that lands each
-// thread's points on the bytes of its own BF16 rows (the uniform kernel, whose
-// strided lines and backward passes take this way; every thread converts its
-// own bytes, with no barrier); or, in many-instance phases, FP32 contiguous
+// thread's points on the bytes of its own BF16 rows (the uniform kernel; every
+// thread converts its own bytes, with no barrier); or, in many-instance phases, FP32 contiguous
 // lines as a TMA tile (two 128 x 32-float boxes with 128-byte swizzle), or BF16
 // planes, the head and tail rows as one TMA tile.
 enum BLoad { kTmaContiguous = 0, kInPlace = 1, kTmaPlanes = 2 };
 
-// FULL: every row block has BR rows (2N a multiple of 128).  GRAD: backward
-// passes, whose input element is 2 grad * psi (the factors come through their
-// own ring; two stages).  ACC: the batch's |.|^2 summed in shared memory.
-template <bool FULL, bool GRAD, bool ACC>
+// The first adjoint pass of a backward call outside a chain: its input element
+// is 2 grad * psi, the factors coming through their own ring.  (All other BF16
+// passes are ffx_planes.cu's.)  FULL: every row block has BR rows (2N a multiple
+// of 128).
+template <bool FULL>
 __global__ void __launch_bounds__(BTHREADS, 1)
     dense_bf16_kernel(const DenseArgs a, const unsigned char* __restrict__ Tblk, int* err) {
-  constexpr int BSTAGES = bstages(GRAD, ACC);
   extern __shared__ __align__(1024) unsigned char bsm_raw[];
   // the stages on a 1024-byte boundary (the launch adds 1 KB for it)
   unsigned char* const bsm = bsm_raw + ((1024u - (smem_u32(bsm_raw) & 1023u)) & 1023u);
-  __shared__ __align__(8) uint64_t full_bar[BSMAX], empty_bar[BSMAX], copy_bar[BSMAX];
+  __shared__ __align__(8) uint64_t full_bar[BSTAGES], empty_bar[BSTAGES], copy_bar[BSTAGES];
   __shared__ __align__(8) uint64_t accf_bar[2], acce_bar[2], done_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int s_abort;
@@ -185,7 +174,6 @@ __global__ void __launch_bounds__(BTHREADS, 1)
   const int64_t items = ((a.ncols + BL - 1) / BL) * mtiles;
   const int64_t my_items = (items - blockIdx.x + gridDim.x - 1) / gridDim.x;
   if (my_items <= 0) return;
-  const int nb = ACC ? (int)a.batch : 1;
   const bool unsplit = a.unsplit != 0;
 
   if (warp == BMMA_WARP) tmem_alloc(&tmem_slot, BCOLS);
@@ -214,7 +202,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     const int t = tid;
     const int64_t inner = a.inner;
     const bool contiguous = (inner == 1);
-    const int64_t total = my_items * nb * kchunks;
+    const int64_t total = my_items * kchunks;
     unsigned char* graw = bsm + BSTAGES * BSTAGE;  // gradient factors, one slot per stage (backward)
     // this thread's 4 core-matrix rows of a chunk: line n_i, K group kp_i
     // (contiguous: two lines, n_0 = n_1 and n_2 = n_3; strided: one), at byte
@@ -230,17 +218,16 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     // the input tile), on the stage's "copy" barrier; in place, every thread
     // copies its points (item i's first two complex points onto its head row
     // X_hi + off_i, the next two onto its tail row X_lo + off_i).  The
-    // chunk's position (item iw, realization ib, K chunk ikc) advances
-    // incrementally; the lines' offsets are computed once per item and
-    // realization.
+    // chunk's position (item iw, K chunk ikc) advances incrementally; the lines'
+    // offsets are computed once per item.
     int64_t ci = 0, iw = blockIdx.x;
-    int ib = 0, ikc = 0, is = 0;
+    int ikc = 0, is = 0;
     long long ilb[2] = {-1, -1};
     int ibr[2] = {0, 0};
     bool lines_ok = false;
-    int last_u[BSMAX];
+    int last_u[BSTAGES];
 #pragma unroll
-    for (int q = 0; q < BSMAX; ++q) last_u[q] = -1;
+    for (int q = 0; q < BSTAGES; ++q) last_u[q] = -1;
     auto issue = [&]() -> bool {
       if (ci < total) {
         const int64_t u = ci / BSTAGES;
@@ -269,8 +256,8 @@ __global__ void __launch_bounds__(BTHREADS, 1)
           last_u[is] = (int)(u & 1);
         }
         if (!lines_ok) {
-          ilb[0] = bline(a, ct * BL + item_line(0), ib, ibr[0]);
-          if (contiguous) ilb[1] = bline(a, ct * BL + item_line(2), ib, ibr[1]);
+          ilb[0] = bline(a, ct * BL + item_line(0), ibr[0]);
+          if (contiguous) ilb[1] = bline(a, ct * BL + item_line(2), ibr[1]);
           lines_ok = true;
         }
         const uint32_t gdst0 = smem_u32(graw + is * BGRAD_CHUNK) + (uint32_t)t * 16;
@@ -298,7 +285,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
                         valid ? 8 : 0);
             }
           }
-          if (GRAD) {
+          {
             const int64_t gaddr = valid && a.grad_shared ? addr - (int64_t)ibr[li] * a.M : addr;
             const uint32_t gd = gdst0 + (uint32_t)(i * BPROD * 16);
 #pragma unroll
@@ -312,10 +299,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         if (++ikc == kchunks) {
           ikc = 0;
           lines_ok = false;
-          if (++ib == nb) {
-            ib = 0;
-            iw += gridDim.x;
-          }
+          iw += gridDim.x;
         }
       } else {
         asm volatile("cp.async.commit_group;" ::: "memory");  // an empty group past the end keeps the count
@@ -345,7 +329,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       }
 #pragma unroll
       for (int i = 0; i < BITEMS; ++i) {
-        if (GRAD) {
+        {
           // the input element is 2 grad * psi
           const float4 g = gs[i * BPROD];
           const float g4[4] = {2.f * g.x, 2.f * g.y, 2.f * g.z, 2.f * g.w};
@@ -370,7 +354,7 @@ __global__ void __launch_bounds__(BTHREADS, 1)
         if (last_u[q] >= 0) mbar_wait_own(smem_u32(&copy_bar[q]), (uint32_t)last_u[q], &s_abort);
   } else if (warp == BMMA_WARP) {
     // ---------------- products: the whole warp, one elected lane issuing ----------------
-    int64_t sub = 0, u = 0;
+    int64_t u = 0;
     int s = 0;
     bool ok = true;
     // descriptor words of both operands' core matrices (see mma_lo)
@@ -381,46 +365,44 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       // whole row blocks: X_hi against [T_hi; T_lo] (the T chunk's 256 rows,
       // head rows then tail rows) in one N = 256 product into the adjacent
       // accumulators [d1 | d2] -- the operand X_hi is read once for both
-      for (int b = 0; ok && b < nb; ++b, ++sub) {
-        const int buf = (int)(sub & 1);
-        const int64_t v = sub >> 1;
-        ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
+      const int buf = (int)(it & 1);
+      const int64_t v = it >> 1;
+      ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
+      if (!ok) break;
+      tc_fence_after();
+      const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
+#pragma unroll 1
+      for (int kc = 0; kc < kchunks; ++kc) {
+        ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
+             mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
         if (!ok) break;
         tc_fence_after();
-        const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
-#pragma unroll 1
-        for (int kc = 0; kc < kchunks; ++kc) {
-          ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-               mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
-          if (!ok) break;
-          tc_fence_after();
-          const uint32_t th = ((smem_base + (uint32_t)(s * BSTAGE)) >> 4) | lo_core, tl = th + BPART / 16;
-          const uint32_t xh = th + BTCHUNK / 16, xl = xh + BPART / 16;
+        const uint32_t th = ((smem_base + (uint32_t)(s * BSTAGE)) >> 4) | lo_core, tl = th + BPART / 16;
+        const uint32_t xh = th + BTCHUNK / 16, xl = xh + BPART / 16;
 #pragma unroll
-          for (uint32_t ks = 0; ks < BKC / 16; ++ks) {
-            const uint32_t o = ks * (2 * BCORE / 16);
-            const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
-            if (unsplit) {
-              mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
+        for (uint32_t ks = 0; ks < BKC / 16; ++ks) {
+          const uint32_t o = ks * (2 * BCORE / 16);
+          const uint32_t more = (kc == 0 && ks == 0) ? 0u : 1u;
+          if (unsplit) {
+            mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
+          } else {
+            if (FULL) {
+              mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc_bf16(BL, 2 * BR), more);
             } else {
-              if (FULL) {
-                mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc_bf16(BL, 2 * BR), more);
-              } else {
-                mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
-                mma_lo<hi_core, hi_core>(d2, xh + o, tl + o, idesc, more);
-              }
-              mma_lo<hi_core, hi_core>(d2, xl + o, th + o, idesc, 1u);
+              mma_lo<hi_core, hi_core>(d1, xh + o, th + o, idesc, more);
+              mma_lo<hi_core, hi_core>(d2, xh + o, tl + o, idesc, more);
             }
+            mma_lo<hi_core, hi_core>(d2, xl + o, th + o, idesc, 1u);
           }
-          if (elect_one()) {
-            mma_commit(smem_u32(&empty_bar[s]));
-            if (kc == kchunks - 1) mma_commit(smem_u32(&accf_bar[buf]));
-          }
-          __syncwarp();
-          if (++s == BSTAGES) {
-            s = 0;
-            ++u;
-          }
+        }
+        if (elect_one()) {
+          mma_commit(smem_u32(&empty_bar[s]));
+          if (kc == kchunks - 1) mma_commit(smem_u32(&accf_bar[buf]));
+        }
+        __syncwarp();
+        if (++s == BSTAGES) {
+          s = 0;
+          ++u;
         }
       }
     }
@@ -435,11 +417,6 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     const int r = q * 32 + lane;                             // line within the item
     const int64_t inner = a.inner;
     const bool contiguous = (inner == 1);
-    float* racc = reinterpret_cast<float*>(bsm + BSTAGES * BSTAGE);  // accumulating launches only
-    if (ACC)
-      for (int j0 = j_first; j0 < BR; j0 += 32)
-        for (int m = 0; m < 8; ++m) racc[(j0 / 2 + m) * BL + r] = 0.f;
-    int64_t sub = 0;
     bool ok = true;
     for (int64_t it = 0; ok && it < my_items; ++it) {
       const int64_t w = blockIdx.x + it * gridDim.x;
@@ -447,81 +424,48 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       const int mt = (int)(w % mtiles);
       const int nbase = mt * (BR / 2);
       const int rows = FULL ? BR : brow_count(N, mt);
-      for (int b = 0; b < nb; ++b, ++sub) {
-        const int buf = (int)(sub & 1);
-        const int64_t v = sub >> 1;
-        // lane 0 polls; the outcome is the warp's (its tensor-memory loads need the whole warp)
-        bool got = true;
-        if (lane == 0) got = mbar_wait(smem_u32(&accf_bar[buf]), (uint32_t)(v & 1), &s_abort);
-        ok = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
-        if (!ok) break;
-        tc_fence_after();
-        int br;
-        const long long base = bline(a, ct * BL + r, b, br);
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BR);
-        uint32_t x[16], z[16];
-        tmem_ld16(taddr + (uint32_t)j_first, x);
-        tmem_ld16(taddr + (uint32_t)(BR + j_first), z);  // unsplit: not written, not used
+      const int buf = (int)(it & 1);
+      const int64_t v = it >> 1;
+      // lane 0 polls; the outcome is the warp's (its tensor-memory loads need the whole warp)
+      bool got = true;
+      if (lane == 0) got = mbar_wait(smem_u32(&accf_bar[buf]), (uint32_t)(v & 1), &s_abort);
+      ok = __shfl_sync(0xffffffffu, got ? 1 : 0, 0) != 0;
+      if (!ok) break;
+      tc_fence_after();
+      int br;
+      const long long base = bline(a, ct * BL + r, br);
+      const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(buf * 2 * BR);
+      uint32_t x[16], z[16];
+      tmem_ld16(taddr + (uint32_t)j_first, x);
+      tmem_ld16(taddr + (uint32_t)(BR + j_first), z);  // unsplit: not written, not used
 #pragma unroll 1
-        for (int j0 = j_first; j0 < rows; j0 += 32) {
-          tmem_wait_ld();
-          float y[16];
+      for (int j0 = j_first; j0 < rows; j0 += 32) {
+        tmem_wait_ld();
+        float y[16];
 #pragma unroll
-          for (int m = 0; m < 16; ++m)
-            y[m] = unsplit ? __uint_as_float(x[m]) : __uint_as_float(x[m]) + __uint_as_float(z[m]);
-          if (j0 + 32 < rows) {
-            // the next columns, in flight while these are written
-            tmem_ld16(taddr + (uint32_t)(j0 + 32), x);
-            tmem_ld16(taddr + (uint32_t)(BR + j0 + 32), z);
-          }
-          const int n0 = nbase + j0 / 2;  // complex outputs n0 .. n0 + 7 of this line
-          if (ACC) {
-#pragma unroll
-            for (int m = 0; m < 8; ++m)
-              racc[(j0 / 2 + m) * BL + r] += y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
-          } else if (base >= 0) {
-            if (a.out_c) {
-              if (contiguous) {
-                float4* o = reinterpret_cast<float4*>(a.out_c + base + n0);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) o[m] = make_float4(y[4 * m], y[4 * m + 1], y[4 * m + 2], y[4 * m + 3]);
-              } else {
-#pragma unroll
-                for (int m = 0; m < 8; ++m) a.out_c[base + (int64_t)(n0 + m) * inner] = make_float2(y[2 * m], y[2 * m + 1]);
-              }
-            } else {
-              float dd[8];
-#pragma unroll
-              for (int m = 0; m < 8; ++m) dd[m] = y[2 * m] * y[2 * m] + y[2 * m + 1] * y[2 * m + 1];
-              if (contiguous) {
-                float4* o = reinterpret_cast<float4*>(a.out_d + base + n0);
-                o[0] = make_float4(dd[0], dd[1], dd[2], dd[3]);
-                o[1] = make_float4(dd[4], dd[5], dd[6], dd[7]);
-              } else {
-#pragma unroll
-                for (int m = 0; m < 8; ++m) a.out_d[base + (int64_t)(n0 + m) * inner] = dd[m];
-              }
-            }
-          }
-          __syncwarp();  // the next columns are read by the whole warp
+        for (int m = 0; m < 16; ++m)
+          y[m] = unsplit ? __uint_as_float(x[m]) : __uint_as_float(x[m]) + __uint_as_float(z[m]);
+        if (j0 + 32 < rows) {
+          // the next columns, in flight while these are written
+          tmem_ld16(taddr + (uint32_t)(j0 + 32), x);
+          tmem_ld16(taddr + (uint32_t)(BR + j0 + 32), z);
         }
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&acce_bar[buf]));
-        if (ACC && b == nb - 1) {
-          if (base >= 0) {
-            const int64_t o0 = base - (int64_t)br * a.M + (int64_t)nbase * inner;
-#pragma unroll 1
-            for (int j0 = j_first; j0 < rows; j0 += 32) {
-              const int m0 = j0 / 2;
+        const int n0 = nbase + j0 / 2;  // complex outputs n0 .. n0 + 7 of this line
+        if (base >= 0) {
+          if (contiguous) {
+            float4* o = reinterpret_cast<float4*>(a.out_c + base + n0);
 #pragma unroll
-              for (int m = m0; m < m0 + 8; ++m) a.out_d[o0 + (int64_t)m * inner] += racc[m * BL + r];
-            }
+            for (int m = 0; m < 4; ++m) o[m] = make_float4(y[4 * m], y[4 * m + 1], y[4 * m + 2], y[4 * m + 3]);
+          } else {
+#pragma unroll
+            for (int m = 0; m < 8; ++m) a.out_c[base + (int64_t)(n0 + m) * inner] = make_float2(y[2 * m], y[2 * m + 1]);
           }
-          for (int j0 = j_first; j0 < BR; j0 += 32)
-            for (int m = 0; m < 8; ++m) racc[(j0 / 2 + m) * BL + r] = 0.f;
         }
+        __syncwarp();  // the next columns are read by the whole warp
       }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acce_bar[buf]));
     }
   }
 
@@ -1189,27 +1133,16 @@ size_t dense_bf16_t_bytes(int N) { return (size_t)((2 * N + BR - 1) / BR) * ((2 
 
 namespace {
 
-// the kernel's variants, indexed [FULL][kind], kind 0 plain, 1 ACC, 2 GRAD
 using BKernel = void (*)(const DenseArgs, const unsigned char*, int*);
-constexpr int kBKinds = 3;
-BKernel bf16_kernel(bool full, int kind) {
-  static const BKernel k[2][kBKinds] = {
-      {dense_bf16_kernel<false, false, false>, dense_bf16_kernel<false, false, true>,
-       dense_bf16_kernel<false, true, false>},
-      {dense_bf16_kernel<true, false, false>, dense_bf16_kernel<true, false, true>,
-       dense_bf16_kernel<true, true, false>}};
-  return k[full ? 1 : 0][kind];
-}
-int bf16_kind_smem(int kind) { return bsmem_launch(kind == 2, kind == 1); }
+BKernel bf16_kernel(bool full) { return full ? dense_bf16_kernel<true> : dense_bf16_kernel<false>; }
 
 }  // namespace
 
 cudaError_t dense_bf16_prepare() {
   cudaError_t e = cudaSuccess;
-  for (int f = 0; f < 2 && e == cudaSuccess; ++f)
-    for (int k = 0; k < kBKinds && e == cudaSuccess; ++k)
-      e = cudaFuncSetAttribute((const void*)bf16_kernel(f == 1, k), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               bf16_kind_smem(k));
+  for (bool f : {false, true})
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute((const void*)bf16_kernel(f), cudaFuncAttributeMaxDynamicSharedMemorySize, BSMEM_LAUNCH);
   return e;
 }
 
@@ -1264,9 +1197,8 @@ bool many_bf16_plane_map(const uint32_t* head, int N, int64_t lines, int64_t pla
 }
 
 cudaError_t launch_dense_bf16(const DenseArgs& a, const unsigned char* Tblk, int* err, int grid, cudaStream_t s) {
-  const bool full = (2 * a.N) % BR == 0;
-  const int kind = a.grad ? 2 : (a.acc ? 1 : 0);  // backward passes never accumulate over the batch
-  bf16_kernel(full, kind)<<<grid, BTHREADS, bf16_kind_smem(kind), s>>>(a, Tblk, err);
+  if (!a.grad || !a.out_c) return cudaErrorInvalidValue;
+  bf16_kernel((2 * a.N) % BR == 0)<<<grid, BTHREADS, BSMEM_LAUNCH, s>>>(a, Tblk, err);
   return cudaGetLastError();
 }
 
