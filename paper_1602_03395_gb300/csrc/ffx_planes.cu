@@ -1,7 +1,7 @@
-// Passes of a BF16 chain (and per-axis BF16 passes over contiguous lines) on
-// the tensor cores: the per-axis map of lines of N points (N a multiple of 32
-// from 64 up to 1024), input as BF16 planes, tcgen05 kind::f16 products
-// accumulated in FP32 in tensor memory.
+// Passes of a BF16 chain and per-axis BF16 passes (contiguous or strided lines)
+// on the tensor cores: the per-axis map of lines of N points (N = 64, 96, 128, 192
+// and multiples of 128 up to 1024), input as BF16 planes or FP32 lines split in
+// shared memory, tcgen05 kind::f16 products accumulated in FP32 in tensor memory.
 //
 // Planes.  A field is a head plane bf16(v) and a tail plane bf16(v - bf16(v)),
 // each 4 bytes a point, in which every 16 consecutive points keep their 16
@@ -28,12 +28,13 @@
 // an item (the kernel this one replaced: 0.095 ms per 256^3 pass).  For N =
 // 64, 96 and 128 (RB = N) T is resident in shared memory and only X streams.
 //
-// One persistent block of 384 threads per SM, warp-specialised.
+// One persistent block of 384 threads per SM (512 with FP32 input: four producer
+// warps split the tiles), warp-specialised.
 //  * warp 0 (one thread): copies.  Per chunk of 32 points, once the products
 //    of the chunk that had its stage have freed it: the X tile (head and tail,
 //    128 lines x 64 values, one 3-D TMA tile with 128-byte swizzle) and, when
 //    streaming, T's chunk (one bulk copy), on the stage's "full" barrier.
-//  * warp 1 (one thread): products.  Per chunk first those of the real
+//  * warp 1 (one elected lane issues): products.  Per chunk first those of the real
 //    accumulators, then those of the imaginary ones: the real half of an item
 //    is complete half a chunk before the imaginary one, and the next item's
 //    real half starts while the imaginary half is read back, so one set of
@@ -817,9 +818,12 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
 //    reads with its lines' points oinner apart (kInPoints).
 // Order of the products: step 1 of item i + 1, then step 2 of item i; of the
 // epilogue: E1 of item i, then E2 of item i - 1: the products of one step hide
-// the other step's epilogue.  Shared memory bounds it: 448 KB of operands and
-// 128 KB of copies, splits and operand stores an item, 5600 clocks against 3072 of
-// products at full rate; HBM 16 bytes a point.
+// the other step's epilogue.  What bounds it is the epilogue warps' chain of both
+// (8500 clocks an item, on a shared-memory port that also serves 448 KB of
+// operands and 256 KB of copies, splits and operand stores: 5600 clocks) against
+// 3072 of products at full rate.  2^24 points: 74 us, 3.6 TB/s of its 16 bytes a
+// point; as two passes 98 us.  (Sixteen epilogue warps, eight a step, with 80
+// registers a thread: 82 us.)
 constexpr int SST = 3;  // stages
 constexpr int SA2 = 4 * 2 * 64 * 128;  // the second operand: 4 parts x 2 squares x 64 rows
 constexpr int ssmem() { return 4 * ptchunk(64) + SA2 + SST * PX + 1024; }

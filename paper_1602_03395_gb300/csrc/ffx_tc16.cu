@@ -1099,7 +1099,7 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
 
 // The split of a backward call's adjoint chain: x = 2 g psi (psi the forward
 // field, g the density gradient: per realization, or one [M] array shared by
-// the batch), into BF16 head and tail planes as bf16_split_kernel does.
+// the batch), into BF16 head and tail planes.
 __global__ void __launch_bounds__(256) bf16_split_grad_kernel(const float4* __restrict__ field,
                                                                const float2* __restrict__ grad, uint2* __restrict__ hi,
                                                                uint2* __restrict__ lo, int64_t n2, int64_t m2,

@@ -69,8 +69,9 @@ def test_plane_passes(ffx, dims, lam, batch):
     assert rel_l2(rough, dens) < UNSPLIT_TOL
 
 
-# passes that fill the chip read their FP32 lines themselves (all lengths but
-# 192): whole and ragged last tiles, chains and single passes, several row blocks
+# passes that fill the chip read their FP32 lines themselves (chains of 192-point
+# lines excepted): whole and ragged last tiles, chains and single passes, several
+# row blocks
 FP32_CASES = [
     ((96, 64, 256), (4, 5, 6), 4),     # chain: 24576 lines of 256
     ((64, 1024), (5, 6), 160),         # chain: 10240 lines of 1024, eight row blocks
