@@ -666,8 +666,8 @@ bool bf16_adjoint_ok(const ffx_plan_s* p) {
 // (plane_square_kernel): 64 points each, the first axis one whose pass keeps T
 // resident, or none (2-D lattices; their ensemble sums stay with the passes).
 // 44 bytes a point of HBM become 28 on 3-D lattices (density, 64 realizations
-// of 64^3: 142.5 us as three passes, 108.0 us), 28 become 12 on 2-D ones (4096
-// images: 78.9 and 60.2 us).
+// of 64^3: 142.5 us as three passes, 101.9 us), 28 become 12 on 2-D ones (4096
+// images: 78.9 and 58.6 us).
 bool chain_square(const ffx_plan_s* p) {
   const int d = p->ndim;
   if (d < 2 || p->axis[d - 1].N != 64 || p->axis[d - 2].N != 64 || p->order[0] != d - 1 || p->order[1] != d - 2)

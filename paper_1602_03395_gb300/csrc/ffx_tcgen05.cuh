@@ -69,11 +69,14 @@ __device__ __forceinline__ bool mbar_test(uint32_t mbar, uint32_t parity) {
 }
 
 // Bounded wait for the phase of the given parity; gives up (false) when the
-// block aborts or the poll budget runs out (then it sets the abort flag).
+// block aborts or the poll budget runs out (then it sets the abort flag).  The
+// flag is read at every sixteenth poll: it lies in shared memory, whose port the
+// products' operands need (read at every poll: 64 realizations of 64^3 108.4 us
+// instead of 101.8, 4 column images of 128^3 101.8 instead of 98.0).
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity, volatile int* abort_flag) {
   for (long long i = 0; i < kSpinLimit; ++i) {
     if (mbar_test(mbar, parity)) return true;
-    if (*abort_flag) return false;
+    if ((i & 15) == 15 && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
@@ -241,7 +244,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint32_t mbar, uint32_t parity
         : "r"(mbar), "r"(parity)
         : "memory");
     if (done) return true;
-    if (*abort_flag) return false;
+    if ((i & 15) == 15 && *abort_flag) return false;
   }
   *abort_flag = 1;
   return false;
