@@ -174,9 +174,13 @@ struct ffx_plan_s {
   // workspace buffers, grown on demand: [0], [1] the passes' fields; [2] the
   // detector densities, or a positive-P pair's first field; [3] its second;
   // [4] the BF16 planes a per-axis BF16 pass splits its FP32 input into; [5]
-  // partial densities of an ensemble sum's groups
+  // partial densities of an ensemble sum's groups (ensure_sum)
   void* ws[kWs] = {};
   size_t ws_bytes[kWs] = {};
+  // smaller buffers that [5] has outgrown: captured graphs may still write them
+  // (at most one a power of two)
+  void* retired[64] = {};
+  int n_retired = 0;
   int64_t launches = 0;  // kernels the plan's calls have launched (ffx_plan_launch_count)
   void* stage[2] = {nullptr, nullptr};  // ffx_expand_host: device copies of the input and the densities
   size_t stage_bytes[2] = {0, 0};
@@ -290,6 +294,43 @@ int ensure_bytes(ffx_plan_s* p, int which, size_t need) {
 
 int ensure_ws(ffx_plan_s* p, int which, int64_t batch) {
   return ensure_bytes(p, which, (size_t)batch * (size_t)p->M * sizeof(float2));
+}
+
+// The partial densities of an ensemble sum (ws[5]) take at most kSumBytes, or
+// one density if that is larger.
+constexpr size_t kSumBytes = size_t(256) << 20;
+int64_t max_sum_groups(const ffx_plan_s* p, int64_t batch) {
+  return std::min<int64_t>(batch, std::max<int64_t>(1, (int64_t)(kSumBytes / (p->M * sizeof(float)))));
+}
+
+// ws[5] for an ensemble sum over `batch` realizations.  The number of groups
+// does not grow with the batch (1-D lines of 2048 points at lam = 20: 518 groups
+// of 1024 realizations, 608 of 608), so the buffer holds the most groups that any
+// batch up to this one, rounded up to a power of two, can take: a smaller batch
+// finds it large enough.  A buffer that a larger batch outgrows lives on with the
+// plan, because a graph captured with it still writes it; the powers of two keep
+// the sum of all below twice the largest.
+int ensure_sum(ffx_plan_s* p, int64_t batch) {
+  int64_t most = 1;
+  while (most < batch) most *= 2;
+  const size_t need = (size_t)max_sum_groups(p, most) * (size_t)p->M * sizeof(float);
+  if (need <= p->ws_bytes[kWsSum]) return FFX_OK;
+  void* grown = nullptr;
+  cudaError_t e = cudaMalloc(&grown, need);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(FFX_ENOMEM, "workspace of %zu bytes: %s", need, cudaGetErrorString(e));
+  }
+  if (p->ws[kWsSum]) p->retired[p->n_retired++] = p->ws[kWsSum];
+  p->ws[kWsSum] = grown;
+  p->ws_bytes[kWsSum] = need;
+  return FFX_OK;
+}
+
+void free_workspace(ffx_plan_s* p) {
+  for (int w = 0; w < kWs; ++w)
+    if (p->ws[w]) cudaFree(p->ws[w]);
+  for (int k = 0; k < p->n_retired; ++k) cudaFree(p->retired[k]);
 }
 
 bool inplace_ok(const Axis& ax) {
@@ -514,8 +555,7 @@ bool tm32_sum(const Axis& ax, int cform, const float2* in, const float* out_d) {
 // resident blocks times realizations each: the fewest groups within 5% of the
 // fewest steps, and one group unless that saves a fifth of them.  (The mean of
 // 512 realizations of one 2048-point line, lam = 20, on the FFT engine of
-// ffx_pass.cuh: 97 ms in one group, 0.41 ms in 512.)  The partial densities take at most kSumBytes.
-constexpr size_t kSumBytes = size_t(256) << 20;
+// ffx_pass.cuh: 97 ms in one group, 0.41 ms in 512.)
 int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, bool tm32, int64_t lines,
                    int64_t inner, int64_t batch) {
   if (batch * lines < kDenseFewLines && cform == FFX_FORM_DENSE) return 1;  // the few-lines kernel
@@ -544,7 +584,7 @@ int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, 
     }
     return (tiles + cap - 1) / cap;
   };
-  const int64_t gmax = std::min<int64_t>(batch, std::max<int64_t>(1, (int64_t)(kSumBytes / (p->M * sizeof(float)))));
+  const int64_t gmax = max_sum_groups(p, batch);
   auto cost = [&](int64_t g) -> int64_t {
     const int64_t rem = batch % g;
     return steps(g * lines) * (batch / g) + (rem ? steps(rem * lines) : 0);
@@ -589,7 +629,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   if (groups > 1 || tm32) {
     // partial densities of the groups, then their sum
     const size_t bytes = (size_t)groups * (size_t)p->M * sizeof(float);
-    if ((rc = ensure_bytes(p, kWsSum, bytes))) return rc;
+    if ((rc = ensure_sum(p, batch))) return rc;
     float* part = (float*)p->ws[kWsSum];
     if (tm32) {
       rc = run_pass(p, j, adjoint, cform, {outer, inner, p->M, batch, lines, groups}, in, nullptr, 0, nullptr, part, acc,
@@ -1561,8 +1601,7 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
   if (rc == FFX_OK) rc = plan_fusion(p);
   cudaStreamDestroy(s);
   if (rc != FFX_OK) {
-    for (int w = 0; w < kWs; ++w)
-      if (p->ws[w]) cudaFree(p->ws[w]);
+    free_workspace(p);
     if (p->dense_mem) cudaFree(p->dense_mem);
     if (p->tc_mem) cudaFree(p->tc_mem);
     if (p->host_err) cudaFreeHost(p->host_err);
@@ -1613,8 +1652,7 @@ int ffx_plan_destroy(ffx_plan_t p) {
     delete p;
     return FFX_OK;
   }
-  for (int w = 0; w < kWs; ++w)
-    if (p->ws[w]) cudaFree(p->ws[w]);
+  free_workspace(p);
   if (p->dense_mem) cudaFree(p->dense_mem);
   if (p->tc_mem) cudaFree(p->tc_mem);
   if (p->host_err) cudaFreeHost(p->host_err);

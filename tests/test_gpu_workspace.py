@@ -1,0 +1,53 @@
+"""A plan's workspace across calls with other batches and under graph capture:
+what one call prepares stays valid for the graphs that use it, and a call that
+needs no more than an earlier one can be captured."""
+
+import numpy as np
+import pytest
+import torch
+
+from gpu_common import random_field, rel_l2, require_gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ffx():
+    return require_gpu()
+
+
+def fields(dims, batch, seed=1):
+    return to_dev(random_field(np.random.default_rng(seed), (batch,) + dims))
+
+
+def capture(call):
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        call()
+    return graph
+
+
+# plans whose sums run in more groups at a smaller batch (the lines of 2048), and
+# in partial densities of one group (32 points on the tensor cores)
+@pytest.mark.parametrize("dims,lam,form,batch,smaller,larger", [
+    ((2048,), (20,), "auto", 1024, 608, 2500),
+    ((32,), (5,), "tc", 700, 300, 5000),
+])
+def test_sum_graph_outlives_other_batches(ffx, dims, lam, form, batch, smaller, larger):
+    x = fields(dims, larger)
+    with ffx.Plan(dims, (0.2,), 4.0, lam, form=form, accumulate=True) as plan:
+        want = ffx.ffx_expand(plan, x[:batch])
+        held = plan.workspace_bytes(1)
+        ffx.ffx_expand(plan, x[:smaller])
+        assert plan.workspace_bytes(1) == held  # (a graph may hold the buffer)
+        out = torch.zeros_like(want)
+        graph = capture(lambda: ffx.ffx_expand(plan, x[:batch], out))
+        ffx.ffx_expand(plan, x[:smaller])
+        ffx.ffx_expand(plan, x)  # grows the workspace
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, want)
+        assert plan.device_errors() == 0
