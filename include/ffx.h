@@ -89,8 +89,11 @@ extern "C" {
 #define FFX_TUNE        0x20u
 /* ffx_expand writes the SUM over the batch of |Psibar|^2, added to what
  * out_density holds ([M_0..M_{d-1}], out += sum_b rho_b), instead of one
- * density per realization.  The order of the sum depends on the
- * lattice and the batch alone (deterministic). */
+ * density per realization.  The sum may run over groups of realizations whose
+ * partial sums are added in order (see ffx_expand); its order depends on the
+ * lattice, the batch, the device, the 16-byte alignment of the buffers and
+ * whether the partial sums' memory is there, never on timing: a repeated call
+ * gives the same bits. */
 #define FFX_ACCUMULATE  0x10u
 /* Keep one launch per axis pass.  Without it, a plan with two or three axes
  * that all take a dense form with at most 64 points runs ffx_expand and
@@ -261,8 +264,12 @@ int64_t ffx_plan_points(ffx_plan_t plan);
  *               Must not overlap psi0.
  *  stream       cudaStream_t or NULL.
  *
- * Uses the plan's workspace (batch * M complex64 for d >= 2), grown on demand:
- * the first call with a larger batch allocates (cudaMalloc, host-synchronous).
+ * Uses the plan's workspace (up to two fields of batch * M complex64), grown on
+ * demand: the first call with a larger batch allocates (cudaMalloc,
+ * host-synchronous).  With FFX_ACCUMULATE the partial sums of the groups take up to
+ * 256 MB more, or one density if that is larger; a call that cannot have
+ * them (no memory, or its stream is being captured before an uncaptured call
+ * with at least this batch) sums in one group and needs none.
  */
 int ffx_expand(ffx_plan_t plan, const void* psi0, int64_t batch, float* out_density,
                void* stream);

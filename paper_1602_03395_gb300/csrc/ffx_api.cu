@@ -296,6 +296,12 @@ int ensure_ws(ffx_plan_s* p, int which, int64_t batch) {
   return ensure_bytes(p, which, (size_t)batch * (size_t)p->M * sizeof(float2));
 }
 
+// Whether the stream is being captured into a graph (nothing may be allocated).
+bool capturing(cudaStream_t stream) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
+}
+
 // The partial densities of an ensemble sum (ws[5]) take at most kSumBytes, or
 // one density if that is larger.
 constexpr size_t kSumBytes = size_t(256) << 20;
@@ -309,22 +315,23 @@ int64_t max_sum_groups(const ffx_plan_s* p, int64_t batch) {
 // batch up to this one, rounded up to a power of two, can take: a smaller batch
 // finds it large enough.  A buffer that a larger batch outgrows lives on with the
 // plan, because a graph captured with it still writes it; the powers of two keep
-// the sum of all below twice the largest.
-int ensure_sum(ffx_plan_s* p, int64_t batch) {
+// the sum of all below twice the largest.  False where there is none and none can
+// be had (no memory, or the stream is being captured): the sum then runs in one
+// group, which needs no partial densities.
+bool ensure_sum(ffx_plan_s* p, int64_t batch, cudaStream_t stream) {
   int64_t most = 1;
   while (most < batch) most *= 2;
   const size_t need = (size_t)max_sum_groups(p, most) * (size_t)p->M * sizeof(float);
-  if (need <= p->ws_bytes[kWsSum]) return FFX_OK;
+  if (need <= p->ws_bytes[kWsSum]) return true;
   void* grown = nullptr;
-  cudaError_t e = cudaMalloc(&grown, need);
-  if (e != cudaSuccess) {
+  if (capturing(stream) || cudaMalloc(&grown, need) != cudaSuccess) {
     cudaGetLastError();
-    return fail(FFX_ENOMEM, "workspace of %zu bytes: %s", need, cudaGetErrorString(e));
+    return false;
   }
   if (p->ws[kWsSum]) p->retired[p->n_retired++] = p->ws[kWsSum];
   p->ws[kWsSum] = grown;
   p->ws_bytes[kWsSum] = need;
-  return FFX_OK;
+  return true;
 }
 
 void free_workspace(ffx_plan_s* p) {
@@ -625,11 +632,14 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   if (acc && batch > 1) {
     tm32 = !io && tm32_sum(ax, cform, in, out_d);
     groups = sum_groups(p, ax, cform, io || (inner == 1 && ax.pl_t[0]), tm32, lines, inner, batch);
+    if ((groups > 1 || tm32) && !ensure_sum(p, batch, stream)) {
+      groups = 1;
+      tm32 = false;
+    }
   }
   if (groups > 1 || tm32) {
     // partial densities of the groups, then their sum
     const size_t bytes = (size_t)groups * (size_t)p->M * sizeof(float);
-    if ((rc = ensure_sum(p, batch))) return rc;
     float* part = (float*)p->ws[kWsSum];
     if (tm32) {
       rc = run_pass(p, j, adjoint, cform, {outer, inner, p->M, batch, lines, groups}, in, nullptr, 0, nullptr, part, acc,

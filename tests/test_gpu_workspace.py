@@ -51,3 +51,20 @@ def test_sum_graph_outlives_other_batches(ffx, dims, lam, form, batch, smaller, 
             torch.cuda.synchronize()
             assert torch.equal(out, want)
         assert plan.device_errors() == 0
+
+
+# a one-dimensional sum needs no workspace: its first call can be captured (the
+# groups of lines, and 32-point sums, run without their partial densities then)
+@pytest.mark.parametrize("dims,lam,form,batch", [
+    ((2048,), (20,), "auto", 64), ((512,), (20,), "auto", 100), ((32,), (5,), "tc", 300),
+])
+def test_first_sum_of_a_plan_can_be_captured(ffx, dims, lam, form, batch):
+    x = fields(dims, batch)
+    with ffx.Plan(dims, (0.2,), 4.0, lam, form=form, accumulate=True) as plan:
+        out = torch.zeros(dims, device="cuda")
+        graph = capture(lambda: ffx.ffx_expand(plan, x, out))
+        graph.replay()
+        direct = ffx.ffx_expand(plan, x)
+        assert plan.device_errors() == 0
+    # two orders of one FP32 sum: a few 1e-7
+    assert rel_l2(out.cpu().numpy(), direct.cpu().numpy()) < 2e-6
