@@ -302,6 +302,22 @@ bool capturing(cudaStream_t stream) {
   return cudaStreamIsCapturing(stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone;
 }
 
+// The same for a call that can do without the buffer: false, with what there was
+// left in place, if the stream is being captured or the memory is not there.
+bool try_ws(ffx_plan_s* p, int which, int64_t batch, cudaStream_t stream) {
+  const size_t need = (size_t)batch * (size_t)p->M * sizeof(float2);
+  if (need <= p->ws_bytes[which]) return true;
+  void* grown = nullptr;
+  if (capturing(stream) || cudaMalloc(&grown, need) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (p->ws[which]) cudaFree(p->ws[which]);
+  p->ws[which] = grown;
+  p->ws_bytes[which] = need;
+  return true;
+}
+
 // The partial densities of an ensemble sum (ws[5]) take at most kSumBytes, or
 // one density if that is larger.
 constexpr size_t kSumBytes = size_t(256) << 20;
@@ -445,13 +461,14 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.in_points = io->points;
       d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
       d.oouter = outer / d.oinner;
-    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_fp32(ax.N, d.ncols, p->sms)) {
+    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_fp32(ax.N, d.ncols, p->sms) &&
+               try_ws(p, kWsSplit, batch * M / p->M, stream)) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
-      // cores' layout instead of converting them on the way
+      // cores' layout instead of converting them on the way.  Without the
+      // planes' buffer (a capture whose uncaptured calls were large enough to
+      // need none) the pass splits the lines itself all the same.
       const int64_t plane = batch * M;
-      int rc = ensure_ws(p, kWsSplit, plane / p->M);
-      if (rc) return rc;
       e = launch_plane_split(in, nullptr, 0, M, (uint32_t*)p->ws[kWsSplit], plane, plane, d.unsplit, p->sms, stream);
       if (e != cudaSuccess) return cuda_fail(e, "BF16 split of a pass input");
       ++p->launches;

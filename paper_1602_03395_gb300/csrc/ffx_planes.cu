@@ -1615,11 +1615,16 @@ cudaError_t launch_plane_split(const float2* in, const float* grad, int grad_sha
                     unsplit);
 }
 
-int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
+namespace {
+int64_t pass_tiles(int N, int64_t ncols, int sms, bool pair, int64_t* at_once) {
   // one pair of blocks per two SMs, or one block per SM
-  const bool pair = pair_pass(N, ncols, sms);
   *at_once = std::max(1, pair ? sms / 2 : sms);
   return pair ? pair_items(N, ncols) : (ncols + PL - 1) / PL * (N / single_rows(N));
+}
+}  // namespace
+
+int64_t plane_pass_tiles(int N, int64_t ncols, int sms, int64_t* at_once) {
+  return pass_tiles(N, ncols, sms, pair_pass(N, ncols, sms), at_once);
 }
 
 bool plane_pass_fp32(int N, int64_t ncols, int sms) {
@@ -1645,14 +1650,15 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
     a.oinner = a.inner;
   }
   const bool f32 = !a.in_bf;
-  const bool pair = pair_pass(a.N, a.ncols, sms);
+  // (contiguous FP32 lines of these lengths are split on pairs alone, however few)
+  const bool pair = pair_pass(a.N, a.ncols, sms) || (f32 && a.inner == 1 && pair_length(a.N));
   const int out = a.out_bf ? (a.grad ? kOutGrad : kOutPlanes)
                            : a.out_c ? kOutComplex : a.acc ? kOutSum : kOutDensity;
   const bool strided = plane_pass_strided(a.inner);
   const int in = strided ? kInStrided : a.in_points ? kInPoints : f32 ? kInF32 : kInPlanes;
   if (strided && (!f32 || a.out_bf)) return cudaErrorInvalidValue;
   if (a.grad && (!a.out_bf || f32 || !(pair || a.N <= 128))) return cudaErrorInvalidValue;
-  if ((a.inner != 1 && !strided) || (f32 && !pair && !strided && a.N > 128 && a.N != 192) || (a.in_points && a.N > 128))
+  if ((a.inner != 1 && !strided) || (a.in_points && a.N > 128))
     return cudaErrorInvalidValue;
   // [plane][line][2N values]: every realization's lines, the tail plane
   // bf_plane points after the head plane; or the FP32 lines; or a square
@@ -1667,7 +1673,7 @@ cudaError_t launch_plane_pass(const DenseArgs& args, const unsigned char* Tblk, 
           : !row_map(&xmap, a.in_bf, 2 * a.N, a.batch * a.outer, a.unsplit ? 1 : 2, a.bf_plane * 4, PL, true))
     return cudaErrorInvalidValue;
   int64_t at_once;
-  int64_t grid = std::min(plane_pass_tiles(a.N, a.ncols, sms, &at_once), at_once);
+  int64_t grid = std::min(pass_tiles(a.N, a.ncols, sms, pair, &at_once), at_once);
   if (grid < 1) grid = 1;
   if (pair) {
     grid *= 2;

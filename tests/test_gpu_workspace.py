@@ -68,3 +68,26 @@ def test_first_sum_of_a_plan_can_be_captured(ffx, dims, lam, form, batch):
         assert plan.device_errors() == 0
     # two orders of one FP32 sum: a few 1e-7
     assert rel_l2(out.cpu().numpy(), direct.cpu().numpy()) < 2e-6
+
+
+# passes over contiguous FP32 lines: large calls split them in the kernel, small
+# ones in a launch of its own into workspace that the large call did not need
+@pytest.mark.parametrize("dims,lam,batch,smaller,accumulate", [
+    ((96,), (5,), 19537, 40, False),
+    ((192,), (7,), 9801, 70, False),
+    ((384,), (5,), 13001, 100, False),
+    ((384,), (5,), 13001, 1, False),
+    ((1024,), (9,), 5000, 300, False),
+    ((256,), (9,), 20000, 130, True),
+])
+def test_smaller_call_can_be_captured(ffx, dims, lam, batch, smaller, accumulate):
+    x = fields(dims, batch)
+    with ffx.Plan(dims, (0.2,), 4.0, lam, form="tc", bf16=True, accumulate=accumulate) as plan:
+        ffx.ffx_expand(plan, x)
+        out = torch.zeros(dims if accumulate else (smaller,) + dims, device="cuda")
+        graph = capture(lambda: ffx.ffx_expand(plan, x[:smaller], out))
+        graph.replay()
+        direct = ffx.ffx_expand(plan, x[:smaller])
+        assert plan.device_errors() == 0
+    # the same split operands and FP32 sums of their products: a few 1e-7
+    assert rel_l2(out.cpu().numpy(), direct.cpu().numpy()) < 2e-6
