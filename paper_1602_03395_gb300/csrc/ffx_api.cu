@@ -765,6 +765,10 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
   const bool square = chain_square(p);
   int rc;
   if ((!square && (rc = ensure_ws(p, 0, batch))) || ((!square || d > 2) && (rc = ensure_ws(p, 1, batch)))) return rc;
+  // A square call leaves one or both fields unused.  They are made all the same
+  // where they can be: the plan's other calls up to this batch (gradients,
+  // smaller batches) use them, and may be captured after this one.
+  if (square) try_ws(p, 0, batch, s), try_ws(p, 1, batch, s);
   const int64_t plane = batch * p->M;
   const int unsplit = (p->flags & FFX_TC_UNSPLIT) ? 1 : 0;
   const uint32_t* cur_bf = nullptr;

@@ -91,3 +91,23 @@ def test_smaller_call_can_be_captured(ffx, dims, lam, batch, smaller, accumulate
         assert plan.device_errors() == 0
     # the same split operands and FP32 sums of their products: a few 1e-7
     assert rel_l2(out.cpu().numpy(), direct.cpu().numpy()) < 2e-6
+
+
+# after a forward call whose last two axes run in one launch: the gradient at the
+# same batch and a smaller forward call that takes the axes one by one
+@pytest.mark.parametrize("dims,lam,batch,smaller", [((64, 64), (5, 8), 1217, 100), ((64, 64, 64), (5, 3, 7), 20, 3)])
+def test_other_calls_after_a_square_call_can_be_captured(ffx, dims, lam, batch, smaller):
+    x = fields(dims, batch)
+    w = torch.rand((batch,) + dims, device="cuda")
+    with ffx.Plan(dims, (0.2,) * len(dims), 4.0, lam, form="tc", bf16=True, fused=False) as plan:
+        assert plan.chain_square(batch) and not plan.chain_square(smaller)
+        ffx.ffx_expand(plan, x)
+        grad, out = torch.zeros_like(x), torch.zeros_like(w[:smaller])
+        graph = capture(lambda: ffx.ffx_expand_backward(plan, x, w, grad))
+        small = capture(lambda: ffx.ffx_expand(plan, x[:smaller], out))
+        graph.replay()
+        small.replay()
+        want = ffx.ffx_expand_backward(plan, x, w)
+        assert torch.equal(grad, want)
+        assert torch.equal(out, ffx.ffx_expand(plan, x[:smaller]))
+        assert plan.device_errors() == 0
