@@ -419,6 +419,10 @@ struct PassGeom {
   int64_t groups;      // 32-point tensor-core sums: DenseArgs::groups (0: none)
 };
 
+// Whether the axis' tensor-core passes over lines whose points are `inner` apart
+// run on launch_plane_pass (no gradient on load, not the 64-point tensor-memory kernel).
+bool plane_route(const Axis& ax, int64_t inner) { return ax.pl_t[0] && (inner == 1 || plane_pass_strided(inner)); }
+
 // Launch one pass of axis j (forward or adjoint) in the form cform, or, with
 // `io`, a pass of a BF16 chain.
 int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, const float2* in, const float* grad,
@@ -461,7 +465,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.in_points = io->points;
       d.oinner = p->M / ax.N;  // the realization's (or each group's) transposed lines
       d.oouter = outer / d.oinner;
-    } else if (ax.pl_t[0] && !tm64 && !grad && inner == 1 && !plane_pass_fp32(ax.N, d.ncols, p->sms) &&
+    } else if (plane_route(ax, inner) && !tm64 && !grad && inner == 1 && !plane_pass_fp32(ax.N, d.ncols, p->sms) &&
                try_ws(p, kWsSplit, batch * M / p->M, stream)) {
       // contiguous FP32 lines: split into BF16 planes first (an HBM-bound
       // pass), so that the pass loads its operands straight into the tensor
@@ -476,7 +480,7 @@ int run_pass(ffx_plan_s* p, int j, bool adjoint, int cform, const PassGeom& gm, 
       d.bf_plane = plane;
       d.in = nullptr;
     }
-    if (io || (ax.pl_t[0] && !tm64 && !grad && (inner == 1 || plane_pass_strided(inner))))
+    if (io || (plane_route(ax, inner) && !tm64 && !grad))
       e = launch_plane_pass(d, ax.pl_t[adjoint ? 1 : 0], p->dev_err, p->sms, stream);
     else if (ax.bf_th && adjoint && !tm64 && grad)
       e = launch_dense_bf16(d, ax.bf_th, p->dev_err, (int)grid, stream);
@@ -583,6 +587,11 @@ bool tm32_sum(const Axis& ax, int cform, const float2* in, const float* out_d) {
 int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, bool tm32, int64_t lines,
                    int64_t inner, int64_t batch) {
   if (batch * lines < kDenseFewLines && cform == FFX_FORM_DENSE) return 1;  // the few-lines kernel
+  const bool fft = cform == FFX_FORM_PAPER || cform == FFX_FORM_FOLD, line3 = fft && line3_supported(ax.N, inner, ax.g);
+  const PassKernelInfo& info = cform == FFX_FORM_PAPER ? ax.paper : ax.foldk;
+  const int64_t fft_cap = line3 ? 2 * (int64_t)p->sms : cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold;
+  const int fft_per = line3 ? line3_lines(ax.N)
+                      : fft ? pass_lines_per_tile(info, choose_qg(info, lines, ax.lam, (int)fft_cap)) : 1;
   auto steps = [&](int64_t ncols) -> int64_t {  // waves of a launch over ncols lines
     int64_t tiles, cap;
     if (cform == FFX_FORM_TC && tm32) {
@@ -596,37 +605,49 @@ int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, 
     } else if (cform == FFX_FORM_DENSE) {
       tiles = ax.N <= kDenseInPlaceMaxN ? dense_small_tiles(ax.N, ncols) : dense_tiles(ax.N, ncols);
       cap = ax.N <= kDenseInPlaceMaxN ? ax.grid_dense_small : ax.grid_dense;
-    } else if (line3_supported(ax.N, inner, ax.g)) {
-      const int per = line3_lines(ax.N);
-      tiles = (ncols + per - 1) / per;
-      cap = 2 * (int64_t)p->sms;
     } else {
-      const PassKernelInfo& info = cform == FFX_FORM_PAPER ? ax.paper : ax.foldk;
-      cap = cform == FFX_FORM_PAPER ? ax.grid_paper : ax.grid_fold;
-      const int per = pass_lines_per_tile(info, choose_qg(info, lines, ax.lam, (int)cap));
-      tiles = (ncols + per - 1) / per;
+      tiles = (ncols + fft_per - 1) / fft_per;
+      cap = fft_cap;
     }
     return (tiles + cap - 1) / cap;
   };
   const int64_t gmax = max_sum_groups(p, batch);
-  auto cost = [&](int64_t g) -> int64_t {
+  // us of the partial densities' traffic
+  auto traffic = [&](int64_t g) { return (double)g * (double)p->M * 8e-6 / 5.0; };
+  // A step of the plane passes is short (2-3 us), so the choice among group counts
+  // weighs a remainder's launch as two steps, and the partial densities' traffic
+  // (512 realizations of 96x64: 47.2 us in 256 groups, 53.5 in 257 and a
+  // remainder; 1001 of 128x64: 76.6 us in 1001 groups, 67.4 in 251 and a remainder).
+  const bool short_steps = cform == FFX_FORM_TC && planes;
+  auto all_steps = [&](int64_t g) -> double {
     const int64_t rem = batch % g;
-    return steps(g * lines) * (batch / g) + (rem ? steps(rem * lines) : 0);
+    return (double)(steps(g * lines) * (batch / g) + (rem ? steps(rem * lines) : 0));
   };
-  // candidates: every g up to 64, then each an eighth more, and the most
-  auto next = [&](int64_t g) { return g >= gmax ? gmax + 1 : std::min(gmax, g < 64 ? g + 1 : g + g / 8); };
-  const int64_t one = cost(1);
-  int64_t best = one;
-  for (int64_t g = 2; g <= gmax; g = next(g)) best = std::min(best, cost(g));
+  auto cost = [&](int64_t g) -> double {
+    return all_steps(g) + (short_steps ? (batch % g ? 2.0 : 0.0) + 0.25 * traffic(g) : 0.0);
+  };
+  // candidates: every g up to 64, then each an eighth more, and the most; and those
+  // of up to 32 realizations each, among which are the ones without a remainder
+  auto candidates = [&](auto&& take) {
+    for (int64_t g = 2; g <= gmax; g = g >= gmax ? gmax + 1 : std::min(gmax, g < 64 ? g + 1 : g + g / 8)) take(g);
+    for (int64_t k = 2; k <= 32; ++k) {
+      const int64_t g = (batch + k - 1) / k;
+      if (g > 64 && g <= gmax) take(g);
+    }
+  };
+  const double one = cost(1);
+  double best = one;
+  candidates([&](int64_t g) { best = std::min(best, cost(g)); });
   if (5 * best > 4 * one) return 1;
+  int64_t few = gmax;
+  candidates([&](int64_t g) {
+    if (g < few && 20 * cost(g) <= 21 * best) few = g;
+  });
   // a step is at least ~2 us, in the FFT forms ~2 us a term; the partial
   // densities cost ~6 us of launches and their traffic, and have to be gained
   // twice over (256x16x64 x 7: 85 us in one group, 100 us in several)
-  const double step_us = cform == FFX_FORM_PAPER || cform == FFX_FORM_FOLD ? 2.0 * ax.lam : 2.0;
-  for (int64_t g = 2; g <= gmax; g = next(g))
-    if (20 * cost(g) <= 21 * best)
-      return (double)(one - cost(g)) * step_us > 2.0 * (6.0 + (double)g * (double)p->M * 8e-6 / 5.0) ? g : 1;
-  return 1;
+  const double step_us = fft ? 2.0 * ax.lam : 2.0;
+  return (all_steps(1) - all_steps(few)) * step_us > 2.0 * (6.0 + traffic(few)) ? few : 1;
 }
 
 // Launch one pass of axis j (forward or adjoint) with the axis's form, or,
@@ -648,7 +669,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   bool tm32 = false;
   if (acc && batch > 1) {
     tm32 = !io && tm32_sum(ax, cform, in, out_d);
-    groups = sum_groups(p, ax, cform, io || (inner == 1 && ax.pl_t[0]), tm32, lines, inner, batch);
+    groups = sum_groups(p, ax, cform, io || plane_route(ax, inner), tm32, lines, inner, batch);
     if ((groups > 1 || tm32) && !ensure_sum(p, batch, stream)) {
       groups = 1;
       tm32 = false;
