@@ -715,11 +715,11 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
       // ---------------- products: the whole warp, one elected lane issuing ----------------
       int64_t u = 0;
       int s = 0;
-      bool ok = !RES || mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
+      if (RES) mbar_wait_all<IN == kInStrided>(smem_u32(&t_bar), 0u, &s_abort);
       constexpr uint32_t major = POINTS ? kMajorA : 0u;
       const uint32_t id1 = idesc_bf16(PL, RB) | major, id2 = idesc_bf16(PL, 2 * RB) | major;
 #pragma unroll 1
-      for (int64_t sub = 0; ok && sub < my_items * nb; ++sub) {
+      for (int64_t sub = 0; sub < my_items * nb; ++sub) {
         const int buf = NBUF == 2 ? (int)(sub & 1) : 0;
         const int64_t v = NBUF == 2 ? sub >> 1 : sub;
         const uint32_t prev = (uint32_t)((v - 1) & 1);
@@ -727,9 +727,8 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
 #pragma unroll 1
         for (int kc = 0; kc < kchunks; ++kc) {
           const bool last = kc == kchunks - 1;
-          ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-               (kc > 0 || v == 0 || mbar_wait(smem_u32(&acce_bar[2 * buf]), prev, &s_abort));
-          if (!ok) break;
+          mbar_wait_all<IN == kInStrided>(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
+          if (kc == 0 && v > 0) mbar_wait_all<IN == kInStrided>(smem_u32(&acce_bar[2 * buf]), prev, &s_abort);
           tc_fence_after();
           const uint32_t st = stages + (uint32_t)(s * STAGE);
           const uint32_t tb = RES ? t_res + (uint32_t)(kc * TCH) : st + (uint32_t)PX;
@@ -745,8 +744,7 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
             __syncwarp();
           }
           if (kc == 0 && v > 0) {
-            ok = mbar_wait(smem_u32(&acce_bar[2 * buf + 1]), prev, &s_abort);
-            if (!ok) break;
+            mbar_wait_all<IN == kInStrided>(smem_u32(&acce_bar[2 * buf + 1]), prev, &s_abort);
             tc_fence_after();
           }
           half(std::true_type(), dim);
@@ -922,7 +920,7 @@ __global__ void __launch_bounds__(PTHREADS_F32, 1)
       __syncwarp();
     } else if (warp == 1) {
       // ---------------- products: the whole warp, one elected lane issuing ----------------
-      bool ok = mbar_wait(smem_u32(&t_bar), 0u, &s_abort);
+      mbar_wait_all(smem_u32(&t_bar), 0u, &s_abort);
       const uint32_t id1 = idesc_bf16(PL, RB), id2 = idesc_bf16(PL, 2 * RB);
       const uint32_t dre1 = tmem, dim1 = dre1 + 2 * RB, dre2 = tmem + 4 * RB, dim2 = dre2 + 2 * RB;
       int s = 0;
@@ -932,22 +930,20 @@ __global__ void __launch_bounds__(PTHREADS_F32, 1)
         __syncwarp();
       };
 #pragma unroll 1
-      for (int64_t i = 0; ok && i <= my_items; ++i) {
+      for (int64_t i = 0; i <= my_items; ++i) {
         const uint32_t prev = (uint32_t)((i - 1) & 1);
         if (i < my_items) {  // step 1 of item i
 #pragma unroll 1
           for (int kc = 0; kc < 2; ++kc) {
-            ok = mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-                 (kc > 0 || i == 0 || mbar_wait(smem_u32(&d1e_bar[0]), prev, &s_abort));
-            if (!ok) break;
+            mbar_wait_all(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
+            if (kc == 0 && i > 0) mbar_wait_all(smem_u32(&d1e_bar[0]), prev, &s_abort);
             tc_fence_after();
             const XLines x(stages + (uint32_t)(s * PX));
             const uint32_t tb = t1 + (uint32_t)(kc * TCH);
             plane_half<1, RB, false>(dre1, x, tb, tb, id1, id2, kc == 0, unsplit);
             if (kc == 1) commit(&d1f_bar[0]);
             if (kc == 0 && i > 0) {
-              ok = mbar_wait(smem_u32(&d1e_bar[1]), prev, &s_abort);
-              if (!ok) break;
+              mbar_wait_all(smem_u32(&d1e_bar[1]), prev, &s_abort);
               tc_fence_after();
             }
             plane_half<1, RB, true>(dim1, x, tb, tb, id1, id2, kc == 0, unsplit);
@@ -958,12 +954,10 @@ __global__ void __launch_bounds__(PTHREADS_F32, 1)
               ++u;
             }
           }
-          if (!ok) break;
         }
         if (i > 0) {  // step 2 of item i - 1
-          ok = mbar_wait(smem_u32(&a2f_bar), prev, &s_abort) &&
-               (i == 1 || mbar_wait(smem_u32(&d2e_bar[0]), (uint32_t)(i & 1), &s_abort));
-          if (!ok) break;
+          mbar_wait_all(smem_u32(&a2f_bar), prev, &s_abort);
+          if (i > 1) mbar_wait_all(smem_u32(&d2e_bar[0]), (uint32_t)(i & 1), &s_abort);
           tc_fence_after();
 #pragma unroll
           for (int kc = 0; kc < 2; ++kc)
@@ -972,8 +966,7 @@ __global__ void __launch_bounds__(PTHREADS_F32, 1)
                                      kc == 0, unsplit);
           commit(&d2f_bar[0]);
           if (i > 1) {
-            ok = mbar_wait(smem_u32(&d2e_bar[1]), (uint32_t)(i & 1), &s_abort);
-            if (!ok) break;
+            mbar_wait_all(smem_u32(&d2e_bar[1]), (uint32_t)(i & 1), &s_abort);
             tc_fence_after();
           }
 #pragma unroll
@@ -1308,13 +1301,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(in_fp32(IN) ? PTHREA
           const uint32_t ph = (uint32_t)(u & 1);
           const uint32_t st0 = stages + (uint32_t)(s0 * QSTAGE), st1 = st0 + QSTAGE;
           const bool last = kc == kchunks - 2;
-          ok = mbar_wait_cluster(smem_u32(&full_bar[s0]), ph, &s_abort) &&
+          ok = ok && mbar_wait_cluster(smem_u32(&full_bar[s0]), ph, &s_abort) &&
                (kc > 0 || sub == 0 || mbar_wait_cluster(smem_u32(&acce_bar[0]), prev, &s_abort));
-          if (!ok) break;
           tc_fence_after();
           plane_half<2, RB, false>(dre, X(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
-          ok = mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
-          if (!ok) break;
+          ok = ok && mbar_wait_cluster(smem_u32(&full_bar[s1]), ph, &s_abort);
           tc_fence_after();
           plane_half<2, RB, false>(dre, X(st1), st1 + PX, st1 + PX + QTP, id1, id2, false, unsplit);
           if (last) {
@@ -1322,8 +1313,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(in_fp32(IN) ? PTHREA
             __syncwarp();
           }
           if (kc == 0 && sub > 0) {
-            ok = mbar_wait_cluster(smem_u32(&acce_bar[1]), prev, &s_abort);
-            if (!ok) break;
+            ok = ok && mbar_wait_cluster(smem_u32(&acce_bar[1]), prev, &s_abort);
             tc_fence_after();
           }
           plane_half<2, RB, true>(dim, X(st0), st0 + PX, st0 + PX + QTP, id1, id2, kc == 0, unsplit);
@@ -1341,6 +1331,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(in_fp32(IN) ? PTHREA
             ++u;
           }
         }
+        // between its products the warp cannot leave (see mbar_wait_all); between
+        // items it does, its lanes together, so that the odd CTA's copies stop too
+        // (those land on this CTA's barriers, which nothing waits for after an abort)
+        ok = __all_sync(0xffffffffu, ok);
       }
       // whatever happened, the tensor cores finish this warp's work before exit
       if (elect_one()) mma2_commit(smem_u32(&done_bar));

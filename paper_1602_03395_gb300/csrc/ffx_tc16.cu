@@ -356,10 +356,9 @@ __global__ void __launch_bounds__(BTHREADS, 1)
     // ---------------- products: the whole warp, one elected lane issuing ----------------
     int64_t u = 0;
     int s = 0;
-    bool ok = true;
     // descriptor words of both operands' core matrices (see mma_lo)
     constexpr uint32_t hi_core = (uint32_t)(BSBO >> 4) | (1u << 14), lo_core = (uint32_t)(BCORE >> 4) << 16;
-    for (int64_t it = 0; ok && it < my_items; ++it) {
+    for (int64_t it = 0; it < my_items; ++it) {
       const int mt = (int)((blockIdx.x + it * gridDim.x) % mtiles);
       const uint32_t idesc = idesc_bf16(BL, FULL ? BR : brow_count(N, mt));
       // whole row blocks: X_hi against [T_hi; T_lo] (the T chunk's 256 rows,
@@ -367,15 +366,13 @@ __global__ void __launch_bounds__(BTHREADS, 1)
       // accumulators [d1 | d2] -- the operand X_hi is read once for both
       const int buf = (int)(it & 1);
       const int64_t v = it >> 1;
-      ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
-      if (!ok) break;
+      if (v >= 1) mbar_wait_all<true>(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
       tc_fence_after();
       const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
 #pragma unroll 1
       for (int kc = 0; kc < kchunks; ++kc) {
-        ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-             mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
-        if (!ok) break;
+        mbar_wait_all<true>(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort);
+        mbar_wait_all<true>(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
         tc_fence_after();
         const uint32_t th = ((smem_base + (uint32_t)(s * BSTAGE)) >> 4) | lo_core, tl = th + BPART / 16;
         const uint32_t xh = th + BTCHUNK / 16, xl = xh + BPART / 16;
@@ -940,7 +937,6 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
     // ---------------- products: the whole warp, one elected lane issuing ----------------
     int64_t sub = 0, u = 0;
     int s = 0;
-    bool ok = true;
     // descriptor words (see mma_lo): T's core matrices, and X's, the in-place
     // producers' core matrices or the swizzled TMA tile
     constexpr uint32_t hi_core = (uint32_t)(BSBO >> 4) | (1u << 14), lo_core = (uint32_t)(BCORE >> 4) << 16;
@@ -949,22 +945,20 @@ __global__ void __launch_bounds__(BTHREADS, 1) dense_bf16_many_kernel(const TcPa
     constexpr uint32_t xstep = SW ? 2 : 2 * BCORE / 16;  // a K step's bytes / 16
     constexpr uint32_t id_whole = idesc_bf16(BL, 2 * BR);
     BItems<false> mi(P, first, last);
-    for (; ok && mi.more(); mi.next(), ++sub) {
+    for (; mi.more(); mi.next(), ++sub) {
       const int rows = brow_count(mi.d.N, mi.item.mt);
       const int kchunks = (2 * mi.d.N + BKC - 1) / BKC;
       const uint32_t idesc = idesc_bf16(BL, rows);
       const bool whole = rows == BR;
       const int buf = (int)(sub & 1);
       const int64_t v = sub >> 1;
-      ok = v < 1 || mbar_wait(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
-      if (!ok) break;
+      if (v >= 1) mbar_wait_all<true>(smem_u32(&acce_bar[buf]), (uint32_t)((v - 1) & 1), &s_abort);
       tc_fence_after();
       const uint32_t d1 = tmem + (uint32_t)(buf * 2 * BR), d2 = d1 + BR;
 #pragma unroll 1
       for (int kc = 0; kc < kchunks; ++kc) {
-        ok = mbar_wait(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort) &&
-             (PLANES || mbar_wait(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort));
-        if (!ok) break;
+        mbar_wait_all<true>(smem_u32(&copy_bar[s]), (uint32_t)(u & 1), &s_abort);
+        if (!PLANES) mbar_wait_all<true>(smem_u32(&full_bar[s]), (uint32_t)(u & 1), &s_abort);
         tc_fence_after();
         const uint32_t st = smem_base + (uint32_t)(s * BSTAGE);
         const uint32_t th = (st >> 4) | lo_core, tl = th + BPART / 16;
