@@ -426,7 +426,11 @@ int ffx_plan_output_axis(ffx_plan_t plan, int axis, double* x0, double* step);
 int ffx_fringe_phase(const float* image, int64_t rows, int64_t ny, int64_t row_stride, int64_t y_stride,
                      double y0, double dy, double D, double t, double* out_phase, void* stream);
 
-/* Bytes of plan-owned workspace a call with this batch uses. */
+/* Bytes of workspace the plan holds after an ffx_expand call with this batch on
+ * 16-byte aligned buffers, with what it holds already: the fields between the
+ * passes, split input planes, and an ensemble sum's partial densities.  (Other
+ * entry points may need one or two fields more, see each.)  A many-instance plan:
+ * its packed workspace.  -1 on a bad argument. */
 int64_t ffx_workspace_bytes(ffx_plan_t plan, int64_t batch);
 
 /* 1 if the plan's streaming tensor-core passes take BF16 operands

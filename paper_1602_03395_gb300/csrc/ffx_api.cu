@@ -181,6 +181,7 @@ struct ffx_plan_s {
   // (at most one a power of two)
   void* retired[64] = {};
   int n_retired = 0;
+  size_t retired_bytes = 0;
   int64_t launches = 0;  // kernels the plan's calls have launched (ffx_plan_launch_count)
   void* stage[2] = {nullptr, nullptr};  // ffx_expand_host: device copies of the input and the densities
   size_t stage_bytes[2] = {0, 0};
@@ -334,17 +335,23 @@ int64_t max_sum_groups(const ffx_plan_s* p, int64_t batch) {
 // the sum of all below twice the largest.  False where there is none and none can
 // be had (no memory, or the stream is being captured): the sum then runs in one
 // group, which needs no partial densities.
-bool ensure_sum(ffx_plan_s* p, int64_t batch, cudaStream_t stream) {
+size_t sum_bytes(const ffx_plan_s* p, int64_t batch) {
   int64_t most = 1;
   while (most < batch) most *= 2;
-  const size_t need = (size_t)max_sum_groups(p, most) * (size_t)p->M * sizeof(float);
+  return (size_t)max_sum_groups(p, most) * (size_t)p->M * sizeof(float);
+}
+bool ensure_sum(ffx_plan_s* p, int64_t batch, cudaStream_t stream) {
+  const size_t need = sum_bytes(p, batch);
   if (need <= p->ws_bytes[kWsSum]) return true;
   void* grown = nullptr;
   if (capturing(stream) || cudaMalloc(&grown, need) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
-  if (p->ws[kWsSum]) p->retired[p->n_retired++] = p->ws[kWsSum];
+  if (p->ws[kWsSum]) {
+    p->retired[p->n_retired++] = p->ws[kWsSum];
+    p->retired_bytes += p->ws_bytes[kWsSum];
+  }
   p->ws[kWsSum] = grown;
   p->ws_bytes[kWsSum] = need;
   return true;
@@ -650,6 +657,20 @@ int64_t sum_groups(const ffx_plan_s* p, const Axis& ax, int cform, bool planes, 
   return (all_steps(1) - all_steps(few)) * step_us > 2.0 * (6.0 + traffic(few)) ? few : 1;
 }
 
+// How an ensemble sum's last pass runs: its groups, and whether it is the 32-point
+// kernel that sums groups itself.  The partial densities are needed where `tm32`
+// or groups > 1.
+struct SumPlan {
+  int64_t groups;
+  bool tm32;
+  bool partial() const { return tm32 || groups > 1; }
+};
+SumPlan plan_sum(const ffx_plan_s* p, const Axis& ax, int cform, bool chain, const float2* in, const float* out_d,
+                 int64_t lines, int64_t inner, int64_t batch) {
+  const bool tm32 = !chain && tm32_sum(ax, cform, in, out_d);
+  return {sum_groups(p, ax, cform, chain || plane_route(ax, inner), tm32, lines, inner, batch), tm32};
+}
+
 // Launch one pass of axis j (forward or adjoint) with the axis's form, or,
 // with `io`, a pass of a BF16 chain.
 int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* grad, int grad_shared,
@@ -665,17 +686,14 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   const int64_t lines = outer * inner;
   const int cform = call_form(p, ax, acc ? lines : batch * lines);  // this call's form
   int rc = FFX_OK;
-  int64_t groups = 1;
-  bool tm32 = false;
+  SumPlan sum = {1, false};
   if (acc && batch > 1) {
-    tm32 = !io && tm32_sum(ax, cform, in, out_d);
-    groups = sum_groups(p, ax, cform, io || plane_route(ax, inner), tm32, lines, inner, batch);
-    if ((groups > 1 || tm32) && !ensure_sum(p, batch, stream)) {
-      groups = 1;
-      tm32 = false;
-    }
+    sum = plan_sum(p, ax, cform, io != nullptr, in, out_d, lines, inner, batch);
+    if (sum.partial() && !ensure_sum(p, batch, stream)) sum = {1, false};
   }
-  if (groups > 1 || tm32) {
+  const int64_t groups = sum.groups;
+  const bool tm32 = sum.tm32;
+  if (sum.partial()) {
     // partial densities of the groups, then their sum
     const size_t bytes = (size_t)groups * (size_t)p->M * sizeof(float);
     float* part = (float*)p->ws[kWsSum];
@@ -883,6 +901,55 @@ int chain_bf16_split_adjoint(ffx_plan_s* p, const float2* field, const float* gr
   ++p->launches;
   trace_end(p, s, rec);
   return chain_bf16_adjoint(p, 1, batch, out, s);
+}
+
+// Bytes of every workspace buffer that ffx_expand over `batch` realizations in
+// 16-byte aligned buffers has the plan hold.
+void expand_needs(const ffx_plan_s* p, int64_t batch, size_t* need) {
+  const size_t field = (size_t)batch * (size_t)p->M * sizeof(float2);
+  const int d = p->ndim;
+  if (batch <= p->fused) {
+    need[0] = field;
+    if (p->fused_tc && d > 2) need[1] = field;
+    return;
+  }
+  const float2* const in = (const float2*)(uintptr_t)16;
+  const float* const out = (const float*)(uintptr_t)16;
+  const bool chain = bf16_chain_ok(p, batch, in, nullptr, out);
+  if (chain) {
+    need[0] = need[1] = field;
+  } else if (d > 1) {
+    need[0] = field;
+    for (int k = 1; k < d - 1; ++k)
+      if (!inplace_ok(p->axis[p->order[k]])) need[1] = field;
+  }
+  const int last = p->order[d - 1];
+  int64_t groups = 1, outer, inner;
+  if (p->acc && batch > 1) {
+    const Axis& ax = p->axis[last];
+    axis_outer_inner(p, last, &outer, &inner);
+    const int64_t lines = outer * inner;
+    const SumPlan sum =
+        plan_sum(p, ax, call_form(p, ax, lines), chain, in, out, lines, chain ? 1 : inner, batch);
+    groups = sum.groups;
+    if (sum.partial()) need[kWsSum] = sum_bytes(p, batch);
+  }
+  // the split of the contiguous axis' lines, where its pass does not split them itself
+  const Axis& ax = p->axis[d - 1];
+  const bool acc = p->acc && last == d - 1;
+  const int64_t real = p->M / ax.N;
+  if (chain || !plane_route(ax, 1) || call_form(p, ax, acc ? real : batch * real) != FFX_FORM_TC) return;
+  auto split = [&](int64_t lines, int64_t planes) {
+    const int64_t items = dense_tc_tiles(ax.N, lines);
+    const bool tm64 = ax.N == 64 && !acc && items <= 4 * std::max<int64_t>(1, std::min<int64_t>(items, p->sms));
+    if (!tm64 && !plane_pass_fp32(ax.N, lines, p->sms)) need[kWsSplit] = std::max(need[kWsSplit], planes * (field / batch));
+  };
+  if (!acc) {
+    split(batch * real, batch);
+  } else {
+    split(groups * real, batch / groups * groups);
+    if (batch % groups) split(batch % groups * real, batch % groups);
+  }
 }
 
 // Run a chain of passes (forward or adjoint) from `in` (read only) into
@@ -1772,10 +1839,13 @@ int ffx_plan_device_errors(ffx_plan_t p) {
 
 int64_t ffx_workspace_bytes(ffx_plan_t p, int64_t batch) {
   if (!p || batch < 0) return -1;
-  int64_t total = 0;
-  for (int w = 0; w < kWs; ++w) total += (int64_t)p->ws_bytes[w];
-  const int64_t need = batch * p->M * (int64_t)sizeof(float2);
-  return total > need ? total : need;
+  if (p->many) return batch * p->M * (int64_t)sizeof(float2);
+  size_t need[kWs] = {};
+  if (batch > 0) expand_needs(p, batch, need);
+  size_t total = p->retired_bytes;
+  for (int w = 0; w < kWs; ++w) total += std::max(need[w], p->ws_bytes[w]);
+  if (need[kWsSum] > p->ws_bytes[kWsSum]) total += p->ws_bytes[kWsSum];  // kept beside the larger one
+  return (int64_t)total;
 }
 
 int ffx_launches_per_call(ffx_plan_t p, int backward) {

@@ -111,3 +111,30 @@ def test_other_calls_after_a_square_call_can_be_captured(ffx, dims, lam, batch, 
         assert torch.equal(grad, want)
         assert torch.equal(out, ffx.ffx_expand(plan, x[:smaller]))
         assert plan.device_errors() == 0
+
+
+# workspace_bytes against what the plan holds after the call (batch 0 adds nothing):
+# fused calls, chains, squares, passes with and without a split launch, FFT forms,
+# sums in groups, growing and shrinking batches
+@pytest.mark.parametrize("dims,lam,form,accumulate,batches", [
+    ((64, 64, 64), (5, 3, 7), "auto", False, (1, 4, 20, 3)),
+    ((64, 64), (5, 8), "tc", False, (3, 1217)),
+    ((32, 16, 48), (3, 4, 5), "auto", False, (1, 40)),
+    ((96, 96, 96), (3, 4, 5), "auto", False, (1, 5)),
+    ((48, 96, 192), (7, 11, 4), "auto", False, (2, 1, 5)),
+    ((384,), (5,), "tc", False, (100, 13001, 300)),
+    ((256, 64, 48), (1, 2, 1), "auto", False, (3,)),
+    ((16, 512), (3, 6), "fold", True, (2, 77)),
+    ((2048,), (20,), "auto", True, (1, 608, 700, 300, 2500)),
+    ((32, 32, 64), (5, 6, 7), "tc", True, (2, 45)),
+    ((96, 64), (5, 9), "auto", True, (61, 331, 1000)),
+    ((48, 256), (5, 9), "tc", True, (100, 7)),
+    ((256,), (9,), "tc", True, (1000, 20000, 30)),
+])
+def test_workspace_bytes(ffx, dims, lam, form, accumulate, batches):
+    x = fields(dims, max(batches))
+    with ffx.Plan(dims, (0.2,) * len(dims), 4.0, lam, form=form, accumulate=accumulate) as plan:
+        for batch in batches:
+            told = plan.workspace_bytes(batch)
+            ffx.ffx_expand(plan, x[:batch])
+            assert plan.workspace_bytes(0) == told == plan.workspace_bytes(batch)
