@@ -740,7 +740,8 @@ def measure_workload(args, torch, dist, world, rank, local, dev, ffx, w, primary
     fused_call = plan.fused and B_ <= plan.fused_max_batch  # all d passes in one launch
     call_forms = plan.call_forms(B_)  # the kernel each axis runs at this batch
     # BF16 chain: one launch splits the input into BF16 planes, then the passes
-    # (a chain whose first pass runs on CTA pairs has no split launch)
+    # (a chain whose first pass splits its FP32 lines itself, or covers the last
+    # two axes, has no split launch)
     chain = plan.bf16_chain(B_) and args.column is None
     split = chain and plan.chain_split(B_)
     square = chain and plan.chain_square(B_)  # one launch covers the last two axes

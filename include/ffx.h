@@ -449,7 +449,8 @@ int ffx_plan_axis_form(ffx_plan_t plan, int axis);
  * with a batch of one.  A call that runs as a BF16 chain
  * (ffx_plan_bf16_chain) makes one more where ffx_plan_chain_split says so: the
  * split of its input into BF16 planes (in ffx_expand_backward: the forward half of a 3-D plan),
- * and one fewer where ffx_plan_chain_square says so. */
+ * and one fewer where ffx_plan_chain_square says so.  An ensemble sum in groups of
+ * realizations makes one more (the sum of the groups), or two (a remainder). */
 int ffx_launches_per_call(ffx_plan_t plan, int backward);
 
 /* The largest batch for which ffx_expand and ffx_expand_field run as one

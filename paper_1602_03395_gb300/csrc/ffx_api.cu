@@ -788,15 +788,18 @@ bool chain_splits(const ffx_plan_s* p, int64_t batch) {
   return !chain_square(p) && !plane_pass_splits(ax.N, batch * (p->M / ax.N), p->sms);
 }
 
+// Whether a chain may read `in`.
+bool chain_reads(const ffx_plan_s* p, const void* in) { return in != p->ws[0] && in != p->ws[1]; }
+
 // The forward map of a batch as a BF16 chain: the input split into BF16
 // planes in ws[1] (head plane, then tail plane: 8 bytes a point, the size of
 // a complex64 field), then the passes in the plan's order (the last axis
 // first), each reading planes and writing planes (ws[0], ws[1], ...), the
 // last one the caller's field (out_c) or densities (out_d, summed over the
 // batch with FFX_ACCUMULATE).  With chain_square the first two passes are one
-// that writes ws[1].  `in` is read by the split (or the first pass,
-// which writes ws[0]) alone, so out_c may equal it; it must not be ws[1] or, if
-// the first pass reads it, ws[0].
+// that writes ws[1].  `in` is read by the first launch alone (the split, or a
+// pass that writes ws[0] or ws[1]), so out_c may equal it; it must not be a
+// field workspace (chain_reads).
 // With `grad` (3-D) the last pass writes planes of 2 grad times the field to ws[0].
 int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, float* out_d, cudaStream_t s,
                const float* grad = nullptr, int grad_shared = 0) {
@@ -960,9 +963,8 @@ int chain_into(ffx_plan_s* p, const int* axes, bool adjoint, const float2* in, c
                int grad_shared, int64_t batch, float2* out, int alt_ws, cudaStream_t s) {
   const int d = p->ndim;
   // forward fields take the BF16 chain (its planes live in ws[0] and ws[1])
-  // unless the input is ws[1], which its split writes, or the output is the
-  // buffer its last pass reads
-  if (!adjoint && !grad && axes == p->order && (const void*)in != p->ws[1] && (void*)out != p->ws[(d - 2) & 1] &&
+  // unless the input is one of them or the output is the buffer its last pass reads
+  if (!adjoint && !grad && axes == p->order && chain_reads(p, in) && (void*)out != p->ws[(d - 2) & 1] &&
       bf16_chain_ok(p, batch, in, out, nullptr))
     return chain_bf16(p, in, batch, out, nullptr, s);
   float2* outs[3];
@@ -1638,11 +1640,8 @@ int ffx_plan_dispersion(ffx_plan_t* out, int ndim, const int64_t* dims, const do
           e = launch_plane_build_t(ax.T, ax.pl_t[0], ax.N, s);
           if (e == cudaSuccess) e = launch_plane_build_t(ax.TH, ax.pl_t[1], ax.N, s);
           const bool square = ndim > 1 && p->axis[ndim - 1].N == 64 && p->axis[ndim - 2].N == 64;
-          int64_t inner = 1;
-          for (int k = j + 1; k < ndim; ++k) inner *= p->axis[k].N;
           if (e == cudaSuccess)
-            e = plane_pass_prepare(ax.N, square && j == 0, ndim == 3 && j == 0,
-                                   j < ndim - 1);
+            e = plane_pass_prepare(ax.N, square && j == 0, ndim == 3 && j == 0, j < ndim - 1);
           if (e == cudaSuccess && square) e = plane_square_prepare();
         }
         if (e == cudaSuccess)
@@ -1896,7 +1895,7 @@ int ffx_plan_call_form(ffx_plan_t p, int axis, int64_t batch) {
 int forward_density(ffx_plan_s* p, const int* axes, const float2* in, int64_t batch, float* out_d,
                     cudaStream_t s) {
   const int d = p->ndim;
-  if (axes == p->order && (const void*)in != p->ws[1] && bf16_chain_ok(p, batch, in, nullptr, out_d))
+  if (axes == p->order && chain_reads(p, in) && bf16_chain_ok(p, batch, in, nullptr, out_d))
     return chain_bf16(p, in, batch, nullptr, out_d, s);
   const float2* cur = in;
   int rc;
@@ -2120,8 +2119,7 @@ int ffx_expand_backward(ffx_plan_t p, const void* psi0, const float* grad_densit
   // grad_psi0 (ws[1] as the alternate)
   if ((rc = ensure_ws(p, 0, batch))) return rc;
   float2* field = (float2*)p->ws[0];
-  if (psi0 != p->ws[0] && psi0 != p->ws[1] && chain_grad(p, batch) &&
-      bf16_chain_ok(p, batch, psi0, grad_psi0, nullptr)) {
+  if (chain_reads(p, psi0) && chain_grad(p, batch) && bf16_chain_ok(p, batch, psi0, grad_psi0, nullptr)) {
     if ((rc = ensure_ws(p, 1, batch)) ||
         (rc = chain_bf16(p, (const float2*)psi0, batch, nullptr, nullptr, s, grad_density, p->acc)))
       return rc;

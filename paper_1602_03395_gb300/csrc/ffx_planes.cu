@@ -1353,7 +1353,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(in_fp32(IN) ? PTHREA
       asm volatile("setmaxnreg.dec.sync.aligned.u32 104;");
       const uint32_t full0 = map_rank(smem_u32(&full_bar[0]), 0u);
       split_tiles<QST>(
-          lane, total, raw_bar, &s_abort, 
+          lane, total, raw_bar, &s_abort,
           [&](int st) {
             if constexpr (STRIDED)
               split_points(psm + st * QSTAGE, warp - 12, lane, unsplit);
@@ -1473,8 +1473,9 @@ struct PVariant {
     if constexpr (!RES || in_fp32(IN)) return nullptr;
     else return plane_pass_kernel<RB, RES, kOutGrad, IN>;
   }
-  static constexpr PKernel planes() {  // strided lines, FP32 lines of 192: no chain
-    if constexpr (IN == kInStrided || (IN == kInF32 && !RES)) return nullptr;
+  // strided lines, FP32 lines of 192: no chain; a square pass's parts: a last pass
+  static constexpr PKernel planes() {
+    if constexpr (IN == kInStrided || IN == kInPoints || (IN == kInF32 && !RES)) return nullptr;
     else return plane_pass_kernel<RB, RES, kOutPlanes, IN>;
   }
   static constexpr PKernel fn[kPOuts] = {

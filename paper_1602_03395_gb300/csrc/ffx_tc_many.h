@@ -78,10 +78,10 @@ bool many_bf16_line_map(const float2* base, int N, int64_t lines, void* map);
 // points: the head plane at `head` (16-byte aligned), the tail plane `plane`
 // pairs after it (4 * plane a multiple of 16).
 bool many_bf16_plane_map(const uint32_t* head, int N, int64_t lines, int64_t plane, void* map);
-// The grid of launch_bf16_split for n points.
-int bf16_split_grid(int64_t n, int sms);
-// A backward chain's split (launch_bf16_split_grad's kernel) as a graph node:
+// A backward chain's split of 2 g psi into planes, as a graph node:
 // kernel(field float4*, grad float2*, hi uint2*, lo uint2*, n2, m2, shared, unsplit).
 const void* bf16_split_grad_func();
+// The grid of that split for n points.
+int bf16_split_grid(int64_t n, int sms);
 
 }  // namespace ffx

@@ -285,7 +285,8 @@ class Plan:
     def launches_per_call(self, backward: bool = False, batch: int = 1) -> int:
         """Passes a call makes (one launch for a fused call), plus the input
         split of a BF16 chain.  A per-axis BF16 pass over contiguous FP32
-        lines adds its own split launch; launch_count() counts exactly."""
+        lines may add its own split launch, an ensemble sum in groups of
+        realizations one or two more; launch_count() counts exactly."""
         n = len(self.dims)
         # a BF16 chain adds the split of its input, unless its first pass takes
         # the FP32 input itself; one launch may cover its last two axes (the
