@@ -297,7 +297,8 @@ int ffx_expand_host(ffx_plan_t plan, const void* psi0_host, int64_t batch, float
 /*
  * ffx_expand_field -- the complex field Psibar itself, [batch][M...] complex64.
  * out_field may equal psi0 (in place); otherwise the two must not overlap.
- * Needs no workspace.  The phase of Psibar is that of the magnified lattice,
+ * Uses the plan's workspace as ffx_expand does (passes that can run in place need
+ * none).  The phase of Psibar is that of the magnified lattice,
  * which Sec. 5.4 warns is not fit for further evolution; its density is exact.
  */
 int ffx_expand_field(ffx_plan_t plan, const void* psi0, int64_t batch, void* out_field,
@@ -313,7 +314,7 @@ int ffx_expand_field(ffx_plan_t plan, const void* psi0, int64_t batch, void* out
  *                i dL/dIm(psi0) (PyTorch's convention for complex inputs).
  *                T^H is the adjoint of the per-axis maps, applied in reverse
  *                axis order; T psi0 is recomputed, not stored.
- *  Uses the plan's workspace (batch * M complex64).
+ *  Uses the plan's workspace (up to two fields of batch * M complex64).
  */
 int ffx_expand_backward(ffx_plan_t plan, const void* psi0, const float* grad_density,
                         int64_t batch, void* grad_psi0, void* stream);
@@ -376,7 +377,8 @@ int ffx_supported_length(int64_t n);
  *                (+=) with FFX_ACCUMULATE (summed over the batch).  Entry =
  *                lam_axis * spacing_axis * sum over the axis of |Psibar|^2
  *                (the magnified lattice's spacing along the axis, eq. wbx).
- *  The map runs with the integrated axis as the last pass.  Small lattices
+ *  The map runs with the integrated axis as the last pass, or, as a BF16 chain
+ *  (ffx_plan_bf16_chain), in the plan's own order.  Small lattices
  *  that fuse (ffx_plan_fused) sum inside the fused launch; otherwise the
  *  densities go to plan workspace and one more launch sums them.  Sums run in
  *  a fixed order (deterministic).  Not for many-instance plans

@@ -772,8 +772,8 @@ bool bf16_adjoint_ok(const ffx_plan_s* p) {
 // (plane_square_kernel): 64 points each, the first axis one whose pass keeps T
 // resident, or none (2-D lattices; their ensemble sums stay with the passes).
 // 44 bytes a point of HBM become 28 on 3-D lattices (density, 64 realizations
-// of 64^3: 142.5 us as three passes, 101.9 us), 28 become 12 on 2-D ones (4096
-// images: 78.9 and 58.6 us).
+// of 64^3: 142.5 us as three passes, 95.6 us), 28 become 12 on 2-D ones (4096
+// images: 78.9 and 52.0 us).
 bool chain_square(const ffx_plan_s* p) {
   const int d = p->ndim;
   if (d < 2 || p->axis[d - 1].N != 64 || p->axis[d - 2].N != 64 || p->order[0] != d - 1 || p->order[1] != d - 2)
@@ -861,8 +861,8 @@ int chain_bf16(ffx_plan_s* p, const float2* in, int64_t batch, float2* out_c, fl
 // the field itself, from which the adjoint half starts: calls that fill the
 // chip (the chain's input is not split apart either) and a last pass whose
 // kernel does so.  Its epilogue then reads 4 bytes a point more; the separate
-// split reads and writes 20 (backward calls: 256^3 499 -> 461 us, 64
-// realizations of 64^3 336 -> 290 us with the square pass, 20 of 96x64x96 261 ->
+// split reads and writes 20 (backward calls: 256^3 499 -> 444 us, 64
+// realizations of 64^3 336 -> 277 us with the square pass, 20 of 96x64x96 261 ->
 // 251 us).
 bool chain_grad(const ffx_plan_s* p, int64_t batch) {
   const Axis& ax = p->axis[p->order[p->ndim - 1]];
@@ -1985,7 +1985,7 @@ int ffx_expand_column(ffx_plan_t p, const void* psi0, int64_t batch, int axis, f
   }
   // (the sum takes whole densities, so the passes may run in any order: that of
   // the BF16 chain where the call can take one.  128^3 x 4: 158 us with strided
-  // FP32 passes ahead of the integrated axis, 106 us as a chain.)
+  // FP32 passes ahead of the integrated axis, 96 us as a chain.)
   const int* passes = bf16_chain_ok(p, batch, psi0, nullptr, rho) ? p->order : axes;
   if ((rc = forward_density(p, passes, (const float2*)psi0, batch, rho, s))) return rc;
   int64_t outer, inner;

@@ -816,12 +816,12 @@ __global__ void __launch_bounds__(in_fp32(IN) ? PTHREADS_F32 : PTHREADS, 1)
 //    reads with its lines' points oinner apart (kInPoints).
 // Order of the products: step 1 of item i + 1, then step 2 of item i; of the
 // epilogue: E1 of item i, then E2 of item i - 1: the products of one step hide
-// the other step's epilogue.  What bounds it is the epilogue warps' chain of both
-// (8500 clocks an item, on a shared-memory port that also serves 448 KB of
-// operands and 256 KB of copies, splits and operand stores: 5600 clocks) against
-// 3072 of products at full rate.  2^24 points: 74 us, 3.6 TB/s of its 16 bytes a
-// point; as two passes 98 us.  (Sixteen epilogue warps, eight a step, with 80
-// registers a thread: 82 us.)
+// the other step's epilogue.  What bounds it is the epilogue warps' chain of both,
+// on a shared-memory port that also serves 448 KB of operands and 256 KB of
+// copies, splits and operand stores an item (5600 clocks, against 3072 of products
+// at full rate).  2^24 points: 67 us, 4.0 TB/s of its 16 bytes a point; as two
+// passes 98 us.  (Sixteen epilogue warps, eight a step, with 80 registers a
+// thread, took 84.6 us where eight took 76.5.)
 constexpr int SST = 3;  // stages
 constexpr int SA2 = 4 * 2 * 64 * 128;  // the second operand: 4 parts x 2 squares x 64 rows
 constexpr int ssmem() { return 4 * ptchunk(64) + SA2 + SST * PX + 1024; }
