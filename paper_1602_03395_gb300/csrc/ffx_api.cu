@@ -327,26 +327,26 @@ int64_t max_sum_groups(const ffx_plan_s* p, int64_t batch) {
 }
 
 // ws[5] for an ensemble sum over `batch` realizations.  The number of groups
-// does not grow with the batch (1-D lines of 2048 points at lam = 20: 518 groups
+// does not grow with the batch (1-D lines of 2048 points at lam = 20: 512 groups
 // of 1024 realizations, 608 of 608), so the buffer holds the most groups that any
 // batch up to this one, rounded up to a power of two, can take: a smaller batch
 // finds it large enough.  A buffer that a larger batch outgrows lives on with the
 // plan, because a graph captured with it still writes it; the powers of two keep
-// the sum of all below twice the largest.  False where there is none and none can
-// be had (no memory, or the stream is being captured): the sum then runs in one
-// group, which needs no partial densities.
+// the sum of all below twice the largest.  False where it cannot be had (no memory,
+// or the stream is being captured) and the `groups` of this call do not fit what
+// there is: the sum then runs in one group, which needs no partial densities.
 size_t sum_bytes(const ffx_plan_s* p, int64_t batch) {
   int64_t most = 1;
   while (most < batch) most *= 2;
   return (size_t)max_sum_groups(p, most) * (size_t)p->M * sizeof(float);
 }
-bool ensure_sum(ffx_plan_s* p, int64_t batch, cudaStream_t stream) {
+bool ensure_sum(ffx_plan_s* p, int64_t batch, int64_t groups, cudaStream_t stream) {
   const size_t need = sum_bytes(p, batch);
   if (need <= p->ws_bytes[kWsSum]) return true;
   void* grown = nullptr;
   if (capturing(stream) || cudaMalloc(&grown, need) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return (size_t)groups * (size_t)p->M * sizeof(float) <= p->ws_bytes[kWsSum];
   }
   if (p->ws[kWsSum]) {
     p->retired[p->n_retired++] = p->ws[kWsSum];
@@ -689,7 +689,7 @@ int run_axis(ffx_plan_s* p, int j, bool adjoint, const float2* in, const float* 
   SumPlan sum = {1, false};
   if (acc && batch > 1) {
     sum = plan_sum(p, ax, cform, io != nullptr, in, out_d, lines, inner, batch);
-    if (sum.partial() && !ensure_sum(p, batch, stream)) sum = {1, false};
+    if (sum.partial() && !ensure_sum(p, batch, sum.groups, stream)) sum = {1, false};
   }
   const int64_t groups = sum.groups;
   const bool tm32 = sum.tm32;

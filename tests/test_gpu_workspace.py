@@ -138,3 +138,15 @@ def test_workspace_bytes(ffx, dims, lam, form, accumulate, batches):
             told = plan.workspace_bytes(batch)
             ffx.ffx_expand(plan, x[:batch])
             assert plan.workspace_bytes(0) == told == plan.workspace_bytes(batch)
+
+
+# a capture at a batch above those called before, whose groups fit what is there
+def test_captured_sum_uses_the_groups_that_fit(ffx):
+    dims, batch = (2048,), 700
+    x = fields(dims, batch)
+    with ffx.Plan(dims, (0.2,), 4.0, (20,), accumulate=True) as plan:
+        ffx.ffx_expand(plan, x[:512])
+        out = torch.zeros(dims, device="cuda")
+        graph = capture(lambda: ffx.ffx_expand(plan, x, out))
+        graph.replay()
+        assert torch.equal(out, ffx.ffx_expand(plan, x))
